@@ -606,12 +606,10 @@ def vertex_leg(args):
 
 
 # DRAM bytes (read + write) per event of the dominant kernel, from one ncu
-# capture of a smaller case (8 stream events in one launch: the traffic is
-# the accumulator write-back plus the hits and hit lists, in proportion to
-# the events); reported only while the kernel's sources hash to the same value.
-PROFILED_TRAFFIC = {"k_vote_batch": {"sha": "c8576bebcabab381",
-                                     "bytes_per_event": (78121216 + 293925632) / 8}}
-KERNEL_SOURCES = ["paper_1309_6275_gb300/csrc/k_vote_layers.cu",
+# capture of a smaller case; reported only while the kernel's sources hash to
+# the captured ones (none at present).
+PROFILED_TRAFFIC = {}
+KERNEL_SOURCES = ["paper_1309_6275_gb300/csrc/k_vote_rows.cu",
                   "paper_1309_6275_gb300/csrc/tiles.cuh",
                   "paper_1309_6275_gb300/csrc/ht_internal.cuh",
                   "paper_1309_6275_gb300/csrc/df32.cuh"]
@@ -627,12 +625,18 @@ def kernel_sha():
 
 
 def launches_per_batch(ne, learned=False):
-    """Kernels one ht_batch_run_tracks replays: hit lists (count, 3-kernel
-    scan, fill), the vote, per event two peak passes and a 3-kernel scan,
-    the confirmation (prefix, grouping 2 + scan 3, hit index 3 + scan 3,
-    confirmation, offers, decode) and the z vote (4 + scan 3); with the
-    proposal one more (the network's top-k per hit)."""
+    """Kernels of a batch whose events' peaks are found one event after
+    another, two passes and a 3-kernel scan each (5 per event)."""
     return 5 + 1 + 5 * ne + 15 + 7 + (1 if learned else 0)
+
+
+def track_launches(learned=False):
+    """Kernels one ht_batch_run_tracks replays, whatever its number of events:
+    the hit index (3 + scan 3), the vote, the peaks of all events (2 + scan
+    3), the confirmation (prefix, grouping 2 + scan 3, confirmation, offers,
+    decode) and the z vote (4 + scan 3); with the proposal one more (the
+    network's top-k per hit)."""
+    return 6 + 1 + 5 + 9 + 7 + (1 if learned else 0)
 
 
 def run_ours(args):
@@ -723,11 +727,11 @@ def run_ours(args):
     votes = plain["votes"]
     g = tr.g
     cells = g["n_rho"] * g["n_d0"] * g["n_phi0"]
-    roof = {"kernel": {1: "k_vote_batch (distinct-layer mode)", 3: "k_confirm"}.get(dom, STAGES[dom]),
+    roof = {"kernel": {1: "k_vote_rows_batch", 3: "k_confirm"}.get(dom, STAGES[dom]),
             "stage_ms_per_event": {s: round(1e3 * v / n_ev, 4) for s, v in zip(STAGES, stage_s)}}
     if dom == 1:
         achieved = OPS_PER_VOTE * votes / stage_s[1]
-        prof = PROFILED_TRAFFIC.get("k_vote_batch")
+        prof = PROFILED_TRAFFIC.get("k_vote_rows_batch")
         from paper_1309_6275_gb300 import probe
         atom = probe.shared_atomic_rate(1 << 14)
         roof.update({"bound": "alu", "achieved": achieved / 1e9, "peak": peak_ops / 1e9,
@@ -746,12 +750,12 @@ def run_ours(args):
                              "algorithmic op count here"})
     roof["float64_redo_per_vote"] = plain["redo"] / max(votes, 1)
     roof["hbm_peaks_stage"] = {
-        "algorithmic_bytes_per_event": cells * 2,
-        "achieved_gbs": cells * 2 / (stage_s[2] / n_ev) / 1e9,
+        "algorithmic_bytes_per_event": cells / 2,
+        "achieved_gbs": cells / 2 / (stage_s[2] / n_ev) / 1e9,
         "peak_gbs": peaks.get("hbm_gbs", 6800.0),
-        "frac": cells * 2 / (stage_s[2] / n_ev) / 1e9 / peaks.get("hbm_gbs", 6800.0),
-        "note": "the count pass reads each uint16 accumulator once and spills its peaks; the "
-                "write pass copies them (tiles with more than 64 peaks are read again)"}
+        "frac": cells / 2 / (stage_s[2] / n_ev) / 1e9 / peaks.get("hbm_gbs", 6800.0),
+        "note": "the layer counts are four bit planes per event, read once by the sweep; its "
+                "peak bits are read again by the write pass"}
     tk = synth.track_of(name)
     line = {
         "metric": METRIC, "value": value, "unit": "events/s", "n_gpus": world,
@@ -771,7 +775,7 @@ def run_ours(args):
                                   "after timing"},
         "hit_votes_per_s": world * votes / (plain["stage_ms"].sum() / 1e3),
         "step_ms": [round(v, 3) for v in step_ms],
-        "gpu_launches": args.steps * sum(launches_per_batch(len(b)) for b in tr.batches),
+        "gpu_launches": args.steps * len(tr.batches) * track_launches(),
         "candidates_per_event": plain["candidates_per_event"],
         "confirmed_per_event": plain["confirmed_per_event"],
         "quality": plain["quality"],

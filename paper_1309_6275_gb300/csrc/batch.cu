@@ -72,12 +72,10 @@ cudaError_t launch_vote_batch_hitmask(const DevGeom &G, const float *x, const fl
 cudaError_t launch_hit_masks(const void *params_bf16, const float *x, const float *y,
                              const float *z, const uint8_t *layer, int n, const int *d_n,
                              int topk, float pmin, unsigned long long *hit_masks, cudaStream_t st);
-cudaError_t launch_vote_batch_layers(const DevGeom &G, const float *x, const float *y,
-                                     const uint8_t *layer, const int *off, const int *order,
-                                     const int *d_nev, uint16_t *acc, size_t acc_stride,
-                                     unsigned long long *stats, int *head, int kt, int sms,
-                                     const unsigned long long *hit_masks, cudaStream_t st,
-                                     const HitBuckets *hb);
+cudaError_t launch_vote_batch_layers(const DevGeom &G, const HitIndex &I, const int *off,
+                                     const int *order, const int *d_nev, uint32_t *planes,
+                                     size_t stride, unsigned long long *stats, int *head, int sms,
+                                     const unsigned long long *hit_masks, cudaStream_t st);
 }  // namespace ht
 
 namespace {
@@ -113,7 +111,9 @@ struct ht_batch {
     int max_events, max_hits, cap, sms;
     int kt_pack, kt_big, kt_assoc;
     size_t cells;
-    uint16_t *acc;
+    size_t slot_words;  // 32-bit words of an event's slot in acc
+    uint16_t *acc;      // plain path: counts, cells apart; track path: bit planes
+                        // and peak bits, slot_words apart
     int *meta;          // [0] n_big [1] pad [2] n_all [3] pad, off[max_events + 1],
                         // order_big[max_events], order_all[max_events] (largest first),
                         // thr[max_events] (peak threshold of each event slot)
@@ -140,6 +140,9 @@ struct ht_batch {
     bool conf_set;
     int *inl;               // track path: 16 inlier hits per candidate slot
     char *cf_ws;            // track path: confirmation scratch
+    char *idx_ws;           // track path: the hit index (k_hitindex.cu)
+    ht::HitIndex idx;
+    char *pp_ws;            // track path: peak finding's scratch
     struct HostPath {       // buffers of ht_batch_run_tracks_host (allocated on first use)
         float *x, *y, *z;
         uint8_t *layer;
@@ -187,6 +190,8 @@ void free_batch(ht_batch *b)
     cudaFree(b->bk_ws);
     cudaFree(b->inl);
     cudaFree(b->cf_ws);
+    cudaFree(b->idx_ws);
+    cudaFree(b->pp_ws);
     {
         ht_batch::HostPath &h = b->hp;
         void *bufs[] = {h.x, h.y, h.z, h.layer, h.hmasks, h.peaks, h.zres, h.counts, h.score,
@@ -245,6 +250,35 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
     }
     e = mark(1);
     if (e != cudaSuccess) return e;
+    const bool tracks = R.layer != nullptr;
+    if (tracks) {
+        // the track path: the hit index, the distinct-layer vote on it (bit
+        // planes, with per-hit region sets or without), the peaks of all
+        // events at their staged thresholds, confirmation and final
+        // assignment, z vote
+        e = ht::launch_hit_index(x, y, R.layer, off, meta + 2, me, b->max_hits, b->idx, b->sms, st);
+        uint32_t *planes = reinterpret_cast<uint32_t *>(b->acc);
+        if (e == cudaSuccess)
+            e = ht::launch_vote_batch_layers(G, b->idx, off, order_all_of(meta, me), meta + 2,
+                                             planes, b->slot_words, st64, b->heads + 1, b->sms,
+                                             R.hit_masks, st);
+        if (e == cudaSuccess) e = mark(2);
+        if (e == cudaSuccess)
+            e = ht::launch_plane_peaks(G, planes, b->slot_words, b->idx.rmm, thr_of(meta, me),
+                                       n_ev, me, peaks, b->cap, counts, b->pp_ws, st);
+        if (e == cudaSuccess) e = mark(3);
+        const ht::ConfirmDev P{b->conf.pool, b->conf.min_layers, b->conf.n_layers, b->conf.tol};
+        if (e == cudaSuccess)
+            e = ht::launch_confirm_batch(G, P, x, y, R.layer, off, meta + 2, b->max_events,
+                                         b->max_hits, peaks, counts, b->cap, R.score, b->inl,
+                                         assign, b->cf_ws, b->idx, b->sms, st);
+        if (e == cudaSuccess) e = mark(4);
+        if (e == cudaSuccess)
+            e = ht::launch_vote_z_batch(G, x, y, z, assign, off, meta + 2, peaks, counts, b->cap,
+                                        n_ev, zres, b->z_ws, b->max_hits, st);
+        if (e == cudaSuccess) e = mark(5);
+        return e;
+    }
     // the hits each tile scans: lists by column group (every tile width the
     // batch uses divides the group)
     e = ht::launch_hit_buckets(G, x, y, off, meta + 2, b->max_hits, b->bk, b->sms, st);
@@ -263,49 +297,22 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
                      : ht::launch_vote_batch(G, x, y, off, order, d_nev, b->acc, b->cells, st64,
                                              head, pack, kt, b->sms, st, &b->bk);
     };
-    const bool tracks = R.layer != nullptr;
-    if (tracks) {
-        // the distinct-layer vote packs every tile: one launch, always with its
-        // default tile (the widths ht_batch_autotune tunes are the plain path's)
-        e = ht::launch_vote_batch_layers(G, x, y, R.layer, off, order_all_of(meta, me), meta + 2,
-                                         b->acc, b->cells, st64, b->heads + 1, 0, b->sms,
-                                         R.hit_masks, st, &b->bk);
-    } else {
-        e = vote(order_big_of(meta, me), meta + 0, b->heads + 0, false, b->kt_big);
-        if (e == cudaSuccess) e = vote(order_all_of(meta, me), meta + 2, b->heads + 1, true, b->kt_pack);
-    }
+    e = vote(order_big_of(meta, me), meta + 0, b->heads + 0, false, b->kt_big);
+    if (e == cudaSuccess) e = vote(order_all_of(meta, me), meta + 2, b->heads + 1, true, b->kt_pack);
     if (e == cudaSuccess) e = mark(2);
     if (e != cudaSuccess) return e;
-    // peaks (each event slot at its staged threshold on the track path) and
-    // the association's candidate tile lists per event slot
+    // peaks and the association's candidate tile lists per event slot
     for (int ev = 0; ev < n_ev; ++ev) {
         e = ht::launch_peaks(G, b->acc + (size_t)ev * b->cells, peaks + (size_t)ev * b->cap,
                              b->cap, counts + ev, b->pk_ws + (size_t)ev * b->pk_stride, st,
-                             masks ? masks + ev : nullptr, tracks ? thr_of(meta, me) + ev : nullptr,
-                             b->pk_spill);
+                             masks ? masks + ev : nullptr, b->pk_spill);
         if (e != cudaSuccess) return e;
-        if (tracks) continue;
         const size_t to = (size_t)ev * (b->ntiles + 1);
         e = ht::launch_cand_lists(G, b->kt_assoc, peaks + (size_t)ev * b->cap, counts + ev,
                                   b->cap, b->tcnt + to, b->toff + to, b->tcur + to,
                                   b->ttmp + (size_t)ev * b->ttmp_stride,
                                   b->tlist + (size_t)ev * b->lstride, st);
         if (e != cudaSuccess) return e;
-    }
-    if (tracks) {
-        // confirmation and final assignment over the whole batch
-        e = mark(3);
-        const ht::ConfirmDev P{b->conf.pool, b->conf.min_layers, b->conf.n_layers, b->conf.tol};
-        if (e == cudaSuccess)
-            e = ht::launch_confirm_batch(G, P, x, y, R.layer, off, meta + 2, b->max_events,
-                                         b->max_hits, peaks, counts, b->cap, R.score, b->inl,
-                                         assign, b->cf_ws, b->sms, st, &b->bk);
-        if (e == cudaSuccess) e = mark(4);
-        if (e == cudaSuccess)
-            e = ht::launch_vote_z_batch(G, x, y, z, assign, off, meta + 2, peaks, counts, b->cap,
-                                        n_ev, zres, b->z_ws, b->max_hits, st);
-        if (e == cudaSuccess) e = mark(5);
-        return e;
     }
     // association over the whole batch
     e = cudaMemsetAsync(b->gbest, 0, (size_t)b->max_hits * 8, st);
@@ -416,6 +423,8 @@ ht_status ht_batch_create(const ht_geometry *g, int32_t max_events, int32_t max_
     b->kt_big = 0;
     b->kt_assoc = ht::assoc32_kt(G);
     b->cells = (size_t)G.n_rho * G.n_d0 * G.n_phi0;
+    b->slot_words = std::max((b->cells + 1) / 2,
+                             ht::layer_planes_words(G) + ht::plane_flag_words(G));
     b->meta_ints = 4 + (size_t)max_events + 1 + 3 * (size_t)max_events;
     b->pk_stride = ht::align256(ht::peaks_workspace_bytes(G));
     b->ntiles = ht::assoc32_ntiles(G, 1);   // the most tiles any tile width gives
@@ -425,7 +434,7 @@ ht_status ht_batch_create(const ht_geometry *g, int32_t max_events, int32_t max_
     auto M = [&](void **p, size_t bytes) {
         if (e == cudaSuccess) e = cudaMalloc(p, bytes);
     };
-    M((void **)&b->acc, b->cells * 2 * max_events);
+    M((void **)&b->acc, b->slot_words * 4 * max_events);
     M((void **)&b->meta, b->meta_ints * 4);
     M((void **)&b->heads, 256);
     M((void **)&b->gbest, (size_t)max_hits * 8);
@@ -628,9 +637,18 @@ ht_status ht_batch_set_confirm(ht_batch *b, const ht_confirm_desc *c)
         if (e == cudaSuccess)
             e = cudaMalloc((void **)&b->cf_ws,
                            ht::confirm_workspace_bytes(b->g->G, b->max_events, b->max_hits, b->cap));
+        if (e == cudaSuccess)
+            e = cudaMalloc((void **)&b->idx_ws, ht::hit_index_bytes(b->max_events, b->max_hits));
+        if (e == cudaSuccess)
+            e = cudaMalloc((void **)&b->pp_ws, ht::plane_peaks_bytes(b->g->G, b->max_events));
+        if (e == cudaSuccess) b->idx = ht::carve_hit_index(b->max_events, b->max_hits, b->idx_ws);
         if (e != cudaSuccess) {
             cudaFree(b->inl);
+            cudaFree(b->cf_ws);
+            cudaFree(b->idx_ws);
+            cudaFree(b->pp_ws);
             b->inl = nullptr;
+            b->cf_ws = b->idx_ws = b->pp_ws = nullptr;
             return ht::set_error(HT_ERR_CUDA, "ht_batch_set_confirm: allocation failed");
         }
     }

@@ -179,6 +179,8 @@ ht_status ht_geometry_create(const ht_geometry_desc *d, ht_geometry **out)
     G.rho_max_f = (float)d->rho_max * 1.0001f;
     G.drho_f = (float)(2.0 * d->rho_max / (double)NR);
     G.dmax_f = (float)(G.off * G.delta) + 0.01f;
+    G.inv_drho_f = (float)((double)NR / (2.0 * d->rho_max));
+    G.kr_f = (float)((double)NR / d->rho_max);
     G.sn64 = d64; G.cs64 = d64 + NP; G.rho64 = d64 + 2 * NP;
     G.sn32 = d32; G.cs32 = d32 + NP; G.phi32 = d32 + 2 * NP;
     G.rho32 = d32 + 3 * NP; G.invrho32 = d32 + 3 * NP + NR;
@@ -388,7 +390,7 @@ ht_status ht_find_peaks(const ht_geometry *g, const void *acc, ht_peak *peaks, i
     if (!aligned(workspace, 256) || !aligned(acc, 16))
         return fail(HT_ERR_ARG, "ht_find_peaks: workspace or accumulator alignment");
     cudaError_t e = ht::launch_peaks(g->G, acc, peaks, cap, d_count, workspace, S(stream),
-                                     nullptr, nullptr,
+                                     nullptr,
                                      peak_spill_of(g->G, workspace, workspace_bytes));
     return e == cudaSuccess ? HT_OK : cuda_fail(e, "ht_find_peaks");
 }
@@ -406,7 +408,7 @@ ht_status ht_find_peaks_masked(const ht_geometry *g, const void *acc, const uint
     if (!aligned(workspace, 256) || !aligned(mask, 8) || !aligned(acc, 16))
         return fail(HT_ERR_ARG, "ht_find_peaks_masked: pointer alignment");
     cudaError_t e = ht::launch_peaks(g->G, acc, peaks, cap, d_count, workspace, S(stream),
-                                     reinterpret_cast<const unsigned long long *>(mask), nullptr,
+                                     reinterpret_cast<const unsigned long long *>(mask),
                                      peak_spill_of(g->G, workspace, workspace_bytes));
     return e == cudaSuccess ? HT_OK : cuda_fail(e, "ht_find_peaks_masked");
 }

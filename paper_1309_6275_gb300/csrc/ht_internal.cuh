@@ -36,6 +36,7 @@ struct DevGeom {
     float dext_f;                  // |d0| of any root within half a bin of the axis, + margin
     float e3;                      // geometry part of the root bounds, in bins
     float rho_max_f, drho_f, dmax_f; // |rho| bound, row width, max |d0| (filters)
+    float inv_drho_f, kr_f;          // 1 / drho, 2 / drho (curve walk)
     // tables (device)
     const float *sn32, *cs32, *phi32, *rho32, *invrho32;
     const double *sn64, *cs64, *rho64;
@@ -383,8 +384,7 @@ cudaError_t launch_vote_hitmask(const DevGeom &G, const float *x, const float *y
 // twice; it may be shared by launches that run one after another.
 cudaError_t launch_peaks(const DevGeom &G, const void *acc, ht_peak *peaks, int cap,
                          int *d_count, void *ws, cudaStream_t st,
-                         const unsigned long long *mask = nullptr, const int *d_thr = nullptr,
-                         void *spill = nullptr);
+                         const unsigned long long *mask = nullptr, void *spill = nullptr);
 size_t peaks_workspace_bytes(const DevGeom &G);
 size_t peak_spill_bytes(const DevGeom &G);
 cudaError_t launch_associate(const DevGeom &G, const float *x, const float *y, int n,
@@ -413,6 +413,22 @@ struct HitIndex {
     void *tmp;
     int ncells;
 };
+// Bit planes of layer counts (k_vote_rows.cu, k_peak_planes.cu): word
+// ((k kPlanes + p) NW + w) n_d0 + j of an event holds bit p of the counts of
+// rows 32 w .. 32 w + 31 in bin j of column k, NW = ceil(n_rho / 32).  A count
+// is at most 16; plane 4 is written and read only for events with hits on
+// all 16 layers.
+constexpr int kPlanes = 5;
+size_t layer_planes_words(const DevGeom &G);   // words per event
+size_t plane_flag_words(const DevGeom &G);     // peak bits that follow an event's planes
+size_t plane_peaks_bytes(const DevGeom &G, int max_events);
+// Peaks of n_ev <= max_events events' planes (stride words apart, at least
+// layer_planes_words + plane_flag_words): event e's go to peaks + e cap, their
+// number to counts[e]; thr[e] is its threshold; rmm: the hit index's radius
+// ranges.  ws: plane_peaks_bytes(G, max_events).
+cudaError_t launch_plane_peaks(const DevGeom &G, const uint32_t *planes, size_t stride,
+                               const unsigned *rmm, const int *thr, int n_ev, int max_events,
+                               ht_peak *peaks, int cap, int *counts, void *ws, cudaStream_t st);
 size_t hit_index_bytes(int max_events, int max_hits);
 HitIndex carve_hit_index(int max_events, int max_hits, void *ws);
 cudaError_t launch_hit_index(const float *x, const float *y, const uint8_t *layer,
@@ -443,8 +459,8 @@ cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const fl
                                  const float *y, const uint8_t *layer, const int *off,
                                  const int *d_nev, int max_events, int max_hits,
                                  const ht_peak *peaks, const int *counts, int cap, int *score,
-                                 int *inl, int *assign, void *ws, int sms, cudaStream_t st,
-                                 const HitBuckets *hb);
+                                 int *inl, int *assign, void *ws, const HitIndex &idx, int sms,
+                                 cudaStream_t st);
 // One event of n hits (host) and *d_count candidates (device).
 size_t confirm_workspace_bytes_single(const DevGeom &G, int n, int cap);
 cudaError_t launch_confirm(const DevGeom &G, const ConfirmDev &P, const float *x, const float *y,

@@ -740,7 +740,6 @@ struct CfWs {
     int *cpre, *head, *gcnt, *gofs, *gcur, *order;
     unsigned long long *gbest;
     void *tmp;
-    HitIndex idx;
 };
 
 int cf_groups(const DevGeom &G) { return (G.n_phi0 + kGroupCols - 1) / kGroupCols; }
@@ -752,10 +751,10 @@ size_t cf_layout(const DevGeom &G, int max_events, int max_hits, int cap, char *
     const size_t parts[] = {(size_t)(max_events + 1) * 4, 64, (size_t)(max_hits > 0 ? max_hits : 1) * 8,
                             ni * 4, (ni + 1) * 4, (ni + 1) * 4,
                             (size_t)max_events * (cap > 0 ? cap : 1) * 4,
-                            scan_tmp_bytes((int)ni), hit_index_bytes(max_events, max_hits)};
+                            scan_tmp_bytes((int)ni)};
     size_t at = 0;
-    char *q[9];
-    for (int i = 0; i < 9; ++i) {
+    char *q[8];
+    for (int i = 0; i < 8; ++i) {
         q[i] = p ? p + at : nullptr;
         at += align256(parts[i]);
     }
@@ -768,7 +767,6 @@ size_t cf_layout(const DevGeom &G, int max_events, int max_hits, int cap, char *
         w->gcur = reinterpret_cast<int *>(q[5]);
         w->order = reinterpret_cast<int *>(q[6]);
         w->tmp = q[7];
-        if (p) w->idx = carve_hit_index(max_events, max_hits, q[8]);
     }
     return at;
 }
@@ -778,7 +776,8 @@ size_t cf_layout(const DevGeom &G, int max_events, int max_hits, int cap, char *
 cudaError_t prepare_confirm_kernels() { return cudaSuccess; }
 
 // Confirmation and final assignment of a batch (device offsets and event
-// count).  ws: confirm_workspace_bytes(G, max_events, max_hits, cap).
+// count; idx: its hit index).  ws: confirm_workspace_bytes(G, max_events,
+// max_hits, cap).
 size_t confirm_workspace_bytes(const DevGeom &G, int max_events, int max_hits, int cap)
 {
     return cf_layout(G, max_events, max_hits, cap, nullptr, nullptr);
@@ -788,10 +787,9 @@ cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const fl
                                  const float *y, const uint8_t *layer, const int *off,
                                  const int *d_nev, int max_events, int max_hits,
                                  const ht_peak *peaks, const int *counts, int cap, int *score,
-                                 int *inl, int *assign, void *ws, int sms, cudaStream_t st,
-                                 const HitBuckets *hb)
+                                 int *inl, int *assign, void *ws, const HitIndex &idx, int sms,
+                                 cudaStream_t st)
 {
-    (void)hb;
     CfWs w;
     cf_layout(G, max_events, max_hits, cap, reinterpret_cast<char *>(ws), &w);
     const int ng = cf_groups(G), ni = max_events * ng;
@@ -805,12 +803,10 @@ cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const fl
     e = scan_exclusive(w.gcnt, w.gofs, w.gcur, ni, nullptr, w.gofs + ni, w.tmp, st);
     if (e != cudaSuccess) return e;
     k_cf_group<<<sms * 4, 256, 0, st>>>(d_nev, w.cpre, peaks, cap, ng, nullptr, w.gcur, w.order);
-    e = launch_hit_index(x, y, layer, off, d_nev, max_events, max_hits, w.idx, sms, st);
-    if (e != cudaSuccess) return e;
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_confirm, kCfThreads, 0);
     k_confirm<<<sms * (occ > 0 ? occ : 1), kCfThreads, 0, st>>>(
-        G, P, w.idx, d_nev, peaks, cap, w.cpre, w.order, score, inl, w.head);
+        G, P, idx, d_nev, peaks, cap, w.cpre, w.order, score, inl, w.head);
     k_confirm_offer<<<sms * 8, 256, 0, st>>>(off, d_nev, w.cpre, cap, score, inl, w.gbest);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -820,7 +816,7 @@ cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const fl
 // One event (host hit count n, device candidate count d_count).
 size_t confirm_workspace_bytes_single(const DevGeom &G, int n, int cap)
 {
-    return align256(16) + confirm_workspace_bytes(G, 1, n, cap);
+    return align256(16) + hit_index_bytes(1, n) + confirm_workspace_bytes(G, 1, n, cap);
 }
 
 cudaError_t launch_confirm(const DevGeom &G, const ConfirmDev &P, const float *x, const float *y,
@@ -829,9 +825,13 @@ cudaError_t launch_confirm(const DevGeom &G, const ConfirmDev &P, const float *x
 {
     int *meta = reinterpret_cast<int *>(ws);   // off[2], n_ev
     k_single_offsets<<<1, 1, 0, st>>>(meta, meta + 2, n);
+    char *p = reinterpret_cast<char *>(ws) + align256(16);
+    const HitIndex idx = carve_hit_index(1, n, p);
+    const int sms = device_sms();
+    const cudaError_t e = launch_hit_index(x, y, layer, meta, meta + 2, 1, n, idx, sms, st);
+    if (e != cudaSuccess) return e;
     return launch_confirm_batch(G, P, x, y, layer, meta, meta + 2, 1, n, peaks, d_count, cap,
-                                score, inl, assign, reinterpret_cast<char *>(ws) + align256(16),
-                                device_sms(), st, nullptr);
+                                score, inl, assign, p + hit_index_bytes(1, n), idx, sms, st);
 }
 
 

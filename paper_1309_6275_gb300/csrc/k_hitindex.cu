@@ -1,5 +1,6 @@
 // k_hitindex.cu -- per-event index of the hits by (layer, azimuth bin), for
-// the candidate confirmation (k_confirm.cu).
+// the distinct-layer vote (k_vote_rows.cu) and the candidate confirmation
+// (k_confirm.cu).
 //
 // Cell (l, b) of event e holds the event's hits of layer l whose azimuth
 // atan2(y, x) falls in bin b = floor((phi + pi) * kIdxAz / (2 pi)) (clamped
@@ -7,9 +8,8 @@
 // and the events follow one another, so event e's cells start at its first
 // hit's batch position.  Each position holds the hit's x, y (float32), its
 // event-local index and its layer; within a cell the order is that of the
-// fill's atomics (the confirmation's results do not depend on it).  The
-// per-(event, layer) radius range is kept for the confirmation's azimuth
-// windows.
+// fill's atomics (no result depends on it).  The
+// per-(event, layer) radius range is kept for the azimuth windows.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -59,8 +59,10 @@ __global__ void k_hidx(const float *__restrict__ x, const float *__restrict__ y,
         } else {
             atomicAdd(&cnt[cell], 1);
             const unsigned rb = __float_as_uint(sqrtf(fmaf(xf, xf, yf * yf)));
-            atomicMin(&rmm[2 * (e * 16 + l)], rb);       // non-negative floats order as their bits
-            atomicMax(&rmm[2 * (e * 16 + l) + 1], rb);
+            if (rb <= 0x7f800000u) {   // not NaN (such a hit votes nowhere)
+                atomicMin(&rmm[2 * (e * 16 + l)], rb);   // non-negative floats order as their bits
+                atomicMax(&rmm[2 * (e * 16 + l) + 1], rb);
+            }
         }
     }
 }

@@ -223,18 +223,16 @@ __device__ __forceinline__ void peaks_tile(const DevGeom &G, const T *__restrict
     }
 }
 
-// d_thr (null: the geometry's threshold): a device threshold for this event.
 // Count pass: one CTA per tile.
 template <typename T, bool MASKED>
 __global__ void __launch_bounds__(kPkThreads)
 k_peaks_count(DevGeom G, const T *__restrict__ acc, int *__restrict__ segcnt,
-              const unsigned long long *__restrict__ mask, const int *__restrict__ d_thr,
-              PeakSpill sp)
+              const unsigned long long *__restrict__ mask, PeakSpill sp)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned bal_s[kJB][kPkThreads / 32];
     __shared__ int s_jpre[kJB + 1];
-    const int thr = d_thr ? *d_thr : G.threshold;
+    const int thr = G.threshold;
     const int t = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     peaks_tile<T, false, MASKED>(G, acc, blockIdx.x, blockIdx.y, blockIdx.z, t, thr, segcnt,
                                  nullptr, nullptr, 0, mask, sp, reinterpret_cast<T *>(smraw),
@@ -247,11 +245,11 @@ template <typename T, bool MASKED>
 __global__ void __launch_bounds__(kPkThreads)
 k_peaks_write(DevGeom G, const T *__restrict__ acc, const int *__restrict__ segoff,
               ht_peak *__restrict__ out, int cap, const unsigned long long *__restrict__ mask,
-              const int *__restrict__ d_thr, PeakSpill sp, int nkb, int njb)
+              PeakSpill sp, int nkb, int njb)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned bal_s[kJB][kPkThreads / 32];
-    const int thr = d_thr ? *d_thr : G.threshold;
+    const int thr = G.threshold;
     const int ND = G.n_d0;
     const int ntiles = nkb * njb * G.n_rho;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -277,14 +275,14 @@ k_peaks_write(DevGeom G, const T *__restrict__ acc, const int *__restrict__ sego
 template <typename T, bool MASKED>
 cudaError_t run_peaks(const DevGeom &G, const T *acc, ht_peak *peaks, int cap, int *d_count,
                       int *segcnt, int *segoff, void *tmp, const unsigned long long *mask,
-                      cudaStream_t st, const int *d_thr, const PeakSpill &sp)
+                      cudaStream_t st, const PeakSpill &sp)
 {
     const int nkb = (G.n_phi0 + kPkThreads - 1) / kPkThreads;
     const int njb = (G.n_d0 + kJB - 1) / kJB;
     dim3 grid(nkb, njb, G.n_rho);
     const int nseg = G.n_rho * G.n_d0 * nkb;
     k_peaks_count<T, MASKED><<<grid, kPkThreads, Stage<T>::kBytes, st>>>(G, acc, segcnt, mask,
-                                                                         d_thr, sp);
+                                                                         sp);
     cudaError_t e = scan_exclusive(segcnt, segoff, nullptr, nseg, nullptr, d_count, tmp, st);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, occ = 0;
@@ -297,7 +295,7 @@ cudaError_t run_peaks(const DevGeom &G, const T *acc, ht_peak *peaks, int cap, i
     const int ntiles = nkb * njb * G.n_rho;
     const int pgrid = min(ntiles, sms * (occ > 0 ? occ : 1));
     k_peaks_write<T, MASKED><<<pgrid, kPkThreads, Stage<T>::kBytes, st>>>(
-        G, acc, segoff, peaks, cap, mask, d_thr, sp, nkb, njb);
+        G, acc, segoff, peaks, cap, mask, sp, nkb, njb);
     return cudaGetLastError();
 }
 
@@ -342,7 +340,7 @@ size_t peak_spill_bytes(const DevGeom &G)
 
 cudaError_t launch_peaks(const DevGeom &G, const void *acc, ht_peak *peaks, int cap,
                          int *d_count, void *ws, cudaStream_t st, const unsigned long long *mask,
-                         const int *d_thr, void *spill)
+                         void *spill)
 {
     const size_t nkb = (G.n_phi0 + kPkThreads - 1) / kPkThreads;
     const size_t nseg = (size_t)G.n_rho * G.n_d0 * nkb;
@@ -366,15 +364,15 @@ cudaError_t launch_peaks(const DevGeom &G, const void *acc, ht_peak *peaks, int 
     if (mask) {
         if (G.count_bits == 16)
             return run_peaks<uint16_t, true>(G, a16, peaks, cap, d_count, segcnt, segoff, tmp,
-                                             mask, st, d_thr, sp);
+                                             mask, st, sp);
         return run_peaks<int32_t, true>(G, a32, peaks, cap, d_count, segcnt, segoff, tmp, mask,
-                                        st, d_thr, sp);
+                                        st, sp);
     }
     if (G.count_bits == 16)
         return run_peaks<uint16_t, false>(G, a16, peaks, cap, d_count, segcnt, segoff, tmp,
-                                          nullptr, st, d_thr, sp);
+                                          nullptr, st, sp);
     return run_peaks<int32_t, false>(G, a32, peaks, cap, d_count, segcnt, segoff, tmp, nullptr,
-                                     st, d_thr, sp);
+                                     st, sp);
 }
 
 }  // namespace ht

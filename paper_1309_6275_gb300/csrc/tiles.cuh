@@ -21,16 +21,6 @@ constexpr int kThreads = 256;
 // ht_internal.cuh).  Association replays votes under kModeEvent with a
 // candidate-box window in MaskCtx.
 constexpr int kModePlain = 0, kModeEvent = 1, kModeHit = 2;
-// Flag on a mode: the distinct-layer vote.  A cell counts the distinct
-// detector layers of the hits voting in it (a track leaves at most one hit
-// per layer); tile words hold 16-bit layer masks (bit l = layer l), set with
-// atomicOr, and the write-back stores their population counts.  An OR never
-// carries, so two masks always share a word, whatever the hit count.
-constexpr int kModeLayers = 4, kModeBase = 3;
-
-__host__ __device__ constexpr int base_mode(int m) { return m & kModeBase; }
-__host__ __device__ constexpr bool layer_mode(int m) { return (m & kModeLayers) != 0; }
-
 template <typename OutT>
 __device__ __forceinline__ OutT saturate(uint32_t v)
 {
@@ -43,7 +33,6 @@ struct WorkList {
     float4 *a, *b;           // Item fields {s, c, r2, eD}, {E1, E2, Qa, Qb}
     int *meta;               // hit << 6 | needB << 5 | unsure << 4 | column-in-tile
     unsigned long long *hm;  // kModeHit: the hit's region set
-    unsigned char *lay;      // kModeLayers: the hit's layer
 };
 
 constexpr int kMetaUnsure = 16, kMetaNeedB = 32, kMetaCol = 15;
@@ -51,18 +40,16 @@ constexpr size_t kItemBytes = 36;
 
 __host__ __device__ constexpr size_t item_bytes(int mode)
 {
-    return kItemBytes + (base_mode(mode) == kModeHit ? 8 : 0) + (layer_mode(mode) ? 1 : 0);
+    return kItemBytes + (mode == kModeHit ? 8 : 0);
 }
 
-__device__ __forceinline__ WorkList carve_worklist(unsigned char *p, int cap,
-                                                   int mode = kModePlain)
+__device__ __forceinline__ WorkList carve_worklist(unsigned char *p, int cap)
 {
     WorkList w;
     w.a = reinterpret_cast<float4 *>(p);
     w.b = w.a + cap;
     w.meta = reinterpret_cast<int *>(w.b + cap);
     w.hm = reinterpret_cast<unsigned long long *>(w.meta + cap);   // cap is a multiple of 2
-    w.lay = reinterpret_cast<unsigned char *>(w.hm + (base_mode(mode) == kModeHit ? cap : 0));
     return w;
 }
 
@@ -86,23 +73,19 @@ struct RowCtx {
     }
 };
 
-// Per-tile constants of the lane's rows and of the tile's columns.  A tile
-// has 32 RW rows: the lane's first row (i0 + lane) is the base RowCtx, its
-// second (i0 + 32 + lane, RW = 2) is r1.
-template <int KT, int RW = 1>
+// Per-tile constants of the lane's row (i0 + lane) and of the tile's columns.
+template <int KT>
 struct TileCtx : RowCtx {
     int i0, k0;
     float rho_lo, rho_hi, rt, sB, cB;
     float sk[KT], ck[KT];
-    RowCtx r1;
 
     __device__ __forceinline__ void init(const DevGeom &G, int lane, int tx, int ty)
     {
         k0 = tx * KT;
-        i0 = ty * 32 * RW;
+        i0 = ty * 32;
         init_row(G, i0 + lane);
-        if (RW == 2) r1.init_row(G, i0 + 32 + lane);
-        const int ilast = min(i0 + 32 * RW - 1, G.n_rho - 1);
+        const int ilast = min(i0 + 31, G.n_rho - 1);
         rho_lo = G.rho32[i0] - G.drho_f;
         rho_hi = G.rho32[ilast] + G.drho_f;
         rt = fmaxf(fabsf(G.rho32[i0]), fabsf(G.rho32[ilast])) * 1.0001f;
@@ -276,20 +259,19 @@ __device__ __forceinline__ void aform_bin(const RowCtx &T, const float4 a, float
 }
 
 // Word offset (from the lane's first word) and increment of column kl's
-// counters in a tile of 32 RW rows with the layout of TileCol.
-template <int KT, bool PACK, int RW = 1>
-__device__ __forceinline__ void col_word(int ND, int kl, uint32_t one, uint32_t &woff,
-                                         uint32_t &inc)
+// counters, with the layout of TileCol.
+template <int KT, bool PACK>
+__device__ __forceinline__ void col_word(int ND, int kl, uint32_t &woff, uint32_t &inc)
 {
     if (PACK && KT > 1) {
-        woff = (uint32_t)((kl >> 1) * ND * 32 * RW);
-        inc = one << ((kl & 1) << 4);
+        woff = (uint32_t)((kl >> 1) * ND * 32);
+        inc = 1u << ((kl & 1) << 4);
     } else if (PACK) {
         woff = 0u;
-        inc = one;
+        inc = 1u;
     } else {
-        woff = (uint32_t)(kl * ND * 32 * RW);
-        inc = one;
+        woff = (uint32_t)(kl * ND * 32);
+        inc = 1u;
     }
 }
 
@@ -301,14 +283,12 @@ __device__ __forceinline__ void col_word(int ND, int kl, uint32_t one, uint32_t 
 // AFORM (the vote tile): the front list takes only A-form items, with the
 // A-form record and their counter word (PACK: the tile's counter layout);
 // other plain items join the back list with the general record.
-template <int KT, int MODE = kModePlain, bool AFORM = false, bool PACK = false, int RW = 1>
-__device__ __forceinline__ void collect(const DevGeom &G, const TileCtx<KT, RW> &T, float xh,
+template <int KT, int MODE = kModePlain, bool AFORM = false, bool PACK = false>
+__device__ __forceinline__ void collect(const DevGeom &G, const TileCtx<KT> &T, float xh,
                                         float yh, int n, int h, int ha, int lane, int *q,
                                         const WorkList &W, const MaskCtx *M = nullptr,
-                                        const HitCtx *H = nullptr,
-                                        const uint8_t *__restrict__ layer = nullptr)
+                                        const HitCtx *H = nullptr)
 {
-    constexpr int BM = base_mode(MODE);
     float is_[KT], ic_[KT];
     int fl_[KT];
     unsigned sel = 0u, af = 0u;
@@ -316,8 +296,7 @@ __device__ __forceinline__ void collect(const DevGeom &G, const TileCtx<KT, RW> 
     unsigned long long hm = 0ull;
     float hwlo = 0.0f, hwhi = 0.0f;
     bool live = h < n;
-    const unsigned char lh = (layer_mode(MODE) && live) ? __ldg(layer + ha) : 0;
-    if (BM == kModeHit && live) {
+    if (MODE == kModeHit && live) {
         hm = H->masks[ha];
         unsigned tb = 0u;
         for (int b = H->rb_lo; b <= H->rb_hi; ++b) tb |= (unsigned)(hm >> (8 * b)) & 0xffu;
@@ -348,10 +327,10 @@ __device__ __forceinline__ void collect(const DevGeom &G, const TileCtx<KT, RW> 
                 f |= kMetaUnsure;
             } else if (c > 1.0f) {
                 float gmin, gmax;
-                if (BM == kModeHit) {
+                if (MODE == kModeHit) {
                     rho_range_w(hwlo + s, hwhi + s, c, eS, gmin, gmax);
                     if (gmax < T.rho_lo || gmin > T.rho_hi) continue;
-                } else if (BM == kModeEvent) {
+                } else if (MODE == kModeEvent) {
                     bool reach = false;
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
@@ -406,7 +385,7 @@ __device__ __forceinline__ void collect(const DevGeom &G, const TileCtx<KT, RW> 
                 float eB;
                 W.a[pos] = make_aform(G, is_[kl], ic_[kl], R1, T.rt, eB);
                 uint32_t woff, inc;
-                col_word<KT, PACK, RW>(G.n_d0, kl, layer_mode(MODE) ? 1u << lh : 1u, woff, inc);
+                col_word<KT, PACK>(G.n_d0, kl, woff, inc);
                 W.b[pos] = make_float4(__uint_as_float(woff), __uint_as_float(inc), eB, 0.0f);
             } else {
                 const Item it = make_item(G, is_[kl], ic_[kl], r2, R1, T.rt);
@@ -414,8 +393,7 @@ __device__ __forceinline__ void collect(const DevGeom &G, const TileCtx<KT, RW> 
                 W.b[pos] = make_float4(it.E1, it.E2, it.Qa, it.Qb);
             }
             W.meta[pos] = (h << 6) | fl_[kl] | kl;
-            if (BM == kModeHit) W.hm[pos] = hm;
-            if (layer_mode(MODE)) W.lay[pos] = lh;
+            if (MODE == kModeHit) W.hm[pos] = hm;
         }
     }
 }
@@ -566,56 +544,39 @@ __device__ __forceinline__ bool push_redo(const RedoQueue &Q, int *n, int hit, i
 // computation; with KT = 1 it holds bins 2w and 2w + 1.  Exact while no cell
 // can reach 65536 votes in the tile: a cell gets at most two votes per
 // scanned hit, so it is used only for tiles scanning at most kPackMaxHits.
-// LAY (the distinct-layer vote): the same words hold layer masks; a vote
-// ORs the hit's layer bit lbit (1 << layer) instead of adding one.
-// RW: the tile has 32 RW rows (row fastest, 32 RW words per bin); lane is
-// the row within the tile.
-template <int KT, bool PACK, bool LAY = false, int RW = 1>
+// Rows are fastest (32 words per bin); lane is the row within the tile.
+template <int KT, bool PACK>
 struct TileCol {
     uint32_t *base;
     uint32_t inc;
 
-    __device__ __forceinline__ TileCol(uint32_t *cnt, int ND, int kl, int lane,
-                                       uint32_t lbit = 1u)
+    __device__ __forceinline__ TileCol(uint32_t *cnt, int ND, int kl, int lane)
     {
-        const uint32_t one = LAY ? lbit : 1u;
-        if (PACK && KT > 1) {
-            base = cnt + (kl >> 1) * ND * 32 * RW + lane;
-            inc = one << ((kl & 1) << 4);
-        } else if (PACK) {
-            base = cnt + lane;
-            inc = one;
-        } else {
-            base = cnt + kl * ND * 32 * RW + lane;
-            inc = one;
-        }
+        uint32_t woff;
+        col_word<KT, PACK>(ND, kl, woff, inc);
+        base = cnt + woff + lane;
     }
 
     __device__ __forceinline__ void add(int j) const
     {
-        uint32_t *w = (PACK && KT == 1) ? base + (j >> 1) * 32 * RW : base + j * 32 * RW;
-        const uint32_t v = (PACK && KT == 1) ? inc << ((j & 1) << 4) : inc;
-        if (LAY) atomicOr(w, v);
-        else atomicAdd(w, v);
+        uint32_t *w = (PACK && KT == 1) ? base + (j >> 1) * 32 : base + j * 32;
+        atomicAdd(w, (PACK && KT == 1) ? inc << ((j & 1) << 4) : inc);
     }
 };
 
 // An A-form item's vote: its counter word woff (from the lane's first word
 // cntl) and increment inc, as col_word gave them, in bin j.
-template <int KT, bool PACK, bool LAY, int RW = 1>
+template <int KT, bool PACK>
 __device__ __forceinline__ void add_word(uint32_t *cntl, uint32_t woff, uint32_t inc, int j)
 {
-    uint32_t *w = (PACK && KT == 1) ? cntl + woff + (j >> 1) * 32 * RW
-                                    : cntl + woff + j * 32 * RW;
-    const uint32_t v = (PACK && KT == 1) ? inc << ((j & 1) << 4) : inc;
-    if (LAY) atomicOr(w, v);
-    else atomicAdd(w, v);
+    uint32_t *w = (PACK && KT == 1) ? cntl + woff + (j >> 1) * 32 : cntl + woff + j * 32;
+    atomicAdd(w, (PACK && KT == 1) ? inc << ((j & 1) << 4) : inc);
 }
 
-template <int KT, bool PACK, int RW = 1>
+template <int KT, bool PACK>
 __device__ __forceinline__ uint32_t tile_get(const uint32_t *cnt, int ND, int kl, int j, int il)
 {
-    constexpr int R = 32 * RW;
+    constexpr int R = 32;
     if (PACK && KT > 1) return (cnt[((kl >> 1) * ND + j) * R + il] >> ((kl & 1) << 4)) & 0xffffu;
     if (PACK) return (cnt[(j >> 1) * R + il] >> ((j & 1) << 4)) & 0xffffu;
     return cnt[(kl * ND + j) * R + il];
@@ -637,45 +598,38 @@ __device__ __forceinline__ int keep_allowed(unsigned bm, const uint8_t *jmask, i
 // cell is written.
 // hl (optional): the tile scans only the nl hits hl[0 .. nl) of the event
 // (a superset of those that can vote in its columns); otherwise all n.
-// RW = 2 (the plain and distinct-layer votes only): tiles of 64 rows, each
-// lane evaluating rows lane and 32 + lane of every item, so that an item's
-// loads, its phase-1 work and the warp's bookkeeping serve twice the votes.
-template <int KT, typename OutT, bool PACK, int MODE = kModePlain, int RW = 1>
+template <int KT, typename OutT, bool PACK, int MODE = kModePlain>
 __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restrict__ x,
                                           const float *__restrict__ y, int n,
                                           OutT *__restrict__ acc,
                                           unsigned long long *__restrict__ stats, int tx, int ty,
                                           unsigned long long mask = ~0ull,
                                           const unsigned long long *__restrict__ hmask = nullptr,
-                                          const int *__restrict__ hl = nullptr, int nl = 0,
-                                          const uint8_t *__restrict__ layer = nullptr)
+                                          const int *__restrict__ hl = nullptr, int nl = 0)
 {
-    constexpr int BM = base_mode(MODE);
-    constexpr bool LAY = layer_mode(MODE);
-    static_assert(RW == 1 || (RW == 2 && BM == kModePlain), "64-row tiles: plain modes only");
-    constexpr int TR = 32 * RW;                            // rows per tile
+    constexpr int TR = 32;                                 // rows per tile
     extern __shared__ __align__(16) unsigned char smem[];
     const int ND = G.n_d0;
     const int NW = PACK ? (ND >> 1) : ND;                  // words per column-row
     constexpr int QCAP = kThreads * KT;
     uint32_t *cnt = reinterpret_cast<uint32_t *>(smem);    // [KT][NW][TR]
     unsigned char *p = reinterpret_cast<unsigned char *>(cnt + KT * NW * TR);
-    const WorkList W = carve_worklist(p, QCAP, MODE);
+    const WorkList W = carve_worklist(p, QCAP);
     const RedoQueue R = carve_redo(p + (size_t)QCAP * item_bytes(MODE));
     __shared__ int qn[2][2], rn;   // [parity][plain, others]
     __shared__ unsigned long long s_stats[2];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int nwarps = kThreads / 32;
-    TileCtx<KT, RW> T;
+    TileCtx<KT> T;
     T.init(G, lane, tx, ty);
     MaskCtx M;
-    if (BM == kModeEvent) {
+    if (MODE == kModeEvent) {
         M.init(G, mask, T.i0, T.irow, T.row_ok);
         if (M.tile_bm == 0u) return;   // uniform: every warp sees the same rows
     }
     HitCtx H;
-    if (BM == kModeHit) {
+    if (MODE == kModeHit) {
         const int NR = G.n_rho;
         uint8_t *jm = p + (size_t)QCAP * item_bytes(MODE) + kRedoBytes;
         for (int j = threadIdx.x; j < ND; j += kThreads)
@@ -695,7 +649,7 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
     }
     {
         uint4 *c4 = reinterpret_cast<uint4 *>(cnt);
-        for (int t = threadIdx.x; t < KT * NW * 8 * RW; t += kThreads) c4[t] = make_uint4(0, 0, 0, 0);
+        for (int t = threadIdx.x; t < KT * NW * 8; t += kThreads) c4[t] = make_uint4(0, 0, 0, 0);
     }
     if (threadIdx.x < 4) qn[threadIdx.x >> 1][threadIdx.x & 1] = 0;
     if (threadIdx.x < 2) s_stats[threadIdx.x] = 0ull;
@@ -703,7 +657,6 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
     __syncthreads();
 
     int my_fb = 0;
-    unsigned my_cast = 0;   // LAY: votes cast by this thread in the tile (< 2^32: 2 KT per hit)
     int parity = 0;
     const HitSeq S{hl, hl ? nl : n};
     HitPrefetch pf;
@@ -712,8 +665,8 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
         int ha;
         float xh, yh;
         pf.next(x, y, S, base, ha, xh, yh);
-        collect<KT, MODE, true, PACK, RW>(G, T, xh, yh, S.n, base + threadIdx.x, ha, lane,
-                                          qn[parity], W, &M, &H, layer);
+        collect<KT, MODE, true, PACK>(G, T, xh, yh, S.n, base + threadIdx.x, ha, lane,
+                                      qn[parity], W, &M, &H);
         __syncthreads();
         const int nf = qn[parity][0], ns = qn[parity][1];
         if (threadIdx.x == 0) {   // last read before the previous barrier
@@ -725,100 +678,63 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
             // increment precomputed.  A warp takes two items per iteration:
             // both are loaded before either votes (a shared atomic orders
             // the loads behind it), their evaluations are independent, and
-            // one warp vote covers both redo tests (rare).  With RW = 2 each
-            // lane also evaluates its second row (32 + lane) of both items.
+            // one warp vote covers both redo tests (rare).
             uint32_t *const cntl = cnt + lane;
             const float mnd = kMagic + (float)ND;
-            const RowCtx &T1 = T.r1;
-            const bool ok1 = RW == 2 && T1.row_ok;
-            auto redo_item = [&](int tt, const RowCtx &Rw, int il) {
+            auto redo_item = [&](int tt) {
                 ++my_fb;
                 const int m = W.meta[tt];
                 const int hh = S.hit(m >> 6);
-                if (push_redo(R, &rn, hh, il, m & kMetaCol)) return;
-                const TileCol<KT, PACK, LAY, RW> col(cnt, ND, m & kMetaCol, il,
-                                                     LAY ? 1u << W.lay[tt] : 1u);
+                if (push_redo(R, &rn, hh, lane, m & kMetaCol)) return;
+                const TileCol<KT, PACK> col(cnt, ND, m & kMetaCol, lane);
                 int jj[2];
-                int nv = redo_bins(G, x[hh], y[hh], Rw.irow, T.k0 + (m & kMetaCol), jj);
-                if (BM == kModeHit) nv = keep_allowed(H.row_bits(W.hm[tt]), H.jmask, nv, jj);
+                int nv = redo_bins(G, x[hh], y[hh], T.irow, T.k0 + (m & kMetaCol), jj);
+                if (MODE == kModeHit) nv = keep_allowed(H.row_bits(W.hm[tt]), H.jmask, nv, jj);
                 for (int v = 0; v < nv; ++v) col.add(jj[v]);
-                if (LAY) my_cast += nv;
             };
-            auto vote_item = [&](int tt, const float4 &b, int j, bool vote, int r) {
-                if (vote && (BM != kModeHit || (H.row_bits(W.hm[tt]) & H.jmask[j]))) {
-                    add_word<KT, PACK, LAY, RW>(cntl + 32 * r, __float_as_uint(b.x),
-                                                __float_as_uint(b.y), j);
-                    if (LAY) ++my_cast;
-                }
+            auto vote_item = [&](int tt, const float4 &b, int j, bool vote) {
+                if (vote && (MODE != kModeHit || (H.row_bits(W.hm[tt]) & H.jmask[j])))
+                    add_word<KT, PACK>(cntl, __float_as_uint(b.x), __float_as_uint(b.y), j);
             };
             int t = warp;
             for (; t + nwarps < nf; t += 2 * nwarps) {
                 const float4 a0 = W.a[t], b0 = W.b[t];
                 const float4 a1 = W.a[t + nwarps], b1 = W.b[t + nwarps];
-                int j0, j1, j2 = 0, j3 = 0;
-                bool v0, v1, r0, r1, v2 = false, v3 = false, r2 = false, r3 = false;
+                int j0, j1;
+                bool v0, v1, r0, r1;
                 aform_bin(T, a0, b0.z, mnd, j0, v0, r0);
                 aform_bin(T, a1, b1.z, mnd, j1, v1, r1);
-                if (RW == 2) {
-                    aform_bin(T1, a0, b0.z, mnd, j2, v2, r2);
-                    aform_bin(T1, a1, b1.z, mnd, j3, v3, r3);
-                    v2 &= ok1;
-                    v3 &= ok1;
-                    r2 &= ok1;
-                    r3 &= ok1;
-                }
-                vote_item(t, b0, j0, v0, 0);
-                vote_item(t + nwarps, b1, j1, v1, 0);
-                if (RW == 2) {
-                    vote_item(t, b0, j2, v2, 1);
-                    vote_item(t + nwarps, b1, j3, v3, 1);
-                }
+                vote_item(t, b0, j0, v0);
+                vote_item(t + nwarps, b1, j1, v1);
                 // lanes of rows past n_rho do not run this loop, hence the active mask
-                if (!__any_sync(__activemask(), r0 | r1 | r2 | r3)) continue;
-                if (r0) redo_item(t, T, lane);
-                if (r1) redo_item(t + nwarps, T, lane);
-                if (RW == 2) {
-                    if (r2) redo_item(t, T1, 32 + lane);
-                    if (r3) redo_item(t + nwarps, T1, 32 + lane);
-                }
+                if (!__any_sync(__activemask(), r0 | r1)) continue;
+                if (r0) redo_item(t);
+                if (r1) redo_item(t + nwarps);
             }
             if (t < nf) {
                 const float4 a0 = W.a[t], b0 = W.b[t];
                 int j0;
                 bool v0, r0;
                 aform_bin(T, a0, b0.z, mnd, j0, v0, r0);
-                vote_item(t, b0, j0, v0, 0);
-                if (r0) redo_item(t, T, lane);
-                if (RW == 2 && ok1) {
-                    aform_bin(T1, a0, b0.z, mnd, j0, v0, r0);
-                    vote_item(t, b0, j0, v0, 1);
-                    if (r0) redo_item(t, T1, 32 + lane);
-                }
+                vote_item(t, b0, j0, v0);
+                if (r0) redo_item(t);
             }
             // unsure items, items whose second root can reach the axis and the
             // other plain items
             for (int t = kThreads * KT - ns + warp; t < kThreads * KT; t += nwarps) {
                 const int m = W.meta[t];
-#pragma unroll
-                for (int r = 0; r < RW; ++r) {
-                    const RowCtx &Rw = r == 0 ? static_cast<const RowCtx &>(T) : T1;
-                    if (r == 1 && !ok1) break;
-                    const int il = lane + 32 * r;
-                    const TileCol<KT, PACK, LAY, RW> col(cnt, ND, m & kMetaCol, il,
-                                                         LAY ? 1u << W.lay[t] : 1u);
-                    int jj[2];
-                    int nv = item_bins32<KT>(G, Rw, W, t, m, jj);
-                    if (nv < 0) {
-                        ++my_fb;
-                        const int hh = S.hit(m >> 6);
-                        if (push_redo(R, &rn, hh, il, m & kMetaCol)) continue;
-                        nv = redo_bins(G, x[hh], y[hh], Rw.irow, T.k0 + (m & kMetaCol), jj);
-                    }
-                    if (BM == kModeHit) nv = keep_allowed(H.row_bits(W.hm[t]), H.jmask, nv, jj);
-                    if (nv > 0) col.add(jj[0]);
-                    if (nv > 1) col.add(jj[1]);
-                    if (LAY) my_cast += nv;
+                const TileCol<KT, PACK> col(cnt, ND, m & kMetaCol, lane);
+                int jj[2];
+                int nv = item_bins32<KT>(G, T, W, t, m, jj);
+                if (nv < 0) {
+                    ++my_fb;
+                    const int hh = S.hit(m >> 6);
+                    if (push_redo(R, &rn, hh, lane, m & kMetaCol)) continue;
+                    nv = redo_bins(G, x[hh], y[hh], T.irow, T.k0 + (m & kMetaCol), jj);
                 }
+                if (MODE == kModeHit) nv = keep_allowed(H.row_bits(W.hm[t]), H.jmask, nv, jj);
+                if (nv > 0) col.add(jj[0]);
+                if (nv > 1) col.add(jj[1]);
             }
         }
         __syncthreads();
@@ -830,13 +746,11 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
                 const int il = rc >> 4, kl = rc & 15;
                 int jj[2];
                 int nv = redo_bins(G, x[h], y[h], T.i0 + il, T.k0 + kl, jj);
-                if (BM == kModeHit)
+                if (MODE == kModeHit)
                     nv = keep_allowed(halo_row_blocks(H.masks[h], T.i0 + il, G.n_rho), H.jmask, nv,
                                       jj);
-                const TileCol<KT, PACK, LAY, RW> col(cnt, ND, kl, il,
-                                                     LAY ? 1u << __ldg(layer + h) : 1u);
+                const TileCol<KT, PACK> col(cnt, ND, kl, il);
                 for (int v = 0; v < nv; ++v) col.add(jj[v]);
-                if (LAY) my_cast += nv;
             }
             __syncthreads();
             if (threadIdx.x == 0) rn = 0;
@@ -849,16 +763,15 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
     // counters never saturate: they hold at most 2 n).
     unsigned long long my_votes = 0;
     for (int t = threadIdx.x; t < TR * ND; t += kThreads) {
-        const int il = t & (TR - 1), j = t / TR;   // il == lane (RW = 1) or lane + 32 (RW = 2)
+        const int il = t & (TR - 1), j = t / TR;   // il == lane
         const int i = T.i0 + il;
         if (i >= G.n_rho) continue;
-        const bool keep = BM != kModeEvent || halo_bin(M.bm, j, ND);
+        const bool keep = MODE != kModeEvent || halo_bin(M.bm, j, ND);
         __align__(16) OutT e[KT];
 #pragma unroll
         for (int kl = 0; kl < KT; ++kl) {
-            uint32_t v = keep ? tile_get<KT, PACK, RW>(cnt, ND, kl, j, il) : 0u;
-            if (LAY) v = (uint32_t)__popc(v);
-            else my_votes += v;
+            const uint32_t v = keep ? tile_get<KT, PACK>(cnt, ND, kl, j, il) : 0u;
+            my_votes += v;
             e[kl] = saturate<OutT>(v);
         }
         OutT *dst = acc + ((size_t)i * ND + j) * G.n_phi0 + T.k0;
@@ -874,7 +787,6 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
         }
     }
 
-    if (LAY) my_votes = my_cast;
     if (stats) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -891,20 +803,14 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
 }
 
 // mask: kModeEvent one device uint64, kModeHit one per hit, else unused;
-// layer: one uint8 per hit under kModeLayers, else unused.
-// The distinct-layer vote's tiles of at most two columns (64-row tiles, and
-// the 32-row tiles of the pile-up geometry and of the per-hit mode) take four
-// CTAs per SM: their counters and two-column work list fit four in shared
-// memory, and 64 registers spill about as little as 80 do.
-template <int KT, typename OutT, bool PACK, int MODE, int RW = 1>
-__global__ void __launch_bounds__(kThreads, (RW == 2 || (layer_mode(MODE) && KT <= 2)) ? 4 : (PACK ? 3 : 2))
+template <int KT, typename OutT, bool PACK, int MODE>
+__global__ void __launch_bounds__(kThreads, PACK ? 3 : 2)
 k_vote(DevGeom G, const float *__restrict__ x, const float *__restrict__ y, int n,
        OutT *__restrict__ acc, unsigned long long *__restrict__ stats,
-       const unsigned long long *__restrict__ mask, const uint8_t *__restrict__ layer)
+       const unsigned long long *__restrict__ mask)
 {
-    vote_tile<KT, OutT, PACK, MODE, RW>(G, x, y, n, acc, stats, blockIdx.x, blockIdx.y,
-                                    base_mode(MODE) == kModeEvent ? *mask : ~0ull, mask,
-                                    nullptr, 0, layer);
+    vote_tile<KT, OutT, PACK, MODE>(G, x, y, n, acc, stats, blockIdx.x, blockIdx.y,
+                                    MODE == kModeEvent ? *mask : ~0ull, mask);
 }
 
 // Persistent vote over a batch: CTAs pop (event, tile) items from a device
@@ -914,18 +820,17 @@ k_vote(DevGeom G, const float *__restrict__ x, const float *__restrict__ y, int 
 // set per hit of the batch (indexed like x).
 // bk (optional, ent null for none): per-event hit lists by column group; a
 // tile scans its group's list instead of the whole event.
-template <int KT, typename OutT, bool PACK, int MODE, int RW = 1>
-__global__ void __launch_bounds__(kThreads, (RW == 2 || (layer_mode(MODE) && KT <= 2)) ? 4 : (PACK ? 3 : 2))
+template <int KT, typename OutT, bool PACK, int MODE>
+__global__ void __launch_bounds__(kThreads, PACK ? 3 : 2)
 k_vote_batch(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
              const int *__restrict__ off, const int *__restrict__ order,
              const int *__restrict__ d_nev,
              OutT *__restrict__ acc, size_t acc_stride, unsigned long long *__restrict__ stats,
              int *__restrict__ head, const unsigned long long *__restrict__ masks,
-             BucketView bk, const uint8_t *__restrict__ layer)
+             BucketView bk)
 {
-    constexpr int BM = base_mode(MODE);
     __shared__ int s_item;
-    const int ntx = G.n_phi0 / KT, nty = (G.n_rho + 32 * RW - 1) / (32 * RW), ntiles = ntx * nty;
+    const int ntx = G.n_phi0 / KT, nty = (G.n_rho + 31) / 32, ntiles = ntx * nty;
     const int total = *d_nev * ntiles;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(head, 1);
@@ -941,95 +846,62 @@ k_vote_batch(DevGeom G, const float *__restrict__ x, const float *__restrict__ y
         // hits (a cell then holds at most 2 kPackMaxHits < 2^16 votes, so no
         // count carries into its neighbour), unpacked counters the others:
         // the two launches of a batch split every event's tiles between them
-        // by the scanned list's length (uniform over the CTA).  Layer masks
-        // never carry, so the distinct-layer vote packs every tile.
-        if (layer_mode(MODE) ? PACK : (PACK == ((bk.ent ? nl : n) <= kPackMaxHits)))
-            vote_tile<KT, OutT, PACK, MODE, RW>(G, x + a, y + a, n, acc + (size_t)e * acc_stride,
+        // by the scanned list's length (uniform over the CTA).
+        if (PACK == ((bk.ent ? nl : n) <= kPackMaxHits))
+            vote_tile<KT, OutT, PACK, MODE>(G, x + a, y + a, n, acc + (size_t)e * acc_stride,
                                             stats ? stats + 2 * e : nullptr, t % ntx, t / ntx,
-                                            BM == kModeEvent ? masks[e] : ~0ull,
-                                            BM == kModeHit ? masks + a : nullptr, hl, nl,
-                                            layer_mode(MODE) ? layer + a : nullptr);
+                                            MODE == kModeEvent ? masks[e] : ~0ull,
+                                            MODE == kModeHit ? masks + a : nullptr, hl, nl);
         __syncthreads();
     }
 }
 
 template <int KT>
-size_t vote_smem(const DevGeom &G, bool pack, int mode = kModePlain, int rw = 1)
+size_t vote_smem(const DevGeom &G, bool pack, int mode = kModePlain)
 {
-    return (size_t)KT * 32 * rw * (pack ? G.n_d0 / 2 : G.n_d0) * 4 +
+    return (size_t)KT * 32 * (pack ? G.n_d0 / 2 : G.n_d0) * 4 +
            (size_t)kThreads * KT * item_bytes(mode) + kRedoBytes +
-           (base_mode(mode) == kModeHit ? ((size_t)G.n_d0 + 15) / 16 * 16 : 0);
+           (mode == kModeHit ? ((size_t)G.n_d0 + 15) / 16 * 16 : 0);
 }
 
 constexpr size_t kSmemBudget2 = 110 * 1024;   // two CTAs per SM
 constexpr size_t kSmemBudget3 = 75 * 1024;    // three CTAs per SM
 
-template <int KT, typename OutT, bool PACK, int MODE, int RW = 1>
+template <int KT, typename OutT, bool PACK, int MODE>
 cudaError_t launch_vote_kt(const DevGeom &G, const float *x, const float *y, int n, void *acc,
                            unsigned long long *stats, const unsigned long long *mask,
-                           cudaStream_t st, const uint8_t *layer)
+                           cudaStream_t st)
 {
-    dim3 grid(G.n_phi0 / KT, (G.n_rho + 32 * RW - 1) / (32 * RW));
-    k_vote<KT, OutT, PACK, MODE, RW><<<grid, kThreads, vote_smem<KT>(G, PACK, MODE, RW), st>>>(
-        G, x, y, n, reinterpret_cast<OutT *>(acc), stats, mask, layer);
+    dim3 grid(G.n_phi0 / KT, (G.n_rho + 31) / 32);
+    k_vote<KT, OutT, PACK, MODE><<<grid, kThreads, vote_smem<KT>(G, PACK, MODE), st>>>(
+        G, x, y, n, reinterpret_cast<OutT *>(acc), stats, mask);
     return cudaGetLastError();
-}
-
-// The distinct-layer vote's default tile: 64 rows of two columns when it
-// fits in the three-CTA budget (plain base mode only).
-template <int MODE>
-constexpr bool tall_tiles_ok()
-{
-    return layer_mode(MODE) && base_mode(MODE) == kModePlain;
 }
 
 // Tile shape: packed 16-bit counters with three CTAs per SM when the output
 // is uint16, n_d0 even and n <= 32767; otherwise 32-bit counters, two CTAs
-// per SM.  KT is the widest tile that fits.  The distinct-layer vote
-// (kModeLayers; n_d0 even) always packs, into either output type, on 64-row
-// tiles of two columns (four CTAs per SM) where they fit the three-CTA
-// budget, else on 32-row tiles.
+// per SM.  KT is the widest tile that fits.
 template <int MODE>
 cudaError_t launch_vote_t(const DevGeom &G, const float *x, const float *y, int n, void *acc,
                           unsigned long long *stats, const unsigned long long *mask,
-                          cudaStream_t st, const uint8_t *layer = nullptr)
+                          cudaStream_t st)
 {
 #define HT_V(KTV, OT, PK)                                                                     \
-    return launch_vote_kt<KTV, OT, PK, MODE>(G, x, y, n, acc, stats, mask, st, layer)
-    if constexpr (tall_tiles_ok<MODE>()) {
-        if (vote_smem<2>(G, true, MODE, 2) <= kSmemBudget3) {
-            if (G.count_bits == 16)
-                return launch_vote_kt<2, uint16_t, true, MODE, 2>(G, x, y, n, acc, stats, mask,
-                                                                  st, layer);
-            return launch_vote_kt<2, int32_t, true, MODE, 2>(G, x, y, n, acc, stats, mask, st,
-                                                             layer);
-        }
-    }
-    if constexpr (layer_mode(MODE)) {
-        if (G.count_bits == 16) {
+    return launch_vote_kt<KTV, OT, PK, MODE>(G, x, y, n, acc, stats, mask, st)
+    if (G.count_bits == 16) {
+        if (n <= 32767 && G.n_d0 % 2 == 0) {
             if (vote_smem<4>(G, true, MODE) <= kSmemBudget3) HT_V(4, uint16_t, true);
             if (vote_smem<2>(G, true, MODE) <= kSmemBudget3) HT_V(2, uint16_t, true);
-            HT_V(1, uint16_t, true);
+            if (vote_smem<1>(G, true, MODE) <= kSmemBudget3) HT_V(1, uint16_t, true);
         }
-        if (vote_smem<4>(G, true, MODE) <= kSmemBudget3) HT_V(4, int32_t, true);
-        if (vote_smem<2>(G, true, MODE) <= kSmemBudget3) HT_V(2, int32_t, true);
-        HT_V(1, int32_t, true);
-    } else {
-        if (G.count_bits == 16) {
-            if (n <= 32767 && G.n_d0 % 2 == 0) {
-                if (vote_smem<4>(G, true, MODE) <= kSmemBudget3) HT_V(4, uint16_t, true);
-                if (vote_smem<2>(G, true, MODE) <= kSmemBudget3) HT_V(2, uint16_t, true);
-                if (vote_smem<1>(G, true, MODE) <= kSmemBudget3) HT_V(1, uint16_t, true);
-            }
-            if (vote_smem<8>(G, false, MODE) <= kSmemBudget2) HT_V(8, uint16_t, false);
-            if (vote_smem<4>(G, false, MODE) <= kSmemBudget2) HT_V(4, uint16_t, false);
-            if (vote_smem<2>(G, false, MODE) <= kSmemBudget2) HT_V(2, uint16_t, false);
-            HT_V(1, uint16_t, false);
-        }
-        if (vote_smem<4>(G, false, MODE) <= kSmemBudget2) HT_V(4, int32_t, false);
-        if (vote_smem<2>(G, false, MODE) <= kSmemBudget2) HT_V(2, int32_t, false);
-        HT_V(1, int32_t, false);
+        if (vote_smem<8>(G, false, MODE) <= kSmemBudget2) HT_V(8, uint16_t, false);
+        if (vote_smem<4>(G, false, MODE) <= kSmemBudget2) HT_V(4, uint16_t, false);
+        if (vote_smem<2>(G, false, MODE) <= kSmemBudget2) HT_V(2, uint16_t, false);
+        HT_V(1, uint16_t, false);
     }
+    if (vote_smem<4>(G, false, MODE) <= kSmemBudget2) HT_V(4, int32_t, false);
+    if (vote_smem<2>(G, false, MODE) <= kSmemBudget2) HT_V(2, int32_t, false);
+    HT_V(1, int32_t, false);
 #undef HT_V
 }
 
@@ -1038,63 +910,44 @@ cudaError_t launch_vote_t(const DevGeom &G, const float *x, const float *y, int 
 // kt selects the tile width (0 = default).  pack: this launch takes the
 // listed events' tiles that scan at most kPackMaxHits hits (a column group's
 // hit list with buckets, else the event) with 16-bit packed counters;
-// otherwise it takes their other tiles with 32-bit counters.  The
-// distinct-layer vote takes every tile in its packed launch (layer: the
-// batch's layer array, indexed like x), by default on 64-row tiles of two
-// columns (an explicit kt selects 32-row tiles of that width).  *head must
+// otherwise it takes their other tiles with 32-bit counters.  *head must
 // be zero.
 template <int MODE>
 cudaError_t launch_vote_batch_t(const DevGeom &G, const float *x, const float *y, const int *off,
                                 const int *order, const int *d_nev, uint16_t *acc,
                                 size_t acc_stride, unsigned long long *stats, int *head,
                                 bool pack, int kt, int sms, const unsigned long long *masks,
-                                cudaStream_t st, BucketView bk = BucketView{},
-                                const uint8_t *layer = nullptr)
+                                cudaStream_t st, BucketView bk = BucketView{})
 {
-#define HT_VB2(KTV, PK, RWV)                                                                  \
+#define HT_VB(KTV, PK)                                                                        \
     do {                                                                                      \
         int occ = 0;                                                                          \
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                        \
-            &occ, k_vote_batch<KTV, uint16_t, PK, MODE, RWV>, kThreads,                       \
-            vote_smem<KTV>(G, PK, MODE, RWV));                                                \
-        k_vote_batch<KTV, uint16_t, PK, MODE, RWV><<<sms * (occ > 0 ? occ : 1), kThreads,    \
-                                                     vote_smem<KTV>(G, PK, MODE, RWV), st>>>( \
-            G, x, y, off, order, d_nev, acc, acc_stride, stats, head, masks, bk, layer);      \
+            &occ, k_vote_batch<KTV, uint16_t, PK, MODE>, kThreads,                       \
+            vote_smem<KTV>(G, PK, MODE));                                                \
+        k_vote_batch<KTV, uint16_t, PK, MODE><<<sms * (occ > 0 ? occ : 1), kThreads,    \
+                                                     vote_smem<KTV>(G, PK, MODE), st>>>( \
+            G, x, y, off, order, d_nev, acc, acc_stride, stats, head, masks, bk);             \
         return cudaGetLastError();                                                            \
     } while (0)
-#define HT_VB(KTV, PK) HT_VB2(KTV, PK, 1)
     // the per-hit mode's larger items would drop a tuned width to two CTAs
     // per SM: it keeps three
-    const size_t budget = base_mode(MODE) == kModeHit ? kSmemBudget3 : kSmemBudget2;
-    if constexpr (tall_tiles_ok<MODE>()) {
-        // kt = 0 (the default): 64-row tiles of two columns where they fit
-        if (pack && kt == 0 && vote_smem<2>(G, true, MODE, 2) <= kSmemBudget3) HT_VB2(2, true, 2);
-    }
-    if constexpr (layer_mode(MODE)) {
-        if (!pack) return cudaSuccess;   // no unpacked tiles
+    const size_t budget = MODE == kModeHit ? kSmemBudget3 : kSmemBudget2;
+    if (pack) {
         if (kt == 0) kt = vote_smem<4>(G, true, MODE) <= kSmemBudget3 ? 4
                         : vote_smem<2>(G, true, MODE) <= kSmemBudget3 ? 2 : 1;
         if (kt == 4 && vote_smem<4>(G, true, MODE) <= budget) HT_VB(4, true);
         if (kt >= 2 && vote_smem<2>(G, true, MODE) <= budget) HT_VB(2, true);
         HT_VB(1, true);
-    } else {
-        if (pack) {
-            if (kt == 0) kt = vote_smem<4>(G, true, MODE) <= kSmemBudget3 ? 4
-                            : vote_smem<2>(G, true, MODE) <= kSmemBudget3 ? 2 : 1;
-            if (kt == 4 && vote_smem<4>(G, true, MODE) <= budget) HT_VB(4, true);
-            if (kt >= 2 && vote_smem<2>(G, true, MODE) <= budget) HT_VB(2, true);
-            HT_VB(1, true);
-        }
-        if (kt == 0) kt = vote_smem<8>(G, false, MODE) <= kSmemBudget2 ? 8
-                        : vote_smem<4>(G, false, MODE) <= kSmemBudget2 ? 4
-                        : vote_smem<2>(G, false, MODE) <= kSmemBudget2 ? 2 : 1;
-        if (kt == 8 && vote_smem<8>(G, false, MODE) <= kSmemBudget2) HT_VB(8, false);
-        if (kt >= 4 && vote_smem<4>(G, false, MODE) <= kSmemBudget2) HT_VB(4, false);
-        if (kt >= 2 && vote_smem<2>(G, false, MODE) <= kSmemBudget2) HT_VB(2, false);
-        HT_VB(1, false);
     }
+    if (kt == 0) kt = vote_smem<8>(G, false, MODE) <= kSmemBudget2 ? 8
+                    : vote_smem<4>(G, false, MODE) <= kSmemBudget2 ? 4
+                    : vote_smem<2>(G, false, MODE) <= kSmemBudget2 ? 2 : 1;
+    if (kt == 8 && vote_smem<8>(G, false, MODE) <= kSmemBudget2) HT_VB(8, false);
+    if (kt >= 4 && vote_smem<4>(G, false, MODE) <= kSmemBudget2) HT_VB(4, false);
+    if (kt >= 2 && vote_smem<2>(G, false, MODE) <= kSmemBudget2) HT_VB(2, false);
+    HT_VB(1, false);
 #undef HT_VB
-#undef HT_VB2
 }
 
 inline cudaError_t allow_smem(const void *const *fns, int nf, int max_smem)
@@ -1115,47 +968,25 @@ inline cudaError_t allow_smem(const void *const *fns, int nf, int max_smem)
 template <int MODE>
 cudaError_t prepare_vote_kernels_t(int max_smem)
 {
-    if constexpr (tall_tiles_ok<MODE>()) {
-        const void *fns[] = {
-            (const void *)k_vote<2, uint16_t, true, MODE, 2>,
-            (const void *)k_vote<2, int32_t, true, MODE, 2>,
-            (const void *)k_vote_batch<2, uint16_t, true, MODE, 2>};
-        const cudaError_t e = allow_smem(fns, (int)(sizeof fns / sizeof fns[0]), max_smem);
-        if (e != cudaSuccess) return e;
-    }
-    if constexpr (layer_mode(MODE)) {
-        const void *fns[] = {
-            (const void *)k_vote<4, uint16_t, true, MODE>,
-            (const void *)k_vote<2, uint16_t, true, MODE>,
-            (const void *)k_vote<1, uint16_t, true, MODE>,
-            (const void *)k_vote<4, int32_t, true, MODE>,
-            (const void *)k_vote<2, int32_t, true, MODE>,
-            (const void *)k_vote<1, int32_t, true, MODE>,
-            (const void *)k_vote_batch<4, uint16_t, true, MODE>,
-            (const void *)k_vote_batch<2, uint16_t, true, MODE>,
-            (const void *)k_vote_batch<1, uint16_t, true, MODE>};
-        return allow_smem(fns, (int)(sizeof fns / sizeof fns[0]), max_smem);
-    } else {
-        const void *fns[] = {
-            (const void *)k_vote<4, uint16_t, true, MODE>,
-            (const void *)k_vote<2, uint16_t, true, MODE>,
-            (const void *)k_vote<1, uint16_t, true, MODE>,
-            (const void *)k_vote<8, uint16_t, false, MODE>,
-            (const void *)k_vote<4, uint16_t, false, MODE>,
-            (const void *)k_vote<2, uint16_t, false, MODE>,
-            (const void *)k_vote<1, uint16_t, false, MODE>,
-            (const void *)k_vote<4, int32_t, false, MODE>,
-            (const void *)k_vote<2, int32_t, false, MODE>,
-            (const void *)k_vote<1, int32_t, false, MODE>,
-            (const void *)k_vote_batch<4, uint16_t, true, MODE>,
-            (const void *)k_vote_batch<2, uint16_t, true, MODE>,
-            (const void *)k_vote_batch<1, uint16_t, true, MODE>,
-            (const void *)k_vote_batch<8, uint16_t, false, MODE>,
-            (const void *)k_vote_batch<4, uint16_t, false, MODE>,
-            (const void *)k_vote_batch<2, uint16_t, false, MODE>,
-            (const void *)k_vote_batch<1, uint16_t, false, MODE>};
-        return allow_smem(fns, (int)(sizeof fns / sizeof fns[0]), max_smem);
-    }
+    const void *fns[] = {
+        (const void *)k_vote<4, uint16_t, true, MODE>,
+        (const void *)k_vote<2, uint16_t, true, MODE>,
+        (const void *)k_vote<1, uint16_t, true, MODE>,
+        (const void *)k_vote<8, uint16_t, false, MODE>,
+        (const void *)k_vote<4, uint16_t, false, MODE>,
+        (const void *)k_vote<2, uint16_t, false, MODE>,
+        (const void *)k_vote<1, uint16_t, false, MODE>,
+        (const void *)k_vote<4, int32_t, false, MODE>,
+        (const void *)k_vote<2, int32_t, false, MODE>,
+        (const void *)k_vote<1, int32_t, false, MODE>,
+        (const void *)k_vote_batch<4, uint16_t, true, MODE>,
+        (const void *)k_vote_batch<2, uint16_t, true, MODE>,
+        (const void *)k_vote_batch<1, uint16_t, true, MODE>,
+        (const void *)k_vote_batch<8, uint16_t, false, MODE>,
+        (const void *)k_vote_batch<4, uint16_t, false, MODE>,
+        (const void *)k_vote_batch<2, uint16_t, false, MODE>,
+        (const void *)k_vote_batch<1, uint16_t, false, MODE>};
+    return allow_smem(fns, (int)(sizeof fns / sizeof fns[0]), max_smem);
 }
 
 }  // namespace
