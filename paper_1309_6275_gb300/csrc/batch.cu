@@ -138,7 +138,6 @@ struct ht_batch {
     ht::HitBuckets bk;
     ht_confirm_desc conf;   // track path parameters (set by ht_batch_set_confirm)
     bool conf_set;
-    int *inl;               // track path: 16 inlier hits per candidate slot
     char *cf_ws;            // track path: confirmation scratch
     char *idx_ws;           // track path: the hit index (k_hitindex.cu)
     ht::HitIndex idx;
@@ -188,7 +187,6 @@ void free_batch(ht_batch *b)
     cudaFree(b->z_ws);
     cudaFree(b->mass);
     cudaFree(b->bk_ws);
-    cudaFree(b->inl);
     cudaFree(b->cf_ws);
     cudaFree(b->idx_ws);
     cudaFree(b->pp_ws);
@@ -269,9 +267,9 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
         if (e == cudaSuccess) e = mark(3);
         const ht::ConfirmDev P{b->conf.pool, b->conf.min_layers, b->conf.n_layers, b->conf.tol};
         if (e == cudaSuccess)
-            e = ht::launch_confirm_batch(G, P, x, y, R.layer, off, meta + 2, b->max_events,
-                                         b->max_hits, peaks, counts, b->cap, R.score, b->inl,
-                                         assign, b->cf_ws, b->idx, b->sms, st);
+            e = ht::launch_confirm_batch(G, P, off, meta + 2, b->max_events, b->max_hits, peaks,
+                                         counts, b->cap, R.score, nullptr, assign, b->cf_ws,
+                                         b->idx, b->sms, st);
         if (e == cudaSuccess) e = mark(4);
         if (e == cudaSuccess)
             e = ht::launch_vote_z_batch(G, x, y, z, assign, off, meta + 2, peaks, counts, b->cap,
@@ -632,22 +630,18 @@ ht_status ht_batch_set_confirm(ht_batch *b, const ht_confirm_desc *c)
             return ht::set_error(HT_ERR_CUDA, "ht_batch_set_confirm: staging wait");
         b->meta_pending = false;
     }
-    if (!b->inl) {
-        cudaError_t e = cudaMalloc((void **)&b->inl, (size_t)b->max_events * b->cap * 16 * 4);
-        if (e == cudaSuccess)
-            e = cudaMalloc((void **)&b->cf_ws,
-                           ht::confirm_workspace_bytes(b->g->G, b->max_events, b->max_hits, b->cap));
+    if (!b->cf_ws) {
+        cudaError_t e = cudaMalloc((void **)&b->cf_ws,
+                                   ht::confirm_workspace_bytes(b->max_events, b->max_hits));
         if (e == cudaSuccess)
             e = cudaMalloc((void **)&b->idx_ws, ht::hit_index_bytes(b->max_events, b->max_hits));
         if (e == cudaSuccess)
             e = cudaMalloc((void **)&b->pp_ws, ht::plane_peaks_bytes(b->g->G, b->max_events));
         if (e == cudaSuccess) b->idx = ht::carve_hit_index(b->max_events, b->max_hits, b->idx_ws);
         if (e != cudaSuccess) {
-            cudaFree(b->inl);
             cudaFree(b->cf_ws);
             cudaFree(b->idx_ws);
             cudaFree(b->pp_ws);
-            b->inl = nullptr;
             b->cf_ws = b->idx_ws = b->pp_ws = nullptr;
             return ht::set_error(HT_ERR_CUDA, "ht_batch_set_confirm: allocation failed");
         }

@@ -335,7 +335,7 @@ ht_status ht_vote_layers(const ht_geometry *g, const float *x, const float *y,
 size_t ht_confirm_workspace_size(const ht_geometry *g, int32_t n_hits, int32_t cap)
 {
     if (!g) return 0;
-    return ht::confirm_workspace_bytes_single(g->G, n_hits > 0 ? n_hits : 0, cap > 0 ? cap : 0);
+    return ht::confirm_workspace_bytes_single(n_hits > 0 ? n_hits : 0);
 }
 
 ht_status ht_confirm(const ht_geometry *g, const ht_confirm_desc *c, const float *x,
@@ -352,7 +352,7 @@ ht_status ht_confirm(const ht_geometry *g, const ht_confirm_desc *c, const float
     if (c->pool < 0 || c->min_layers < 1 || c->n_layers < 1 || c->n_layers > 16 ||
         !(c->tol > 0.0))
         return fail(HT_ERR_ARG, "ht_confirm: parameters out of range");
-    if (workspace_bytes < ht::confirm_workspace_bytes_single(g->G, n_hits, cap) ||
+    if (workspace_bytes < ht::confirm_workspace_bytes_single(n_hits) ||
         !aligned(workspace, 256))
         return fail(HT_ERR_ARG, "ht_confirm: workspace too small or misaligned");
     const ht::ConfirmDev P{c->pool, c->min_layers, c->n_layers, c->tol};

@@ -441,9 +441,10 @@ struct ConfirmDev {
     double tol;
 };
 // Batch: event e's hits at x[off[e] ..), candidates peaks[e cap ..), kept
-// counts min(counts[e], cap); score (n_ev cap), inl (16 n_ev cap) and
-// assign (batch hit index) written.  ws: confirm_workspace_bytes.
-size_t confirm_workspace_bytes(const DevGeom &G, int max_events, int max_hits, int cap);
+// counts min(counts[e], cap); idx: the batch's hit index; score (n_ev cap),
+// inl (16 n_ev cap, or null) and assign (batch hit index) written.  ws:
+// confirm_workspace_bytes.
+size_t confirm_workspace_bytes(int max_events, int max_hits);
 cudaError_t prepare_confirm_kernels();
 // Compact found tracks of a batch (k_confirm.cu): tracks[tfirst[e] ..
 // tfirst[e + 1]) are event e's confirmed candidates in candidate order (the
@@ -455,14 +456,13 @@ cudaError_t launch_track_compact(const int *off, const int *d_nev, int max_event
                                  const int *score, const ht_zres *zres, const int *assign,
                                  ht_track_out *tracks, int tcap, int *tfirst, int *ntot,
                                  int *assign_out, void *ws, int sms, cudaStream_t st);
-cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const float *x,
-                                 const float *y, const uint8_t *layer, const int *off,
+cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const int *off,
                                  const int *d_nev, int max_events, int max_hits,
                                  const ht_peak *peaks, const int *counts, int cap, int *score,
                                  int *inl, int *assign, void *ws, const HitIndex &idx, int sms,
                                  cudaStream_t st);
 // One event of n hits (host) and *d_count candidates (device).
-size_t confirm_workspace_bytes_single(const DevGeom &G, int n, int cap);
+size_t confirm_workspace_bytes_single(int n);
 cudaError_t launch_confirm(const DevGeom &G, const ConfirmDev &P, const float *x, const float *y,
                            const uint8_t *layer, int n, const ht_peak *peaks, const int *d_count,
                            int cap, int *score, int *inl, int *assign, void *ws, cudaStream_t st);

@@ -16,17 +16,30 @@
 // Then each hit goes to the confirmed candidate that lists it with the most
 // inlier layers, ties to the smallest candidate index.
 //
-// One warp per candidate, persistent over the candidates of a batch grouped
-// by (event, column group).  A candidate scans only the hits of each layer
-// whose azimuth can give a root near its bin (a per-event index by layer and
-// azimuth, k_hitindex.cu; a superset of the pool).  Each of those hits
-// gets the vote's exact bin decision (guarded float32, then double-float,
-// then float64 in the definition's operation order), so own and pool
-// membership are exactly the vote's.  The seed circle is float64 in the definition's order;
-// distances are estimated in float32 with an error bound, and the float64
-// distance of the definition is computed for every hit the bound cannot
-// settle, so every decision is the definition's.  The results are
-// bit-identical to the float64 plain definition.
+// A warp per candidate, persistent over the batch's candidates, on the hit
+// index by layer and azimuth (k_hitindex.cu).  Nearly every candidate fails,
+// so the work goes in the order that lets it fail early:
+//  1. the own hits: only the azimuth cells whose hits can have a root in the
+//     candidate's one bin (about a quarter of its pool's); own(h) from the
+//     signs of the circle equation at the bin's two edges;
+//  2. the seed circle's float32 frame, for up to 32 candidates at once, a
+//     lane each (its float64 products would otherwise take the float64 pipe
+//     a warp at a time);
+//  3. the cells that circle crosses on every layer, and the float32 distance
+//     of their hits with an error bound: hits on fewer than min_layers
+//     layers end the candidate;
+//  4. only then pool(h), per-layer contenders, and the float64 distance of
+//     the definition where the bound cannot settle a layer.
+// Every decision that float32 cannot prove is the vote's exact bin decision
+// (double-float, then float64 in the definition's operation order) or the
+// definition's float64 distance, so the results are bit-identical to the
+// float64 plain definition.
+//
+// Bound by latency and issue (59% of slots; index loads and fixed latencies
+// lead the stalls): 1540 warp instructions per candidate, where scanning and
+// binning the whole pool (435 hits) with a frame per warp took 6800.  Stage on
+// GB300: 25 events of 2k-60k hits (1.25 M candidates) 11.7 -> 2.3 ms, 25 of 10k
+// hits (2.7 M) 16.7 -> 4.6, two of 50k (512 x 256 x 1024) 8.7 -> 1.6.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -180,11 +193,20 @@ __device__ __forceinline__ bool seed_frame(float x1, float y1, float x2, float y
 }
 
 constexpr int kCfThreads = 128, kCfWarps = kCfThreads / 32;
-constexpr int kCfCap = 384;        // pool hits held per pass (more: further passes)
-constexpr int kCfBlk = 256;        // 32-hit blocks of a scan whose pool counts are kept
+constexpr int kCfCap = 128;        // hits near the circle held per pass (more: further passes)
+constexpr int kCfChunk = 32;       // candidates of a warp's chunk, at most
+
+// A candidate's seeds and, once computed, its float32 seed frame with the
+// circle's implicit form |P|^2 kap - 2 P.g + h = 0, g = kap P1 + n (towards
+// the centre from the origin), h = kap |P1|^2 + 2 P1.n.
+struct CfSeed {
+    int pa, pb, pc, ev;     // index positions (pa < 0: none), event
+    SeedFrame F;
+    float psi, gn, h;       // azimuth and length of g
+};
 
 struct CfWarp {
-    int n_own[16], own_pos[16];
+    int own_pos[16];
     int best_h[16];
     double best_d[16];
     // per layer, over the pool hits of the pass: least lower and upper bound
@@ -192,38 +214,59 @@ struct CfWarp {
     // pass's positions [qs, qe) (the pool is in layer order)
     unsigned lbmin[16], ubmin[16];
     int ncont[16], cq[16], qs[16], qe[16];
-    int rs[32], rp[33];     // runs of index positions scanned: start, exclusive prefix of lengths
-    unsigned short blk[kCfBlk];   // pool hits of each 32-hit block of the first pass
+    int2 rr[32];            // non-empty runs scanned: start less the positions before it, layer
     int pool_p[kCfCap], pool_h[kCfCap];   // index position and event-local hit index
     float pool_lo[kCfCap], pool_hi[kCfCap];   // bounds on the hit's float64 distance
     unsigned char pool_l[kCfCap];
-    SeedFrame F;            // the candidate's float32 seed frame
-    double xc, yc, R;       // and its float64 seed circle, once computed
-    int seed_pos[3];        // index positions of the three seed hits
+    double xc, yc, R;       // the float64 seed circle, once computed
+    CfSeed seed[kCfChunk];
 };
 
 // The warps' state of k_confirm (at namespace scope, so that the functions
 // that take a warp's index address it as shared memory).
 __shared__ CfWarp g_cfw[kCfWarps];
 
-// The hits a candidate scans: the t-th of the runs W.rs / W.rp of the
-// event's hit index (k_hitindex.cu).
-struct HitView {
-    const float *x, *y;
-    const int *h;
-    const uint8_t *l;
-    int wid;   // the warp's state in g_cfw
-    int n;     // total positions
+// The hits a candidate scans: runs of positions of the event's hit index
+// (k_hitindex.cu), lane r's run being [start, start + len).  Position t of
+// the sequence belongs to the run that covers it; at(base) gives every
+// lane its position base + lane (p) and layer (l), or false past the end.
+struct Runs {
+    int excl, len, n;
+    int wid;
 
-    __device__ __forceinline__ int pos(int t) const
+    __device__ __forceinline__ void set(int start, int len_, int layer, int wid_, int lane)
     {
-        int lo = 0, hi = 31;   // the last run r with rp[r] <= t
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (g_cfw[wid].rp[mid] <= t) lo = mid;
-            else hi = mid - 1;
+        constexpr unsigned kAll = 0xffffffffu;
+        wid = wid_;
+        len = len_;
+        int incl = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kAll, incl, o);
+            if (lane >= o) incl += v;
         }
-        return g_cfw[wid].rs[lo] + (t - g_cfw[wid].rp[lo]);
+        excl = incl - len;
+        n = __shfl_sync(kAll, incl, 31);
+        const unsigned ne = __ballot_sync(kAll, len > 0);
+        __syncwarp();   // the previous runs' readers are done
+        if (len > 0)
+            g_cfw[wid].rr[__popc(ne & ((1u << lane) - 1u))] = make_int2(start - excl, layer);
+        __syncwarp();
+    }
+
+    __device__ __forceinline__ bool at(int base, int lane, int &p, int &l) const
+    {
+        constexpr unsigned kAll = 0xffffffffu;
+        const int d = excl - base;
+        const unsigned m = __reduce_or_sync(kAll, len > 0 && d > 0 && d < 32 ? 1u << d : 0u);
+        const int c0 = __popc(__ballot_sync(kAll, len > 0 && d <= 0)) - 1;
+        const bool ok = base + lane < n;
+        if (ok) {
+            const int2 r = g_cfw[wid].rr[c0 + __popc(m & (kAll >> (31 - lane)))];
+            p = r.x + base + lane;
+            l = r.y;
+        }
+        return ok;
     }
 };
 
@@ -240,10 +283,9 @@ __device__ __forceinline__ int event_of(const int *cpre, int n_ev, int f)
     return lo;
 }
 
-// Azimuth window of the hits of one layer that can have a root within
-// d0 in [lo, hi] (cm) in column (rho, phi0_k); returns its runs of index
-// cells as bins [b0, b1] (b1 - b0 + 1 >= kIdxAz or full: the whole layer;
-// empty: no hit can).  A root d0 of the circle equation gives
+// Azimuth window [w0, w1] (radians, near phik) of the hits of one layer that
+// can have a root within d0 in [lo, hi] (cm) in column (rho, phi0_k); full:
+// any hit of the layer, empty: none.  A root d0 of the circle equation gives
 //   s = -(2 d0 + rho (d0^2 + r^2)) / (2 u),   u = 1 + rho d0,
 // with ds/dd0 = -(u^2 + 1 - rho^2 r^2) / (2 u^2) and ds/d(r^2) = -rho / (2 u):
 // for u > 0, s is monotone in r^2 (sign -rho), and in d0 (decreasing) while
@@ -258,11 +300,11 @@ __device__ __forceinline__ int event_of(const int *cpre, int n_ev, int f)
 // proven the whole layer is scanned.
 __device__ __forceinline__ void layer_window(float rho, float phik, float lo, float hi,
                                              float rmin, float rmax, bool &full, bool &empty,
-                                             int &b0, int &b1)
+                                             float &w0, float &w1)
 {
     full = false;
     empty = !(rmin <= rmax);
-    b0 = b1 = 0;
+    w0 = w1 = 0.0f;
     if (empty) return;
     const float tl = fmaf(rho, lo, 1.0f), th = fmaf(rho, hi, 1.0f);
     const float tmin = fminf(tl, th);
@@ -297,206 +339,299 @@ __device__ __forceinline__ void layer_window(float rho, float phik, float lo, fl
         empty = true;
         return;
     }
-    const float dmax = asinf(fminf(a_hi, 1.0f)), dmin = asinf(fmaxf(a_lo, -1.0f));
-    const float k = kIdxAz / 6.28318531f;
-    b0 = (int)floorf((phik - dmax - 2e-3f + 3.14159265f) * k);
-    b1 = (int)floorf((phik - dmin + 2e-3f + 3.14159265f) * k);
-    if (b1 - b0 + 1 >= kIdxAz) full = true;
+    w0 = phik - asinf(fminf(a_hi, 1.0f)) - 2e-3f;
+    w1 = phik - asinf(fmaxf(a_lo, -1.0f)) + 2e-3f;
 }
 
-// One pass over a candidate's hit sequence: collects the pool hits of rank
-// [r0, r0 + kCfCap) into the warp's list (in sequence order) and, when
-// count_own (the first pass, r0 = 0), the own hits per layer.  Returns the
-// total number of pool hits (first pass).  Every scanned hit gets the
-// vote's exact bin decision in the candidate's column, one hit per lane
-// (the index windows already hold few hits far from the pool, so no cheaper
-// screen pays for itself).  The first pass keeps each 32-hit block's pool
-// count, so a later pass evaluates only the blocks whose pool hits can fall
-// in its rank range.
-__device__ __noinline__ int scan_pool(const DevGeom &G, const HitView V, int i, int j, int k,
-                                      int pool, int r0, bool count_own, int lane)
+// Azimuth window [w0, w1] of the hits of one layer (radii in [rmin, rmax])
+// with c > 0 in the column at phik whose distance from the seed circle is
+// below tolw.  On the circle's implicit form a point at signed distance t
+// gives kap |P|^2 - 2 P.g + h = t (2 + kap t), so with q = cos(psi_hit - psi)
+//   |kap r^2 + h - 2 r |g| q| <= T,   T = tolw (2 + kap tolw):
+// q lies between (kap r + (h -+ T) / r) / (2 |g|) at the ends of the radius
+// range, or at the interior minimum sqrt(kap h) / |g| of kap r + h / r, and
+// the hit on either side of psi.  Each side is kept where it meets the
+// half-plane c > 0, their hull is the window.  Margins: 4e-6 of the terms'
+// sizes and 1e-5 cm on T (float32 rounding of g and h and of the sums), and
+// 2e-3 rad on the azimuth (acos near 1 for argument errors below 2e-6).
+__device__ __forceinline__ void circle_window(const CfSeed &C, float phik, float tolw, float rmin,
+                                              float rmax, bool &full, bool &empty, float &w0,
+                                              float &w1)
 {
-    CfWarp &W = g_cfw[V.wid];
+    constexpr float kHalf = 1.57079633f + 4e-3f;   // c > 0, with a margin
+    full = false;
+    empty = !(rmin <= rmax);
+    w0 = phik - kHalf;
+    w1 = phik + kHalf;
+    if (empty) return;
+    const float k = C.F.kap, x1 = C.F.x1, y1 = C.F.y1;
+    if (!(rmin >= 1e-3f) || !(C.gn >= 1e-3f) || !(C.F.B0 < 1e30f)) {
+        full = true;
+        return;
+    }
+    const float p1 = fabsf(x1) + fabsf(y1), W = rmax + p1;
+    const float tw = tolw + fmaf(C.F.B2, W * W, fmaf(2.0f * C.F.B1, W, C.F.B0));
+    const float T = fmaf(tw, fmaf(k, tw, 2.0f), 1e-5f) +
+                    4e-6f * (k * fmaf(rmax, rmax, p1 * p1) + 2.0f * p1 + 2.0f * rmax * C.gn);
+    const float ig = 0.5f / C.gn;
+    const float ia = 1.0f / rmin, ib = 1.0f / rmax;
+    const float qa = fmaf(k, rmin, C.h * ia), qb = fmaf(k, rmax, C.h * ib);
+    float lo = fminf(qa, qb);
+    if (C.h > k * rmin * rmin && C.h < k * rmax * rmax) lo = fminf(lo, 1.9999f * sqrtf(k * C.h));
+    const float qlo = fmaf(-T, ia, lo) * ig - 2e-6f;
+    const float qhi = fmaf(T, ia, fmaxf(qa, qb)) * ig + 2e-6f;
+    if (qlo > 1.0f || qhi < -1.0f) {
+        empty = true;
+        return;
+    }
+    const float a1 = acosf(fminf(qhi, 1.0f)), a2 = acosf(fmaxf(qlo, -1.0f));
+    if (!(a2 - a1 <= 1.0f)) return;   // wide: every hit with c > 0
+    const float mid = 0.5f * (a1 + a2), hw = 0.5f * (a2 - a1) + 2e-3f;
+    float l0 = 1e9f, h0 = -1e9f;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        float d = (side ? C.psi - mid : C.psi + mid) - phik;   // to [-pi, pi]
+        d = fmaf(-6.28318531f, rintf(d * 0.159154943f), d);
+        const float a = fmaxf(d - hw, -kHalf), b = fminf(d + hw, kHalf);
+        if (a <= b) {
+            l0 = fminf(l0, a);
+            h0 = fmaxf(h0, b);
+        }
+    }
+    empty = !(l0 <= h0);
+    w0 = phik + l0;
+    w1 = phik + h0;
+}
+
+// Lane (layer l, part) of a layer's window as a run of index positions: the
+// window's cells, in two parts when they wrap.
+__device__ __forceinline__ void window_run(const int *__restrict__ offs, int cell0, int part,
+                                           bool full, bool empty, float w0, float w1, int &start,
+                                           int &len)
+{
+    start = len = 0;
+    if (empty) return;
+    const float k = kIdxAz / 6.28318531f;
+    const int b0 = (int)floorf((w0 + 3.14159265f) * k), b1 = (int)floorf((w1 + 3.14159265f) * k);
+    const int nb = b1 - b0 + 1;
+    const int *o = offs + cell0;
+    int a = 0, b = kIdxAz;   // cells [a, b)
+    if (full || nb >= kIdxAz) {
+        if (part) return;
+    } else {
+        const int b0m = b0 & (kIdxAz - 1);
+        const bool wrap = b0m + nb > kIdxAz;
+        if (part && !wrap) return;
+        a = part ? 0 : b0m;
+        b = part ? b0m + nb - kIdxAz : wrap ? kIdxAz : b0m + nb;
+    }
+    start = o[a];
+    len = o[b] - start;
+}
+
+// Whether the root of a hit in column (rho, phi0) that grows through F = 0 is
+// between da and db (cm): F(d) = rho d^2 + 2 (1 + rho s) d + rho r^2 + 2 s of
+// the circle equation is linear in s and r^2, so its signs at the two ends
+// decide, without a square root.  dF/dd = 2 (1 + rho (s + d)), and where that
+// is positive at both ends F is monotone between them: one root there when
+// F(da) < 0 < F(db), else none (the other root, if any, is outside).
+// Returns 0 (no root), 1 (a root), or 2: too close to an end for float32,
+// or dF/dd or the sign of c not proven.  The bound is first order (u = 2^-24,
+// taken four times): s is within 3u R1, r^2 within 2u, the tables' rho within
+// u, da and db within 2u of themselves:
+//   u (11 R1 + 6 |rho| R1^2 + 12 dmax).
+struct EdgePair {
+    float ka, la, kb, lb, ma, mb, ce, rho;
+
+    __device__ __forceinline__ void init(const DevGeom &G, float rho_, int j0, int j1)
+    {
+        rho = rho_;
+        const float da = ((float)j0 - G.off_f) * G.delta_f, db = ((float)j1 - G.off_f) * G.delta_f;
+        ka = fmaf(rho * da, da, 2.0f * da);
+        kb = fmaf(rho * db, db, 2.0f * db);
+        la = fmaf(2.0f * rho, da, 2.0f);
+        lb = fmaf(2.0f * rho, db, 2.0f);
+        ma = fmaf(rho, da, 1.0f);
+        mb = fmaf(rho, db, 1.0f);
+        ce = 12.0f * G.dext_f;
+    }
+
+    __device__ __forceinline__ int root(float x, float y, float sk, float ck) const
+    {
+        const float s = fmaf(x, sk, -(y * ck)), c = fmaf(x, ck, y * sk);
+        const float R1 = fabsf(x) + fabsf(y);
+        const float Ec = (kSafe * 3.0f * kEps) * R1;
+        const float base = rho * fmaf(x, x, y * y);
+        const float Fa = fmaf(la, s, ka + base), Fb = fmaf(lb, s, kb + base);
+        const float e = (kSafe * kEps) * fmaf(fmaf(6.0f * fabsf(rho), R1, 11.0f), R1, ce);
+        const float m = fminf(fmaf(rho, s, ma), fmaf(rho, s, mb));
+        if (c < -Ec) return 0;
+        if (!(c > Ec && m > 0.05f)) return 2;
+        if (Fa > e || Fb < -e) return 0;
+        return Fa < -e && Fb > e ? 1 : 2;
+    }
+};
+
+// The same by the vote's exact bin decision: a bin in [j0, j1).
+static __device__ __noinline__ bool exact_root(const DevGeom &G, int i, int k, float x, float y,
+                                               int j0, int j1)
+{
     ColumnCtx C;
     C.init(G, i, k);
-    const unsigned lt = (1u << lane) - 1u;
-    int rank = 0;
-    for (int base = 0; base < V.n; base += 32) {
-        const int b = base >> 5;
-        if (!count_own && b < kCfBlk) {   // uniform
-            const int cnt = W.blk[b];
-            if (rank + cnt <= r0) {
-                rank += cnt;
-                continue;
-            }
-            if (rank >= r0 + kCfCap) break;
-        }
-        const int t = base + lane;
-        int p = -1, l = 0;
-        bool own = false, inp = false;
-        if (t < V.n) {
-            p = V.pos(t);
-            int jj[2];
-            const int nv = column_bins(G, C, V.x[p], V.y[p], jj);
-            for (int v = 0; v < nv; ++v) {
-                own |= jj[v] == j;
-                inp |= abs(jj[v] - j) <= pool;
-            }
-            if (inp) l = V.l[p];
-        }
-        if (count_own && own) {
-            atomicAdd(&W.n_own[l], 1);
-            W.own_pos[l] = p;   // read only where the layer holds exactly one own hit
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, inp);
-        const int r = rank + __popc(bal & lt);
-        if (inp && r >= r0 && r < r0 + kCfCap) {
-            W.pool_p[r - r0] = p;
-            W.pool_h[r - r0] = V.h[p];
-            W.pool_l[r - r0] = (unsigned char)l;
-        }
-        if (count_own && lane == 0 && b < kCfBlk) W.blk[b] = (unsigned short)__popc(bal);
-        rank += __popc(bal);
-    }
-    __syncwarp();
-    return rank;
+    int jj[2];
+    const int nv = column_bins(G, C, x, y, jj);
+    bool in = false;
+    for (int v = 0; v < nv; ++v) in |= jj[v] >= j0 && jj[v] < j1;
+    return in;
 }
 
-// The runs of index positions a candidate of event e in column (rho_i,
-// phi0_k) with bin j scans: per layer its azimuth window (layer_window) for
-// d0 within two bins beyond the pool, as one or two runs of cells (the
-// window may wrap); lane r takes run r = 2 l + part.
-__device__ __forceinline__ void candidate_runs(const DevGeom &G, const ConfirmDev &P,
-                                               const HitIndex &I, int e, int i, int j, int k,
-                                               CfWarp &W, HitView &V, int lane)
+// The seeds of one candidate of event e: scans, per layer, the hits whose
+// azimuth can give a root in its bin, and takes the layers with one own hit.
+__device__ __forceinline__ void find_seeds(const DevGeom &G, const ConfirmDev &P,
+                                           const HitIndex &I, int e, const ht_peak pk, CfSeed &out,
+                                           int wid, int lane)
 {
-    const int l = lane >> 1, part = lane & 1;
-    int start = 0, len = 0;
-    if (l < P.n_layers) {
-        const float lo = ((float)(j - P.pool - 2) - G.off_f) * G.delta_f;
-        const float hi = ((float)(j + P.pool + 3) - G.off_f) * G.delta_f;
-        const float rmin = __uint_as_float(I.rmm[2 * (e * 16 + l)]);
-        const float rmax = __uint_as_float(I.rmm[2 * (e * 16 + l) + 1]);
-        bool full, empty;
-        int b0, b1;
-        layer_window(G.rho32[i], G.phi32[k], lo, hi, rmin, rmax, full, empty, b0, b1);
-        const int base = (e * 16 + l) * kIdxAz;
-        if (full) {
-            if (part == 0) {
-                start = I.offs[base];
-                len = I.offs[base + kIdxAz] - start;
+    constexpr unsigned kAll = 0xffffffffu;
+    CfWarp &W = g_cfw[wid];
+    const float rho = G.rho32[pk.i_rho], phik = G.phi32[pk.k_phi0];
+    Runs R;
+    {
+        const int l = lane >> 1;
+        int start = 0, len = 0;
+        if (l < P.n_layers) {
+            // the bin's edges, a hundredth of a bin and 1e-4 cm beyond
+            const float jo = (float)pk.j_d0 - G.off_f;
+            const float lo = fmaf(jo - 0.01f, G.delta_f, -1e-4f);
+            const float hi = fmaf(jo + 1.01f, G.delta_f, 1e-4f);
+            const float rmin = __uint_as_float(I.rmm[2 * (e * 16 + l)]);
+            const float rmax = __uint_as_float(I.rmm[2 * (e * 16 + l) + 1]);
+            bool full, empty;
+            float w0, w1;
+            layer_window(rho, phik, lo, hi, rmin, rmax, full, empty, w0, w1);
+            window_run(I.offs, (e * 16 + l) * kIdxAz, lane & 1, full, empty, w0, w1, start, len);
+        }
+        R.set(start, len, l, wid, lane);
+    }
+    const float sk = G.sn32[pk.k_phi0], ck = G.cs32[pk.k_phi0];
+    EdgePair E;
+    E.init(G, rho, pk.j_d0, pk.j_d0 + 1);
+    unsigned once = 0u, twice = 0u;   // layers with an own hit, with more
+    for (int base = 0; base < R.n; base += 32) {
+        int p = 0, l = 0;
+        int st = 0;
+        if (R.at(base, lane, p, l)) {
+            const float x = I.x[p], y = I.y[p];
+            st = E.root(x, y, sk, ck);
+            if (st == 2)
+                st = exact_root(G, pk.i_rho, pk.k_phi0, x, y, pk.j_d0, pk.j_d0 + 1) ? 1 : 0;
+        }
+        const bool own = st == 1;
+        const unsigned bo = __ballot_sync(kAll, own);
+        if (bo) {
+            const unsigned m = __reduce_or_sync(kAll, own ? 1u << l : 0u);
+            if (__popc(bo) != __popc(m)) {   // a layer twice in this step
+                const unsigned peers = __match_any_sync(kAll, own ? l : 32 + lane);
+                twice |= __reduce_or_sync(kAll, own && __popc(peers) > 1 ? 1u << l : 0u);
             }
-        } else if (!empty) {
-            const int b0m = ((b0 % kIdxAz) + kIdxAz) % kIdxAz, nb = b1 - b0 + 1;
-            if (b0m + nb <= kIdxAz) {
-                if (part == 0) {
-                    start = I.offs[base + b0m];
-                    len = I.offs[base + b0m + nb] - start;
-                }
-            } else if (part == 0) {
-                start = I.offs[base + b0m];
-                len = I.offs[base + kIdxAz] - start;
-            } else {
-                start = I.offs[base];
-                len = I.offs[base + b0m + nb - kIdxAz] - start;
-            }
+            twice |= once & m;
+            once |= m;
+            if (own) W.own_pos[l] = p;   // read only where the layer holds exactly one own hit
         }
     }
-    int incl = len;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    W.rs[lane] = start;
-    W.rp[lane + 1] = incl;
-    if (lane == 0) W.rp[0] = 0;
     __syncwarp();
-    V.n = W.rp[32];
+    // the first, the last, and the layer between them nearest their middle
+    // (the smaller on a tie)
+    const unsigned seeds = once & ~twice;
+    int pa = -1, pb = -1, pc = -1;
+    if (__popc(seeds) >= 3) {
+        const int la = __ffs(seeds) - 1, lc = 31 - __clz(seeds), t2 = la + lc;
+        const unsigned inner = seeds & ~(1u << la) & ~(1u << lc);
+        const unsigned low = inner & ((2u << (t2 >> 1)) - 1u), high = inner & ~low;
+        const int l1 = 31 - __clz(low), l2 = __ffs(high) - 1;   // -1: none
+        const int lb = !high ? l1 : !low ? l2 : t2 - 2 * l1 <= 2 * l2 - t2 ? l1 : l2;
+        pa = W.own_pos[la];
+        pb = W.own_pos[lb];
+        pc = W.own_pos[lc];
+    }
+    if (lane == 0) {
+        out.pa = pa;
+        out.pb = pb;
+        out.pc = pc;
+        out.ev = e;
+    }
+    __syncwarp();   // own_pos is reused
 }
 
-// Confirmation of one candidate by one warp (see the file comment).  Writes
-// score[slot] (0 = not confirmed) and inl[16 slot + l].
+// The seed frame of one candidate (a lane per candidate: the float64
+// products of up to 32 candidates at once).
+__device__ __forceinline__ void make_frame(const HitIndex &I, CfSeed &C)
+{
+    if (C.pa < 0) return;
+    SeedFrame F;
+    if (!seed_frame(I.x[C.pa], I.y[C.pa], I.x[C.pb], I.y[C.pb], I.x[C.pc], I.y[C.pc], F)) {
+        C.pa = -1;
+        return;
+    }
+    const float gx = fmaf(F.kap, F.x1, F.nx), gy = fmaf(F.kap, F.y1, F.ny);
+    C.F = F;
+    C.psi = atan2f(gy, gx);
+    C.gn = sqrtf(fmaf(gx, gx, gy * gy));
+    C.h = fmaf(F.kap, fmaf(F.x1, F.x1, F.y1 * F.y1), 2.0f * fmaf(F.x1, F.nx, F.y1 * F.ny));
+}
+
+// Confirmation of one candidate with a seed frame, by one warp.  Returns the
+// number of inlier layers when it is confirmed (W.best_h[l] of lanes with
+// in_l: the inlier hits), else 0.
 //
-// Distances: the float32 estimate of seed_frame and its bound give every
-// pool hit an interval [lo, hi] holding its float64 distance.  Per layer
-// the contenders are the hits with lo at most the layer's least hi and
-// below tol; the layer's nearest hit is one of them.  A layer without a
+// Distances: the float32 estimate of seed_frame and its bound give a hit an
+// interval [lo, hi] holding its float64 distance.  Only hits with lo below
+// tol can be inliers: the scan, over the azimuth cells the circle crosses,
+// keeps those, and where they lie on fewer than min_layers layers the
+// candidate is not confirmed.  Otherwise the pool's hits among them are
+// found, and per layer the contenders: the hits with lo at most the layer's
+// least hi; the layer's nearest hit is one of them.  A layer without a
 // contender has no inlier, a single contender certainly below tol is the
-// inlier, and otherwise the float64 distances of the contenders decide
-// (the definition's seed circle is computed then, once per candidate).
-// When fewer than min_layers layers can hold an inlier the candidate is not
-// confirmed, without any float64 distance.  Pools larger than kCfCap go in
-// passes of kCfCap hits, every contender by its float64 distance.
-__device__ __forceinline__ void confirm_one(const DevGeom &G, const ConfirmDev &P,
-                                            const HitIndex &I, int e, const ht_peak pk,
-                                            size_t slot, float tol_lo, float tol_hi,
-                                            int *__restrict__ score, int *__restrict__ inl,
-                                            int wid, int lane)
+// inlier, and otherwise the float64 distances of the contenders decide (the
+// definition's seed circle is computed then, once per candidate).  More than
+// kCfCap hits go in passes of kCfCap, every contender by its float64
+// distance.
+__device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P,
+                                           const HitIndex &I, const ht_peak pk, const CfSeed &C,
+                                           float tol_lo, float tol_hi, int wid, int lane,
+                                           bool &in_l)
 {
     CfWarp &W = g_cfw[wid];
     constexpr unsigned kAll = 0xffffffffu;
     const float kInf = __int_as_float(0x7f800000);
-    HitView V{I.x, I.y, I.h, I.l, wid, 0};
-    candidate_runs(G, P, I, e, pk.i_rho, pk.j_d0, pk.k_phi0, W, V, lane);
-    if (lane < 16) {
-        W.n_own[lane] = 0;
-        W.best_h[lane] = -1;
-        W.best_d[lane] = 0.0;
-    }
-    __syncwarp();
-    const long long tol_bits = __double_as_longlong(P.tol);
-    const SeedFrame &F = W.F;
-    bool ok = false, exact = false, rejected = false;
-    const int npool = scan_pool(G, V, pk.i_rho, pk.j_d0, pk.k_phi0, P.pool, 0, true, lane);
+    const int e = C.ev;
+    const float rho = G.rho32[pk.i_rho], phik = G.phi32[pk.k_phi0];
+    Runs R;
     {
-        // seed layers (every lane computes the same)
-        int la = -1, lb = -1, lc = -1, ns = 0;
-        for (int l = 0; l < P.n_layers; ++l)
-            if (W.n_own[l] == 1) {
-                if (la < 0) la = l;
-                lc = l;
-                ++ns;
-            }
-        int gap = 1 << 30;
-        for (int l = la + 1; ns >= 3 && l < lc; ++l)
-            if (W.n_own[l] == 1 && abs(2 * l - (la + lc)) < gap) {
-                gap = abs(2 * l - (la + lc));
-                lb = l;
-            }
-        if (ns >= 3) {
-            if (lane == 0) {
-                const int pa = W.own_pos[la], pb = W.own_pos[lb], pc = W.own_pos[lc];
-                const bool f = seed_frame(V.x[pa], V.y[pa], V.x[pb], V.y[pb], V.x[pc], V.y[pc], W.F);
-                W.seed_pos[0] = f ? pa : -1;
-                W.seed_pos[1] = pb;
-                W.seed_pos[2] = pc;
-            }
-            __syncwarp();
-            ok = W.seed_pos[0] >= 0;
+        const int l = lane >> 1;
+        int start = 0, len = 0;
+        if (l < P.n_layers) {
+            const float rmin = __uint_as_float(I.rmm[2 * (e * 16 + l)]);
+            const float rmax = __uint_as_float(I.rmm[2 * (e * 16 + l) + 1]);
+            bool full, empty;
+            float w0, w1;
+            circle_window(C, phik, tol_hi, rmin, rmax, full, empty, w0, w1);
+            window_run(I.offs, (e * 16 + l) * kIdxAz, lane & 1, full, empty, w0, w1, start, len);
         }
+        R.set(start, len, l, wid, lane);
     }
-    for (int r0 = 0; ok && r0 < npool; r0 += kCfCap) {
-        if (r0 > 0) scan_pool(G, V, pk.i_rho, pk.j_d0, pk.k_phi0, P.pool, r0, false, lane);
-        const bool single = npool <= kCfCap;
-        const int nq = min(npool - r0, kCfCap);
-        if (lane < 16) {
-            W.lbmin[lane] = W.ubmin[lane] = 0x7f800000u;   // +inf
-            W.ncont[lane] = 0;
-            W.qs[lane] = kCfCap;
-            W.qe[lane] = 0;
-        }
-        __syncwarp();
-        // the bounds of every pool hit, and their least values per layer
-        // (the pool is in layer order: each layer is one run of lanes)
-        for (int q0 = 0; q0 < nq; q0 += 32) {
-            const int q = q0 + lane;
-            int l = 16;
+    in_l = false;
+    const SeedFrame F = C.F;
+    int total = 0;
+    // hits of rank [r0, r0 + kCfCap) near the circle, in layer order; returns
+    // their layers
+    auto scan = [&](int r0) {
+        unsigned lm = 0u;
+        int rank = 0;
+        for (int base = 0; base < R.n; base += 32) {
+            int p = 0, l = 0;
             float lo = kInf, hi = kInf;
-            if (q < nq) {
-                const int p = W.pool_p[q];
-                l = W.pool_l[q];
-                const float wx = V.x[p] - F.x1, wy = V.y[p] - F.y1;
+            if (R.at(base, lane, p, l)) {
+                const float wx = I.x[p] - F.x1, wy = I.y[p] - F.y1;
                 const float w2 = fmaf(wx, wx, wy * wy);
                 const float wn = fmaf(wx, F.nx, wy * F.ny);
                 const float num = fmaf(F.kap, w2, -2.0f * wn);
@@ -506,10 +641,80 @@ __device__ __forceinline__ void confirm_one(const DevGeom &G, const ConfirmDev &
                 const float dl = __fsub_rd(d, er);
                 lo = dl > 0.0f ? dl : 0.0f;   // +0 (the bits order as the values)
                 hi = __fadd_ru(d, er);
-                W.pool_lo[q] = lo;
-                W.pool_hi[q] = hi;
             }
-            float slo = lo, shi = hi;
+            const bool near = lo < tol_hi;
+            const unsigned bal = __ballot_sync(kAll, near);
+            if (!bal) continue;
+            const int r = rank + __popc(bal & ((1u << lane) - 1u)) - r0;
+            if (near && r >= 0 && r < kCfCap) {
+                W.pool_p[r] = p;
+                W.pool_l[r] = (unsigned char)l;
+                W.pool_lo[r] = lo;
+                W.pool_hi[r] = hi;
+            }
+            lm |= __reduce_or_sync(kAll, near ? 1u << l : 0u);
+            rank += __popc(bal);
+        }
+        total = rank;
+        return lm;
+    };
+    if (__popc(scan(0)) < P.min_layers) return 0;
+    if (lane < 16) {
+        W.best_h[lane] = -1;
+        W.best_d[lane] = 0.0;
+    }
+    const long long tol_bits = __double_as_longlong(P.tol);
+    const bool single = total <= kCfCap;
+    const int jp0 = max(pk.j_d0 - P.pool, 0), jp1 = min(pk.j_d0 + P.pool + 1, G.n_d0);
+    EdgePair E;
+    E.init(G, rho, jp0, jp1);
+    const float sk = G.sn32[pk.k_phi0], ck = G.cs32[pk.k_phi0];
+    bool exact = false;
+    for (int r0 = 0; r0 < total; r0 += kCfCap) {
+        if (r0 > 0) scan(r0);
+        int nq = min(total - r0, kCfCap);
+        __syncwarp();
+        // the pool's hits among them, kept in order
+        int kept = 0;
+        for (int q0 = 0; q0 < nq; q0 += 32) {
+            const int q = q0 + lane;
+            int p = 0, st = 0;
+            unsigned char l = 0;
+            float lo = 0.0f, hi = 0.0f;
+            if (q < nq) {
+                p = W.pool_p[q];
+                l = W.pool_l[q];
+                lo = W.pool_lo[q];
+                hi = W.pool_hi[q];
+                const float x = I.x[p], y = I.y[p];
+                st = E.root(x, y, sk, ck);
+                if (st == 2) st = exact_root(G, pk.i_rho, pk.k_phi0, x, y, jp0, jp1) ? 1 : 0;
+            }
+            const unsigned bal = __ballot_sync(kAll, st == 1);
+            if (st == 1) {
+                const int r = kept + __popc(bal & ((1u << lane) - 1u));
+                W.pool_p[r] = p;   // r <= q: read before
+                W.pool_l[r] = l;
+                W.pool_lo[r] = lo;
+                W.pool_hi[r] = hi;
+                W.pool_h[r] = I.h[p];
+            }
+            kept += __popc(bal);
+            __syncwarp();
+        }
+        nq = kept;
+        if (lane < 16) {
+            W.lbmin[lane] = W.ubmin[lane] = 0x7f800000u;   // +inf
+            W.ncont[lane] = 0;
+            W.qs[lane] = kCfCap;
+            W.qe[lane] = 0;
+        }
+        __syncwarp();
+        // the least bounds per layer (each layer is one run of positions)
+        for (int q0 = 0; q0 < nq; q0 += 32) {
+            const int q = q0 + lane;
+            const int l = q < nq ? W.pool_l[q] : 16;
+            float slo = q < nq ? W.pool_lo[q] : kInf, shi = q < nq ? W.pool_hi[q] : kInf;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const float olo = __shfl_down_sync(kAll, slo, o);
@@ -532,15 +737,11 @@ __device__ __forceinline__ void confirm_one(const DevGeom &G, const ConfirmDev &
         if (single) {
             // layers that can hold an inlier at all: too few, not confirmed
             const bool can = lane < P.n_layers && __uint_as_float(W.lbmin[lane]) < tol_hi;
-            if (__popc(__ballot_sync(kAll, can)) < P.min_layers) {
-                rejected = true;
-                break;
-            }
+            if (__popc(__ballot_sync(kAll, can)) < P.min_layers) return 0;
         }
         for (int q = lane; q < nq; q += 32) {
             const int l = W.pool_l[q];
-            const float lo = W.pool_lo[q];
-            if (lo <= __uint_as_float(W.ubmin[l]) && lo < tol_hi) {
+            if (W.pool_lo[q] <= __uint_as_float(W.ubmin[l])) {
                 atomicAdd(&W.ncont[l], 1);
                 W.cq[l] = q;   // read only where the layer has one contender
             }
@@ -558,11 +759,9 @@ __device__ __forceinline__ void confirm_one(const DevGeom &G, const ConfirmDev &
         }
         const unsigned need_m = __ballot_sync(kAll, need);
         if (need_m != 0u && !exact) {
-            if (lane == 0) {
-                const int pa = W.seed_pos[0], pb = W.seed_pos[1], pc = W.seed_pos[2];
-                circle3((double)V.x[pa], (double)V.y[pa], (double)V.x[pb], (double)V.y[pb],
-                        (double)V.x[pc], (double)V.y[pc], W.xc, W.yc, W.R);
-            }
+            if (lane == 0)
+                circle3((double)I.x[C.pa], (double)I.y[C.pa], (double)I.x[C.pb], (double)I.y[C.pb],
+                        (double)I.x[C.pc], (double)I.y[C.pc], W.xc, W.yc, W.R);
             __syncwarp();
             exact = true;
         }
@@ -572,10 +771,9 @@ __device__ __forceinline__ void confirm_one(const DevGeom &G, const ConfirmDev &
             long long bk = 0x7fffffffffffffffll;   // none: above every distance's bits
             int bh = -1;
             for (int q = W.qs[l] + lane; q < W.qe[l]; q += 32) {
-                const float lo = W.pool_lo[q];
-                if (!(lo <= ub && lo < tol_hi)) continue;
+                if (!(W.pool_lo[q] <= ub)) continue;
                 const int p = W.pool_p[q], h = W.pool_h[q];
-                const long long key = __double_as_longlong(circle_dist(V.x[p], V.y[p], W.xc, W.yc, W.R));
+                const long long key = __double_as_longlong(circle_dist(I.x[p], I.y[p], W.xc, W.yc, W.R));
                 if (key < bk || (key == bk && h < bh)) {
                     bk = key;
                     bh = h;
@@ -600,67 +798,65 @@ __device__ __forceinline__ void confirm_one(const DevGeom &G, const ConfirmDev &
         }
         __syncwarp();
     }
-    const bool in_l = ok && !rejected && lane < P.n_layers && W.best_h[lane] >= 0 &&
-                      __double_as_longlong(W.best_d[lane]) < tol_bits;
+    in_l = lane < P.n_layers && W.best_h[lane] >= 0 &&
+           __double_as_longlong(W.best_d[lane]) < tol_bits;
     const int sc = __popc(__ballot_sync(kAll, in_l));
-    const bool conf = ok && !rejected && sc >= P.min_layers;
-    if (lane < 16) inl[slot * 16 + lane] = conf && in_l ? W.best_h[lane] : -1;
-    if (lane == 0) score[slot] = conf ? sc : 0;
-    __syncwarp();
+    return sc >= P.min_layers ? sc : 0;
 }
 
-// Confirmation of every kept candidate of a batch.  The candidates are
-// ordered by (event, column group of kGroupCols columns) in order[] (flattened
-// indices; cpre is the exclusive prefix of the kept counts), so that the
-// consecutive candidates are nearby columns of one event; each warp takes
-// chunks of kCfChunk consecutive entries from a device counter (*head, zero
-// at launch) and confirms them one after another.  I: the batch's hit index
-// (k_hitindex.cu).
-constexpr int kCfChunk = 8;
-
-__global__ void __launch_bounds__(kCfThreads, 6)
-k_confirm(DevGeom G, ConfirmDev P, HitIndex I, const int *__restrict__ d_nev,
-          const ht_peak *__restrict__ peaks, int cap, const int *__restrict__ cpre,
-          const int *__restrict__ order, int *__restrict__ score, int *__restrict__ inl,
-          int *__restrict__ head)
+// Confirmation of every kept candidate of a batch (cpre: exclusive prefix of
+// the events' kept counts), persistent: each warp takes chunks of consecutive
+// candidates from a device counter (*head, zero at launch; as many as keep
+// every warp busy, at most kCfChunk).  Of a chunk it finds the seeds
+// candidate by candidate, the seed frames all at once (a lane each), then
+// confirms candidate by candidate.  A confirmed candidate's inliers offer
+// the key score << 32 | (2^32 - 1 - m) to their hits: the largest wins (most
+// inlier layers, then the smallest candidate index); gbest (batch hit index)
+// must be zero, k_assoc_final_batch decodes it.  score per slot (0 = not
+// confirmed); inl (may be null): 16 inlier hits per slot, -1 none.  I: the
+// batch's hit index (k_hitindex.cu).
+__global__ void __launch_bounds__(kCfThreads, 8)
+k_confirm(DevGeom G, ConfirmDev P, HitIndex I, const int *__restrict__ off,
+          const int *__restrict__ d_nev, const ht_peak *__restrict__ peaks, int cap,
+          const int *__restrict__ cpre, int *__restrict__ score, int *__restrict__ inl,
+          unsigned long long *__restrict__ gbest, int *__restrict__ head)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    CfWarp &W = g_cfw[wid];
     const int n_ev = *d_nev;
     const int total = cpre[n_ev];
+    const int chunk = min(max(total / (int)(gridDim.x * kCfWarps * 2), 1), kCfChunk);
     float tol_hi = (float)P.tol;   // tol rounded up to float32
     if ((double)tol_hi < P.tol) tol_hi = nextafterf(tol_hi, 3.0e38f);
     float tol_lo = (float)P.tol;   // and down
     if ((double)tol_lo > P.tol) tol_lo = nextafterf(tol_lo, 0.0f);
-    // each warp claims its own chunks (its state in g_cfw is private and it
-    // synchronises only itself), so a warp never waits for its CTA's others
     for (;;) {
         int c = 0;
         if (lane == 0) c = atomicAdd(head, 1);
-        const int t0 = __shfl_sync(0xffffffffu, c, 0) * kCfChunk;
-        if (t0 >= total) break;
-        const int t1 = min(t0 + kCfChunk, total);
-        for (int t = t0; t < t1; ++t) {
-            const int f = __ldg(order + t);
-            const int e = event_of(cpre, n_ev, f);
-            const size_t slot = (size_t)e * cap + (f - cpre[e]);
-            confirm_one(G, P, I, e, peaks[slot], slot, tol_lo, tol_hi, score, inl, warp, lane);
+        const long long t64 = (long long)__shfl_sync(0xffffffffu, c, 0) * chunk;
+        if (t64 >= total) break;
+        const int t0 = (int)t64, n = min(chunk, total - t0);
+        int e = event_of(cpre, n_ev, t0);
+        for (int q = 0; q < n; ++q) {
+            while (t0 + q >= cpre[e + 1]) ++e;   // t < cpre[n_ev]
+            find_seeds(G, P, I, e, peaks[(size_t)e * cap + (t0 + q - cpre[e])], W.seed[q], wid, lane);
         }
-    }
-}
-
-// Candidates of each (event, column group) item: counts, then positions.
-__global__ void k_cf_group(const int *__restrict__ d_nev, const int *__restrict__ cpre,
-                           const ht_peak *__restrict__ peaks, int cap, int ngroups,
-                           int *__restrict__ gcnt, int *__restrict__ gcur, int *__restrict__ order)
-{
-    const int n_ev = *d_nev;
-    const int total = cpre[n_ev];
-    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < total; f += gridDim.x * blockDim.x) {
-        const int e = event_of(cpre, n_ev, f);
-        const int k = peaks[(size_t)e * cap + (f - cpre[e])].k_phi0;
-        const int it = e * ngroups + k / kGroupCols;
-        if (gcur) order[atomicAdd(&gcur[it], 1)] = f;
-        else atomicAdd(&gcnt[it], 1);
+        if (lane < n) make_frame(I, W.seed[lane]);
+        __syncwarp();
+        for (int q = 0; q < n; ++q) {
+            const CfSeed &C = W.seed[q];
+            const int m = t0 + q - cpre[C.ev];
+            const size_t slot = (size_t)C.ev * cap + m;
+            bool in_l = false;
+            int sc = 0;
+            if (C.pa >= 0) sc = confirm_one(G, P, I, peaks[slot], C, tol_lo, tol_hi, wid, lane, in_l);
+            if (lane == 0) score[slot] = sc;
+            if (inl && lane < 16) inl[slot * 16 + lane] = sc > 0 && in_l ? W.best_h[lane] : -1;
+            if (sc > 0 && in_l)
+                atomicMax(&gbest[off[C.ev] + W.best_h[lane]],
+                          ((unsigned long long)sc << 32) | (0xffffffffull - (unsigned)m));
+            __syncwarp();
+        }
     }
 }
 
@@ -692,32 +888,6 @@ k_cand_prefix(const int *__restrict__ counts, const int *__restrict__ d_nev, int
     if (threadIdx.x == 1023) cpre[n_ev] = part[1023];
 }
 
-// Final assignment: every inlier of a confirmed candidate offers the key
-// score << 32 | (2^32 - 1 - m) to its hit; the largest wins (most inlier
-// layers, then the smallest candidate index).  gbest (batch hit index) must
-// be zero; k_assoc_final_batch decodes it.
-__global__ void k_confirm_offer(const int *__restrict__ off, const int *__restrict__ d_nev,
-                                const int *__restrict__ cpre, int cap,
-                                const int *__restrict__ score, const int *__restrict__ inl,
-                                unsigned long long *__restrict__ gbest)
-{
-    const int n_ev = *d_nev;
-    const long long total = (long long)cpre[n_ev] * 16;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const int f = (int)(t >> 4), l = (int)(t & 15);
-        const int e = event_of(cpre, n_ev, f);
-        const int m = f - cpre[e];
-        const size_t slot = (size_t)e * cap + m;
-        const int sc = score[slot];
-        if (sc <= 0) continue;
-        const int h = inl[slot * 16 + l];
-        if (h < 0) continue;
-        atomicMax(&gbest[off[e] + h],
-                  ((unsigned long long)sc << 32) | (0xffffffffull - (unsigned)m));
-    }
-}
-
 __global__ void k_single_offsets(int *__restrict__ off, int *__restrict__ nev, int n)
 {
     off[0] = 0;
@@ -730,31 +900,21 @@ __global__ void k_single_offsets(int *__restrict__ off, int *__restrict__ nev, i
 cudaError_t launch_assoc_final_batch(const unsigned long long *gbest, const int *off,
                                      const int *d_nev, int *assign, int max_hits, cudaStream_t st);
 
-size_t scan_tmp_bytes(int n_cap);
-cudaError_t scan_exclusive(const int *in, int *out, int *out2, int n_cap, const int *d_n,
-                           int *total, void *tmp, cudaStream_t st);
-
 namespace {
 
 struct CfWs {
-    int *cpre, *head, *gcnt, *gofs, *gcur, *order;
+    int *cpre, *head;
     unsigned long long *gbest;
-    void *tmp;
 };
 
-int cf_groups(const DevGeom &G) { return (G.n_phi0 + kGroupCols - 1) / kGroupCols; }
-
 // Carves (p non-null) or sizes the confirmation workspace.
-size_t cf_layout(const DevGeom &G, int max_events, int max_hits, int cap, char *p, CfWs *w)
+size_t cf_layout(int max_events, int max_hits, char *p, CfWs *w)
 {
-    const size_t ni = (size_t)max_events * cf_groups(G);
-    const size_t parts[] = {(size_t)(max_events + 1) * 4, 64, (size_t)(max_hits > 0 ? max_hits : 1) * 8,
-                            ni * 4, (ni + 1) * 4, (ni + 1) * 4,
-                            (size_t)max_events * (cap > 0 ? cap : 1) * 4,
-                            scan_tmp_bytes((int)ni)};
+    const size_t parts[] = {(size_t)(max_events + 1) * 4, 64,
+                            (size_t)(max_hits > 0 ? max_hits : 1) * 8};
     size_t at = 0;
-    char *q[8];
-    for (int i = 0; i < 8; ++i) {
+    char *q[3];
+    for (int i = 0; i < 3; ++i) {
         q[i] = p ? p + at : nullptr;
         at += align256(parts[i]);
     }
@@ -762,11 +922,6 @@ size_t cf_layout(const DevGeom &G, int max_events, int max_hits, int cap, char *
         w->cpre = reinterpret_cast<int *>(q[0]);
         w->head = reinterpret_cast<int *>(q[1]);
         w->gbest = reinterpret_cast<unsigned long long *>(q[2]);
-        w->gcnt = reinterpret_cast<int *>(q[3]);
-        w->gofs = reinterpret_cast<int *>(q[4]);
-        w->gcur = reinterpret_cast<int *>(q[5]);
-        w->order = reinterpret_cast<int *>(q[6]);
-        w->tmp = q[7];
     }
     return at;
 }
@@ -776,47 +931,38 @@ size_t cf_layout(const DevGeom &G, int max_events, int max_hits, int cap, char *
 cudaError_t prepare_confirm_kernels() { return cudaSuccess; }
 
 // Confirmation and final assignment of a batch (device offsets and event
-// count; idx: its hit index).  ws: confirm_workspace_bytes(G, max_events,
-// max_hits, cap).
-size_t confirm_workspace_bytes(const DevGeom &G, int max_events, int max_hits, int cap)
+// count; idx: its hit index; inl may be null).  ws: confirm_workspace_bytes(
+// max_events, max_hits).
+size_t confirm_workspace_bytes(int max_events, int max_hits)
 {
-    return cf_layout(G, max_events, max_hits, cap, nullptr, nullptr);
+    return cf_layout(max_events, max_hits, nullptr, nullptr);
 }
 
-cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const float *x,
-                                 const float *y, const uint8_t *layer, const int *off,
+cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const int *off,
                                  const int *d_nev, int max_events, int max_hits,
                                  const ht_peak *peaks, const int *counts, int cap, int *score,
                                  int *inl, int *assign, void *ws, const HitIndex &idx, int sms,
                                  cudaStream_t st)
 {
     CfWs w;
-    cf_layout(G, max_events, max_hits, cap, reinterpret_cast<char *>(ws), &w);
-    const int ng = cf_groups(G), ni = max_events * ng;
+    cf_layout(max_events, max_hits, reinterpret_cast<char *>(ws), &w);
     cudaError_t e = cudaMemsetAsync(w.head, 0, 4, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.gbest, 0, (size_t)max_hits * 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.gcnt, 0, (size_t)ni * 4, st);
     if (e != cudaSuccess) return e;
     k_cand_prefix<<<1, 1024, 0, st>>>(counts, d_nev, cap, w.cpre);
-    // candidates by (event, column group): counts, offsets, positions
-    k_cf_group<<<sms * 4, 256, 0, st>>>(d_nev, w.cpre, peaks, cap, ng, w.gcnt, nullptr, nullptr);
-    e = scan_exclusive(w.gcnt, w.gofs, w.gcur, ni, nullptr, w.gofs + ni, w.tmp, st);
-    if (e != cudaSuccess) return e;
-    k_cf_group<<<sms * 4, 256, 0, st>>>(d_nev, w.cpre, peaks, cap, ng, nullptr, w.gcur, w.order);
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_confirm, kCfThreads, 0);
     k_confirm<<<sms * (occ > 0 ? occ : 1), kCfThreads, 0, st>>>(
-        G, P, idx, d_nev, peaks, cap, w.cpre, w.order, score, inl, w.head);
-    k_confirm_offer<<<sms * 8, 256, 0, st>>>(off, d_nev, w.cpre, cap, score, inl, w.gbest);
+        G, P, idx, off, d_nev, peaks, cap, w.cpre, score, inl, w.gbest, w.head);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_assoc_final_batch(w.gbest, off, d_nev, assign, max_hits, st);
 }
 
 // One event (host hit count n, device candidate count d_count).
-size_t confirm_workspace_bytes_single(const DevGeom &G, int n, int cap)
+size_t confirm_workspace_bytes_single(int n)
 {
-    return align256(16) + hit_index_bytes(1, n) + confirm_workspace_bytes(G, 1, n, cap);
+    return align256(16) + hit_index_bytes(1, n) + confirm_workspace_bytes(1, n);
 }
 
 cudaError_t launch_confirm(const DevGeom &G, const ConfirmDev &P, const float *x, const float *y,
@@ -830,7 +976,7 @@ cudaError_t launch_confirm(const DevGeom &G, const ConfirmDev &P, const float *x
     const int sms = device_sms();
     const cudaError_t e = launch_hit_index(x, y, layer, meta, meta + 2, 1, n, idx, sms, st);
     if (e != cudaSuccess) return e;
-    return launch_confirm_batch(G, P, x, y, layer, meta, meta + 2, 1, n, peaks, d_count, cap,
+    return launch_confirm_batch(G, P, meta, meta + 2, 1, n, peaks, d_count, cap,
                                 score, inl, assign, p + hit_index_bytes(1, n), idx, sms, st);
 }
 
