@@ -16,9 +16,18 @@
 // fitted again with `iters2` steps (the outlier rejection of a track fit).
 //
 // Design (GB300): candidates' hit lists by counting sort (count, scan,
-// scatter); one warp per candidate, lanes over its hits, the normal
-// equations summed with warp shuffles in float64 (a few dozen flops per
-// hit: the float64 rate is no bottleneck) and solved by lane 0.
+// scatter), then a pass that settles the candidates with too few hits and
+// lists the others.  The float64 pipe bounds the fit: a warp's float64
+// instruction takes about 16 cycles of an SM however few of its lanes work, so
+// a warp per candidate (ten hits on 32 lanes, and every lane repeating the
+// sine, the Cholesky factor and the substitutions) spends most of it on idle
+// or repeated lanes.  A candidate of up to kFitSmall hits is fitted by one
+// thread, its hits in turn, its hit selection kept as a bit mask, the sine
+// and cosine computed once per parameter vector; by eight lanes where the
+// candidates would not fill the GPU one to a thread (64 threads per SM: two
+// warps keep its float64 pipe busy).  Larger candidates take a warp each.
+// GB300, 21,855 candidates of 7 to 10 hits, road, cut and eight steps: 3.67 ->
+// 0.265 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -58,66 +67,9 @@ __global__ void k_fit_lists(const int *__restrict__ off, int n_ev,
     }
 }
 
-__device__ __forceinline__ double wsum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 __device__ __forceinline__ double half_f(double rho, double d0, double s, double r2)
 {
     return 0.5 * (rho * d0 * d0 + 2.0 * (1.0 + rho * s) * d0 + rho * r2 + 2.0 * s);
-}
-
-// A hit selection: the hits whose residual at q is at most w in magnitude
-// (w = infinity: every hit).
-struct Sel {
-    double q[3];
-    double w;
-};
-
-// Normal equations of the selected hits of list[b .. b + nh) at p: A (6
-// unique entries), J^T r, sum r^2 and their number; every lane gets them.
-__device__ __forceinline__ void normal_eq(const float *__restrict__ x,
-                                          const float *__restrict__ y,
-                                          const int *__restrict__ list, int b, int nh,
-                                          const double p[3], const Sel &S, int lane,
-                                          double A[6], double g[3], double &rr, int &nk)
-{
-    double sn, cs, qs, qc;
-    sincos(p[2], &sn, &cs);
-    sincos(S.q[2], &qs, &qc);
-    double a[6] = {0, 0, 0, 0, 0, 0}, gg[3] = {0, 0, 0}, s2 = 0;
-    int k = 0;
-    for (int t = lane; t < nh; t += 32) {
-        const int h = list[b + t];
-        const double xh = (double)x[h], yh = (double)y[h];
-        if (S.w < 1e300) {
-            const double sq = xh * qs - yh * qc;
-            if (!(fabs(half_f(S.q[0], S.q[1], sq, xh * xh + yh * yh)) <= S.w)) continue;
-        }
-        ++k;
-        const double s = xh * sn - yh * cs, c = xh * cs + yh * sn;
-        const double r2 = xh * xh + yh * yh;
-        const double rho = p[0], d0 = p[1];
-        const double r = half_f(rho, d0, s, r2);
-        const double j0 = 0.5 * (d0 * d0 + 2.0 * s * d0 + r2);
-        const double j1 = rho * d0 + 1.0 + rho * s;
-        const double j2 = (1.0 + rho * d0) * c;
-        a[0] += j0 * j0; a[1] += j0 * j1; a[2] += j0 * j2;
-        a[3] += j1 * j1; a[4] += j1 * j2; a[5] += j2 * j2;
-        gg[0] += j0 * r; gg[1] += j1 * r; gg[2] += j2 * r;
-        s2 += r * r;
-    }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) A[i] = wsum(a[i]);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) g[i] = wsum(gg[i]);
-    rr = wsum(s2);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-    nk = k;
 }
 
 // Cholesky of the symmetric 3 x 3 matrix {A0 A1 A2; . A3 A4; . . A5}:
@@ -144,91 +96,162 @@ struct FitArgs {
     int n_phi0, min_hits, iters, iters2;
 };
 
-// Gauss-Newton steps on the hits that S selects; false (and p kept) when
-// the normal matrix is not positive definite.
-__device__ __forceinline__ bool gauss_newton(const float *__restrict__ x,
-                                             const float *__restrict__ y,
-                                             const int *__restrict__ list, int b, int nh,
-                                             double p[3], const Sel &S, int iters, int lane)
-{
-    double A[6], g[3], rr, L[6];
-    int nk;
-    for (int it = 0; it < iters; ++it) {
-        normal_eq(x, y, list, b, nh, p, S, lane, A, g, rr, nk);
-        if (!chol3(A, L)) return false;               // same sums on every lane
-        // forward then backward substitution: L z = g, L^T dp = z
-        const double z0 = g[0] / L[0];
-        const double z1 = (g[1] - L[1] * z0) / L[2];
-        const double z2 = (g[2] - L[3] * z0 - L[4] * z1) / L[5];
-        const double d2 = z2 / L[5];
-        const double d1 = (z1 - L[4] * d2) / L[2];
-        const double d0 = (z0 - L[1] * d1 - L[3] * d2) / L[0];
-        p[0] -= d0;
-        p[1] -= d1;
-        p[2] -= d2;
-    }
-    return true;
-}
+constexpr int kFitSmall = 32;       // hits of a candidate fitted by one thread or eight lanes
+constexpr int kFitThreads = 64;     // small blocks spread few candidates over the SMs
 
-// One warp per candidate (grid.y = event, warps stride over its candidates).
-__global__ void __launch_bounds__(256)
-k_fit_tracks(FitArgs F, const float *__restrict__ x, const float *__restrict__ y,
-             const ht_peak *__restrict__ peaks, const int *__restrict__ counts, int cap,
-             const int *__restrict__ cnt, const int *__restrict__ start,
-             const int *__restrict__ list, ht_track *__restrict__ out)
-{
-    const int e = blockIdx.y, lane = threadIdx.x & 31;
-    const int nwarps = gridDim.x * (blockDim.x >> 5);
-    const int nc = min(counts[e], cap);
-    for (int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); m < nc; m += nwarps) {
-        const size_t slot = (size_t)e * cap + m;
-        const int nh = cnt[slot], b = start[slot];
-        ht_track T;
-        T.n_hits = nh;
-        T.reserved = 0;
-        const ht_peak pk = peaks[slot];
-        double p[3] = {F.rho64[pk.i_rho], ((double)pk.j_d0 - F.half_nd) * F.delta,
-                       (double)(2 * pk.k_phi0 + 1 - F.n_phi0) * F.pi_over_np};
-        if (nh < F.min_hits) {
-            T.rho = p[0]; T.d0 = p[1]; T.phi0 = p[2];
-            T.sig_rho = T.sig_d0 = T.sig_phi0 = nan("");
-            T.chi2 = nanf("");
-            T.status = 0;
-            if (lane == 0) out[slot] = T;
-            continue;
+// One candidate's hits as W consecutive lanes of a warp see them: lane sub
+// takes hits sub, sub + W, ... of list[b .. b + nh).  keep: bit i selects the
+// lane's i-th hit (up to kFitSmall per lane); with more hits than that the
+// selection is evaluated at each use (q, w).
+template <int W>
+struct Fitter {
+    const float *x, *y;
+    const int *list;
+    int nh, sub;
+    double p[3], sn, cs;   // parameters, sine and cosine of phi0
+    double q[5], w;        // selection: residual at q (with its sine, cosine) at most w
+    unsigned keep;
+
+    __device__ __forceinline__ double sum(double v) const
+    {
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, W);
+        return v;
+    }
+
+    __device__ __forceinline__ int sum(int v) const
+    {
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, W);
+        return v;
+    }
+
+    __device__ __forceinline__ bool selected(double xh, double yh) const
+    {
+        if (!(w < 1e300)) return true;
+        return fabs(half_f(q[0], q[1], xh * q[3] - yh * q[4], xh * xh + yh * yh)) <= w;
+    }
+
+    __device__ __forceinline__ void set_p()
+    {
+        sincos(p[2], &sn, &cs);
+    }
+
+    // Selects the hits within width of the circle p; returns their number.
+    __device__ __forceinline__ int select(double width)
+    {
+        q[0] = p[0]; q[1] = p[1]; q[2] = p[2]; q[3] = sn; q[4] = cs;
+        w = width;
+        keep = 0u;
+        int k = 0;
+        for (int t = sub, i = 0; t < nh; t += W, ++i) {
+            const int h = list[t];
+            if (!selected((double)x[h], (double)y[h])) continue;
+            ++k;
+            if (i < 32) keep |= 1u << i;
         }
-        int status = 1;
-        double A[6], g[3], rr, L[6];
-        int nk;
-        Sel S;
-        S.q[0] = p[0]; S.q[1] = p[1]; S.q[2] = p[2];
-        S.w = F.road > 0.0 ? F.road : 1e308;
-        // the road: hits near the cell-centre circle
-        normal_eq(x, y, list, b, nh, p, S, lane, A, g, rr, nk);
-        bool few = nk < F.min_hits;
-        if (!few) {
-            if (!gauss_newton(x, y, list, b, nh, p, S, F.iters, lane)) status = -1;
-            if (status == 1 && F.cut > 0.0) {
-                // the outlier cut: hits near the fitted circle, fitted again
-                S.q[0] = p[0]; S.q[1] = p[1]; S.q[2] = p[2];
-                S.w = F.cut * F.sigma;
-                normal_eq(x, y, list, b, nh, p, S, lane, A, g, rr, nk);
-                few = nk < F.min_hits;
-                if (!few && !gauss_newton(x, y, list, b, nh, p, S, F.iters2, lane)) status = -1;
+        return sum(k);
+    }
+
+    // Normal equations of the selected hits at p: A (6 unique entries), J^T r
+    // and sum r^2; every lane gets them.
+    __device__ __forceinline__ void normal_eq(double A[6], double g[3], double &rr) const
+    {
+        double a[6] = {0, 0, 0, 0, 0, 0}, gg[3] = {0, 0, 0}, s2 = 0;
+        const double rho = p[0], d0 = p[1];
+        for (int t = sub, i = 0; t < nh; t += W, ++i) {
+            if (i < 32 && !((keep >> i) & 1u)) continue;
+            const int h = list[t];
+            const double xh = (double)x[h], yh = (double)y[h];
+            if (i >= 32 && !selected(xh, yh)) continue;
+            const double s = xh * sn - yh * cs, c = xh * cs + yh * sn;
+            const double r2 = xh * xh + yh * yh;
+            const double r = half_f(rho, d0, s, r2);
+            const double j0 = 0.5 * (d0 * d0 + 2.0 * s * d0 + r2);
+            const double j1 = rho * d0 + 1.0 + rho * s;
+            const double j2 = (1.0 + rho * d0) * c;
+            a[0] += j0 * j0; a[1] += j0 * j1; a[2] += j0 * j2;
+            a[3] += j1 * j1; a[4] += j1 * j2; a[5] += j2 * j2;
+            gg[0] += j0 * r; gg[1] += j1 * r; gg[2] += j2 * r;
+            s2 += r * r;
+        }
+#pragma unroll
+        for (int i = 0; i < 6; ++i) A[i] = sum(a[i]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) g[i] = sum(gg[i]);
+        rr = sum(s2);
+    }
+
+    // Gauss-Newton steps on the selected hits; false (and p kept) when the
+    // normal matrix is not positive definite.  All W lanes hold the same sums,
+    // so they leave together; lanes of other candidates may go on (active:
+    // this one still steps).
+    __device__ __forceinline__ bool steps(int iters, bool active)
+    {
+        for (int it = 0; it < iters; ++it) {
+            double A[6], g[3], rr, L[6];
+            normal_eq(A, g, rr);
+            if (active && !chol3(A, L)) active = false;
+            if (active) {
+                // forward then backward substitution: L z = g, L^T dp = z
+                const double z0 = g[0] / L[0];
+                const double z1 = (g[1] - L[1] * z0) / L[2];
+                const double z2 = (g[2] - L[3] * z0 - L[4] * z1) / L[5];
+                const double d2 = z2 / L[5];
+                const double d1 = (z1 - L[4] * d2) / L[2];
+                const double d0 = (z0 - L[1] * d1 - L[3] * d2) / L[0];
+                p[0] -= d0;
+                p[1] -= d1;
+                p[2] -= d2;
+                set_p();
             }
         }
+        return active;
+    }
+
+    // The whole fit of the candidate at peak pk (nh >= min_hits hits; nh = 0
+    // for lanes without a candidate, whose result is not used).
+    __device__ __forceinline__ ht_track fit(const FitArgs &F, const ht_peak pk)
+    {
+        ht_track T;
+        T.reserved = 0;
+        p[0] = F.rho64[pk.i_rho];
+        p[1] = ((double)pk.j_d0 - F.half_nd) * F.delta;
+        p[2] = (double)(2 * pk.k_phi0 + 1 - F.n_phi0) * F.pi_over_np;
+        set_p();
+        // the road: hits near the cell-centre circle
+        int nk = select(F.road > 0.0 ? F.road : 1e308);
+        bool few = nk < F.min_hits;
+        bool ok = steps(F.iters, !few);
+        if (F.cut > 0.0) {
+            // the outlier cut: hits near the fitted circle, fitted again
+            const bool again = ok;
+            const unsigned keep0 = keep;
+            const double q0[5] = {q[0], q[1], q[2], q[3], q[4]}, w0 = w;
+            const int nk2 = select(F.cut * F.sigma);
+            if (again) {
+                nk = nk2;
+                few = nk < F.min_hits;
+            } else {   // the road's selection stays
+                keep = keep0;
+                w = w0;
+#pragma unroll
+                for (int i = 0; i < 5; ++i) q[i] = q0[i];
+            }
+            ok = steps(F.iters2, again && !few);
+        }
         T.rho = p[0]; T.d0 = p[1]; T.phi0 = p[2];
+        T.n_hits = nk;
+        double A[6], g[3], rr, L[6];
+        normal_eq(A, g, rr);
+        T.sig_rho = T.sig_d0 = T.sig_phi0 = nan("");
         if (few) {
-            T.n_hits = nk;
-            T.sig_rho = T.sig_d0 = T.sig_phi0 = nan("");
             T.chi2 = nanf("");
             T.status = 0;
-            if (lane == 0) out[slot] = T;
-            continue;
+            return T;
         }
-        normal_eq(x, y, list, b, nh, p, S, lane, A, g, rr, nk);
-        T.n_hits = nk;
         T.chi2 = (float)(rr / (F.sigma * F.sigma));
+        T.status = ok ? 1 : -1;
         if (chol3(A, L)) {
             // diagonal of (L L^T)^-1 = columns of L^-1 squared and summed
             const double i0 = 1.0 / L[0], i2 = 1.0 / L[2], i5 = 1.0 / L[5];
@@ -240,12 +263,94 @@ k_fit_tracks(FitArgs F, const float *__restrict__ x, const float *__restrict__ y
             T.sig_d0 = sqrt(s2 * (i2 * i2 + i4 * i4));
             T.sig_phi0 = sqrt(s2 * (i5 * i5));
         } else {
-            T.sig_rho = T.sig_d0 = T.sig_phi0 = nan("");
-            status = -1;
+            T.status = -1;
         }
-        T.status = status;
-        if (lane == 0) out[slot] = T;
+        return T;
     }
+};
+
+// Settles the candidates with too few hits and lists the others' slots: those
+// of up to kFitSmall hits from the front of todo (n[0] of them), larger ones
+// from its back (n[1]).  grid.y = event.
+__global__ void __launch_bounds__(256)
+k_fit_split(FitArgs F, const ht_peak *__restrict__ peaks, const int *__restrict__ counts, int cap,
+            const int *__restrict__ start, int ns, ht_track *__restrict__ out,
+            int *__restrict__ todo, int *__restrict__ n)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int e = blockIdx.y, nc = min(counts[e], cap), lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int m0 = blockIdx.x * blockDim.x + threadIdx.x - lane; m0 < nc;
+         m0 += gridDim.x * blockDim.x) {   // uniform over the warp
+        const int m = m0 + lane;
+        const size_t slot = (size_t)e * cap + m;
+        const int nh = m < nc ? start[slot + 1] - start[slot] : -1;
+        const bool fit = nh >= F.min_hits;   // min_hits >= 3
+        const unsigned ms = __ballot_sync(kAll, fit && nh <= kFitSmall);
+        const unsigned mb = __ballot_sync(kAll, fit && nh > kFitSmall);
+        int at = 0;   // one counter per warp and list
+        if (lane == 0 && ms) at = atomicAdd(&n[0], __popc(ms));
+        if (lane == 1 && mb) at = atomicAdd(&n[1], __popc(mb));
+        const int as = __shfl_sync(kAll, at, 0), ab = __shfl_sync(kAll, at, 1);
+        if (fit) {
+            if (nh <= kFitSmall) todo[as + __popc(ms & lt)] = (int)slot;
+            else todo[ns - 1 - (ab + __popc(mb & lt))] = (int)slot;
+        }
+        if (fit || m >= nc) continue;
+        const ht_peak pk = peaks[slot];
+        ht_track T;
+        T.rho = F.rho64[pk.i_rho];
+        T.d0 = ((double)pk.j_d0 - F.half_nd) * F.delta;
+        T.phi0 = (double)(2 * pk.k_phi0 + 1 - F.n_phi0) * F.pi_over_np;
+        T.sig_rho = T.sig_d0 = T.sig_phi0 = nan("");
+        T.chi2 = nanf("");
+        T.n_hits = nh;
+        T.status = 0;
+        T.reserved = 0;
+        out[slot] = T;
+    }
+}
+
+// W lanes per candidate over the list todo[0 .. n) (step 1) or backwards
+// from todo (step -1).
+template <int W>
+__device__ __forceinline__ void fit_list(const FitArgs &F, const float *__restrict__ x,
+                                         const float *__restrict__ y,
+                                         const ht_peak *__restrict__ peaks,
+                                         const int *__restrict__ start,
+                                         const int *__restrict__ list, const int *todo, int step,
+                                         int n, ht_track *__restrict__ out)
+{
+    const int per = (gridDim.x * kFitThreads) / W;
+    const int g0 = (blockIdx.x * kFitThreads + threadIdx.x) / W;
+    const int wfirst = (blockIdx.x * kFitThreads + (threadIdx.x & ~31)) / W;   // the warp's first
+    for (int at = 0; wfirst + at < n; at += per) {   // uniform over the warp
+        const int i = g0 + at;
+        const bool act = i < n;
+        const size_t slot = (size_t)todo[step * (act ? i : wfirst + at)];
+        const int b = start[slot];
+        Fitter<W> f;
+        f.x = x;
+        f.y = y;
+        f.list = list + b;
+        f.nh = act ? start[slot + 1] - b : 0;
+        f.sub = threadIdx.x % W;
+        const ht_track T = f.fit(F, peaks[slot]);
+        if (act && f.sub == 0) out[slot] = T;
+    }
+}
+
+__global__ void __launch_bounds__(kFitThreads)
+k_fit_tracks(FitArgs F, const float *__restrict__ x, const float *__restrict__ y,
+             const ht_peak *__restrict__ peaks, const int *__restrict__ start,
+             const int *__restrict__ list, const int *__restrict__ todo, int ns,
+             const int *__restrict__ n, int dense, ht_track *__restrict__ out)
+{
+    const int small = n[0], big = n[1];
+    // a thread each where the candidates fill `dense` threads, else eight lanes
+    if (small >= dense) fit_list<1>(F, x, y, peaks, start, list, todo, 1, small, out);
+    else fit_list<8>(F, x, y, peaks, start, list, todo, 1, small, out);
+    fit_list<32>(F, x, y, peaks, start, list, todo + ns - 1, -1, big, out);
 }
 
 }  // namespace
@@ -312,9 +417,19 @@ ht_status ht_fit_tracks(const ht_geometry *g, const float *x, const float *y, co
         F.n_phi0 = g->G.n_phi0;
         F.min_hits = min_hits;
         F.iters = iters;
-        ht::k_fit_tracks<<<dim3(64, n_events), 256, 0, st>>>(F, x, y, peaks, d_count, cap, cnt,
-                                                              start, list, out);
-        e = cudaGetLastError();
+        // the cursors are spent: they hold the list of candidates to fit; the
+        // scan's scratch holds its two counts
+        int *n = reinterpret_cast<int *>(tmp);
+        e = cudaMemsetAsync(n, 0, 8, st);
+        if (e == cudaSuccess) {
+            const int sms = ht::device_sms();
+            const int gx = max(1, min((cap + 255) / 256, sms * 8 / min(n_events, sms) + 1));
+            ht::k_fit_split<<<dim3(gx, n_events), 256, 0, st>>>(F, peaks, d_count, cap, start, ns,
+                                                                out, cur, n);
+            ht::k_fit_tracks<<<sms * 8, ht::kFitThreads, 0, st>>>(F, x, y, peaks, start, list, cur,
+                                                                  ns, n, sms * 64, out);
+            e = cudaGetLastError();
+        }
     }
     return e == cudaSuccess ? HT_OK : ht::set_error(HT_ERR_CUDA, cudaGetErrorString(e));
 }
