@@ -633,9 +633,9 @@ def launches_per_batch(ne, learned=False):
 def track_launches(learned=False):
     """Kernels one ht_batch_run_tracks replays, whatever its number of events:
     the hit index (3 + scan 3), the vote, the peaks of all events (2 + scan
-    3), the confirmation (prefix, confirmation, decode) and the z vote (4 +
-    scan 3); with the proposal one more (the network's top-k per hit)."""
-    return 6 + 1 + 5 + 3 + 7 + (1 if learned else 0)
+    3), the confirmation (prefix, confirmation, decode) and the z vote (6);
+    with the proposal one more (the network's top-k per hit)."""
+    return 6 + 1 + 5 + 3 + 6 + (1 if learned else 0)
 
 
 def run_ours(args):

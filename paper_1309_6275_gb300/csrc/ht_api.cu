@@ -190,6 +190,7 @@ ht_status ht_geometry_create(const ht_geometry_desc *d, ht_geometry **out)
     G.dz = 2.0 * d->z0_max / (double)d->n_z0;
     G.z0_max = d->z0_max;
     G.cstep = d->cot_max / (double)d->n_cot;
+    G.inv_dz = 1.0 / G.dz;
     G.inv_dz_f = (float)(1.0 / G.dz);
     G.z0_max_f = (float)d->z0_max;
     G.cstep_f = (float)G.cstep;

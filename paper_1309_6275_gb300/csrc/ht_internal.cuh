@@ -46,6 +46,7 @@ struct DevGeom {
     float inv_delta_lo;                // 1/delta - inv_delta_f
     // z vote
     double dz, z0_max, cstep;      // dz = 2 z0_max / n_z0, cstep = cot_max / n_cot
+    double inv_dz;                 // 1 / dz (a first estimate only)
     float inv_dz_f, z0_max_f, cstep_f;
 };
 
@@ -307,10 +308,12 @@ __device__ __forceinline__ double atan_unit64(double t)
     for (int h = 0; h < 3; ++h)
         t = __ddiv_rn(t, __dadd_rn(1.0, __dsqrt_rn(__dadd_rn(1.0, __dmul_rn(t, t)))));
     const double t2 = __dmul_rn(t, t);
-    double p = __ddiv_rn(1.0, 21.0);
-#pragma unroll 1
-    for (int k = 9; k >= 0; --k)
-        p = __dsub_rn(__ddiv_rn(1.0, (double)(2 * k + 1)), __dmul_rn(t2, p));
+    // 1 / (2k + 1), correctly rounded by the compiler
+    constexpr double inv[10] = {1.0,        1.0 / 3.0,  1.0 / 5.0,  1.0 / 7.0,  1.0 / 9.0,
+                                1.0 / 11.0, 1.0 / 13.0, 1.0 / 15.0, 1.0 / 17.0, 1.0 / 19.0};
+    double p = 1.0 / 21.0;
+#pragma unroll
+    for (int k = 9; k >= 0; --k) p = __dsub_rn(inv[k], __dmul_rn(t2, p));
     return __dmul_rn(8.0, __dmul_rn(t, p));
 }
 

@@ -8,13 +8,23 @@
 // ties to the smallest n n_cot + q.
 //
 // Design (GB300):
-//  * Hits are grouped by candidate in device memory (count, one-CTA scan,
-//    scatter), so every candidate reads only its own hits.
-//  * Candidates with at most 32 hits (nearly all): one warp per candidate,
-//    lane = hit.  For each cot column q every lane bins its hit; the count of
-//    each lane's bin is __match_any_sync's popcount (warp-aggregated, no
-//    histogram in memory) and one redux.sync max over (count, -n) gives the
-//    column's best cell.
+//  * Hits are grouped by candidate in device memory, so every candidate
+//    reads only its own hits.  Their order and place do not matter, so a
+//    candidate with hits takes its range from one running total (a warp's
+//    candidates together) instead of a scan over every candidate slot, and
+//    candidates without hits are settled there.  Single events and batches
+//    share the kernels (global candidate id e * cap + m).
+//  * Candidates with at most 32 hits (nearly all): one warp per candidate.
+//    Lane = hit computes the arc length; then lane = cot column: a lane bins
+//    all the candidate's hits in its columns and counts equal bins by
+//    comparing them pairwise (45 comparisons for ten hits), so the 128
+//    columns are four independent rounds instead of 128 warp-wide matches in
+//    a row.  The float64 arc lengths, where any bin needs them, are computed
+//    for all hits at once (lane = hit); a bin's float64 quotient is a product
+//    unless that lies within 1e-9 of an integer.
+//  * Latency-bound.  Stage on GB300, 25 events of 2k-60k hits: 337 -> 84 us
+//    (most of it was the scan and a warp per empty candidate slot); 25 of 10k
+//    hits: 538 -> 150 us.
 //  * Larger candidates: one CTA per candidate with an n_z0 x n_cot uint32
 //    histogram in shared memory and a block argmax.
 //  * Arithmetic: float32 with a proven error bound per (hit, q); any bin
@@ -27,6 +37,9 @@
 #include "ht_internal.cuh"
 
 namespace ht {
+
+size_t z_big_smem(const DevGeom &G) { return (size_t)G.n_z0 * G.n_cot * 4; }
+
 namespace {
 
 constexpr int kBigThreads = 256;
@@ -92,11 +105,9 @@ __device__ __forceinline__ double arc64(const ZCand &C, float xf, float yf)
     return __ddiv_rn(th, C.rho64);
 }
 
-// z0 bin of one (hit, q): float32 if provably decided, else float64 (L64 is
-// computed on first need and cached by the caller through `have64`).
-__device__ __forceinline__ int z_bin(const DevGeom &G, const ZCand &C, float xf, float yf,
-                                     float z, float L, float eL, int q, bool &have64,
-                                     double &L64)
+// z0 bin of one (hit, q) by float32: -1 outside the axis, -2 too close to an
+// edge to be decided.
+__device__ __forceinline__ int z_bin32(const DevGeom &G, float z, float L, float eL, int q)
 {
     const float t = G.cstep_f * (float)(2 * q + 1 - G.n_cot);
     const float zz = z + G.z0_max_f;
@@ -109,102 +120,91 @@ __device__ __forceinline__ int z_bin(const DevGeom &G, const ZCand &C, float xf,
     const float f = floorf(u);
     const float fr = u - f;
     // u + 1 (u in (-1, 0)) is rounded: only f >= 0 is decided here
-    if (f >= 0.0f && fminf(fr, 1.0f - fr) > err) return (int)f;
-    if (!have64) {
-        L64 = arc64(C, xf, yf);
-        have64 = true;
-    }
+    return f >= 0.0f && fminf(fr, 1.0f - fr) > err ? (int)f : -2;
+}
+
+// The same by the float64 definition, from the hit's arc length L64.
+__device__ __forceinline__ int z_bin64(const DevGeom &G, float z, double L64, int q)
+{
     const double t64 = __dmul_rn((double)(2 * q + 1 - G.n_cot), G.cstep);
     const double z0 = __dsub_rn((double)z, __dmul_rn(L64, t64));
-    const double u64 = __ddiv_rn(__dadd_rn(z0, G.z0_max), G.dz);
+    const double v = __dadd_rn(z0, G.z0_max);
+    // a product settles all but the quotients within 1e-9 of an integer
+    const double w = v * G.inv_dz, f = floor(w);
+    if (fabs(w) < 1e6 && w - f > 1e-9 && w - f < 1.0 - 1e-9)
+        return f >= 0.0 && f < (double)G.n_z0 ? (int)f : -1;
+    const double u64 = __ddiv_rn(v, G.dz);
     if (u64 >= 0.0 && u64 < (double)G.n_z0) return (int)floor(u64);
     return -1;
 }
 
-__global__ void k_z_count(const int *__restrict__ assign, int n, const int *__restrict__ d_count,
-                          int cap, int *__restrict__ cnt)
-{
-    const int ncand = min(*d_count, cap);
-    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) {
-        const int a = assign[h];
-        if (a >= 0 && a < ncand) atomicAdd(&cnt[a], 1);
-    }
-}
+constexpr int kZWarps = 4, kZThreads = 32 * kZWarps;
 
-__global__ void k_z_scatter(const int *__restrict__ assign, int n, const int *__restrict__ d_count,
-                            int cap, int *__restrict__ cur, int *__restrict__ list)
-{
-    const int ncand = min(*d_count, cap);
-    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) {
-        const int a = assign[h];
-        if (a >= 0 && a < ncand) list[atomicAdd(&cur[a], 1)] = h;
-    }
-}
+// One warp's state: a candidate's hits and one round's bins (lane = column).
+struct ZWarp {
+    double L64[32];
+    float z[32], L[32], eL[32];
+    short bin[32][32];   // [hit][lane]
+};
 
 // (z0, cot theta) result of one candidate with 1..32 hits list[o .. o + nh),
-// one warp, lane = hit.  Every lane returns the result.
+// one warp.  Every lane returns the result.
 __device__ __forceinline__ ht_zres z_small_cand(const DevGeom &G, const float *__restrict__ x,
                                                 const float *__restrict__ y,
                                                 const float *__restrict__ z, const ht_peak &pk,
                                                 const int *__restrict__ list, int o, int nh,
-                                                int lane)
+                                                int lane, ZWarp &W)
 {
     const ZCand C = z_cand(G, pk);
-    const bool act = lane < nh;
-    float xf = 0.f, yf = 0.f, zf = 0.f, L = 0.f, eL = 0.f;
-    if (act) {
+    __syncwarp();   // the previous candidate's readers are done
+    float xf = 0.0f, yf = 0.0f;
+    if (lane < nh) {
         const int h = list[o + lane];
         xf = x[h];
         yf = y[h];
-        zf = z[h];
-        arc32(C, xf, yf, L, eL);
+        W.z[lane] = z[h];
+        arc32(C, xf, yf, W.L[lane], W.eL[lane]);
     }
-    bool have64 = false;
-    double L64 = 0.0;
-    unsigned best_c = 0u;
-    int best_idx = 0x7fffffff;
-    for (int q = 0; q < G.n_cot; ++q) {
-        const int nb = act ? z_bin(G, C, xf, yf, zf, L, eL, q, have64, L64) : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, nb);
-        const unsigned key = nb >= 0 ? ((unsigned)__popc(peers) << 16) | (0xffffu - (unsigned)nb) : 0u;
-        const unsigned top = __reduce_max_sync(0xffffffffu, key);
-        if (top) {
-            const unsigned cq = top >> 16;
-            const int idx = (int)(0xffffu - (top & 0xffffu)) * G.n_cot + q;
-            if (cq > best_c || (cq == best_c && idx < best_idx)) {
-                best_c = cq;
+    __syncwarp();
+    bool have64 = false;   // uniform
+    // the lane's best cell: key = count, then smallest index n n_cot + q
+    int best_c = 0, best_idx = 0x7fffffff;
+    for (int q0 = 0; q0 < G.n_cot; q0 += 32) {   // uniform
+        const int q = q0 + lane;
+        const bool col = q < G.n_cot;
+        bool open = false;
+        for (int h = 0; h < nh; ++h) {
+            const int b = col ? z_bin32(G, W.z[h], W.L[h], W.eL[h], q) : -1;
+            W.bin[h][lane] = (short)b;
+            open |= b == -2;
+        }
+        if (__any_sync(0xffffffffu, open)) {
+            // the float64 arc lengths, of all hits at once (lane = hit)
+            if (!have64) {
+                if (lane < nh) W.L64[lane] = arc64(C, xf, yf);
+                have64 = true;
+                __syncwarp();
+            }
+            if (open)
+                for (int h = 0; h < nh; ++h)
+                    if (W.bin[h][lane] == -2) W.bin[h][lane] = (short)z_bin64(G, W.z[h], W.L64[h], q);
+            __syncwarp();
+        }
+        for (int h = 0; h < nh; ++h) {   // (each lane reads what it wrote)
+            const int b = W.bin[h][lane];
+            if (b < 0 || nh - h < best_c) continue;
+            int c = 1;
+            for (int g = h + 1; g < nh; ++g) c += W.bin[g][lane] == b;
+            const int idx = b * G.n_cot + q;
+            if (c > best_c || (c == best_c && idx < best_idx)) {
+                best_c = c;
                 best_idx = idx;
             }
         }
     }
-    return best_c ? ht_zres{best_idx / G.n_cot, best_idx % G.n_cot, (int)best_c}
-                  : ht_zres{-1, -1, 0};
-}
-
-// One warp per candidate with <= 32 hits; larger ones go to the big list.
-__global__ void k_z_small(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
-                          const float *__restrict__ z, const ht_peak *__restrict__ peaks,
-                          const int *__restrict__ d_count, int cap, const int *__restrict__ off,
-                          const int *__restrict__ list, ht_zres *__restrict__ out,
-                          int *__restrict__ big, int *__restrict__ nbig)
-{
-    const int ncand = min(*d_count, cap);
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int m = gw; m < ncand; m += nw) {
-        const int o = off[m], nh = off[m + 1] - o;
-        if (nh == 0) {
-            if (lane == 0) out[m] = ht_zres{-1, -1, 0};
-            continue;
-        }
-        if (nh > 32) {
-            if (lane == 0) big[atomicAdd(nbig, 1)] = m;
-            continue;
-        }
-        const ht_zres r = z_small_cand(G, x, y, z, peaks[m], list, o, nh, lane);
-        if (lane == 0) out[m] = r;
-    }
+    const int top = __reduce_max_sync(0xffffffffu, best_c);
+    const int idx = __reduce_min_sync(0xffffffffu, best_c == top ? best_idx : 0x7fffffff);
+    return top > 0 ? ht_zres{idx / G.n_cot, idx % G.n_cot, top} : ht_zres{-1, -1, 0};
 }
 
 // (z0, cot theta) result of one candidate with any number of hits, one CTA:
@@ -236,9 +236,8 @@ __device__ __forceinline__ ht_zres z_big_cand(const DevGeom &G, const float *__r
         __syncthreads();
         for (int t = threadIdx.x; t < hc * NC; t += kBigThreads) {
             const int hl = t / NC, q = t - hl * NC;
-            bool have64 = false;
-            double L64 = 0.0;
-            const int nbin = z_bin(G, C, sx[hl], sy[hl], sz[hl], sL[hl], seL[hl], q, have64, L64);
+            int nbin = z_bin32(G, sz[hl], sL[hl], seL[hl], q);
+            if (nbin == -2) nbin = z_bin64(G, sz[hl], arc64(C, sx[hl], sy[hl]), q);
             if (nbin >= 0) atomicAdd(&hist[nbin * NC + q], 1u);
         }
     }
@@ -267,23 +266,11 @@ __device__ __forceinline__ ht_zres z_big_cand(const DevGeom &G, const float *__r
     return r;
 }
 
-__global__ void __launch_bounds__(kBigThreads)
-k_z_big(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
-        const float *__restrict__ z, const ht_peak *__restrict__ peaks,
-        const int *__restrict__ off, const int *__restrict__ list,
-        const int *__restrict__ big, const int *__restrict__ nbig, ht_zres *__restrict__ out)
-{
-    const int nb = *nbig;
-    for (int bi = blockIdx.x; bi < nb; bi += gridDim.x) {
-        const int m = big[bi];
-        const ht_zres r = z_big_cand(G, x, y, z, peaks[m], list, off[m], off[m + 1] - off[m]);
-        if (threadIdx.x == 0) out[m] = r;
-    }
-}
-
-// ---------------------------------------------------------------- batches
-// Global candidate id g = e * cap + m (event slot e, candidate m); hits carry
-// batch-wide indices; off[0..n_ev] are the events' hit offsets.
+// ---------------------------------------------------------------- launches
+// Candidates of event slot e: ids e * cap + m, m < min(counts[e], cap); hits
+// carry batch-wide indices, off[0 .. n_ev] are the events' hit offsets (null:
+// one event of n hits).  tot[0]: grouped hits, tot[1]: candidates of up to
+// 32 hits (listed from the front of todo), tot[2]: larger ones (from its back).
 __device__ __forceinline__ int event_of(const int *__restrict__ off, int n_ev, int h)
 {
     int lo = 0, hi = n_ev;          // off[lo] <= h < off[hi]
@@ -294,116 +281,179 @@ __device__ __forceinline__ int event_of(const int *__restrict__ off, int n_ev, i
     return lo;
 }
 
-__global__ void k_zb_group(const int *__restrict__ assign, const int *__restrict__ off,
-                           const int *__restrict__ d_nev, const int *__restrict__ counts,
-                           int cap, int *__restrict__ cnt, int *__restrict__ cur,
-                           int *__restrict__ list)
-{
-    const int n_ev = *d_nev, n = off[n_ev];
-    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) {
+struct ZGroup {
+    const int *off, *d_nev, *counts;   // off, d_nev null: one event
+    int n, cap;
+
+    __device__ __forceinline__ int hits(int &n_ev) const
+    {
+        n_ev = d_nev ? *d_nev : 1;
+        return off ? off[n_ev] : n;
+    }
+    // global id of hit h's candidate, -1 for none
+    __device__ __forceinline__ long long cand(const int *__restrict__ assign, int h, int n_ev) const
+    {
         const int a = assign[h];
-        if (a < 0) continue;
-        const int e = event_of(off, n_ev, h);
-        if (a >= min(counts[e], cap)) continue;
-        const size_t g = (size_t)e * cap + a;
-        if (list) list[atomicAdd(&cur[g], 1)] = h;
-        else atomicAdd(&cnt[g], 1);
+        if (a < 0) return -1;
+        const int e = off ? event_of(off, n_ev, h) : 0;
+        return a < min(counts[e], cap) ? (long long)e * cap + a : -1;
+    }
+};
+
+// cnt = 0 for every kept candidate; grid.y = event slot.
+__global__ void k_z_zero(ZGroup Z, int *__restrict__ cnt, int *__restrict__ tot)
+{
+    const int e = blockIdx.y;
+    if (e >= (Z.d_nev ? *Z.d_nev : 1)) return;
+    if (e == 0 && blockIdx.x == 0 && threadIdx.x < 3) tot[threadIdx.x] = 0;
+    const int nc = min(Z.counts[e], Z.cap);
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < nc; m += gridDim.x * blockDim.x)
+        cnt[(size_t)e * Z.cap + m] = 0;
+}
+
+__global__ void k_z_count(ZGroup Z, const int *__restrict__ assign, int *__restrict__ cnt)
+{
+    int n_ev;
+    const int n = Z.hits(n_ev);
+    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) {
+        const long long g = Z.cand(assign, h, n_ev);
+        if (g >= 0) atomicAdd(&cnt[g], 1);
     }
 }
 
-__global__ void k_zb_small(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
-                           const float *__restrict__ z, const ht_peak *__restrict__ peaks,
-                           const int *__restrict__ counts, const int *__restrict__ d_nev,
-                           int cap, const int *__restrict__ off, const int *__restrict__ list,
-                           ht_zres *__restrict__ out, int *__restrict__ big,
-                           int *__restrict__ nbig)
+// A candidate with hits takes its range of the grouped list and its place in
+// todo (one atomic per warp and counter); one without gets its result.
+__global__ void __launch_bounds__(256)
+k_z_alloc(ZGroup Z, const int *__restrict__ cnt, int *__restrict__ start, int *__restrict__ cur,
+          int *__restrict__ todo, int ns, int *__restrict__ tot, ht_zres *__restrict__ out)
 {
-    const int e = blockIdx.y;
-    if (e >= *d_nev) return;
-    const int ncand = min(counts[e], cap);
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int m = gw; m < ncand; m += nw) {
-        const size_t g = (size_t)e * cap + m;
-        const int o = off[g], nh = off[g + 1] - o;
-        if (nh == 0) {
-            if (lane == 0) out[g] = ht_zres{-1, -1, 0};
-            continue;
+    constexpr unsigned kAll = 0xffffffffu;
+    const int e = blockIdx.y, lane = threadIdx.x & 31;
+    if (e >= (Z.d_nev ? *Z.d_nev : 1)) return;
+    const int nc = min(Z.counts[e], Z.cap);
+    const unsigned lt = (1u << lane) - 1u;
+    for (int m0 = blockIdx.x * blockDim.x + threadIdx.x - lane; m0 < nc;
+         m0 += gridDim.x * blockDim.x) {   // uniform over the warp
+        const int m = m0 + lane;
+        const size_t g = (size_t)e * Z.cap + m;
+        const int nh = m < nc ? cnt[g] : 0;
+        const unsigned any = __ballot_sync(kAll, nh > 0);
+        if (m < nc && nh == 0) out[g] = ht_zres{-1, -1, 0};
+        if (!any) continue;
+        int incl = nh;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kAll, incl, o);
+            if (lane >= o) incl += v;
         }
-        if (nh > 32) {
-            if (lane == 0) big[atomicAdd(nbig, 1)] = (int)g;
-            continue;
-        }
-        const ht_zres r = z_small_cand(G, x, y, z, peaks[g], list, o, nh, lane);
+        const unsigned ms = __ballot_sync(kAll, nh > 0 && nh <= 32);
+        const unsigned mb = __ballot_sync(kAll, nh > 32);
+        int at = 0;
+        if (lane == 31) at = atomicAdd(&tot[0], incl);
+        if (lane == 0 && ms) at = atomicAdd(&tot[1], __popc(ms));
+        if (lane == 1 && mb) at = atomicAdd(&tot[2], __popc(mb));
+        const int base = __shfl_sync(kAll, at, 31), as = __shfl_sync(kAll, at, 0),
+                  ab = __shfl_sync(kAll, at, 1);
+        if (nh == 0) continue;
+        start[g] = cur[g] = base + incl - nh;
+        if (nh <= 32) todo[as + __popc(ms & lt)] = (int)g;
+        else todo[ns - 1 - (ab + __popc(mb & lt))] = (int)g;
+    }
+}
+
+__global__ void k_z_scatter(ZGroup Z, const int *__restrict__ assign, int *__restrict__ cur,
+                            int *__restrict__ list)
+{
+    int n_ev;
+    const int n = Z.hits(n_ev);
+    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) {
+        const long long g = Z.cand(assign, h, n_ev);
+        if (g >= 0) list[atomicAdd(&cur[g], 1)] = h;
+    }
+}
+
+__global__ void __launch_bounds__(kZThreads)
+k_z_small(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
+          const float *__restrict__ z, const ht_peak *__restrict__ peaks,
+          const int *__restrict__ cnt, const int *__restrict__ start,
+          const int *__restrict__ list, const int *__restrict__ todo,
+          const int *__restrict__ tot, ht_zres *__restrict__ out)
+{
+    __shared__ ZWarp s_w[kZWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = tot[1];
+    for (int t = blockIdx.x * kZWarps + warp; t < n; t += gridDim.x * kZWarps) {
+        const int g = todo[t];
+        const ht_zres r = z_small_cand(G, x, y, z, peaks[g], list, start[g], cnt[g], lane, s_w[warp]);
         if (lane == 0) out[g] = r;
     }
 }
 
 __global__ void __launch_bounds__(kBigThreads)
-k_zb_big(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
-         const float *__restrict__ z, const ht_peak *__restrict__ peaks,
-         const int *__restrict__ off, const int *__restrict__ list,
-         const int *__restrict__ big, const int *__restrict__ nbig, ht_zres *__restrict__ out)
+k_z_big(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
+        const float *__restrict__ z, const ht_peak *__restrict__ peaks,
+        const int *__restrict__ cnt, const int *__restrict__ start,
+        const int *__restrict__ list, const int *__restrict__ todo, int ns,
+        const int *__restrict__ tot, ht_zres *__restrict__ out)
 {
-    const int nb = *nbig;
-    for (int bi = blockIdx.x; bi < nb; bi += gridDim.x) {
-        const int g = big[bi];
-        const ht_zres r = z_big_cand(G, x, y, z, peaks[g], list, off[g], off[g + 1] - off[g]);
+    const int n = tot[2];
+    for (int t = blockIdx.x; t < n; t += gridDim.x) {
+        const int g = todo[ns - 1 - t];
+        const ht_zres r = z_big_cand(G, x, y, z, peaks[g], list, start[g], cnt[g]);
         if (threadIdx.x == 0) out[g] = r;
     }
 }
 
-struct ZWs {
-    int *cnt, *off, *cur, *list, *big, *nbig;
-    void *tmp;
-};
-
-ZWs carve(void *ws, int n, int cap)
+size_t z_bytes(size_t ng, int n)
 {
+    return 4 * align256((ng + 1) * 4) + 256 + align256((size_t)(n > 0 ? n : 1) * 4);
+}
+
+cudaError_t run_z(const DevGeom &G, const ZGroup &Z, int n_ev, int max_hits, const float *x,
+                  const float *y, const float *z, const int *assign, const ht_peak *peaks,
+                  ht_zres *out, void *ws, cudaStream_t st)
+{
+    const size_t ng = (size_t)n_ev * Z.cap;
     char *p = reinterpret_cast<char *>(ws);
-    ZWs w;
-    w.cnt = reinterpret_cast<int *>(p); p += align256((size_t)(cap + 1) * 4);
-    w.off = reinterpret_cast<int *>(p); p += align256((size_t)(cap + 1) * 4);
-    w.cur = reinterpret_cast<int *>(p); p += align256((size_t)(cap + 1) * 4);
-    w.big = reinterpret_cast<int *>(p); p += align256((size_t)(cap + 1) * 4);
-    w.nbig = reinterpret_cast<int *>(p); p += 256;
-    w.tmp = p; p += scan_tmp_bytes(cap);
-    w.list = reinterpret_cast<int *>(p);
-    return w;
+    int *cnt = reinterpret_cast<int *>(p); p += align256((ng + 1) * 4);
+    int *start = reinterpret_cast<int *>(p); p += align256((ng + 1) * 4);
+    int *cur = reinterpret_cast<int *>(p); p += align256((ng + 1) * 4);
+    int *todo = reinterpret_cast<int *>(p); p += align256((ng + 1) * 4);
+    int *tot = reinterpret_cast<int *>(p); p += 256;
+    int *list = reinterpret_cast<int *>(p);
+    const int sms = device_sms();
+    const int nb = max(1, min(sms * 8, (max_hits + 255) / 256));
+    const dim3 gc(max(1, min((Z.cap + 255) / 256, sms * 8 / n_ev + 1)), n_ev);
+    k_z_zero<<<gc, 256, 0, st>>>(Z, cnt, tot);
+    k_z_count<<<nb, 256, 0, st>>>(Z, assign, cnt);
+    k_z_alloc<<<gc, 256, 0, st>>>(Z, cnt, start, cur, todo, (int)ng, tot, out);
+    k_z_scatter<<<nb, 256, 0, st>>>(Z, assign, cur, list);
+    k_z_small<<<sms * 8, kZThreads, 0, st>>>(G, x, y, z, peaks, cnt, start, list, todo, tot, out);
+    k_z_big<<<sms * 2, kBigThreads, z_big_smem(G), st>>>(G, x, y, z, peaks, cnt, start, list, todo,
+                                                         (int)ng, tot, out);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
 size_t vote_z_workspace_bytes(const DevGeom &, int n, int cap)
 {
-    return 4 * align256((size_t)(cap + 1) * 4) + 256 + scan_tmp_bytes(cap) +
-           align256((size_t)(n > 0 ? n : 1) * 4);
+    return z_bytes((size_t)(cap > 0 ? cap : 0), n);
 }
-
-size_t z_big_smem(const DevGeom &G) { return (size_t)G.n_z0 * G.n_cot * 4; }
 
 cudaError_t prepare_z_kernels(int max_smem)
 {
-    const void *fns[] = {(const void *)k_z_big, (const void *)k_zb_big};
-    for (const void *f : fns) {
-        cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, f);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 max_smem - (int)fa.sharedSizeBytes);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, (const void *)k_z_big);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute((const void *)k_z_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                max_smem - (int)fa.sharedSizeBytes);
 }
 
-// Batch z vote: candidates of all n_ev event slots at once (global id
-// e * cap + m), hits grouped per candidate with batch-wide indices.
+// Batch z vote: candidates of all n_ev event slots at once.
 size_t vote_z_batch_workspace_bytes(int n_ev, int cap, int max_hits)
 {
-    const size_t ng = (size_t)n_ev * cap;
-    return 4 * align256((ng + 1) * 4) + 256 + scan_tmp_bytes((int)ng) +
-           align256((size_t)(max_hits > 0 ? max_hits : 1) * 4);
+    return z_bytes((size_t)n_ev * cap, max_hits);
 }
 
 cudaError_t launch_vote_z_batch(const DevGeom &G, const float *x, const float *y, const float *z,
@@ -411,29 +461,8 @@ cudaError_t launch_vote_z_batch(const DevGeom &G, const float *x, const float *y
                                 const ht_peak *peaks, const int *counts, int cap, int n_ev,
                                 ht_zres *out, void *ws, int max_hits, cudaStream_t st)
 {
-    const size_t ng = (size_t)n_ev * cap;
-    char *p = reinterpret_cast<char *>(ws);
-    int *cnt = reinterpret_cast<int *>(p); p += align256((ng + 1) * 4);
-    int *zoff = reinterpret_cast<int *>(p); p += align256((ng + 1) * 4);
-    int *cur = reinterpret_cast<int *>(p); p += align256((ng + 1) * 4);
-    int *big = reinterpret_cast<int *>(p); p += align256((ng + 1) * 4);
-    int *nbig = reinterpret_cast<int *>(p); p += 256;
-    void *tmp = p; p += scan_tmp_bytes((int)ng);
-    int *list = reinterpret_cast<int *>(p);
-    cudaError_t e = cudaMemsetAsync(cnt, 0, (ng + 1) * 4, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(nbig, 0, 4, st);
-    if (e != cudaSuccess) return e;
-    const int nb = min(4096, max_hits / 256 + 1);
-    k_zb_group<<<nb, 256, 0, st>>>(assign, off, d_nev, counts, cap, cnt, nullptr, nullptr);
-    e = scan_exclusive(cnt, zoff, cur, (int)ng, nullptr, nullptr, tmp, st);
-    if (e != cudaSuccess) return e;
-    k_zb_group<<<nb, 256, 0, st>>>(assign, off, d_nev, counts, cap, nullptr, cur, list);
-    dim3 gs(max(1, min(device_sms() * 8 / max(n_ev, 1), 1024)), n_ev);
-    k_zb_small<<<gs, 256, 0, st>>>(G, x, y, z, peaks, counts, d_nev, cap, zoff, list, out, big,
-                                   nbig);
-    k_zb_big<<<device_sms() * 2, kBigThreads, z_big_smem(G), st>>>(G, x, y, z, peaks, zoff, list, big,
-                                                           nbig, out);
-    return cudaGetLastError();
+    return run_z(G, ZGroup{off, d_nev, counts, 0, cap}, n_ev, max_hits, x, y, z, assign, peaks, out,
+                 ws, st);
 }
 
 cudaError_t launch_vote_z(const DevGeom &G, const float *x, const float *y, const float *z,
@@ -441,23 +470,8 @@ cudaError_t launch_vote_z(const DevGeom &G, const float *x, const float *y, cons
                           int cap, ht_zres *out, void *ws, cudaStream_t st)
 {
     if (cap == 0) return cudaSuccess;
-    ZWs w = carve(ws, n, cap);
-    cudaError_t e = cudaMemsetAsync(w.cnt, 0, (size_t)(cap + 1) * 4, st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(w.nbig, 0, 4, st);
-    if (e != cudaSuccess) return e;
-    const int nb = n > 0 ? min(4096, (n + 255) / 256) : 1;
-    if (n > 0) k_z_count<<<nb, 256, 0, st>>>(assign, n, d_count, cap, w.cnt);
-    e = scan_exclusive(w.cnt, w.off, w.cur, cap, d_count, nullptr, w.tmp, st);
-    if (e != cudaSuccess) return e;
-    if (n > 0) k_z_scatter<<<nb, 256, 0, st>>>(assign, n, d_count, cap, w.cur, w.list);
-    const int warps_needed = cap;
-    const int blocks = min(device_sms() * 16, (warps_needed + 7) / 8);
-    k_z_small<<<blocks, 256, 0, st>>>(G, x, y, z, peaks, d_count, cap, w.off, w.list, out, w.big,
-                                      w.nbig);
-    k_z_big<<<device_sms() * 2, kBigThreads, z_big_smem(G), st>>>(G, x, y, z, peaks, w.off, w.list, w.big,
-                                                          w.nbig, out);
-    return cudaGetLastError();
+    return run_z(G, ZGroup{nullptr, nullptr, d_count, n, cap}, 1, n, x, y, z, assign, peaks, out,
+                 ws, st);
 }
 
 }  // namespace ht
