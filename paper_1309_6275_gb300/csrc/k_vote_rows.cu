@@ -25,8 +25,8 @@
 //   walk  curves that keep a bin for a word of rows or more: 32 / NWB hits per
 //         step, one lane per (hit, word), each lane walking its word's bins;
 //   edge  steeper ones up to kEdgeSlope bins per row: 8, 16 or 32 lanes per
-//         hit, a lane per bin, whose rows lie between its own crossing and
-//         the previous lane's;
+//         hit, a lane per bin (two beyond 32 bins), whose rows lie between its
+//         own crossing and the previous lane's;
 //   row   the steepest, in the A-form of tiles.cuh: one hit per step, one
 //         lane per row of the hit's row window (the rows whose circles can
 //         reach the axis);
@@ -42,16 +42,16 @@
 // Why here: the tile kernel this replaces evaluated every (hit, row) of a
 // column (52.7 thread instructions per vote; 29.5 lanes) and built each (hit,
 // column) item three times, once per 64-row tile.  Of a 17k-hit event's 24.5k
-// votes per hit, 4.0k runs of rows remain.  Issue-bound now (73% of slots); an
-// edge step takes about 80 instructions for 32 bins, a row step 65 for 32
-// rows.  Vote stage with hit index, GB300, 25 events of 2k-60k hits (256 x 128
-// x 512 cells): 18.3 -> 9.6 ms; 25 of 10k: 11.2 -> 5.9; with top-8 region sets
-// 14.6 -> 6.3; two of 50k (512 x 256 x 1024): 32.2 -> 18.3.
+// votes per hit, 4.0k runs of rows remain.  Issue-bound now (76% of slots).
+// Vote stage with hit index, GB300, 25 events of 2k-60k hits (256 x 128 x 512
+// cells): 18.3 -> 8.5 ms; 25 of 10k: 11.2 -> 5.2; with top-8 region sets 14.6
+// -> 6.1; two of 50k (512 x 256 x 1024): 32.2 -> 17.7.
 //
-// Constants, each measured on those batches: kEdgeSlope 0.6 (0.5 to 0.8 equal,
-// 1.1 6% slower: a steep curve has fewer rows than bins); 3 CTAs of 320
-// threads (4 of 256 spill: 5% slower; 5 with 8 resident layers: 20%); kRes 10
-// layers resident keep three CTAs, and the detector has ten.
+// Constants, each measured on those batches: kEdgeSlope 0.5 (0.45 to 0.6
+// equal, 1.0 5% slower: a steep curve has fewer rows than bins); kWalkSlope
+// 1/64 (1/16 2% slower); two bins per lane beyond 32 bins (one: 10% slower);
+// 3 CTAs of 320 threads (256: 4% slower, 384: 5%); kRes 10 layers resident
+// keep three CTAs, and the detector has ten.
 //
 // In the batch the hits come from the (layer, azimuth) index of
 // k_hitindex.cu: a column scans, per layer, the run of azimuth cells whose
@@ -72,8 +72,8 @@ constexpr int kVrThreads = 320, kVrWarps = kVrThreads / 32;
 constexpr int kRes = 10;              // layers resident in a tile (more: a second round)
 constexpr int kVrRedo = 96;           // redo slots per warp
 constexpr int kVrPad = 4;             // words between rows of words: spreads one bin's words over banks
-constexpr float kWalkSlope = 1.0f / 32.0f;   // bins per row up to which a curve is walked
-constexpr float kEdgeSlope = 0.6f;    // and up to which a lane takes a bin
+constexpr float kWalkSlope = 1.0f / 64.0f;   // bins per row up to which a curve is walked
+constexpr float kEdgeSlope = 0.5f;    // and up to which a lane takes a bin
 constexpr float kWalkEps = 8.0f;      // rows of uncertainty at a crossing
 constexpr float kEdgeEps = 0.25f;     // (an edge lane's at most one row)
 constexpr size_t kVrBitmap = 43 * 1024;
@@ -456,7 +456,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             const int p = s_rs[run] + (ch - s_cp[run]) * 32 + lane;
             bool live = p < s_re[run];
             // ---- one hit per lane: its kind and its constants
-            enum { kWalk, kEdge8, kEdge16, kEdge32, kRow, kKinds, kNone = kKinds };
+            enum { kWalk, kEdge8, kEdge16, kEdge32, kEdge64, kRow, kKinds, kNone = kKinds };
             int kind = kNone;
             // item rows: the window's (bytes 0 and 3) without bytes 1 .. 2 (all when 1 > 2)
             unsigned rest = 0u;
@@ -560,7 +560,8 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                                 } else if (flat ? eps <= kWalkEps
                                                 : eps <= kEdgeEps && c > 2.4e-7f * G.kr_f) {
                                     kind = flat ? kWalk : nbin <= 8.0f ? kEdge8
-                                           : nbin <= 16.0f ? kEdge16 : kEdge32;
+                                           : nbin <= 16.0f ? kEdge16
+                                           : nbin <= 32.0f ? kEdge32 : kEdge64;
                                     ma = make_float4(s, c, eps, jt - G.off_f);
                                     mb.x = nbin;
                                     mb.z = __int_as_float(__float_as_int(mb.z) + (int)jt);
@@ -638,115 +639,142 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             }
             __syncwarp();
 
-            // ---- edge: lane = (hit, bin), 2^lg lanes per hit
+            // ---- edge: lane = (hit, bin)
+            const float jcap = (float)ND - G.off_f - 0.25f;
+            // votes rows r .. last (in one word, or two, or more) of the bin of word wp
+            // (lower edge jo); the virtual bin above the axis has none
+            auto emit = [&](uint32_t *wp, int r, int last, float jo, unsigned long long hs) {
+                if (!(r <= last && jo < jcap)) return;
+                uint32_t m = kAll << (r & 31), m2 = kAll >> (31 - (last & 31));
+                const int w0 = r >> 5, w1 = last >> 5;
+                if (w0 == w1) m &= m2;
+                if (HIT) {
+                    const unsigned jm = S.jmask[(int)(jo + G.off_f + 0.25f)];
+                    m &= allowed(hs, jm, w0);
+                    m2 = w1 > w0 ? m2 & allowed(hs, jm, w1) : 0u;
+                    my_cast += __popc(m) + __popc(m2);
+                } else {
+                    my_cast += last - r + 1;
+                }
+                atomicOr(wp + w0 * NDp, m);
+                if (w1 > w0) {
+                    atomicOr(wp + w1 * NDp, m2);
+                    for (int w = w0 + 1; w < w1; ++w) {   // a run over a whole word
+                        uint32_t mm = kAll;
+                        if (HIT) {
+                            mm = allowed(hs, S.jmask[(int)(jo + G.off_f + 0.25f)], w);
+                            my_cast += __popc(mm);
+                        }
+                        atomicOr(wp + w * NDp, mm);
+                    }
+                }
+            };
+            // up to 32 bins: 2^lg lanes per hit
 #pragma unroll 1
             for (int lg = 3; lg <= 5; ++lg) {
                 const int qb = lg == 3 ? first[kEdge8] : lg == 4 ? first[kEdge16] : first[kEdge32];
-                const int qe = lg == 3 ? first[kEdge16] : lg == 4 ? first[kEdge32] : first[kRow];
+                const int qe = lg == 3 ? first[kEdge16] : lg == 4 ? first[kEdge32] : first[kEdge64];
                 const int width = 1 << lg, sub = lane & (width - 1);
-                const float fsub = (float)sub, jcap = (float)ND - G.off_f - 0.25f;
+                const float fsub = (float)sub;
 #pragma unroll 1
                 for (int q0 = qb; q0 < qe; q0 += 32 >> lg) {
                     const bool act = q0 + (lane >> lg) < qe;
                     const int q = act ? q0 + (lane >> lg) : q0;
                     const float4 a = slot[q].a, b = slot[q].b;
-                    const float s = a.x, c = a.y, c2 = c * c;
-                    const int rab = __float_as_int(b.y);
-                    const int rb = act ? rab >> 16 : -1000;   // no row
+                    const int rab = __float_as_int(b.y), ra1 = (rab & 0xffff) - 1, rb = rab >> 16;
                     unsigned long long hs = 0ull;
                     if (HIT) hs = shm[q];
-                    int up = (rab & 0xffff) - 1;   // the last row settled by the edges above
-                    float jo = a.w - fsub;         // the lane's lower edge, in bins from d0 = 0
-                    // bins left at and below the lane's, the virtual one above the axis counted
-                    float left = b.x - (float)sub;
-                    uint32_t *wp = S.bm + (__float_as_int(b.z) & 0xffff) - sub;
-                    for (;;) {
-                        int lo, hi;
-                        crossing(cross_row(G, jo, s, c, c2, tc), a.z, lo, hi);
-                        const int pv = __shfl_up_sync(kAll, hi, 1, width);
-                        const int before = sub == 0 ? up : max(pv, (rab & 0xffff) - 1);
-                        const bool bin = left > 0.5f;
-                        const int r = before + 1, last = min(lo, rb);
-                        if (bin && r <= last && jo < jcap) {
-                            // the rows r .. last: in one word, or two
-                            uint32_t m = kAll << (r & 31), m2 = kAll >> (31 - (last & 31));
-                            const int w0 = r >> 5, w1 = last >> 5;
-                            if (w0 == w1) m &= m2;
-                            if (HIT) {
-                                const unsigned jm = S.jmask[(int)(jo + G.off_f + 0.25f)];
-                                m &= allowed(hs, jm, w0);
-                                m2 = w1 > w0 ? m2 & allowed(hs, jm, w1) : 0u;
-                                my_cast += __popc(m) + __popc(m2);
-                            } else {
-                                my_cast += last - before;
-                            }
-                            atomicOr(wp + w0 * NDp, m);
-                            if (w1 > w0) {
-                                atomicOr(wp + w1 * NDp, m2);
-                                for (int w = w0 + 1; w < w1; ++w) {   // a run over a whole word
-                                    uint32_t mm = kAll;
-                                    if (HIT) {
-                                        mm = allowed(hs, S.jmask[(int)(jo + G.off_f + 0.25f)], w);
-                                        my_cast += __popc(mm);
-                                    }
-                                    atomicOr(wp + w * NDp, mm);
-                                }
-                            }
-                        }
-                        if (hi > lo && bin) {   // one row within the bound of this edge
-                            if (lo >= before && lo < rb)
-                                push(__float_as_int(b.w), lo + 1, __float_as_int(b.z) >> 16);
-                        }
-                        if (lg < 5 || b.x <= 32.0f) break;   // uniform for 32 lanes
-                        if (!(__shfl_sync(kAll, left, 31) > 1.5f)) break;
-                        up = __shfl_sync(kAll, hi, 31);
-                        jo -= 32.0f;
-                        left -= 32.0f;
-                        wp -= 32;
+                    const float jo = a.w - fsub;   // the lane's lower edge, in bins from d0 = 0
+                    int lo, hi;
+                    crossing(cross_row(G, jo, a.x, a.y, a.y * a.y, tc), a.z, lo, hi);
+                    const int pv = __shfl_up_sync(kAll, hi, 1, width);
+                    const int before = sub == 0 ? ra1 : max(pv, ra1);   // rows settled above
+                    if (act && fsub < b.x) {
+                        emit(S.bm + (__float_as_int(b.z) & 0xffff) - sub, before + 1, min(lo, rb), jo, hs);
+                        // one row within the bound of this edge
+                        if (hi > lo && lo >= before && lo < rb)
+                            push(__float_as_int(b.w), lo + 1, __float_as_int(b.z) >> 16);
                     }
+                }
+            }
+            // more: a lane takes two bins
+#pragma unroll 1
+            for (int q = first[kEdge64]; q < first[kRow]; ++q) {
+                const float4 a = slot[q].a, b = slot[q].b;
+                const int rab = __float_as_int(b.y), rb = rab >> 16;
+                const float s = a.x, c = a.y, c2 = c * c;
+                unsigned long long hs = 0ull;
+                if (HIT) hs = shm[q];
+                int up = (rab & 0xffff) - 1;             // rows settled by the edges above
+                float jo = a.w - (float)(2 * lane), left = b.x - (float)(2 * lane);
+                uint32_t *wp = S.bm + (__float_as_int(b.z) & 0xffff) - 2 * lane;
+#pragma unroll 1
+                for (;;) {
+                    int lo0, hi0, lo1, hi1;
+                    crossing(cross_row(G, jo, s, c, c2, tc), a.z, lo0, hi0);
+                    crossing(cross_row(G, jo - 1.0f, s, c, c2, tc), a.z, lo1, hi1);
+                    const int pv = __shfl_up_sync(kAll, hi1, 1);
+                    const int before = lane == 0 ? up : max(pv, up);
+                    const int mid = max(hi0, before);
+                    if (left > 0.5f) emit(wp, before + 1, min(lo0, rb), jo, hs);
+                    if (left > 1.5f) emit(wp - 1, mid + 1, min(lo1, rb), jo - 1.0f, hs);
+                    if (hi0 > lo0 || hi1 > lo1) {        // a row within the bound of an edge
+                        const int l = __float_as_int(b.z) >> 16, pp = __float_as_int(b.w);
+                        if (hi0 > lo0 && left > 0.5f && lo0 >= before && lo0 < rb) push(pp, lo0 + 1, l);
+                        if (hi1 > lo1 && left > 1.5f && lo1 >= mid && lo1 < rb) push(pp, lo1 + 1, l);
+                    }
+                    if (!(__shfl_sync(kAll, left, 31) > 2.5f)) break;   // uniform
+                    up = __shfl_sync(kAll, hi1, 31);
+                    jo -= 64.0f;
+                    left -= 64.0f;
+                    wp -= 64;
                 }
             }
             __syncwarp();
 
-            // ---- row: lane = row of the window, 64 rows at a time
+            // ---- row: lane = row of the window; a lane's bit and the step of its word
+            // are the same for all its rows
 #pragma unroll 1
             for (int q = first[kRow]; q < first[kKinds]; ++q) {
-                const float mnd = kMagic + (float)ND;
                 const float4 a = slot[q].a, b = slot[q].b;
-                const int rend = __float_as_int(b.y) >> 16, l = __float_as_int(b.z) >> 16;
-                uint32_t *const wp = S.bm + (__float_as_int(b.z) & 0xffff);
-                auto eval = [&](int row, int &j, bool &vote, bool &rd) {
-                    const bool in = row <= rend;
-                    RowCtx R;
-                    R.rho = S.rho[in ? row : 0];
-                    R.rho2 = R.rho * R.rho;
-                    R.arho = fabsf(R.rho);
-                    aform_bin(R, a, b.x, mnd, j, vote, rd);
-                    vote &= in;
-                    rd &= in;
-                };
-                auto cast = [&](int row, int j, bool vote, bool rd) {
-                    if (HIT && vote) {
-                        const unsigned sh = S.rowblk[row];
-                        const unsigned long long hs = shm[q];
-                        const unsigned bits = (unsigned)((hs >> (sh & 63)) | (hs >> ((sh >> 8) & 63)) |
-                                                         (hs >> ((sh >> 16) & 63))) & 0xffu;
-                        vote = (bits & S.jmask[j]) != 0u;
+                const int rend = __float_as_int(b.y) >> 16;
+                int row = (__float_as_int(b.y) & 0xffff) + lane;
+                const uint32_t bit = 1u << (row & 31);
+                uint32_t *wp = S.bm + (__float_as_int(b.z) & 0xffff) + (row >> 5) * NDp;
+                unsigned long long hs = 0ull;
+                if (HIT) hs = shm[q];
+                auto one = [&](int rw, uint32_t *w) {
+                    if (rw > rend) return;
+                    const float rho = S.rho[rw];
+                    const float D = fmaf(-(rho * rho), a.y, 1.0f);
+                    const float den = fmaf(D, rsqrt_approx(D), 1.0f);
+                    const float u = fmaf(-(rho * a.z), rcp_approx(den), a.x);
+                    const float e = fmaf(fabsf(rho), b.x, a.w);
+                    const float lo = __fadd_rd(__fsub_rd(u, e), kMagic);
+                    const float hi = __fadd_rd(__fadd_ru(u, e), kMagic);
+                    const int j = __float_as_int(lo) - kMagicBits;
+                    if (lo == hi) {
+                        bool ok = (unsigned)j < (unsigned)ND;
+                        if (HIT && ok) {
+                            const unsigned sh = S.rowblk[rw];
+                            const unsigned bits = (unsigned)((hs >> (sh & 63)) | (hs >> ((sh >> 8) & 63)) |
+                                                             (hs >> ((sh >> 16) & 63))) & 0xffu;
+                            ok = (bits & S.jmask[j]) != 0u;
+                        }
+                        if (ok) {
+                            atomicOr(w + j, bit);
+                            ++my_cast;
+                        }
+                    } else if (hi >= kMagic && lo < kMagic + (float)ND) {   // not certainly outside
+                        push(__float_as_int(b.w), rw, __float_as_int(b.z) >> 16);
                     }
-                    if (vote) {
-                        atomicOr(wp + (row >> 5) * NDp + j, 1u << (row & 31));
-                        ++my_cast;
-                    }
-                    if (rd) push(__float_as_int(b.w), row, l);
                 };
 #pragma unroll 1
-                for (int r0 = __float_as_int(b.y) & 0xffff; r0 <= rend; r0 += 64) {
-                    int j0, j1 = 0;
-                    bool v0, v1 = false, d0, d1 = false;
-                    eval(r0 + lane, j0, v0, d0);
-                    if (r0 + 32 <= rend) eval(r0 + 32 + lane, j1, v1, d1);   // uniform
-                    cast(r0 + lane, j0, v0, d0);
-                    cast(r0 + 32 + lane, j1, v1, d1);
+                for (int left = rend - (row - lane); left >= 0; left -= 64) {   // uniform
+                    one(row, wp);
+                    if (left >= 32) one(row + 32, wp + NDp);
+                    row += 64;
+                    wp += 2 * NDp;
                 }
             }
             __syncwarp();
