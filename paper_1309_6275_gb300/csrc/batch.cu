@@ -73,8 +73,9 @@ cudaError_t launch_hit_masks(const void *params_bf16, const float *x, const floa
                              const float *z, const uint8_t *layer, int n, const int *d_n,
                              int topk, float pmin, unsigned long long *hit_masks, cudaStream_t st);
 cudaError_t launch_vote_batch_layers(const DevGeom &G, const HitIndex &I, const int *off,
-                                     const int *order, const int *d_nev, uint32_t *planes,
-                                     size_t stride, unsigned long long *stats, int *head, int sms,
+                                     const int *order, const int *d_nev, const int *d_ncell,
+                                     uint32_t *planes, size_t stride, unsigned long long *stats,
+                                     int *heads, int sms,
                                      const unsigned long long *hit_masks, cudaStream_t st);
 }  // namespace ht
 
@@ -114,7 +115,8 @@ struct ht_batch {
     size_t slot_words;  // 32-bit words of an event's slot in acc
     uint16_t *acc;      // plain path: counts, cells apart; track path: bit planes
                         // and peak bits, slot_words apart
-    int *meta;          // [0] n_big [1] pad [2] n_all [3] pad, off[max_events + 1],
+    int *meta;          // [0] n_big [1] events of at least kCellHits hits [2] n_all [3] pad,
+                        // off[max_events + 1],
                         // order_big[max_events], order_all[max_events] (largest first),
                         // thr[max_events] (peak threshold of each event slot)
     int *h_meta;        // pinned staging, same layout
@@ -258,8 +260,8 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
         uint32_t *planes = reinterpret_cast<uint32_t *>(b->acc);
         if (e == cudaSuccess)
             e = ht::launch_vote_batch_layers(G, b->idx, off, order_all_of(meta, me), meta + 2,
-                                             planes, b->slot_words, st64, b->heads + 1, b->sms,
-                                             R.hit_masks, st);
+                                             meta + 1, planes, b->slot_words, st64, b->heads + 1,
+                                             b->sms, R.hit_masks, st);
         if (e == cudaSuccess) e = mark(2);
         if (e == cudaSuccess)
             e = ht::launch_plane_peaks(G, planes, b->slot_words, b->idx.rmm, thr_of(meta, me),
@@ -345,13 +347,15 @@ ht_status stage_meta(ht_batch *b, const int32_t *h_off, int n_ev, cudaStream_t s
     std::stable_sort(idx.begin(), idx.end(), [&](int a, int c) {
         return h_off[a + 1] - h_off[a] > h_off[c + 1] - h_off[c];
     });
-    int nb = 0;
+    int nb = 0, ncell = 0;
     for (int i = 0; i < n_ev; ++i) {
         const int ev = idx[i];
+        if (h_off[ev + 1] - h_off[ev] >= ht::kCellHits) ++ncell;   // a prefix: largest first
         if (h_off[ev + 1] - h_off[ev] > ht::kPackMaxHits) order_big_of(hm, me)[nb++] = ev;
         order_all_of(hm, me)[i] = ev;
     }
     hm[0] = nb;
+    hm[1] = ncell;
     hm[2] = n_ev;
     // peak threshold of each event slot (track path): the first band holding
     // the event's hit count, else the geometry's threshold

@@ -413,6 +413,7 @@ struct HitIndex {
     float *x, *y;
     int *h;
     uint8_t *l;
+    int *unsorted;   // per (event, layer): cells whose hits are not in azimuth order
     void *tmp;
     int ncells;
 };
@@ -437,6 +438,12 @@ HitIndex carve_hit_index(int max_events, int max_hits, void *ws);
 cudaError_t launch_hit_index(const float *x, const float *y, const uint8_t *layer,
                              const int *off, const int *d_nev, int max_events, int max_hits,
                              const HitIndex &I, int sms, cudaStream_t st);
+// Orders the hits of every cell of the first *d_n events of order[] by azimuth.
+cudaError_t launch_hit_sort(const HitIndex &I, const int *order, const int *d_n, int sms,
+                            cudaStream_t st);
+// Events of at least this many hits vote their dense layers cell by cell
+// (k_vote_rows.cu).
+constexpr int kCellHits = 24000;
 
 // Candidate confirmation (k_confirm.cu): parameters as ht_confirm_desc.
 struct ConfirmDev {

@@ -67,11 +67,70 @@ __global__ void k_hidx(const float *__restrict__ x, const float *__restrict__ y,
     }
 }
 
-__global__ void k_hidx_init(unsigned *__restrict__ rmm, int n)
+// One warp per cell of up to 64 hits: each lane counts the hits before its
+// own in azimuth (the sign of a cross product, exact by Kahan's difference of
+// products as long as nothing underflows; collinear hits in index order) and
+// moves them there.  Larger cells, and cells with a hit within 1e-6 cm of the
+// origin, not finite or with a coordinate so small that a product's rounding
+// error could underflow, stay as they are and are counted.
+__global__ void __launch_bounds__(256)
+k_hidx_sort(HitIndex I, const int *__restrict__ order, const int *__restrict__ d_n)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int nw = gridDim.x * (blockDim.x >> 5);
+    const int total = *d_n * 16 * kIdxAz;
+    for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < total; t += nw) {
+        const int el = order[t / (16 * kIdxAz)] * 16 + (t / kIdxAz) % 16;
+        const int cell = el * kIdxAz + t % kIdxAz;
+        const int a = I.offs[cell], n = I.offs[cell + 1] - a;
+        if (n < 2) continue;
+        float x[2], y[2];
+        int h[2], rank[2] = {0, 0};
+        bool ok = n <= 64;
+        if (ok) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int q = lane + 32 * u;
+                const bool in = q < n;
+                x[u] = in ? I.x[a + q] : 1.0f;
+                y[u] = in ? I.y[a + q] : 0.0f;
+                h[u] = in ? I.h[a + q] : 0;
+                const float ax = fabsf(x[u]), ay = fabsf(y[u]);
+                ok = ok && ax + ay > 1e-6f && ax + ay < 1e12f &&
+                     (ax > 1e-12f || ax == 0.0f) && (ay > 1e-12f || ay == 0.0f);
+            }
+        }
+        if (!__all_sync(kAll, ok)) {
+            if (lane == 0) atomicAdd(&I.unsorted[el], 1);
+            continue;
+        }
+        for (int q = 0; q < n; ++q) {
+            const float xq = __shfl_sync(kAll, q < 32 ? x[0] : x[1], q & 31);
+            const float yq = __shfl_sync(kAll, q < 32 ? y[0] : y[1], q & 31);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float w = __fmul_rn(yq, x[u]);
+                const float d = fmaf(xq, y[u], -w) + fmaf(-yq, x[u], w);   // xq y - yq x
+                rank[u] += d > 0.0f || (d == 0.0f && q < lane + 32 * u);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (lane + 32 * u < n) {
+                I.x[a + rank[u]] = x[u];
+                I.y[a + rank[u]] = y[u];
+                I.h[a + rank[u]] = h[u];
+            }
+    }
+}
+
+__global__ void k_hidx_init(unsigned *__restrict__ rmm, int *__restrict__ unsorted, int n)
 {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         rmm[2 * t] = 0x7f800000u;   // +inf: empty layer (min > max)
         rmm[2 * t + 1] = 0u;
+        unsorted[t] = 0;
     }
 }
 
@@ -82,7 +141,8 @@ size_t hit_index_bytes(int max_events, int max_hits)
     const size_t nc = (size_t)max_events * 16 * kIdxAz;
     const size_t mh = (size_t)(max_hits > 0 ? max_hits : 1);
     return 3 * align256((nc + 1) * 4) + align256((size_t)max_events * 16 * 8) +
-           3 * align256(mh * 4) + align256(mh) + scan_tmp_bytes((int)nc);
+           3 * align256(mh * 4) + align256(mh) + align256((size_t)max_events * 16 * 4) +
+           scan_tmp_bytes((int)nc);
 }
 
 HitIndex carve_hit_index(int max_events, int max_hits, void *ws)
@@ -107,6 +167,8 @@ HitIndex carve_hit_index(int max_events, int max_hits, void *ws)
     p += align256(mh * 4);
     I.l = reinterpret_cast<uint8_t *>(p);
     p += align256(mh);
+    I.unsorted = reinterpret_cast<int *>(p);
+    p += align256((size_t)max_events * 16 * 4);
     I.tmp = p;
     I.ncells = (int)nc;
     return I;
@@ -118,13 +180,20 @@ cudaError_t launch_hit_index(const float *x, const float *y, const uint8_t *laye
 {
     cudaError_t e = cudaMemsetAsync(I.cnt, 0, (size_t)I.ncells * 4, st);
     if (e != cudaSuccess) return e;
-    k_hidx_init<<<32, 256, 0, st>>>(I.rmm, max_events * 16);
+    k_hidx_init<<<32, 256, 0, st>>>(I.rmm, I.unsorted, max_events * 16);
     const int grid = sms * 4;
     k_hidx<<<grid, 256, 0, st>>>(x, y, layer, off, d_nev, I.cnt, I.rmm, nullptr, I);
     e = scan_exclusive(I.cnt, I.offs, I.cur, I.ncells, nullptr, I.offs + I.ncells, I.tmp, st);
     if (e != cudaSuccess) return e;
     k_hidx<<<grid, 256, 0, st>>>(x, y, layer, off, d_nev, I.cnt, I.rmm, I.cur, I);
     (void)max_hits;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hit_sort(const HitIndex &I, const int *order, const int *d_n, int sms,
+                            cudaStream_t st)
+{
+    k_hidx_sort<<<sms * 8, 256, 0, st>>>(I, order, d_n);
     return cudaGetLastError();
 }
 

@@ -53,6 +53,25 @@
 // 3 CTAs of 320 threads (256: 4% slower, 384: 5%); kRes 10 layers resident
 // keep three CTAs, and the detector has ten.
 //
+// Cell by cell.  Where many hits of a layer can vote in a column, going
+// through them costs more than going through the column's cells, and that
+// cost does not grow with the hits.  For one radius r the circle of (rho, d0)
+// meets the layer at s = -S, S(rho, d0) = (rho (d0^2 + r^2) + 2 d0) / (2 (1 +
+// rho d0)), so a cell holds a hit's root iff the hit's -s lies between S at
+// the bin's two edges.  The index keeps each layer in azimuth order
+// (k_hidx_sort) and -s is sorted along it, so an edge's place among the hits is
+// a table lookup over s and a step or two along them, and the bits of 32 rows
+// (a lane each) of a bin are one ballot.  Only where a bin depends on a hit
+// within the error bound of an edge is that hit evaluated by the definition.
+// The number of votes telescopes: per row, the hits between the axis' ends.
+// A layer's rows where S is not monotone (tight curls) keep the hit-by-hit
+// vote, as do sparse layers (kCellMin: 160, 300 and 500 time alike), layers
+// whose radii spread, and smaller events: kCellHits = 24000 measured, for 25
+// events of 2k-60k hits on 256 x 128 x 512 cells, 7.49 ms (20000: 7.67, 16000:
+// 7.88, 12000: 8.25, none: 8.67), and for two of 50k hits on 512 x 256 x 1024 14.2 ms
+// instead of 18.1.  It is bound
+// by instructions (3.25 G for 6 events of 30k hits, the issue slots 75% busy).
+//
 // In the batch the hits come from the (layer, azimuth) index of
 // k_hitindex.cu: a column scans, per layer, the run of azimuth cells whose
 // hits can reach it, and a warp's hits have about the same curve, so its
@@ -77,6 +96,10 @@ constexpr float kEdgeSlope = 0.5f;    // and up to which a lane takes a bin
 constexpr float kWalkEps = 8.0f;      // rows of uncertainty at a crossing
 constexpr float kEdgeEps = 0.25f;     // (an edge lane's at most one row)
 constexpr size_t kVrBitmap = 43 * 1024;
+constexpr int kClThreads = 512;       // cell-by-cell tiles: two CTAs of 16 warps per SM
+constexpr int kClMaxHits = 4096;      // hits of a layer in a column's window, at most
+constexpr int kCellMin = 160;         // and at least, to go cell by cell
+constexpr int kClTab = 2048;          // table entries over a layer's s
 
 // Where a tile's hits come from: the batch's hit index (offs set), or an
 // event's arrays in the caller's order (offs null, n hits).
@@ -87,6 +110,7 @@ struct HitSource {
     const int *offs;
     const unsigned *rmm;
     int n;
+    const int *unsorted;      // cells: layers not in azimuth order (index only)
 };
 
 struct VrSlot {
@@ -96,25 +120,31 @@ struct VrSlot {
 // Shared memory of a tile (dynamic), in this order.
 struct VrSmem {
     uint32_t *bm;             // [kRes][NWB][ND + kVrPad]
-    VrSlot *slot;             // [kVrWarps][32]
-    int4 *item;               // [kVrWarps][32]: item rows, layer | flags, position
-    int2 *redo;               // [kVrWarps][kVrRedo]: position, row << 4 | layer
+    VrSlot *slot;             // [warps][32]
+    int4 *item;               // [warps][32]: item rows, layer | flags, position
+    int2 *redo;               // [warps][kVrRedo]: position, row << 4 | layer
+    float *sig;               // CELLS: [kClMaxHits + 1] a layer's -s, over the slots
+    uint16_t *tab;            // CELLS: [kClTab] hits certainly below a bin of s
     float *rho;               // [32 NWB]
-    unsigned long long *hm;   // HIT: [kVrWarps][32] region sets of the slots
+    unsigned long long *hm;   // HIT: [warps][32] region sets of the slots
     uint32_t *rowmask;        // HIT: [NWB][8] rows of the word in or next to rho block b
     uint32_t *rowblk;         // HIT: [32 NWB] rho blocks (x 8) of rows i - 1, i, i + 1
     uint8_t *jmask;           // HIT: [ND] d0 blocks of bins j - 1, j, j + 1
 };
 
-__host__ __device__ constexpr size_t vr_smem(int nwb, int nd, bool hit)
+__host__ __device__ constexpr size_t vr_smem(int nwb, int nd, bool hit, bool cells)
 {
     const size_t rows = (size_t)32 * nwb;
-    size_t b = (size_t)kRes * nwb * (nd + kVrPad) * 4 + (size_t)kVrWarps * 32 * (sizeof(VrSlot) + 16) +
-               (size_t)kVrWarps * kVrRedo * 8 + rows * 4;
+    const size_t warps = cells ? kClThreads / 32 : kVrWarps;
+    size_t b = warps * 32 * (sizeof(VrSlot) + 16) + warps * kVrRedo * 8 +
+               (size_t)kRes * nwb * (nd + kVrPad) * 4 + rows * 4;
     b = (b + 15) / 16 * 16;
-    if (hit) b += (size_t)kVrWarps * 32 * 8 + (size_t)nwb * 32 + rows * 4 + (nd + 15) / 16 * 16;
+    if (hit) b += warps * 32 * 8 + (size_t)nwb * 32 + rows * 4 + (nd + 15) / 16 * 16;
+    if (cells) b += (size_t)kClTab * 2;
     return b;
 }
+static_assert((kClThreads / 32) * 32 * (sizeof(VrSlot) + 16) >= (kClMaxHits + 1) * sizeof(float),
+              "a layer's hits fit the slots' space");
 
 // Words of rows per band: the largest power of two whose bitmap fits, at
 // most 8 (32 rows x 8 words keep three tiles per SM at 128 bins) and no more
@@ -128,25 +158,31 @@ __host__ __device__ inline int vr_nwb(int n_rho, int nd)
     return nwb;
 }
 
-template <int NWB, bool HIT>
+template <int NWB, bool HIT, bool CELLS>
 __device__ __forceinline__ VrSmem vr_carve(unsigned char *p, int nd)
 {
+    constexpr size_t warps = CELLS ? kClThreads / 32 : kVrWarps;
     VrSmem S{};
     // 16-byte items first: the slots, then the rest
     S.slot = reinterpret_cast<VrSlot *>(p);
-    p += (size_t)kVrWarps * 32 * sizeof(VrSlot);
+    S.sig = reinterpret_cast<float *>(p);
+    p += warps * 32 * sizeof(VrSlot);
     S.item = reinterpret_cast<int4 *>(p);
-    p += (size_t)kVrWarps * 32 * 16;
+    p += warps * 32 * 16;
     if (HIT) {
         S.hm = reinterpret_cast<unsigned long long *>(p);
-        p += (size_t)kVrWarps * 32 * 8;
+        p += warps * 32 * 8;
     }
     S.redo = reinterpret_cast<int2 *>(p);
-    p += (size_t)kVrWarps * kVrRedo * 8;
+    p += warps * kVrRedo * 8;
     S.bm = reinterpret_cast<uint32_t *>(p);
     p += (size_t)kRes * NWB * (nd + kVrPad) * 4;
     S.rho = reinterpret_cast<float *>(p);
     p += (size_t)32 * NWB * 4;
+    if (CELLS) {
+        S.tab = reinterpret_cast<uint16_t *>(p);
+        p += (size_t)kClTab * 2;
+    }
     if (HIT) {
         S.rowmask = reinterpret_cast<uint32_t *>(p);
         p += (size_t)NWB * 32;
@@ -289,40 +325,45 @@ __device__ __forceinline__ float row_coord(const DevGeom &G, float s, float c2, 
 // One tile of one event: votes, then the layer counts.
 // PLANES: out is the event's bit planes (see k_peak_planes.cu); otherwise the
 // accumulator of OutT counts.
-template <int NWB, bool HIT, bool PLANES, typename OutT>
+template <int NWB, bool HIT, bool PLANES, bool CELLS, typename OutT>
 __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, int e,
                                         const unsigned long long *__restrict__ hmask,
                                         void *__restrict__ out,
                                         unsigned long long *__restrict__ stats, int k, int band)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_rs[32], s_re[32], s_cp[33];   // runs of positions, chunks before each
+    constexpr int kThr = CELLS ? kClThreads : kVrThreads, kWarps = kThr / 32;
+    // runs of positions [rs, re) (index: layer << 2 | part << 1 | side), chunks
+    // before each, rows first | last << 16 they vote in
+    __shared__ int s_rs[64], s_re[64], s_cp[65], s_row[64];
     __shared__ int s_next, s_more, s_full;
-    __shared__ int s_nredo[kVrWarps];
+    __shared__ int s_nredo[kWarps];
     __shared__ unsigned long long s_stats[2];
+    __shared__ int s_ws[32], s_we[32];   // CELLS: window runs (layer << 1 | part)
+    __shared__ int s_bad, s_val[16];   // CELLS: a cell layer's rows first | last << 16, else -1
     constexpr unsigned kAll = 0xffffffffu;
     constexpr int kBand = 32 * NWB;
     constexpr int IPW = 32 / NWB;                  // hits per walk step
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ND = G.n_d0, NDp = ND + kVrPad, NW = (G.n_rho + 31) / 32;
-    const VrSmem S = vr_carve<NWB, HIT>(smem, ND);
+    const VrSmem S = vr_carve<NWB, HIT, CELLS>(smem, ND);
     const int i0 = band * kBand, nrow = min(kBand, G.n_rho - i0);
     const float tc = 0.5f * (float)(G.n_rho - 1) - (float)i0;   // row of rho = 0
 
-    for (int r = threadIdx.x; r < nrow; r += kVrThreads) S.rho[r] = G.rho32[i0 + r];
+    for (int r = threadIdx.x; r < nrow; r += kThr) S.rho[r] = G.rho32[i0 + r];
     if (HIT) {
         const int NR = G.n_rho;
-        for (int j = threadIdx.x; j < ND; j += kVrThreads)
+        for (int j = threadIdx.x; j < ND; j += kThr)
             S.jmask[j] = (uint8_t)((1u << region_block(max(j - 1, 0), ND)) |
                                    (1u << region_block(j, ND)) |
                                    (1u << region_block(min(j + 1, ND - 1), ND)));
-        for (int r = threadIdx.x; r < kBand; r += kVrThreads) {
+        for (int r = threadIdx.x; r < kBand; r += kThr) {
             const int i = min(i0 + r, NR - 1);
             S.rowblk[r] = (8u * region_block(max(i - 1, 0), NR)) |
                           (8u * region_block(i, NR) << 8) |
                           (8u * region_block(min(i + 1, NR - 1), NR) << 16);
         }
-        for (int q = threadIdx.x; q < NWB * 8; q += kVrThreads) {
+        for (int q = threadIdx.x; q < NWB * 8; q += kThr) {
             const int b = q & 7, f = i0 + 32 * (q >> 3);
             // rows [first of b - 1, first of b + 1] of the word; empty blocks hold none
             const int lo = max(block_first(b, NR) - 1 - f, 0);
@@ -333,7 +374,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
         }
     }
     if (threadIdx.x < 2) s_stats[threadIdx.x] = 0ull;
-    unsigned my_cast = 0u;
+    int my_cast = 0;   // votes (cell rows subtract what lies below the axis)
     int my_fb = 0;
 
     for (int l0 = 0; l0 < 16; l0 += kRes) {
@@ -373,16 +414,8 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             } else if (lane == 0 && (l0 == 0 || s_more)) {
                 end = H.n;
             }
-            const int nch = (end - start + 31) >> 5;
-            int incl = nch;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(kAll, incl, o);
-                if (lane >= o) incl += v;
-            }
-            s_rs[lane] = start;
-            s_re[lane] = end;
-            s_cp[lane + 1] = incl;
+            s_ws[lane] = start;
+            s_we[lane] = end;
             if (lane == 0) {
                 s_cp[0] = 0;
                 s_next = 0;
@@ -390,17 +423,18 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             __syncwarp();
             if (lane == 0 && l0 == 0) s_more = 0;
         }
-        if (threadIdx.x < kVrWarps) s_nredo[threadIdx.x] = 0;
+        if (threadIdx.x < kWarps) s_nredo[threadIdx.x] = 0;
+        if (CELLS && threadIdx.x < 16) s_val[threadIdx.x] = -1;
         __syncthreads();
-        const int nchunk = s_cp[32];
-        if (l0 > 0 && nchunk == 0) continue;   // uniform
+        bool none = true;
+        for (int q = 0; q < 32; ++q) none = none && s_we[q] <= s_ws[q];
+        if (l0 > 0 && none) continue;   // uniform
         {
             uint4 *z4 = reinterpret_cast<uint4 *>(S.bm);
             const int n4 = kRes * NWB * NDp / 4;   // NDp is a multiple of 2, kRes NWB too
-            for (int t = threadIdx.x; t < n4; t += kVrThreads) z4[t] = make_uint4(0, 0, 0, 0);
+            for (int t = threadIdx.x; t < n4; t += kThr) z4[t] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();
-
         VrSlot *const slot = S.slot + warp * 32;
         int4 *const imeta = S.item + warp * 32;
         unsigned long long *const shm = HIT ? S.hm + warp * 32 : nullptr;
@@ -411,7 +445,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             return S.bm + ((l - l0) * NWB + w) * NDp;
         };
         // the definition's votes of one (position, row), any tier
-        auto redo_row = [&](int p, int r, int l) {
+        auto redo_row = [&](int p, int r, int l, bool counted) {
             const unsigned pk = redo_packed(G, H.x[p], H.y[p], i0 + r, k);
             unsigned rb = 0u;
             if (HIT) rb = halo_row_blocks(set_hm(p), i0 + r, G.n_rho);
@@ -420,14 +454,27 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                 const int j = (int)((pk >> (16 * v)) & 0xffffu) - 1;
                 if (j < 0 || (HIT && !(rb & S.jmask[j]))) continue;
                 atomicOr(word0(l, r >> 5) + j, 1u << (r & 31));
-                ++my_cast;
+                if (counted) ++my_cast;
             }
         };
-        auto push = [&](int p, int r, int l) {
+        constexpr int kNotCounted = 1 << 30;   // the row's vote is counted already
+        auto push = [&](int p, int r, int l, int flag = 0) {
             ++my_fb;
             const int q = atomicAdd(&s_nredo[warp], 1);
-            if (q < kVrRedo) redo[q] = make_int2(p, (r << 4) | l);
-            else redo_row(p, r, l);
+            if (q < kVrRedo) redo[q] = make_int2(p, (r << 4) | l | flag);
+            else redo_row(p, r, l, flag == 0);
+        };
+        auto drain = [&]() {   // the warp's redos, a lane each (all lanes call)
+            __syncwarp();
+            const int nr = min(s_nredo[warp], kVrRedo);
+#pragma unroll 1
+            for (int t = lane; t < nr; t += 32) {
+                const int y = redo[t].y;
+                redo_row(redo[t].x, (y & ~kNotCounted) >> 4, y & 15, !(y & kNotCounted));
+            }
+            __syncwarp();
+            if (lane == 0) s_nredo[warp] = 0;
+            __syncwarp();
         };
         // rows [r, last] of word wd (in-word rows) allowed to the set hs in a
         // bin with d0 blocks jm
@@ -439,6 +486,162 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             return al;
         };
 
+        if constexpr (CELLS) {
+            for (int l = l0; l < l1; ++l) {   // uniform
+                const int st0 = s_ws[2 * l], n0 = s_we[2 * l] - st0;
+                const int st1 = s_ws[2 * l + 1], n = n0 + s_we[2 * l + 1] - st1;
+                if (n < kCellMin || n > kClMaxHits || H.unsorted[e * 16 + l] != 0) continue;
+                const float rmin = __uint_as_float(H.rmm[2 * (e * 16 + l)]);
+                const float rmax = __uint_as_float(H.rmm[2 * (e * 16 + l) + 1]);
+                const float dmax = G.dext_f;
+                if (!(rmin >= 1e-3f) || !(rmax < 1e6f)) continue;
+                // |rho| up to which S is monotone over the axis: with u = 1 - |rho| dmax,
+                // 1 + u^2 - rho^2 r^2 >= 0.05 (then dS/dd0 > 0 and sqrt(D) > 0.01)
+                const float rv = fminf(1.95f / (dmax + sqrtf(fmaxf(fmaf(1.95f * rmax, rmax,
+                                                                        -0.95f * dmax * dmax), 0.0f))),
+                                       0.95f / dmax) * 0.9999f;
+                const int vA = (int)fmaxf(ceilf(fmaf(-rv, G.inv_drho_f, tc)), 0.0f);
+                const int vB = (int)fminf(floorf(fmaf(rv, G.inv_drho_f, tc)), (float)(nrow - 1));
+                if (vB - vA < 32) continue;
+                // bound on S at an edge against -s of a hit (cm), first order: S's own
+                // rounding, the layer's spread in r^2, the hit's float32 s; and by how much
+                // hits can be out of order in s: the spread in r, atan2f's 3 ulp at a cell
+                // boundary (twice), the rounding of s
+                const float rt = fmaxf(fabsf(S.rho[vA]), fabsf(S.rho[vB]));
+                const float iu = 0.5f / (1.0f - rt * dmax);
+                const float r2 = 0.5f * fmaf(rmin, rmin, rmax * rmax);
+                const float eE = kEps * fmaf(iu, fmaf(8.0f * rt, fmaf(rmax, rmax, dmax * dmax), 12.0f * dmax),
+                                             4.0f * rmax);
+                const float eR2 = rt * iu * (0.51f * (rmax - rmin) * (rmax + rmin) +
+                                             8.0f * kEps * rmax * rmax);
+                const float eta = 1.01f * (rmax - rmin) + 2.3e-6f * rmax;   // how far out of order
+                const float eps = fmaf(kSafe, eE + eR2 + dot2_err(rmax, 2.0f * rmax), eta);
+                if (!(eps <= 0.05f * G.delta_f)) continue;
+                // ---- the layer's -s in azimuth order; hits with c <= 0 beyond its ends
+                __syncthreads();
+                if (threadIdx.x == 0) s_bad = 0;
+                __syncthreads();
+                {
+                    const float sk = G.sn32[k], ck = G.cs32[k], sl = G.snlo[k], cl = G.cslo[k];
+                    for (int t = threadIdx.x; t < n; t += kThr) {
+                        const int p = t < n0 ? st0 + t : st1 + t - n0;
+                        const float xf = H.x[p], yf = H.y[p];
+                        const float c = dot2(xf, ck, cl, yf, sk, sl);
+                        const float s = dot2(xf, sk, sl, -yf, ck, cl);
+                        const float Ec = (kSafe * 3.0f * kEps) * (fabsf(xf) + fabsf(yf));
+                        if (!(fabsf(c) > Ec)) s_bad = 1;   // sign of c not proven (or NaN)
+                        S.sig[t] = c > 0.0f ? -s : s < 0.0f ? 3.0e38f : -3.0e38f;
+                    }
+                    if (threadIdx.x == 0) S.sig[n] = 3.4e38f;
+                }
+                __syncthreads();
+                if (s_bad) continue;   // uniform
+                // ---- the table: below[q] = hits certainly before bin q = [q, q + 1) / kap - R
+                const float Rr = rmax * 1.001f, kap = (float)kClTab / (2.0f * Rr), k0 = Rr * kap;
+                const float ef = fmaf(2e-6f, Rr, eps + eta);   // and the rounding of a table bin
+                auto tbin = [&](float v) -> int {
+                    return (int)fminf(fmaxf(floorf(fmaf(v, kap, k0)), -1.0f), (float)(kClTab - 1));
+                };
+                for (int t = threadIdx.x; t <= n; t += kThr) {
+                    const int a1 = t < n ? tbin(S.sig[t] + ef) : kClTab - 1;
+                    const int a0 = t > 0 ? tbin(S.sig[t - 1] + ef) : -1;
+                    for (int q = a0 + 1; q <= a1; ++q) S.tab[q] = (uint16_t)t;
+                }
+                __syncthreads();
+                // the first hit not below v, from rank r on (a value past every edge ends
+                // the hits)
+                auto first_at = [&](float v, int r, float &t) -> int {
+                    const float q = fminf(fmaxf(fmaf(v, kap, k0), 0.0f), (float)(kClTab - 1));
+                    r = max(r, (int)S.tab[(int)q]);
+                    t = S.sig[r];
+                    while (t < v) t = S.sig[++r];
+                    return r;
+                };
+                // ---- units of one row word x 32 bins, a lane per row
+                const int nj = (ND + 31) >> 5;
+                for (int u = warp; u < NWB * nj; u += kWarps) {
+                    const int wd = u % NWB, j0 = (u / NWB) << 5, jn = min(32, ND - j0);
+                    const int row = 32 * wd + lane;
+                    const bool ok = row >= vA && row <= vB;
+                    const float rho = S.rho[min(max(row, vA), vB)], rr = rho * r2, rho2 = 2.0f * rho;
+                    uint32_t mine = 0u;
+                    auto hit = [&](int q) -> int { return q < n0 ? st0 + q : st1 + q - n0; };
+                    auto at = [&](int j) -> float {
+                        const float d = ((float)j - G.off_f) * G.delta_f;
+                        return fmaf(fmaf(rho, d, 2.0f), d, rr) * rcp_approx(fmaf(rho2, d, 2.0f));
+                    };
+                    // r: hits below the edge or within the bound of it; those from open on
+                    // are within it and not settled yet
+                    const float v0 = at(j0);
+                    int r = n, open = n;
+                    if (ok) {
+                        float t;
+                        open = r = first_at(v0 - eps, 0, t);
+                        while (t <= v0 + eps) t = S.sig[++r];
+                        if (j0 == 0) {   // the axis' lower end: these are not counted below
+                            my_cast -= r;
+                            for (; open < r; ++open) push(hit(open), row, l);
+                        }
+                    }
+                    bool prev = false;   // the bin below surely holds a hit
+                    for (int jj = 0; jj < jn; ++jj) {
+                        const float v1 = at(j0 + jj + 1);
+                        const int r0 = r;
+                        float t;
+                        r = first_at(v1 - eps, r0, t);
+                        const bool bit = r > r0;
+                        if (open < r0 && !(prev && bit))   // one of the two bins depends on them
+                            for (int q = open; q < r0; ++q) push(hit(q), row, l, kNotCounted);
+                        open = r;
+                        while (t <= v1 + eps) t = S.sig[++r];
+                        prev = bit;
+                        const uint32_t word = __ballot_sync(kAll, bit);
+                        if (lane == jj) mine = word;
+                    }
+                    if (ok) {
+                        const bool end = j0 + jn == ND;   // the axis' upper end
+                        if (end) my_cast += open;
+                        for (; open < r; ++open) push(hit(open), row, l, end ? 0 : kNotCounted);
+                    }
+                    if (mine) atomicOr(word0(l, wd) + j0 + lane, mine);
+                    __syncwarp();
+                    if (s_nredo[warp] >= 32) drain();
+                }
+                if (threadIdx.x == 0) s_val[l] = vA | (vB << 16);   // the other rows go hit by hit
+            }
+            __syncthreads();
+        }
+        // ---- chunks of 32 hits of the runs; a cell layer's runs twice, below and
+        // above its rows
+        if (warp == 0) {
+            int n[2];
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const int q = 2 * lane + side;   // layer << 2 | part << 1 | side
+                int r0 = 0, r1 = nrow - 1;
+                bool use = side == 0;
+                if (CELLS && s_val[lane >> 1] >= 0) {
+                    if (side) r0 = (s_val[lane >> 1] >> 16) + 1;
+                    else r1 = (s_val[lane >> 1] & 0xffff) - 1;
+                    use = r0 <= r1;
+                }
+                s_rs[q] = s_ws[lane];
+                s_re[q] = use ? s_we[lane] : s_ws[lane];
+                s_row[q] = r0 | (max(r1, 0) << 16);
+                n[side] = (s_re[q] - s_rs[q] + 31) >> 5;
+            }
+            int incl = n[0] + n[1];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(kAll, incl, o);
+                if (lane >= o) incl += v;
+            }
+            s_cp[2 * lane + 1] = incl - n[1];
+            s_cp[2 * lane + 2] = incl;
+        }
+        __syncthreads();
+        const int nchunk = s_cp[64];
+
         for (;;) {
             int ch = 0;
             if (lane == 0) ch = atomicAdd(&s_next, 1);
@@ -446,7 +649,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             if (ch >= nchunk) break;
             int run = 0;
             {
-                int hi = 31;   // the last run with s_cp[run] <= ch
+                int hi = 63;   // the last run with s_cp[run] <= ch
                 while (run < hi) {
                     const int mid = (run + hi + 1) >> 1;
                     if (s_cp[mid] <= ch) run = mid;
@@ -464,7 +667,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             float4 ma = make_float4(0.f, 0.f, 0.f, 0.f), mb = ma;
             unsigned long long hm = 0ull;
             if (live) {
-                int l = run >> 1;
+                int l = run >> 2;
                 if (!H.offs) {
                     l = H.l[p] & 15;
                     if (l < l0 || l >= l1) {
@@ -503,15 +706,16 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                 }
                 if (live) {
                     // rows whose circles can reach the (hit's part of the) axis
-                    int ra = 0, rb = nrow - 1;
+                    int ra = CELLS ? s_row[run] & 0xffff : 0;
+                    int rb = CELLS ? s_row[run] >> 16 : nrow - 1;
                     if (c > 1.0f) {
                         float gmin, gmax;
                         rho_range_w(hwlo + s, hwhi + s, c, eR, gmin, gmax);
                         const float fa = floorf(fmaf(gmin, G.inv_drho_f, tc - 0.5f));
                         const float fb = ceilf(fmaf(gmax, G.inv_drho_f, tc + 0.5f));
-                        ra = (int)fmaxf(fa, 0.0f);
-                        rb = (int)fminf(fb, (float)(nrow - 1));
-                        if (!(fa <= (float)(nrow - 1) && fb >= 0.0f)) live = false;
+                        if (!(fa <= (float)rb && fb >= (float)ra)) live = false;
+                        ra = (int)fmaxf(fa, (float)ra);
+                        rb = (int)fminf(fb, (float)rb);
                     }
                     if (live) {
                         // |rho| up to which root B is out of the axis (the conditions of
@@ -794,7 +998,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                     slot[q].b = make_float4(it.E1, it.E2, it.Qa, it.Qb);
                     const bool sure = c > (kSafe * 3.0f * kEps) * R1;   // sign of c proven
                     const bool nb = needs_b(G, rt, s, c, 4e-7f * R1);
-                    imeta[q] = make_int4((int)rest, (H.offs ? run >> 1 : H.l[p] & 15) |
+                    imeta[q] = make_int4((int)rest, (H.offs ? run >> 2 : H.l[p] & 15) |
                                                         (sure ? 32 : 0) | (nb ? 64 : 0), p, 0);
                     if (HIT) shm[q] = hm;
                 }
@@ -842,33 +1046,26 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             }
             // ---- the warp's redos, once they fill its lanes (or its last chunk is done)
             __syncwarp();
-            if (s_nredo[warp] >= 32) {
-                const int nr = min(s_nredo[warp], kVrRedo);
-#pragma unroll 1
-                for (int t = lane; t < nr; t += 32) redo_row(redo[t].x, redo[t].y >> 4, redo[t].y & 15);
-                __syncwarp();
-                if (lane == 0) s_nredo[warp] = 0;
-                __syncwarp();
-            }
+            if (s_nredo[warp] >= 32) drain();
         }
         __syncthreads();
         // every warp's remaining redos, by all threads
         {
             int n = 0;
 #pragma unroll
-            for (int w = 0; w < kVrWarps; ++w) n += min(s_nredo[w], kVrRedo);
+            for (int w = 0; w < kWarps; ++w) n += min(s_nredo[w], kVrRedo);
 #pragma unroll 1
-            for (int t = threadIdx.x; t < n; t += kVrThreads) {
+            for (int t = threadIdx.x; t < n; t += kThr) {
                 int w = 0, q = t;
                 while (q >= min(s_nredo[w], kVrRedo)) q -= min(s_nredo[w++], kVrRedo);
                 const int2 d = S.redo[w * kVrRedo + q];
-                redo_row(d.x, d.y >> 4, d.y & 15);
+                redo_row(d.x, (d.y & ~kNotCounted) >> 4, d.y & 15, !(d.y & kNotCounted));
             }
         }
         __syncthreads();
 
         // ---- the counts: carry-save sum of the layers' bits, 32 rows at a time
-        for (int t = threadIdx.x; t < NWB * ND; t += kVrThreads) {
+        for (int t = threadIdx.x; t < NWB * ND; t += kThr) {
             const int w = t / ND, j = t - w * ND, wg = band * NWB + w;
             if (wg >= NW) continue;
             uint32_t n0 = 0, n1 = 0, n2 = 0, n3 = 0, n4 = 0;
@@ -910,7 +1107,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             cg::cluster_group cluster = cg::this_cluster();
             cluster.sync();
             const int q = (int)cluster.block_rank(), k0 = k - q, npair = NWB * ND;
-            for (int t = threadIdx.x; t < (npair + kVrCluster - 1) / kVrCluster * 4; t += kVrThreads) {
+            for (int t = threadIdx.x; t < (npair + kVrCluster - 1) / kVrCluster * 4; t += kThr) {
                 const int pr = (t >> 2) * kVrCluster + q, w = pr / ND, j = pr - w * ND;
                 const int wg = band * NWB + w;
                 if (pr >= npair || wg >= NW) continue;
@@ -945,7 +1142,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
         }
     }
     if (stats) {
-        unsigned long long v = my_cast;
+        unsigned long long v = (unsigned long long)(long long)my_cast;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             v += __shfl_xor_sync(kAll, v, o);
@@ -961,29 +1158,32 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
     __syncthreads();
 }
 
-// Persistent over the batch's (event, band, column) tiles, events in the order given
-// (largest first).  out: the events' bit planes, out_stride words apart.
-template <int NWB, bool HIT>
-__global__ void __launch_bounds__(kVrThreads, 3)
+// Persistent over the (event, band, column) tiles of a batch's events, in the
+// order given (largest first): CELLS the first *d_ncell (dense layers cell by
+// cell), else the others up to *d_nev (d_ncell null: all).  out: the events'
+// bit planes, out_stride words apart.
+template <int NWB, bool HIT, bool CELLS>
+__global__ void __launch_bounds__(CELLS ? kClThreads : kVrThreads, CELLS ? 2 : 3)
 k_vote_rows_batch(DevGeom G, HitSource H, const int *__restrict__ off,
                   const int *__restrict__ order, const int *__restrict__ d_nev,
-                  uint32_t *__restrict__ out, size_t out_stride,
+                  const int *__restrict__ d_ncell, uint32_t *__restrict__ out, size_t out_stride,
                   unsigned long long *__restrict__ stats, int *__restrict__ head,
                   const unsigned long long *__restrict__ masks)
 {
     __shared__ int s_item;
     const int nb = (G.n_rho + 32 * NWB - 1) / (32 * NWB), nt = nb * G.n_phi0;
-    const int total = *d_nev * nt;
+    const int first = CELLS || !d_ncell ? 0 : *d_ncell;
+    const int total = ((CELLS ? *d_ncell : *d_nev) - first) * nt;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(head, 1);
         __syncthreads();
         const int item = s_item;
         if (item >= total) break;
-        const int e = order[item / nt], t = item % nt;
-        vr_tile<NWB, HIT, true, uint16_t>(G, H, e, HIT ? masks + off[e] : nullptr,
-                                          out + (size_t)e * out_stride,
-                                          stats ? stats + 2 * e : nullptr, t % G.n_phi0,
-                                          t / G.n_phi0);
+        const int e = order[first + item / nt], t = item % nt;
+        vr_tile<NWB, HIT, true, CELLS, uint16_t>(G, H, e, HIT ? masks + off[e] : nullptr,
+                                                 out + (size_t)e * out_stride,
+                                                 stats ? stats + 2 * e : nullptr, t % G.n_phi0,
+                                                 t / G.n_phi0);
     }
 }
 
@@ -994,7 +1194,7 @@ __global__ void __cluster_dims__(kVrCluster, 1, 1) __launch_bounds__(kVrThreads,
 k_vote_rows(DevGeom G, HitSource H, OutT *__restrict__ acc,
             unsigned long long *__restrict__ stats)
 {
-    vr_tile<NWB, false, false, OutT>(G, H, 0, nullptr, acc, stats, blockIdx.x, blockIdx.y);
+    vr_tile<NWB, false, false, false, OutT>(G, H, 0, nullptr, acc, stats, blockIdx.x, blockIdx.y);
 }
 
 }  // namespace
@@ -1008,10 +1208,10 @@ cudaError_t launch_vote_layers(const DevGeom &G, const float *x, const float *y,
                                const uint8_t *layer, int n, void *acc,
                                unsigned long long *stats, cudaStream_t st)
 {
-    const HitSource H{x, y, nullptr, layer, nullptr, nullptr, n};
+    const HitSource H{x, y, nullptr, layer, nullptr, nullptr, n, nullptr};
     const int nwb = vr_nwb(G.n_rho, G.n_d0);
     const dim3 grid(G.n_phi0, (G.n_rho + 32 * nwb - 1) / (32 * nwb));
-    const size_t sm = vr_smem(nwb, G.n_d0, false);
+    const size_t sm = vr_smem(nwb, G.n_d0, false, false);
 #define HT_VR(N)                                                                              \
     do {                                                                                      \
         if (G.count_bits == 16)                                                               \
@@ -1029,41 +1229,74 @@ cudaError_t launch_vote_layers(const DevGeom &G, const float *x, const float *y,
     return cudaGetLastError();
 }
 
-cudaError_t launch_vote_batch_layers(const DevGeom &G, const HitIndex &I, const int *off,
-                                     const int *order, const int *d_nev, uint32_t *planes,
-                                     size_t stride, unsigned long long *stats, int *head, int sms,
-                                     const unsigned long long *hit_masks, cudaStream_t st)
+namespace {
+
+template <int NWB, bool HIT, bool CELLS>
+void run_vote_batch(const DevGeom &G, const HitSource &H, const int *off, const int *order,
+                    const int *d_nev, const int *d_ncell, uint32_t *planes, size_t stride,
+                    unsigned long long *stats, int *head, int sms,
+                    const unsigned long long *hit_masks, cudaStream_t st)
 {
-    const HitSource H{I.x, I.y, I.h, I.l, I.offs, I.rmm, 0};
-    const int nwb = vr_nwb(G.n_rho, G.n_d0);
-#define HT_VRB2(N, HITV)                                                                      \
-    do {                                                                                      \
-        const size_t sm = vr_smem(N, G.n_d0, HITV);                                           \
-        int occ = 0;                                                                          \
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_vote_rows_batch<N, HITV>,       \
-                                                      kVrThreads, sm);                        \
-        k_vote_rows_batch<N, HITV><<<sms * (occ > 0 ? occ : 1), kVrThreads, sm, st>>>(        \
-            G, H, off, order, d_nev, planes, stride, stats, head, hit_masks);                 \
-    } while (0)
-#define HT_VRB(N)                                                                             \
-    do {                                                                                      \
-        if (hit_masks) HT_VRB2(N, true);                                                      \
-        else HT_VRB2(N, false);                                                               \
-    } while (0)
-    if (nwb == 8) HT_VRB(8);
-    else if (nwb == 4) HT_VRB(4);
-    else if (nwb == 2) HT_VRB(2);
-    else HT_VRB(1);
-#undef HT_VRB
-#undef HT_VRB2
+    const size_t sm = vr_smem(NWB, G.n_d0, HIT, CELLS);
+    const int threads = CELLS ? kClThreads : kVrThreads;
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_vote_rows_batch<NWB, HIT, CELLS>, threads,
+                                                  sm);
+    k_vote_rows_batch<NWB, HIT, CELLS><<<sms * (occ > 0 ? occ : 1), threads, sm, st>>>(
+        G, H, off, order, d_nev, d_ncell, planes, stride, stats, head, hit_masks);
+}
+
+template <int NWB>
+cudaError_t run_votes(const DevGeom &G, const HitIndex &I, const int *off, const int *order,
+                      const int *d_nev, const int *d_ncell, uint32_t *planes, size_t stride,
+                      unsigned long long *stats, int *heads, int sms,
+                      const unsigned long long *hit_masks, cudaStream_t st)
+{
+    const HitSource H{I.x, I.y, I.h, I.l, I.offs, I.rmm, 0, I.unsorted};
+    if (hit_masks) {   // a hit's regions restrict its votes: hit by hit
+        run_vote_batch<NWB, true, false>(G, H, off, order, d_nev, nullptr, planes, stride, stats,
+                                         heads, sms, hit_masks, st);
+    } else {
+        const cudaError_t e = launch_hit_sort(I, order, d_ncell, sms, st);
+        if (e != cudaSuccess) return e;
+        run_vote_batch<NWB, false, true>(G, H, off, order, d_nev, d_ncell, planes, stride, stats,
+                                         heads, sms, nullptr, st);
+        run_vote_batch<NWB, false, false>(G, H, off, order, d_nev, d_ncell, planes, stride, stats,
+                                          heads + 1, sms, nullptr, st);
+    }
     return cudaGetLastError();
+}
+
+}  // namespace
+
+// order lists the batch's events, largest first; the first *d_ncell have at
+// least kCellHits hits.  heads: two counters, zero at launch.
+cudaError_t launch_vote_batch_layers(const DevGeom &G, const HitIndex &I, const int *off,
+                                     const int *order, const int *d_nev, const int *d_ncell,
+                                     uint32_t *planes, size_t stride, unsigned long long *stats,
+                                     int *heads, int sms, const unsigned long long *hit_masks,
+                                     cudaStream_t st)
+{
+    const int nwb = vr_nwb(G.n_rho, G.n_d0);
+#define HT_VRB(N)                                                                             \
+    if (nwb == N)                                                                             \
+        return run_votes<N>(G, I, off, order, d_nev, d_ncell, planes, stride, stats, heads,   \
+                            sms, hit_masks, st)
+    HT_VRB(8);
+    HT_VRB(4);
+    HT_VRB(2);
+    HT_VRB(1);
+#undef HT_VRB
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t prepare_layer_vote_kernels(int max_smem)
 {
 #define HT_VRP(N)                                                                             \
     (const void *)k_vote_rows<N, uint16_t>, (const void *)k_vote_rows<N, int32_t>,            \
-        (const void *)k_vote_rows_batch<N, false>, (const void *)k_vote_rows_batch<N, true>
+        (const void *)k_vote_rows_batch<N, false, false>,                                     \
+        (const void *)k_vote_rows_batch<N, true, false>,                                      \
+        (const void *)k_vote_rows_batch<N, false, true>
     const void *fns[] = {HT_VRP(8), HT_VRP(4), HT_VRP(2), HT_VRP(1)};
 #undef HT_VRP
     return allow_smem(fns, (int)(sizeof fns / sizeof fns[0]), max_smem);

@@ -75,8 +75,8 @@ def crossings(geom, x, y, k, t0, TR, rcp_err=0.0, scale=1.0, seed=0):
         dmax = F32(off * delta + 0.01)
         eps = F32(4.0) * (kr * ic * ic * (EPS32 * (dmax + c) + eS + F32(1e-13) * R1) +
                           F32(NR) * (2 * eC * ic + 9 * EPS32))
-        ok &= (slope <= 0.6) & (c * (2 * drho_f + rt) <= 0.97)
-        ok &= np.where(slope <= 1 / 32, eps <= 8.0, (eps <= 0.25) & (c > F32(2.4e-7) * kr))
+        ok &= (slope <= 0.5) & (c * (2 * drho_f + rt) <= 0.97)
+        ok &= np.where(slope <= 1 / 64, eps <= 8.0, (eps <= 0.25) & (c > F32(2.4e-7) * kr))
     sel = np.nonzero(ok)[0]
     x, y, k, s, c, ra, rb, eps = (a[sel] for a in (x, y, k, s, c, ra, rb, eps))
     eps = eps * F32(scale)
@@ -126,3 +126,78 @@ def test_bound_has_teeth():
     x, y, k, t0, _, _ = items(geom, rr, 1000000, seed=5, TR=256)
     n, bad = crossings(geom, x, y, k, t0, 256, rcp_err=2 ** -23.0, scale=1 / 40)
     assert n > 100000 and bad > 0
+
+
+# ------------------------------------------------------------ cell by cell
+def cell_edges(geom, radii, n, seed, scale=1.0, rcp_err=0.0):
+    """Random hits of exact layers against random (row, edge)s of random
+    columns near their roots: (checked, wrong sides)."""
+    NR, ND, NP, rmax_, dh = geom
+    delta = 2.0 * dh / ND
+    off = ND / 2 + 0.5
+    rng = np.random.default_rng(seed)
+    rho64 = (2 * np.arange(NR) + 1 - NR) * (rmax_ / NR)
+    phi = (2 * np.arange(NP) + 1 - NP) * (np.pi / NP)
+    sn64, cs64 = np.sin(phi), np.cos(phi)
+    sn, cs = sn64.astype(F32), cs64.astype(F32)
+    snl, csl = (sn64 - sn).astype(F32), (cs64 - cs).astype(F32)
+    dext = F32((off + 0.5) * delta * 1.0001 + 0.01)
+    checked = wrong = 0
+    for r in radii:
+        ph = rng.uniform(-np.pi, np.pi, n)
+        x, y = (r * np.cos(ph)).astype(F32), (r * np.sin(ph)).astype(F32)
+        rr = np.sqrt(fma32(x, x, (y * y).astype(F32)).astype(np.float64)).astype(F32)
+        rmin, rmax = rr.min(), rr.max()
+        rv = min(1.95 / (dext + np.sqrt(max(1.95 * rmax * rmax - 0.95 * dext * dext, 0.0))),
+                 0.95 / dext) * 0.9999
+        half = (NR - 1) / 2.0
+        drho = 2.0 * rmax_ / NR
+        vA, vB = max(int(np.ceil(half - rv / drho)), 0), min(int(np.floor(half + rv / drho)), NR - 1)
+        if vB <= vA:
+            continue
+        rt = F32(max(abs(rho64[vA]), abs(rho64[vB])))
+        iu = F32(0.5) / (F32(1.0) - rt * dext)
+        r2 = F32(0.5) * fma32(rmin, rmin, F32(rmax * rmax))
+        eE = EPS32 * (iu * (8 * rt * (rmax * rmax + dext * dext) + 12 * dext) + 4 * rmax)
+        eR2 = rt * iu * (F32(0.51) * (rmax - rmin) * (rmax + rmin) + 8 * EPS32 * rmax * rmax)
+        hit = F32(1.25) * EPS32 * rmax + F32(2e-13) * rmax
+        eps = np.float64(4.0 * (eE + eR2 + hit) * scale)   # (without the order's slack)
+        k = rng.integers(0, NP, n)
+        i = rng.integers(vA, vB + 1, n)
+        s = dot2(x, sn[k], snl[k], -y, cs[k], csl[k])
+        c = dot2(x, cs[k], csl[k], y, sn[k], snl[k])
+        rho = rho64[i]
+        X, Y = x.astype(np.float64), y.astype(np.float64)
+        sd, cd = X * sn64[k] - Y * cs64[k], X * cs64[k] + Y * sn64[k]
+        b = 1.0 + rho * sd
+        D = 1.0 - (rho * cd) ** 2
+        ok = (c > F32(12 * U) * (np.abs(x) + np.abs(y))) & (D > 0)
+        with np.errstate(invalid="ignore", divide="ignore"):
+            q = -(b + np.where(b >= 0, 1.0, -1.0) * np.sqrt(D))
+            root = np.where(b >= 0, (rho * (X * X + Y * Y) + 2.0 * sd) / q, q / rho)
+            u = root / delta + off
+        ok &= (u > -3) & (u < ND + 3)
+        j = np.clip(np.floor(np.where(ok, u, 0)) + rng.integers(0, 2, n), 0, ND)
+        d = ((j - off).astype(F32) * F32(delta)).astype(F32)
+        r32 = rho.astype(F32)
+        num = fma32(fma32(r32, d, F32(2.0)), d, (r32 * r2).astype(F32))
+        rc = (1.0 / fma32((F32(2.0) * r32).astype(F32), d, F32(2.0)).astype(np.float64) *
+              (1.0 + rcp_err)).astype(F32)
+        v = (num * rc).astype(F32).astype(np.float64)
+        sig = -s.astype(np.float64)
+        checked += int(ok.sum())
+        wrong += int((ok & (sig > v + eps) & ~(u >= j)).sum())
+        wrong += int((ok & (sig < v - eps) & ~(u < j)).sum())
+    return checked, wrong
+
+
+@pytest.mark.parametrize("name", ["single_64", "event100_256", "pileup_512"])
+def test_side_of_an_edge_by_s(name):
+    """A hit's -s beyond the bound of S(rho, d0 edge) puts its root on that
+    side of the edge."""
+    geom, _ = GEOMS[name]
+    radii = [4.0 + l * 106.0 / 9.0 for l in range(10)]
+    for err in (-2 ** -23.0, 2 ** -23.0):
+        n, bad = cell_edges(geom, radii, 40000, seed=3, rcp_err=err)
+        assert n > 20000 and bad == 0
+

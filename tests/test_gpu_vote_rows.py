@@ -116,3 +116,72 @@ def test_hits_that_vote_nowhere():
     assert np.array_equal(acc.cpu().numpy().view(np.uint16), acc_o)
     assert int(stats[0]) == st["votes"]
     G.close()
+
+
+# Dense events: layers voted cell by cell (24000 hits and more), with the layers
+# and rows that leave that path: tight curls, spread radii, more hits of a cell
+# than are put in order, hits that are not finite, a second round of layers.
+DENSE = {   # n_rho, n_d0, n_phi0, rho_max, d0_half, layers
+    "rings": (64, 64, 32, 0.0114, 20.0, 10),
+    "pileup_like": (130, 66, 24, 0.0228, 30.0, 10),
+    "curled": (96, 32, 16, 0.05, 8.0, 12),
+    "few_bins": (40, 6, 16, 0.0114, 10.0, 8),
+    "clustered": (64, 64, 32, 0.0114, 20.0, 10),
+    "spread": (64, 64, 32, 0.0114, 20.0, 10),
+    "doubled": (64, 64, 32, 0.0114, 20.0, 10),
+    "not_finite": (64, 64, 32, 0.0114, 20.0, 10),
+}
+
+
+def dense(name, seed, n):
+    nr, nd, nphi, rmax, dh, nl = DENSE[name]
+    g = dict(n_rho=nr, n_d0=nd, n_phi0=nphi, rho_max=rmax, d0_half=dh, n_z0=16, n_cot=16,
+             z0_max=20.0, cot_max=3.0, threshold=nl, count_bits=16)
+    rng = np.random.Generator(np.random.Philox(900 + seed))
+    lay = rng.integers(0, nl, n)
+    r = 4.0 + 106.0 * lay / (nl - 1)
+    ph = rng.uniform(-np.pi, np.pi, n)
+    if name == "spread":
+        r = r * np.where(lay % 2 == 0, rng.uniform(0.995, 1.005, n), 1.0)
+    if name == "clustered":
+        c = rng.random(n) < 0.3
+        ph[c] = 0.4 + rng.uniform(0, 0.02, c.sum())
+    if name == "doubled":
+        ph[1::2], lay[1::2], r[1::2] = ph[0::2], lay[0::2], r[0::2]
+    x, y = (r * np.cos(ph)).astype(np.float32), (r * np.sin(ph)).astype(np.float32)
+    if name == "not_finite" and n > 500:
+        x[5], y[77], x[300], x[400], y[400] = np.nan, np.inf, -np.inf, 0.0, 0.0
+    return g, Event(x=x, y=y, z=rng.uniform(-20, 20, n).astype(np.float32),
+                    layer=lay.astype(np.int8), track=np.full(n, -1, np.int32))
+
+
+@pytest.mark.parametrize("name", sorted(DENSE))
+def test_dense_batch(name):
+    """A dense event, a small one and one at the line between the two ways,
+    against the oracle: votes, peaks, confirmation, assignment, z vote."""
+    import torch
+    from paper_1309_6275_gb300 import ht
+    evs = [dense(name, q, n)[1] for q, n in enumerate((25000, 1200, 24000))]
+    g = dense(name, 0, 100)[0]
+    off = np.concatenate([[0], np.cumsum([e.n_hits for e in evs])]).astype(np.int32)
+    cat = lambda k, t: to_dev(np.concatenate([getattr(e, k) for e in evs]).astype(t))
+    cap = 1 << 16
+    G = ht.Geometry(g)
+    B = ht.Batch(G, max_events=4, max_hits=int(off[-1]), cap=cap)
+    B.set_confirm(CP)
+    for _ in range(2):
+        B.run_tracks(cat("x", np.float32), cat("y", np.float32), cat("z", np.float32),
+                     cat("layer", np.uint8), off)
+    torch.cuda.synchronize()
+    for e, ev in enumerate(evs):
+        r = B.event_results(off, e)
+        ok = np.isfinite(ev.x) & np.isfinite(ev.y)   # (no such hit votes)
+        acc, st = oracle.vote_layers(g, ev.x[ok], ev.y[ok], ev.layer[ok])
+        pk, cnt = oracle.peaks(g, acc, cap)
+        assert r["votes"] == st["votes"]
+        assert r["count"] == cnt and np.array_equal(r["peaks"], pk)
+        if ok.all() and cnt < 3000:
+            assert_same_tracks(dict(r, inl=None), dict(oracle_tracks(g, ev, cap, CP), inl=None),
+                               acc=False)
+    B.close()
+    G.close()
