@@ -37,9 +37,10 @@ cudaError_t launch_vote_batch(const DevGeom &G, const float *x, const float *y, 
                               int kt, int sms, cudaStream_t st, const HitBuckets *hb);
 int assoc32_kt(const DevGeom &G);
 int assoc32_ntiles(const DevGeom &G, int kt);
-cudaError_t launch_cand_lists(const DevGeom &G, int kt, const ht_peak *peaks, const int *d_count,
-                              int cap, int *tcnt, int *toff, int *tcur, void *tmp, int *tlist,
-                              cudaStream_t st);
+cudaError_t launch_cand_lists(const DevGeom &G, int kt, int n_ev, const ht_peak *peaks,
+                              const int *d_count, int cap, int *tcnt, int *toff, int *tcur,
+                              size_t tstride, void *tmp, size_t tmp_stride, int *tlist,
+                              size_t lstride, cudaStream_t st);
 cudaError_t launch_assoc_batch(const DevGeom &G, int kt, const float *x, const float *y,
                                const int *off, const int *order, const int *d_nev,
                                const ht_peak *peaks, int cap, const int *toff, size_t tstride,
@@ -127,7 +128,6 @@ struct ht_batch {
     unsigned long long *gbest;
     char *pk_ws;
     size_t pk_stride;
-    char *pk_spill;     // one spill buffer: the events' peak launches run in turn
     int ntiles;
     int *tcnt, *toff, *tcur;
     char *ttmp;
@@ -180,7 +180,6 @@ void free_batch(ht_batch *b)
     cudaFree(b->heads);
     cudaFree(b->gbest);
     cudaFree(b->pk_ws);
-    cudaFree(b->pk_spill);
     cudaFree(b->tcnt);
     cudaFree(b->toff);
     cudaFree(b->tcur);
@@ -301,19 +300,14 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
     if (e == cudaSuccess) e = vote(order_all_of(meta, me), meta + 2, b->heads + 1, true, b->kt_pack);
     if (e == cudaSuccess) e = mark(2);
     if (e != cudaSuccess) return e;
-    // peaks and the association's candidate tile lists per event slot
-    for (int ev = 0; ev < n_ev; ++ev) {
-        e = ht::launch_peaks(G, b->acc + (size_t)ev * b->cells, peaks + (size_t)ev * b->cap,
-                             b->cap, counts + ev, b->pk_ws + (size_t)ev * b->pk_stride, st,
-                             masks ? masks + ev : nullptr, b->pk_spill);
-        if (e != cudaSuccess) return e;
-        const size_t to = (size_t)ev * (b->ntiles + 1);
-        e = ht::launch_cand_lists(G, b->kt_assoc, peaks + (size_t)ev * b->cap, counts + ev,
-                                  b->cap, b->tcnt + to, b->toff + to, b->tcur + to,
-                                  b->ttmp + (size_t)ev * b->ttmp_stride,
-                                  b->tlist + (size_t)ev * b->lstride, st);
-        if (e != cudaSuccess) return e;
-    }
+    // peaks and the association's candidate tile lists of every event slot
+    e = ht::launch_peaks(G, b->acc, b->cells, n_ev, peaks, b->cap, counts, b->pk_ws, b->pk_stride,
+                         b->pk_stride, st, masks);
+    if (e == cudaSuccess)
+        e = ht::launch_cand_lists(G, b->kt_assoc, n_ev, peaks, counts, b->cap, b->tcnt, b->toff,
+                                  b->tcur, (size_t)b->ntiles + 1, b->ttmp, b->ttmp_stride,
+                                  b->tlist, b->lstride, st);
+    if (e != cudaSuccess) return e;
     // association over the whole batch
     e = cudaMemsetAsync(b->gbest, 0, (size_t)b->max_hits * 8, st);
     if (e == cudaSuccess) e = mark(3);
@@ -428,7 +422,7 @@ ht_status ht_batch_create(const ht_geometry *g, int32_t max_events, int32_t max_
     b->slot_words = std::max((b->cells + 1) / 2,
                              ht::layer_planes_words(G) + ht::plane_flag_words(G));
     b->meta_ints = 4 + (size_t)max_events + 1 + 3 * (size_t)max_events;
-    b->pk_stride = ht::align256(ht::peaks_workspace_bytes(G));
+    b->pk_stride = ht::peaks_workspace_bytes(G) + ht::peaks_flag_bytes(G);
     b->ntiles = ht::assoc32_ntiles(G, 1);   // the most tiles any tile width gives
     b->ttmp_stride = ht::scan_tmp_bytes(b->ntiles);
     b->lstride = (size_t)6 * cap;     // a candidate's box touches at most 6 tiles
@@ -441,7 +435,6 @@ ht_status ht_batch_create(const ht_geometry *g, int32_t max_events, int32_t max_
     M((void **)&b->heads, 256);
     M((void **)&b->gbest, (size_t)max_hits * 8);
     M((void **)&b->pk_ws, b->pk_stride * max_events);
-    M((void **)&b->pk_spill, ht::peak_spill_bytes(G));
     M((void **)&b->tcnt, tl);
     M((void **)&b->toff, tl);
     M((void **)&b->tcur, tl);

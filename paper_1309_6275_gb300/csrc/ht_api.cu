@@ -363,19 +363,11 @@ ht_status ht_confirm(const ht_geometry *g, const ht_confirm_desc *c, const float
 }
 
 // The workspace: the segment counts and offsets and the scan's scratch
-// (peaks_workspace_bytes, enough), then the spill buffer that saves the
-// second stencil pass when the workspace also holds it.
+// (peaks_workspace_bytes, enough), then the peak bits that save the second
+// comparison when the workspace also holds them.
 size_t ht_find_peaks_workspace_size(const ht_geometry *g)
 {
-    return g ? ht::align256(ht::peaks_workspace_bytes(g->G)) + ht::peak_spill_bytes(g->G) : 0;
-}
-
-static void *peak_spill_of(const ht::DevGeom &G, void *workspace, size_t workspace_bytes)
-{
-    const size_t a = ht::align256(ht::peaks_workspace_bytes(G));
-    return workspace_bytes >= a + ht::peak_spill_bytes(G)
-               ? reinterpret_cast<char *>(workspace) + a
-               : nullptr;
+    return g ? ht::peaks_workspace_bytes(g->G) + ht::peaks_flag_bytes(g->G) : 0;
 }
 
 ht_status ht_find_peaks(const ht_geometry *g, const void *acc, ht_peak *peaks, int32_t cap,
@@ -390,9 +382,8 @@ ht_status ht_find_peaks(const ht_geometry *g, const void *acc, ht_peak *peaks, i
                     ht::peaks_workspace_bytes(g->G));
     if (!aligned(workspace, 256) || !aligned(acc, 16))
         return fail(HT_ERR_ARG, "ht_find_peaks: workspace or accumulator alignment");
-    cudaError_t e = ht::launch_peaks(g->G, acc, peaks, cap, d_count, workspace, S(stream),
-                                     nullptr,
-                                     peak_spill_of(g->G, workspace, workspace_bytes));
+    cudaError_t e = ht::launch_peaks(g->G, acc, 0, 1, peaks, cap, d_count, workspace, 0,
+                                     workspace_bytes, S(stream));
     return e == cudaSuccess ? HT_OK : cuda_fail(e, "ht_find_peaks");
 }
 
@@ -408,9 +399,9 @@ ht_status ht_find_peaks_masked(const ht_geometry *g, const void *acc, const uint
                     ht::peaks_workspace_bytes(g->G));
     if (!aligned(workspace, 256) || !aligned(mask, 8) || !aligned(acc, 16))
         return fail(HT_ERR_ARG, "ht_find_peaks_masked: pointer alignment");
-    cudaError_t e = ht::launch_peaks(g->G, acc, peaks, cap, d_count, workspace, S(stream),
-                                     reinterpret_cast<const unsigned long long *>(mask),
-                                     peak_spill_of(g->G, workspace, workspace_bytes));
+    cudaError_t e = ht::launch_peaks(g->G, acc, 0, 1, peaks, cap, d_count, workspace, 0,
+                                     workspace_bytes, S(stream),
+                                     reinterpret_cast<const unsigned long long *>(mask));
     return e == cudaSuccess ? HT_OK : cuda_fail(e, "ht_find_peaks_masked");
 }
 

@@ -382,14 +382,17 @@ cudaError_t launch_vote_swept(const DevGeom &G, const float *x, const float *y, 
 cudaError_t launch_vote_hitmask(const DevGeom &G, const float *x, const float *y, int n,
                                 void *acc, unsigned long long *stats,
                                 const unsigned long long *hit_masks, cudaStream_t st);
-// mask (device, or null for every cell): only peaks inside it are reported.
-// spill (peak_spill_bytes, or null): lets the stencil run once instead of
-// twice; it may be shared by launches that run one after another.
-cudaError_t launch_peaks(const DevGeom &G, const void *acc, ht_peak *peaks, int cap,
-                         int *d_count, void *ws, cudaStream_t st,
-                         const unsigned long long *mask = nullptr, void *spill = nullptr);
+// The peaks of n_ev accumulators acc_stride cells apart; peaks are cap apart,
+// counts one, scratch ws_stride bytes.  An event's scratch (ws_bytes) holds at
+// least peaks_workspace_bytes; with peaks_flag_bytes more the second pass
+// writes from peak bits instead of comparing again.  masks (device, or null
+// for every cell): only peaks inside masks[event] are reported.
+cudaError_t launch_peaks(const DevGeom &G, const void *acc, size_t acc_stride, int n_ev,
+                         ht_peak *peaks, int cap, int *d_count, void *ws, size_t ws_stride,
+                         size_t ws_bytes, cudaStream_t st,
+                         const unsigned long long *masks = nullptr);
 size_t peaks_workspace_bytes(const DevGeom &G);
-size_t peak_spill_bytes(const DevGeom &G);
+size_t peaks_flag_bytes(const DevGeom &G);
 cudaError_t launch_associate(const DevGeom &G, const float *x, const float *y, int n,
                              const ht_peak *peaks, const int *d_count, int cap, int *assign,
                              void *ws, cudaStream_t st);
@@ -483,6 +486,9 @@ ht_status set_error(ht_status s, const char *msg);
 size_t scan_tmp_bytes(int n_cap);
 cudaError_t scan_exclusive(const int *in, int *out, int *out2, int n_cap, const int *d_n,
                            int *total, void *tmp, cudaStream_t st);
+cudaError_t scan_exclusive_batch(const int *in, size_t in_stride, int *out, size_t out_stride,
+                                 int *out2, int n, int n_seq, int *total, void *tmp,
+                                 size_t tmp_stride, cudaStream_t st);
 
 }  // namespace ht
 

@@ -3,24 +3,31 @@
 // are the local maxima of the vote space; the threshold reflects the peak
 // finder's tuning for tracks of at least seven hits).
 //
-// Design (GB300, HBM-bound stencil):
-//  * A CTA of 256 threads owns one segment row (i, j-block of 16 d0 bins,
-//    block of 256 phi0 columns).  It first stages rows i-1..i+1 x bins
-//    j0-1..j0+16 x its columns plus one wrapped column on each side into
-//    shared memory with 16-byte loads, all issued before any is used, so a
-//    CTA waits for memory once instead of once per d0 bin; absent rows and
-//    bins read as -1.  Then thread = phi0 column walks the bins keeping, per
-//    row and bin of the rolling 3 x 3 x 3 window, the largest of its three
-//    columns (9 shared loads and 3 three-input maxima per cell); the 26
-//    comparisons become two against the maxima of the preceding and of the
-//    following neighbours.
+// Design (GB300):
+//  * A CTA of 256 threads owns one tile: 16 d0 bins x 256 phi0 columns of a
+//    rho row.  It reads the tile's own cells with 16-byte loads and counts
+//    those at or above the threshold.  Few events fill their accumulator, so
+//    most tiles hold none (a 400-hit event: 45%, and 5 cells on average): such
+//    a tile costs one read of its cells.
+//  * Up to kSparse such cells: a thread per cell compares it with its 26
+//    neighbours, read where they lie (cached lines of tiles next to it).
+//  * More: the CTA stages rows i-1..i+1 x bins j0-1..j0+16 x its columns plus
+//    one wrapped column on each side in shared memory, all loads issued
+//    before any is used; absent rows and bins read as 0.  Then thread = phi0
+//    column walks the bins keeping, per row and bin of the rolling 3 x 3 x 3
+//    window, the largest of its three columns (9 shared loads and 3
+//    three-input maxima per cell); the 26 comparisons become two against the
+//    maxima of the preceding and of the following neighbours.  About 100
+//    instructions per cell: the instruction rate bounds it.
 //  * Compaction keeps increasing logical index l = (i n_d0 + j) n_phi0 + k:
-//    pass 1 counts the peaks of every (i, j, k-block) segment, a
-//    device-wide scan turns counts into offsets (and the total), pass 2
-//    recomputes and writes each peak at its segment offset plus its rank in
-//    the CTA (warp ballots kept per bin, one barrier per pass).  Segments
-//    are ordered by l, so the output is too.
-#include <cuda_runtime.h>
+//    the tile leaves a bit per cell and the count of each (i, j, block of 256
+//    columns) segment, a device-wide scan turns the counts into offsets (and
+//    the total), and a second kernel writes each bit's peak at its segment's
+//    offset plus its rank.  Segments are ordered by l, so the output is too.
+//    A caller whose scratch has no room for the bits gets the tile kernel
+//    again as its second one, writing instead of counting.
+//  * Several events (a batch's, a vertex search's) take one launch of each
+XX#include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "ht_internal.cuh"
@@ -45,257 +52,296 @@ struct Stage {
 };
 constexpr size_t kPkSmemMax = Stage<int32_t>::kBytes;
 
-// Spilled peaks (single stencil pass): the count pass also writes the
-// peaks of every tile that has at most q of them into the tile's q slots, in
-// the tile's l order, with each peak's rank within its segment; tiletot
-// holds every tile's peak count.  The write pass then copies a spilled tile's
-// peaks to their segment offsets and runs the stencil again only for tiles
-// with more than q peaks.  q == 0: no spill (every tile's stencil runs
-// twice).
-struct PeakSpill {
-    ht_peak *pk;
-    int *rk;
-    int *tiletot;
-    int q;
-};
+constexpr int kFlagWords = kPkThreads / 32;     // peak bits of a segment
+constexpr int kSparse = 512;                    // cells compared one by one, at most
 
-// One tile: (rho row i, 16 d0 bins from j0 = jb * kJB, 256 phi0 columns
-// from k0 = kb * kPkThreads), tile index t.  Count pass (!WRITE): the
-// segment counts, the tile's total and, when sp.q allows, the spilled peaks.
-// Write pass: every peak at its segment offset.
+// Count pass: tile (rho row i, 16 d0 bins from j0, 256 phi0 columns from k0)
+// of event e; the peak bits (flags given) and the segment counts.  Scratch of event e lies
+// e * ws_stride bytes after event 0's.
 //
-// MASKED: only cells inside *mask (a learned proposal's regions) can be
+// MASKED: only cells inside masks[e] (a learned proposal's regions) can be
 // peaks; a tile whose bins are all outside reads nothing.  An inside cell's
 // 26 neighbours lie in the mask's halo, which the masked vote fills exactly.
-template <typename T, bool WRITE, bool MASKED>
-__device__ __forceinline__ void peaks_tile(const DevGeom &G, const T *__restrict__ acc, int kb,
-                                           int jb, int i, int t, int thr,
-                                           int *__restrict__ segcnt,
-                                           const int *__restrict__ segoff,
-                                           ht_peak *__restrict__ out, int cap,
-                                           const unsigned long long *__restrict__ mask,
-                                           const PeakSpill &sp, T *sw,
-                                           unsigned (*bal_s)[kPkThreads / 32], int *s_jpre)
+// WRITE: the second pass without peak bits; seg holds the segments' offsets
+// and the peaks go to out.
+template <typename T, bool MASKED, bool WRITE>
+__global__ void __launch_bounds__(kPkThreads)
+k_peaks_tile(DevGeom G, const T *__restrict__ acc, size_t acc_stride, int *__restrict__ segs,
+             uint32_t *__restrict__ flags, size_t ws_stride,
+             const unsigned long long *__restrict__ masks, ht_peak *__restrict__ out, int cap)
 {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ uint32_t s_flag[kJB][kFlagWords];
+    __shared__ int s_n, s_at;
+    __shared__ uint16_t s_hot[kSparse];
     constexpr int kOff = Stage<T>::kOff, kSW = Stage<T>::kSW;
-    const int NP = G.n_phi0, ND = G.n_d0, NR = G.n_rho;
+    T *const sw = reinterpret_cast<T *>(smraw);
+    const int NP = G.n_phi0, ND = G.n_d0, NR = G.n_rho, thr = G.threshold;
     const int nkb = (NP + kPkThreads - 1) / kPkThreads;
+    const int kb = blockIdx.x % nkb, jb = blockIdx.x / nkb, i = blockIdx.y, e = blockIdx.z;
+    acc += e * acc_stride;
+    segs = reinterpret_cast<int *>(reinterpret_cast<char *>(segs) + e * ws_stride);
+    if (flags)
+        flags = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(flags) + e * ws_stride);
     const int k0 = kb * kPkThreads, ncol = min(kPkThreads, NP - k0);
-    const int j0 = jb * kJB, j1 = min(j0 + kJB, ND);
+    const int j0 = jb * kJB, j1 = min(j0 + kJB, ND), nj = j1 - j0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned inside = 0xffu;   // d0 blocks inside the mask in row i's rho block
+    bool any = true;
     if (MASKED) {
-        inside = (unsigned)(*mask >> (8 * region_block(i, NR))) & 0xffu;
+        inside = (unsigned)(masks[e] >> (8 * region_block(i, NR))) & 0xffu;
         const int b0 = region_block(j0, ND), b1 = region_block(j1 - 1, ND);
-        if (!(inside & ((2u << b1) - 1u) & ~((1u << b0) - 1u))) {
-            if (!WRITE) {
-                for (int j = j0 + threadIdx.x; j < j1; j += kPkThreads)
-                    segcnt[(i * ND + j) * nkb + kb] = 0;
-                if (sp.q > 0 && threadIdx.x == 0) sp.tiletot[t] = 0;
-            }
-            return;   // uniform over the CTA
-        }
+        any = (inside & ((2u << b1) - 1u) & ~((1u << b0) - 1u)) != 0u;
     }
-
-    // ---- stage the window: interior columns with 16-byte loads and stores.
-    // Absent rows and bins read as 0: a peak has v >= threshold >= 1, so a 0
-    // neighbour never decides a comparison (as no neighbour at all).
-    constexpr int VEC = 16 / (int)sizeof(T);
-    const int nvec = ncol / VEC;                         // ncol is a multiple of 8
-    for (int v = threadIdx.x; v < kSlices * nvec; v += kPkThreads) {
-        const int sl = v / nvec, q = v - sl * nvec;
-        const int ii = i - 1 + sl / (kJB + 2), jj = j0 - 1 + sl % (kJB + 2);
-        uint4 u = make_uint4(0, 0, 0, 0);
-        if (ii >= 0 && ii < NR && jj >= 0 && jj < ND)
-            u = *reinterpret_cast<const uint4 *>(acc + ((size_t)ii * ND + jj) * NP + k0 + q * VEC);
-        *reinterpret_cast<uint4 *>(sw + sl * kSW + kOff + q * VEC) = u;
-    }
-    // the two wrapped neighbour columns of every slice
-    for (int v = threadIdx.x; v < 2 * kSlices; v += kPkThreads) {
-        const int sl = v >> 1, side = v & 1;
-        const int ii = i - 1 + sl / (kJB + 2), jj = j0 - 1 + sl % (kJB + 2);
-        const int kk = side ? (k0 + ncol) % NP : (k0 + NP - 1) % NP;
-        const bool ok = ii >= 0 && ii < NR && jj >= 0 && jj < ND;
-        sw[sl * kSW + (side ? kOff + ncol : kOff - 1)] =
-            ok ? acc[((size_t)ii * ND + jj) * NP + kk] : (T)0;
-    }
+    if (threadIdx.x < kJB * kFlagWords) (&s_flag[0][0])[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) s_n = s_at = 0;
     __syncthreads();
 
-    // ---- walk the bins.  cm[r][s]: largest of columns k-1, k, k+1 in row
-    // i-1+r at bin j-1+s; c1/n1: the three columns of row i at bins j and
-    // j+1.  A cell is a peak when v >= T, v exceeds every neighbour that
-    // precedes it in l (row i-1, bin j-1 of row i, column k-1 of its own
-    // bin) and is at least every neighbour that follows it (row i+1, bin j+1,
-    // column k+1) -- the two maxima below; across the phi0 wrap the order of
-    // the column neighbours flips.
-    const int c = threadIdx.x;
-    const bool cok = c < ncol;
-    const int k = k0 + c;
-    const int cc = cok ? c : 0;                           // stays inside the staged row
-    // q[-1], q[0], q[1]: columns k - 1, k, k + 1 of slice (r, jj)
-    auto S = [&](int r, int jj) -> const T * {
-        return sw + (r * (kJB + 2) + jj) * kSW + kOff + cc;
-    };
-    int cm[3][3], c1[3], n1[3];
+    // ---- the tile's own cells, and which of them reach the threshold
+    constexpr int VEC = 16 / (int)sizeof(T), kRowVec = kPkThreads / VEC, NV = kJB / VEC;
+    uint4 u[NV];
+    unsigned hot[NV];
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
+    for (int n = 0; n < NV; ++n) {
+        const int v = threadIdx.x + n * kPkThreads, jl = v / kRowVec, q = v % kRowVec;
+        u[n] = make_uint4(0, 0, 0, 0);
+        if (any && jl < nj && q * VEC < ncol)            // ncol is a multiple of 8
+            u[n] = *reinterpret_cast<const uint4 *>(acc + ((size_t)i * ND + j0 + jl) * NP + k0 +
+                                                    q * VEC);
+    }
+    int nhot = 0;
 #pragma unroll
-        for (int sl = 0; sl < 2; ++sl) {
-            const T *q = S(r, sl);
-            const int a = (int)q[-1], b = (int)q[0], d = (int)q[1];
-            cm[r][sl] = __vimax3_s32(a, b, d);
-            if (r == 1 && sl == 1) { c1[0] = a; c1[1] = b; c1[2] = d; }
+    for (int n = 0; n < NV; ++n) {
+        const uint32_t w[4] = {u[n].x, u[n].y, u[n].z, u[n].w};
+        const int jl = (threadIdx.x + n * kPkThreads) / kRowVec;
+        hot[n] = 0u;
+#pragma unroll
+        for (int b = 0; b < VEC; ++b) {
+            const int c = sizeof(T) == 2 ? (int)((w[b >> 1] >> (16 * (b & 1))) & 0xffffu)
+                                         : (int)w[b & 3];
+            hot[n] |= (unsigned)(c >= thr) << b;
         }
-    const bool wrap_lo = k == 0, wrap_hi = k == NP - 1;
-    unsigned mine = 0u;
-    const int nj = j1 - j0;
+        if (MASKED && jl < nj && !((inside >> region_block(j0 + jl, ND)) & 1u)) hot[n] = 0u;
+        nhot += __popc(hot[n]);
+    }
+    const int wsum = __reduce_add_sync(0xffffffffu, nhot);
+    if (lane == 0 && wsum) atomicAdd(&s_n, wsum);
+    __syncthreads();
+    const int total = s_n;
+    if (total > 0 && total <= kSparse) {
+        // ---- few: list them, a thread each
+        if (nhot) {
+            int at = atomicAdd(&s_at, nhot);
 #pragma unroll
-    for (int jl = 0; jl < kJB; ++jl) {
-        if (jl < nj) {   // uniform over the CTA
+            for (int n = 0; n < NV; ++n)
+                for (unsigned h = hot[n]; h; h &= h - 1u)
+                    s_hot[at++] =
+                        (uint16_t)((threadIdx.x + n * kPkThreads) * VEC + __ffs(h) - 1);
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < total; t += kPkThreads) {
+            const int jl = s_hot[t] / kPkThreads, c = s_hot[t] % kPkThreads;
+            const int j = j0 + jl, k = k0 + c;
+            const int km = k == 0 ? NP - 1 : k - 1, kp = k == NP - 1 ? 0 : k + 1;
+            auto row = [&](int ii, int jj, int &a, int &m, int &b) {
+                a = m = b = 0;
+                if (ii < 0 || ii >= NR || jj < 0 || jj >= ND) return;
+                const T *r = acc + ((size_t)ii * ND + jj) * NP;
+                a = (int)r[km];
+                m = (int)r[k];
+                b = (int)r[kp];
+            };
+            int a[9], m[9], b[9];
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const T *q = S(r, jl + 2);
+            for (int r = 0; r < 9; ++r) row(i - 1 + r / 3, j - 1 + r % 3, a[r], m[r], b[r]);
+            int before = 0, after = 0;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) before = max(before, __vimax3_s32(a[r], m[r], b[r]));
+#pragma unroll
+            for (int r = 5; r < 9; ++r) after = max(after, __vimax3_s32(a[r], m[r], b[r]));
+            // the column neighbours of the own bin: across the wrap their order flips
+            before = __vimax3_s32(before, k == 0 ? 0 : a[4], k == NP - 1 ? b[4] : 0);
+            after = __vimax3_s32(after, k == 0 ? a[4] : 0, k == NP - 1 ? 0 : b[4]);
+            if (m[4] > before && m[4] >= after) atomicOr(&s_flag[jl][c >> 5], 1u << (c & 31));
+        }
+    } else if (total > 0) {
+        // ---- many: stage the window, the own cells from the registers
+#pragma unroll
+        for (int n = 0; n < NV; ++n) {
+            const int v = threadIdx.x + n * kPkThreads, jl = v / kRowVec, q = v % kRowVec;
+            if (jl < nj && q * VEC < ncol)
+                *reinterpret_cast<uint4 *>(sw + (kJB + 2 + jl + 1) * kSW + kOff + q * VEC) = u[n];
+        }
+        // Absent rows and bins read as 0: a peak has v >= threshold >= 1, so a 0
+        // neighbour never decides a comparison (as no neighbour at all).
+        const int nvec = ncol / VEC;
+        for (int v = threadIdx.x; v < kSlices * nvec; v += kPkThreads) {
+            const int sl = v / nvec, q = v - sl * nvec;
+            const int r = sl / (kJB + 2), jj = j0 - 1 + sl % (kJB + 2), ii = i - 1 + r;
+            if (r == 1 && jj >= j0 && jj < j1) continue;
+            uint4 w = make_uint4(0, 0, 0, 0);
+            if (ii >= 0 && ii < NR && jj >= 0 && jj < ND)
+                w = *reinterpret_cast<const uint4 *>(acc + ((size_t)ii * ND + jj) * NP + k0 +
+                                                     q * VEC);
+            *reinterpret_cast<uint4 *>(sw + sl * kSW + kOff + q * VEC) = w;
+        }
+        // the two wrapped neighbour columns of every slice
+        for (int v = threadIdx.x; v < 2 * kSlices; v += kPkThreads) {
+            const int sl = v >> 1, side = v & 1;
+            const int ii = i - 1 + sl / (kJB + 2), jj = j0 - 1 + sl % (kJB + 2);
+            const int kk = side ? (k0 + ncol) % NP : (k0 + NP - 1) % NP;
+            const bool ok = ii >= 0 && ii < NR && jj >= 0 && jj < ND;
+            sw[sl * kSW + (side ? kOff + ncol : kOff - 1)] =
+                ok ? acc[((size_t)ii * ND + jj) * NP + kk] : (T)0;
+        }
+        __syncthreads();
+
+        // ---- walk the bins.  cm[r][s]: largest of columns k-1, k, k+1 in row
+        // i-1+r at bin j-1+s; c1/n1: the three columns of row i at bins j and
+        // j+1.  A cell is a peak when v >= T, v exceeds every neighbour that
+        // precedes it in l (row i-1, bin j-1 of row i, column k-1 of its own
+        // bin) and is at least every neighbour that follows it (row i+1, bin j+1,
+        // column k+1) -- the two maxima below; across the phi0 wrap the order of
+        // the column neighbours flips.
+        const int c = threadIdx.x;
+        const bool cok = c < ncol;
+        const int k = k0 + c;
+        const int cc = cok ? c : 0;                           // stays inside the staged row
+        // q[-1], q[0], q[1]: columns k - 1, k, k + 1 of slice (r, jj)
+        auto S = [&](int r, int jj) -> const T * {
+            return sw + (r * (kJB + 2) + jj) * kSW + kOff + cc;
+        };
+        int cm[3][3], c1[3], n1[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int sl = 0; sl < 2; ++sl) {
+                const T *q = S(r, sl);
                 const int a = (int)q[-1], b = (int)q[0], d = (int)q[1];
-                cm[r][2] = __vimax3_s32(a, b, d);
-                if (r == 1) { n1[0] = a; n1[1] = b; n1[2] = d; }
+                cm[r][sl] = __vimax3_s32(a, b, d);
+                if (r == 1 && sl == 1) { c1[0] = a; c1[1] = b; c1[2] = d; }
             }
-            const int v = c1[1];
-            const int before = max(__vimax3_s32(cm[0][0], cm[0][1], cm[0][2]),
-                                   __vimax3_s32(cm[1][0], wrap_lo ? 0 : c1[0],
-                                                wrap_hi ? c1[2] : 0));
-            const int after = max(__vimax3_s32(cm[2][0], cm[2][1], cm[2][2]),
-                                  __vimax3_s32(cm[1][2], wrap_lo ? c1[0] : 0,
-                                               wrap_hi ? 0 : c1[2]));
-            const bool pk = cok && v >= thr && v > before && v >= after &&
-                            (!MASKED || ((inside >> region_block(j0 + jl, ND)) & 1u));
-            const unsigned bal = __ballot_sync(0xffffffffu, pk);
-            if (lane == 0) bal_s[jl][warp] = bal;
-            mine |= (unsigned)pk << jl;
+        const bool wrap_lo = k == 0, wrap_hi = k == NP - 1;
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                cm[r][0] = cm[r][1];
-                cm[r][1] = cm[r][2];
+        for (int jl = 0; jl < kJB; ++jl) {
+            if (jl < nj) {   // uniform over the CTA
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    const T *q = S(r, jl + 2);
+                    const int a = (int)q[-1], b = (int)q[0], d = (int)q[1];
+                    cm[r][2] = __vimax3_s32(a, b, d);
+                    if (r == 1) { n1[0] = a; n1[1] = b; n1[2] = d; }
+                }
+                const int v = c1[1];
+                const int before = max(__vimax3_s32(cm[0][0], cm[0][1], cm[0][2]),
+                                       __vimax3_s32(cm[1][0], wrap_lo ? 0 : c1[0],
+                                                    wrap_hi ? c1[2] : 0));
+                const int after = max(__vimax3_s32(cm[2][0], cm[2][1], cm[2][2]),
+                                      __vimax3_s32(cm[1][2], wrap_lo ? c1[0] : 0,
+                                                   wrap_hi ? 0 : c1[2]));
+                const bool pk = cok && v >= thr && v > before && v >= after &&
+                                (!MASKED || ((inside >> region_block(j0 + jl, ND)) & 1u));
+                const unsigned bal = __ballot_sync(0xffffffffu, pk);
+                if (lane == 0) s_flag[jl][warp] = bal;
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    cm[r][0] = cm[r][1];
+                    cm[r][1] = cm[r][2];
+                }
+                c1[0] = n1[0]; c1[1] = n1[1]; c1[2] = n1[2];
             }
-            c1[0] = n1[0]; c1[1] = n1[1]; c1[2] = n1[2];
         }
     }
     __syncthreads();
-    // rank of the lane's peak in bin jl within its segment (CTA order = l order)
-    auto seg_rank = [&](int jl) {
-        int r = __popc(bal_s[jl][warp] & ((1u << lane) - 1u));
-        for (int w2 = 0; w2 < warp; ++w2) r += __popc(bal_s[jl][w2]);
-        return r;
-    };
-    if constexpr (!WRITE) {
-        for (int jl = threadIdx.x; jl < nj; jl += kPkThreads) {
-            int cnt = 0;
+    if (threadIdx.x < nj * kFlagWords) {   // whole groups of kFlagWords lanes
+        const int jl = threadIdx.x / kFlagWords, w = threadIdx.x % kFlagWords;
+        const size_t seg = ((size_t)i * ND + j0 + jl) * nkb + kb;
+        const uint32_t f = s_flag[jl][w];
+        const unsigned grp = 0xffu << (lane & ~7);
+        int incl = __popc(f);
 #pragma unroll
-            for (int w2 = 0; w2 < kPkThreads / 32; ++w2) cnt += __popc(bal_s[jl][w2]);
-            segcnt[(i * ND + j0 + jl) * nkb + kb] = cnt;
-            if (sp.q > 0) s_jpre[jl + 1] = cnt;
+        for (int o = 1; o < kFlagWords; o <<= 1) {
+            const int below = __shfl_up_sync(grp, incl, o, kFlagWords);
+            if (w >= o) incl += below;
         }
-        if (sp.q > 0) {
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                s_jpre[0] = 0;
-                for (int jl = 0; jl < nj; ++jl) s_jpre[jl + 1] += s_jpre[jl];
-                sp.tiletot[t] = s_jpre[nj];
+        if (WRITE) {
+            const int j = j0 + jl;
+            int pos = segs[seg] + incl - __popc(f);
+            for (uint32_t b = f; b; b &= b - 1u, ++pos) {
+                const int k = k0 + 32 * w + __ffs(b) - 1;
+                if (pos < cap)
+                    out[(size_t)e * cap + pos] =
+                        ht_peak{i, j, k, (int)acc[((size_t)i * ND + j) * NP + k]};
             }
-            __syncthreads();
-            if (s_jpre[nj] <= sp.q) {   // uniform
-                while (mine) {
-                    const int jl = __ffs(mine) - 1;
-                    mine &= mine - 1u;
-                    const int r = seg_rank(jl);
-                    const size_t slot = (size_t)t * sp.q + s_jpre[jl] + r;
-                    sp.pk[slot] = ht_peak{i, j0 + jl, k, (int)S(1, jl + 1)[0]};
-                    sp.rk[slot] = r;
-                }
-            }
-        }
-    } else {
-        while (mine) {
-            const int jl = __ffs(mine) - 1;
-            mine &= mine - 1u;
-            const int pos = segoff[(i * ND + j0 + jl) * nkb + kb] + seg_rank(jl);
-            if (pos < cap) out[pos] = ht_peak{i, j0 + jl, k, (int)S(1, jl + 1)[0]};
+        } else {
+            if (flags) flags[seg * kFlagWords + w] = f;
+            if (w == kFlagWords - 1) segs[seg] = incl;
         }
     }
 }
+static_assert(kFlagWords == 8, "the groups of eight lanes above");
 
-// Count pass: one CTA per tile.
-template <typename T, bool MASKED>
+// Write pass from the bits: a thread per half segment.
+template <typename T>
 __global__ void __launch_bounds__(kPkThreads)
-k_peaks_count(DevGeom G, const T *__restrict__ acc, int *__restrict__ segcnt,
-              const unsigned long long *__restrict__ mask, PeakSpill sp)
+k_peaks_write(DevGeom G, const T *__restrict__ acc, size_t acc_stride,
+              const int *__restrict__ segoff, const uint32_t *__restrict__ flags,
+              size_t ws_stride, int nseg, ht_peak *__restrict__ out, int cap)
 {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ unsigned bal_s[kJB][kPkThreads / 32];
-    __shared__ int s_jpre[kJB + 1];
-    const int thr = G.threshold;
-    const int t = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    peaks_tile<T, false, MASKED>(G, acc, blockIdx.x, blockIdx.y, blockIdx.z, t, thr, segcnt,
-                                 nullptr, nullptr, 0, mask, sp, reinterpret_cast<T *>(smraw),
-                                 bal_s, s_jpre);
-}
-
-// Write pass, persistent over the tiles: a spilled tile is copied, the
-// others run the stencil again.
-template <typename T, bool MASKED>
-__global__ void __launch_bounds__(kPkThreads)
-k_peaks_write(DevGeom G, const T *__restrict__ acc, const int *__restrict__ segoff,
-              ht_peak *__restrict__ out, int cap, const unsigned long long *__restrict__ mask,
-              PeakSpill sp, int nkb, int njb)
-{
-    extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ unsigned bal_s[kJB][kPkThreads / 32];
-    const int thr = G.threshold;
-    const int ND = G.n_d0;
-    const int ntiles = nkb * njb * G.n_rho;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int kb = t % nkb, jb = (t / nkb) % njb, i = t / (nkb * njb);
-        if (sp.q > 0) {
-            const int tot = sp.tiletot[t];
-            if (tot <= sp.q) {   // uniform
-                for (int r = threadIdx.x; r < tot; r += kPkThreads) {
-                    const size_t slot = (size_t)t * sp.q + r;
-                    const ht_peak pk = sp.pk[slot];
-                    const int pos = segoff[(pk.i_rho * ND + pk.j_d0) * nkb + kb] + sp.rk[slot];
-                    if (pos < cap) out[pos] = pk;
-                }
-                continue;
-            }
+    const int e = blockIdx.y, t = blockIdx.x * kPkThreads + threadIdx.x;
+    const int seg = t >> 1, half = t & 1;
+    acc += e * acc_stride;
+    segoff = reinterpret_cast<const int *>(reinterpret_cast<const char *>(segoff) + e * ws_stride);
+    flags = reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(flags) + e * ws_stride);
+    out += (size_t)e * cap;
+    uint4 f = make_uint4(0, 0, 0, 0);
+    if (seg < nseg) f = reinterpret_cast<const uint4 *>(flags)[t];
+    const int mine = __popc(f.x) + __popc(f.y) + __popc(f.z) + __popc(f.w);
+    const int other = __shfl_xor_sync(0xffffffffu, mine, 1);
+    if (!mine) return;
+    int pos = segoff[seg] + (half ? other : 0);
+    const int nkb = (G.n_phi0 + kPkThreads - 1) / kPkThreads;
+    const int r = seg / nkb, i = r / G.n_d0, j = r - i * G.n_d0;
+    const int k0 = (seg - r * nkb) * kPkThreads + half * 128;
+    const uint32_t w[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        for (uint32_t b = w[q]; b; b &= b - 1u, ++pos) {
+            const int k = k0 + 32 * q + __ffs(b) - 1;
+            if (pos < cap) out[pos] = ht_peak{i, j, k, (int)acc[(size_t)r * G.n_phi0 + k]};
         }
-        peaks_tile<T, true, MASKED>(G, acc, kb, jb, i, t, thr, nullptr, segoff, out, cap, mask,
-                                    sp, reinterpret_cast<T *>(smraw), bal_s, nullptr);
-        __syncthreads();   // the staged window is refilled by the next tile
-    }
 }
 
 template <typename T, bool MASKED>
-cudaError_t run_peaks(const DevGeom &G, const T *acc, ht_peak *peaks, int cap, int *d_count,
-                      int *segcnt, int *segoff, void *tmp, const unsigned long long *mask,
-                      cudaStream_t st, const PeakSpill &sp)
+cudaError_t run_peaks(const DevGeom &G, const T *acc, size_t acc_stride, int n_ev, ht_peak *peaks,
+                      int cap, int *d_count, void *ws, size_t ws_stride, bool with_flags,
+                      const unsigned long long *masks, cudaStream_t st)
 {
     const int nkb = (G.n_phi0 + kPkThreads - 1) / kPkThreads;
     const int njb = (G.n_d0 + kJB - 1) / kJB;
-    dim3 grid(nkb, njb, G.n_rho);
     const int nseg = G.n_rho * G.n_d0 * nkb;
-    k_peaks_count<T, MASKED><<<grid, kPkThreads, Stage<T>::kBytes, st>>>(G, acc, segcnt, mask,
-                                                                         sp);
-    cudaError_t e = scan_exclusive(segcnt, segoff, nullptr, nseg, nullptr, d_count, tmp, st);
+    char *p = reinterpret_cast<char *>(ws);
+    int *segcnt = reinterpret_cast<int *>(p);
+    p += align256(((size_t)nseg + 1) * 4);
+    int *segoff = reinterpret_cast<int *>(p);
+    p += align256(((size_t)nseg + 1) * 4);
+    void *const tmp = p;
+    uint32_t *flags =
+        with_flags ? reinterpret_cast<uint32_t *>(p + scan_tmp_bytes(nseg)) : nullptr;
+    const dim3 grid(nkb * njb, G.n_rho, n_ev);
+    k_peaks_tile<T, MASKED, false><<<grid, kPkThreads, Stage<T>::kBytes, st>>>(
+        G, acc, acc_stride, segcnt, flags, ws_stride, masks, nullptr, 0);
+    const cudaError_t e = scan_exclusive_batch(segcnt, ws_stride, segoff, ws_stride, nullptr, nseg,
+                                               n_ev, d_count, tmp, ws_stride, st);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, occ = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_peaks_write<T, MASKED>,
-                                                          kPkThreads, Stage<T>::kBytes);
-    if (e != cudaSuccess) return e;
-    const int ntiles = nkb * njb * G.n_rho;
-    const int pgrid = min(ntiles, sms * (occ > 0 ? occ : 1));
-    k_peaks_write<T, MASKED><<<pgrid, kPkThreads, Stage<T>::kBytes, st>>>(
-        G, acc, segoff, peaks, cap, mask, sp, nkb, njb);
+    if (flags) {
+        const dim3 wgrid((2 * nseg + kPkThreads - 1) / kPkThreads, n_ev);
+        k_peaks_write<T><<<wgrid, kPkThreads, 0, st>>>(G, acc, acc_stride, segoff, flags,
+                                                       ws_stride, nseg, peaks, cap);
+    } else {
+        k_peaks_tile<T, MASKED, true><<<grid, kPkThreads, Stage<T>::kBytes, st>>>(
+            G, acc, acc_stride, segoff, nullptr, ws_stride, masks, peaks, cap);
+    }
     return cudaGetLastError();
 }
 
@@ -305,11 +351,11 @@ cudaError_t run_peaks(const DevGeom &G, const T *acc, ht_peak *peaks, int cap, i
 // memory.  Called once per device.
 cudaError_t prepare_peaks_kernels()
 {
-    const void *fns[] = {
-        (const void *)k_peaks_count<uint16_t, false>, (const void *)k_peaks_write<uint16_t, false>,
-        (const void *)k_peaks_count<uint16_t, true>,  (const void *)k_peaks_write<uint16_t, true>,
-        (const void *)k_peaks_count<int32_t, false>,  (const void *)k_peaks_write<int32_t, false>,
-        (const void *)k_peaks_count<int32_t, true>,   (const void *)k_peaks_write<int32_t, true>};
+#define HT_PKF(T)                                                                             \
+    (const void *)k_peaks_tile<T, false, false>, (const void *)k_peaks_tile<T, true, false>,  \
+        (const void *)k_peaks_tile<T, false, true>, (const void *)k_peaks_tile<T, true, true>
+    const void *fns[] = {HT_PKF(uint16_t), HT_PKF(int32_t)};
+#undef HT_PKF
     for (const void *f : fns) {
         const cudaError_t e =
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPkSmemMax);
@@ -318,61 +364,32 @@ cudaError_t prepare_peaks_kernels()
     return cudaSuccess;
 }
 
+static size_t peak_segments(const DevGeom &G)
+{
+    return (size_t)G.n_rho * G.n_d0 * ((G.n_phi0 + kPkThreads - 1) / kPkThreads);
+}
+
 size_t peaks_workspace_bytes(const DevGeom &G)
 {
-    const size_t nkb = (G.n_phi0 + kPkThreads - 1) / kPkThreads;
-    const size_t nseg = (size_t)G.n_rho * G.n_d0 * nkb;
+    const size_t nseg = peak_segments(G);
     return 2 * align256((nseg + 1) * 4) + scan_tmp_bytes((int)nseg);
 }
 
-// Spill slots per tile: a tile (one row, 16 bins, 256 columns) has at most
-// 1024 peaks (no two peaks are neighbours), usually a few; tiles above this
-// run the stencil twice.
-constexpr int kSpillQ = 64;
+size_t peaks_flag_bytes(const DevGeom &G) { return align256(peak_segments(G) * kFlagWords * 4); }
 
-size_t peak_spill_bytes(const DevGeom &G)
+cudaError_t launch_peaks(const DevGeom &G, const void *acc, size_t acc_stride, int n_ev,
+                         ht_peak *peaks, int cap, int *d_count, void *ws, size_t ws_stride,
+                         size_t ws_bytes, cudaStream_t st, const unsigned long long *masks)
 {
-    const size_t nkb = (G.n_phi0 + kPkThreads - 1) / kPkThreads;
-    const size_t nt = nkb * ((G.n_d0 + kJB - 1) / kJB) * G.n_rho;
-    return align256(nt * 4) + align256(nt * kSpillQ * sizeof(ht_peak)) +
-           align256(nt * kSpillQ * 4);
-}
-
-cudaError_t launch_peaks(const DevGeom &G, const void *acc, ht_peak *peaks, int cap,
-                         int *d_count, void *ws, cudaStream_t st, const unsigned long long *mask,
-                         void *spill)
-{
-    const size_t nkb = (G.n_phi0 + kPkThreads - 1) / kPkThreads;
-    const size_t nseg = (size_t)G.n_rho * G.n_d0 * nkb;
-    char *p = reinterpret_cast<char *>(ws);
-    int *segcnt = reinterpret_cast<int *>(p);
-    int *segoff = reinterpret_cast<int *>(p + align256((nseg + 1) * 4));
-    void *tmp = p + 2 * align256((nseg + 1) * 4);
-    PeakSpill sp{nullptr, nullptr, nullptr, 0};
-    if (spill) {
-        const size_t nt = nkb * ((G.n_d0 + kJB - 1) / kJB) * G.n_rho;
-        char *q = reinterpret_cast<char *>(spill);
-        sp.tiletot = reinterpret_cast<int *>(q);
-        q += align256(nt * 4);
-        sp.pk = reinterpret_cast<ht_peak *>(q);
-        q += align256(nt * kSpillQ * sizeof(ht_peak));
-        sp.rk = reinterpret_cast<int *>(q);
-        sp.q = kSpillQ;
-    }
+    const bool flags = ws_bytes >= peaks_workspace_bytes(G) + peaks_flag_bytes(G);
     const uint16_t *a16 = reinterpret_cast<const uint16_t *>(acc);
     const int32_t *a32 = reinterpret_cast<const int32_t *>(acc);
-    if (mask) {
-        if (G.count_bits == 16)
-            return run_peaks<uint16_t, true>(G, a16, peaks, cap, d_count, segcnt, segoff, tmp,
-                                             mask, st, sp);
-        return run_peaks<int32_t, true>(G, a32, peaks, cap, d_count, segcnt, segoff, tmp, mask,
-                                        st, sp);
-    }
+#define HT_PK(T, M, a)                                                                        \
+    run_peaks<T, M>(G, a, acc_stride, n_ev, peaks, cap, d_count, ws, ws_stride, flags, masks, st)
     if (G.count_bits == 16)
-        return run_peaks<uint16_t, false>(G, a16, peaks, cap, d_count, segcnt, segoff, tmp,
-                                          nullptr, st, sp);
-    return run_peaks<int32_t, false>(G, a32, peaks, cap, d_count, segcnt, segoff, tmp, nullptr,
-                                     st, sp);
+        return masks ? HT_PK(uint16_t, true, a16) : HT_PK(uint16_t, false, a16);
+    return masks ? HT_PK(int32_t, true, a32) : HT_PK(int32_t, false, a32);
+#undef HT_PK
 }
 
 }  // namespace ht
@@ -440,7 +457,7 @@ extern "C" ht_status ht_find_peaks_noalloc(const ht_geometry *g, const void *acc
         }
         scratch = g_noalloc_ptr[dev];
     }
-    e = ht::launch_peaks(g->G, acc, peaks, cap, d_count, scratch,
+    e = ht::launch_peaks(g->G, acc, 0, 1, peaks, cap, d_count, scratch, 0, 0,
                          reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return ht::set_error(HT_ERR_CUDA, cudaGetErrorString(e));
     return HT_OK;

@@ -4,7 +4,8 @@
 // Three launches, all coalesced: per-block sums of 4096-element chunks
 // (1024 threads x 4), one CTA scanning the block sums, per-block rescan with
 // the block's offset.  The element count may live in device memory (graph
-// capture: no host read).
+// capture: no host read).  Several sequences of one length are scanned by the
+// same three launches, a grid row each.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -20,6 +21,13 @@ constexpr int kChunk = kScanT * kPer;
 __device__ __forceinline__ int scan_count(int n_cap, const int *d_n)
 {
     return d_n ? max(0, min(*d_n, n_cap)) : n_cap;
+}
+
+// The grid row's sequence (strides in bytes).
+template <typename T>
+__device__ __forceinline__ T *at_seq(T *p, size_t stride)
+{
+    return reinterpret_cast<T *>(reinterpret_cast<size_t>(p) + blockIdx.y * stride);
 }
 
 // Block-wide exclusive scan of one int per thread (blockDim == kScanT);
@@ -56,9 +64,11 @@ __device__ __forceinline__ int block_exclusive(int v, int &excl)
 }
 
 __global__ void __launch_bounds__(kScanT)
-k_scan_sums(const int *__restrict__ in, int n_cap, const int *__restrict__ d_n,
-            int *__restrict__ sums)
+k_scan_sums(const int *__restrict__ in, size_t in_stride, int n_cap,
+            const int *__restrict__ d_n, int *__restrict__ sums, size_t tmp_stride)
 {
+    in = at_seq(in, in_stride);
+    sums = at_seq(sums, tmp_stride);
     const int n = scan_count(n_cap, d_n);
     const int base = blockIdx.x * kChunk + threadIdx.x * kPer;
     int s = 0;
@@ -70,8 +80,9 @@ k_scan_sums(const int *__restrict__ in, int n_cap, const int *__restrict__ d_n,
 }
 
 __global__ void __launch_bounds__(kScanT)
-k_scan_top(int *__restrict__ sums, int nb)
+k_scan_top(int *__restrict__ sums, size_t tmp_stride, int nb)
 {
+    sums = at_seq(sums, tmp_stride);
     int carry = 0;
     for (int b0 = 0; b0 < nb; b0 += kScanT) {
         const int b = b0 + threadIdx.x;
@@ -86,10 +97,15 @@ k_scan_top(int *__restrict__ sums, int nb)
 }
 
 __global__ void __launch_bounds__(kScanT)
-k_scan_apply(const int *__restrict__ in, int n_cap, const int *__restrict__ d_n,
-             const int *__restrict__ sums, int nb, int *__restrict__ out,
-             int *__restrict__ out2, int *__restrict__ total)
+k_scan_apply(const int *__restrict__ in, size_t in_stride, int n_cap,
+             const int *__restrict__ d_n, const int *__restrict__ sums, size_t tmp_stride, int nb,
+             int *__restrict__ out, size_t out_stride, int *__restrict__ out2,
+             int *__restrict__ total)
 {
+    in = at_seq(in, in_stride);
+    sums = at_seq(sums, tmp_stride);
+    out = at_seq(out, out_stride);
+    if (out2) out2 = at_seq(out2, out_stride);
     const int n = scan_count(n_cap, d_n);
     const int base = blockIdx.x * kChunk + threadIdx.x * kPer;
     int v[kPer], s = 0;
@@ -111,7 +127,7 @@ k_scan_apply(const int *__restrict__ in, int n_cap, const int *__restrict__ d_n,
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         out[n] = sums[nb];
-        if (total) *total = sums[nb];
+        if (total) total[blockIdx.y] = sums[nb];
     }
 }
 
@@ -128,9 +144,26 @@ cudaError_t scan_exclusive(const int *in, int *out, int *out2, int n_cap, const 
     const int nb = (n_cap + kChunk - 1) / kChunk;
     const int nbl = nb > 0 ? nb : 1;
     int *sums = reinterpret_cast<int *>(tmp);
-    k_scan_sums<<<nbl, kScanT, 0, st>>>(in, n_cap, d_n, sums);
-    k_scan_top<<<1, kScanT, 0, st>>>(sums, nbl);
-    k_scan_apply<<<nbl, kScanT, 0, st>>>(in, n_cap, d_n, sums, nbl, out, out2, total);
+    k_scan_sums<<<nbl, kScanT, 0, st>>>(in, 0, n_cap, d_n, sums, 0);
+    k_scan_top<<<1, kScanT, 0, st>>>(sums, 0, nbl);
+    k_scan_apply<<<nbl, kScanT, 0, st>>>(in, 0, n_cap, d_n, sums, 0, nbl, out, 0, out2, total);
+    return cudaGetLastError();
+}
+
+// The same for n_seq sequences of n counts: in, out (and out2) and tmp of
+// sequence s lie s strides (bytes) after the first's, its sum goes to total[s].
+cudaError_t scan_exclusive_batch(const int *in, size_t in_stride, int *out, size_t out_stride,
+                                 int *out2, int n, int n_seq, int *total, void *tmp,
+                                 size_t tmp_stride, cudaStream_t st)
+{
+    const int nb = (n + kChunk - 1) / kChunk;
+    const int nbl = nb > 0 ? nb : 1;
+    int *sums = reinterpret_cast<int *>(tmp);
+    const dim3 grid(nbl, n_seq);
+    k_scan_sums<<<grid, kScanT, 0, st>>>(in, in_stride, n, nullptr, sums, tmp_stride);
+    k_scan_top<<<dim3(1, n_seq), kScanT, 0, st>>>(sums, tmp_stride, nbl);
+    k_scan_apply<<<grid, kScanT, 0, st>>>(in, in_stride, n, nullptr, sums, tmp_stride, nbl, out,
+                                          out_stride, out2, total);
     return cudaGetLastError();
 }
 

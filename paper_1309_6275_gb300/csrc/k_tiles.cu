@@ -223,9 +223,15 @@ __device__ __forceinline__ int tiles_of(const ht_peak &p, int NR, int NP, int KT
 
 __global__ void k_cand_tiles(const ht_peak *__restrict__ peaks, const int *__restrict__ d_count,
                              int cap, int NR, int NP, int KT, int nct, int *__restrict__ tcnt,
-                             int *__restrict__ tcur, int *__restrict__ list)
+                             int *__restrict__ tcur, size_t tstride, int *__restrict__ list,
+                             size_t lstride)
 {
-    const int ncand = min(*d_count, cap);
+    const size_t e = blockIdx.y;   // the event
+    const int ncand = min(d_count[e], cap);
+    peaks += e * cap;
+    if (tcnt) tcnt += e * tstride;
+    if (tcur) tcur += e * tstride;
+    if (list) list += e * lstride;
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < ncand; m += gridDim.x * blockDim.x) {
         int t[kMaxTilesPerCand];
         const int nt = tiles_of(peaks[m], NR, NP, KT, nct, t);
@@ -245,10 +251,15 @@ __global__ void k_cand_tiles(const ht_peak *__restrict__ peaks, const int *__res
 __global__ void __launch_bounds__(256)
 k_cand_hist(const ht_peak *__restrict__ peaks, const int *__restrict__ d_count, int cap, int NR,
             int NP, int KT, int nct, int ntiles, int *__restrict__ tcnt, int *__restrict__ tcur,
-            int *__restrict__ list)
+            size_t tstride, int *__restrict__ list, size_t lstride)
 {
     extern __shared__ int hist[];   // [ntiles]
-    const int ncand = min(*d_count, cap);
+    const size_t e = blockIdx.y;   // the event
+    const int ncand = min(d_count[e], cap);
+    peaks += e * cap;
+    if (tcnt) tcnt += e * tstride;
+    if (tcur) tcur += e * tstride;
+    if (list) list += e * lstride;
     const int per = (ncand + gridDim.x - 1) / gridDim.x;
     const int a = blockIdx.x * per, b = min(ncand, a + per);
     if (a >= b) return;   // uniform over the CTA
@@ -277,20 +288,25 @@ k_cand_hist(const ht_peak *__restrict__ peaks, const int *__restrict__ d_count, 
 
 constexpr int kCandHistMaxTiles = 24 * 1024;   // 96 KB of shared counters
 
-// One pass of the candidate tile lists: counts (list null) or fill.
+// One pass of the candidate tile lists: counts (list null) or fill.  Several
+// events: lists lstride and counters tstride apart, the SMs' CTAs shared out
+// (a small event's pass is its launch and the clearing of its histograms).
 inline void cand_tiles_pass(const ht_peak *peaks, const int *d_count, int cap, int NR, int NP,
-                            int KT, int nct, int ntiles, int *tcnt, int *tcur, int *list,
-                            cudaStream_t st)
+                            int KT, int nct, int ntiles, int *tcnt, int *tcur, size_t tstride,
+                            int *list, size_t lstride, int n_ev, cudaStream_t st)
 {
     if (ntiles <= kCandHistMaxTiles) {
         const int sms = device_sms();
-        k_cand_hist<<<sms, 256, (size_t)ntiles * 4, st>>>(peaks, d_count, cap, NR, NP, KT, nct,
-                                                          ntiles, tcnt, tcur, list);
+        const dim3 grid(n_ev == 1 ? sms : max(1, min(sms, 4 * sms / n_ev)), n_ev);
+        k_cand_hist<<<grid, 256, (size_t)ntiles * 4, st>>>(peaks, d_count, cap, NR, NP, KT, nct,
+                                                           ntiles, tcnt, tcur, tstride, list,
+                                                           lstride);
         return;
     }
     const int nb = min(4096, (cap + 255) / 256 > 0 ? (cap + 255) / 256 : 1);
-    k_cand_tiles<<<nb, 256, 0, st>>>(peaks, d_count, cap, NR, NP, KT, nct, list ? nullptr : tcnt,
-                                     list ? tcur : nullptr, list);
+    k_cand_tiles<<<dim3(nb, n_ev), 256, 0, st>>>(peaks, d_count, cap, NR, NP, KT, nct,
+                                                 list ? nullptr : tcnt, list ? tcur : nullptr,
+                                                 tstride, list, lstride);
 }
 
 // hl (optional): scan only the nl hits hl[0 .. nl) of the event (a superset
@@ -618,11 +634,11 @@ cudaError_t launch_assoc32_kt(const DevGeom &G, const float *x, const float *y, 
     cudaError_t e = cudaMemsetAsync(tcnt, 0, (size_t)ntiles * 4, st);
     if (e != cudaSuccess) return e;
     cand_tiles_pass(peaks, d_count, cap, G.n_rho, G.n_phi0, KT, nct, ntiles, tcnt, nullptr,
-                    nullptr, st);
+                    0, nullptr, 0, 1, st);
     e = scan_exclusive(tcnt, toff, tcur, ntiles, nullptr, nullptr, tmp, st);
     if (e != cudaSuccess) return e;
-    cand_tiles_pass(peaks, d_count, cap, G.n_rho, G.n_phi0, KT, nct, ntiles, nullptr, tcur, tlist,
-                    st);
+    cand_tiles_pass(peaks, d_count, cap, G.n_rho, G.n_phi0, KT, nct, ntiles, nullptr, tcur, 0,
+                    tlist, 0, 1, st);
     dim3 grid(nct, nrt);
     k_assoc32<KT><<<grid, kThreads, assoc32_smem<KT>(G), st>>>(G, x, y, n, peaks, toff, tlist,
                                                                assoc32_lcap<KT>(G), gbest);
@@ -728,21 +744,24 @@ int assoc32_kt(const DevGeom &G)
 
 int assoc32_ntiles(const DevGeom &G, int kt) { return (G.n_phi0 / kt) * ((G.n_rho + 31) / 32); }
 
-// Per-event candidate tile lists (count, scan, scatter) into caller-carved
-// buffers: tcnt/toff/tcur (ntiles + 1), tmp (scan), tlist (6 cap).
-cudaError_t launch_cand_lists(const DevGeom &G, int kt, const ht_peak *peaks, const int *d_count,
-                              int cap, int *tcnt, int *toff, int *tcur, void *tmp, int *tlist,
-                              cudaStream_t st)
+// Candidate tile lists (count, scan, scatter) of n_ev events into
+// caller-carved buffers: tcnt/toff/tcur (ntiles + 1 each, tstride apart), tmp
+// (scan, tmp_stride bytes apart), tlist (6 cap, lstride apart).
+cudaError_t launch_cand_lists(const DevGeom &G, int kt, int n_ev, const ht_peak *peaks,
+                              const int *d_count, int cap, int *tcnt, int *toff, int *tcur,
+                              size_t tstride, void *tmp, size_t tmp_stride, int *tlist,
+                              size_t lstride, cudaStream_t st)
 {
     const int nct = G.n_phi0 / kt, ntiles = assoc32_ntiles(G, kt);
-    cudaError_t e = cudaMemsetAsync(tcnt, 0, (size_t)ntiles * 4, st);
+    cudaError_t e = cudaMemsetAsync(tcnt, 0, tstride * n_ev * 4, st);
     if (e != cudaSuccess) return e;
     cand_tiles_pass(peaks, d_count, cap, G.n_rho, G.n_phi0, kt, nct, ntiles, tcnt, nullptr,
-                    nullptr, st);
-    e = scan_exclusive(tcnt, toff, tcur, ntiles, nullptr, nullptr, tmp, st);
+                    tstride, nullptr, 0, n_ev, st);
+    e = scan_exclusive_batch(tcnt, tstride * 4, toff, tstride * 4, tcur, ntiles, n_ev, nullptr,
+                             tmp, tmp_stride, st);
     if (e != cudaSuccess) return e;
-    cand_tiles_pass(peaks, d_count, cap, G.n_rho, G.n_phi0, kt, nct, ntiles, nullptr, tcur, tlist,
-                    st);
+    cand_tiles_pass(peaks, d_count, cap, G.n_rho, G.n_phi0, kt, nct, ntiles, nullptr, tcur,
+                    tstride, tlist, lstride, n_ev, st);
     return cudaGetLastError();
 }
 

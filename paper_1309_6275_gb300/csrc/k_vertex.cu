@@ -21,6 +21,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -53,6 +54,7 @@ struct VtxArgs {
 };
 
 constexpr int kVtxThreads = 256;
+constexpr int kVtxGroup = 32;     // events per peak launch that the workspace is sized for
 
 __global__ void __launch_bounds__(kVtxThreads)
 k_vertex_vote(VtxArgs A, const ht_peak *__restrict__ peaks, const int *__restrict__ counts,
@@ -140,6 +142,8 @@ __global__ void k_vertex_first(const ht_peak *__restrict__ peaks, const int *__r
     }
     first[e] = lo;
 }
+
+size_t vtx_scratch(const DevGeom &P) { return peaks_workspace_bytes(P) + peaks_flag_bytes(P); }
 
 ht_status vfail(ht_status s, const char *msg) { return set_error(s, msg); }
 
@@ -233,7 +237,7 @@ size_t ht_vertex_accumulator_bytes(const ht_vertex *v)
 
 size_t ht_vertex_workspace_size(const ht_vertex *v)
 {
-    return v ? ht::peaks_workspace_bytes(v->P) : 0;
+    return v ? ht::kVtxGroup * ht::vtx_scratch(v->P) : 0;
 }
 
 ht_status ht_vertex_vote(const ht_vertex *v, const ht_peak *cands, const int32_t *d_count,
@@ -287,9 +291,14 @@ ht_status ht_vertex_find(const ht_vertex *v, const int32_t *acc, int32_t n_event
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const size_t cells = (size_t)v->desc.n_r * v->desc.n_theta;
     cudaError_t e = cudaSuccess;
-    for (int ev = 0; ev < n_events && e == cudaSuccess; ++ev)
-        e = ht::launch_peaks(v->P, acc + ev * cells, out + (size_t)ev * cap, cap, d_count + ev,
-                             workspace, st);
+    // a workspace below one event's full scratch serves the events in turn
+    const size_t each = ht::vtx_scratch(v->P);
+    const int group = (int)std::max((size_t)1, std::min((size_t)ht::kVtxGroup,
+                                                        workspace_bytes / each));
+    for (int ev = 0; ev < n_events && e == cudaSuccess; ev += group)
+        e = ht::launch_peaks(v->P, acc + ev * cells, cells, std::min(group, n_events - ev),
+                             out + (size_t)ev * cap, cap, d_count + ev, workspace, each,
+                             std::min(workspace_bytes, each), st);
     if (e == cudaSuccess) {
         ht::k_vertex_first<<<(n_events + 127) / 128, 128, 0, st>>>(out, d_count, cap, n_events,
                                                                     v->j_keep, d_first);
