@@ -33,8 +33,9 @@
 namespace ht {
 cudaError_t launch_vote_batch(const DevGeom &G, const float *x, const float *y, const int *off,
                               const int *order, const int *d_nev, uint16_t *acc,
-                              size_t acc_stride, unsigned long long *stats, int *head, bool pack,
-                              int kt, int sms, cudaStream_t st, const HitBuckets *hb);
+                              size_t acc_stride, unsigned long long *stats, int *head,
+                              const int *d_big, int *head_big, bool pack, int kt, int sms,
+                              cudaStream_t st, const HitBuckets *hb);
 int assoc32_kt(const DevGeom &G);
 int assoc32_ntiles(const DevGeom &G, int kt);
 cudaError_t launch_cand_lists(const DevGeom &G, int kt, int n_ev, const ht_peak *peaks,
@@ -57,7 +58,8 @@ cudaError_t prepare_batch_kernels(int max_smem);
 cudaError_t launch_vote_batch_masked(const DevGeom &G, const float *x, const float *y,
                                      const int *off, const int *order, const int *d_nev,
                                      uint16_t *acc, size_t acc_stride, unsigned long long *stats,
-                                     int *head, bool pack, int kt, int sms,
+                                     int *head, const int *d_big, int *head_big, bool pack,
+                                     int kt, int sms,
                                      const unsigned long long *masks, cudaStream_t st,
                                      const HitBuckets *hb);
 cudaError_t launch_region_mask(const void *params_bf16, const float *x, const float *y,
@@ -67,7 +69,8 @@ cudaError_t launch_region_mask(const void *params_bf16, const float *x, const fl
 cudaError_t launch_vote_batch_hitmask(const DevGeom &G, const float *x, const float *y,
                                       const int *off, const int *order, const int *d_nev,
                                       uint16_t *acc, size_t acc_stride,
-                                      unsigned long long *stats, int *head, bool pack, int kt,
+                                      unsigned long long *stats, int *head, const int *d_big,
+                                      int *head_big, bool pack, int kt,
                                       int sms, const unsigned long long *hit_masks,
                                       cudaStream_t st, const HitBuckets *hb);
 cudaError_t launch_hit_masks(const void *params_bf16, const float *x, const float *y,
@@ -285,19 +288,22 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
     // vote: the tiles whose hit lists pass the packed-counter limit (only
     // events above it can have such tiles), then every other tile of every
     // event with packed counters
-    auto vote = [&](const int *order, const int *d_nev, int *head, bool pack, int kt) {
+    auto vote = [&](const int *order, const int *d_nev, int *head, const int *d_big,
+                    int *head_big, bool pack, int kt) {
         if (R.hit_masks)
             return ht::launch_vote_batch_hitmask(G, x, y, off, order, d_nev, b->acc, b->cells,
-                                                 st64, head, pack, kt, b->sms, R.hit_masks, st,
-                                                 &b->bk);
+                                                 st64, head, d_big, head_big, pack, kt, b->sms,
+                                                 R.hit_masks, st, &b->bk);
         return masks ? ht::launch_vote_batch_masked(G, x, y, off, order, d_nev, b->acc, b->cells,
-                                                    st64, head, pack, kt, b->sms, masks, st,
-                                                    &b->bk)
+                                                    st64, head, d_big, head_big, pack, kt, b->sms,
+                                                    masks, st, &b->bk)
                      : ht::launch_vote_batch(G, x, y, off, order, d_nev, b->acc, b->cells, st64,
-                                             head, pack, kt, b->sms, st, &b->bk);
+                                             head, d_big, head_big, pack, kt, b->sms, st, &b->bk);
     };
-    e = vote(order_big_of(meta, me), meta + 0, b->heads + 0, false, b->kt_big);
-    if (e == cudaSuccess) e = vote(order_all_of(meta, me), meta + 2, b->heads + 1, true, b->kt_pack);
+    e = vote(order_big_of(meta, me), meta + 0, b->heads + 0, nullptr, nullptr, false, b->kt_big);
+    if (e == cudaSuccess)
+        e = vote(order_all_of(meta, me), meta + 2, b->heads + 1, meta + 0, b->heads + 3, true,
+                 b->kt_pack);
     if (e == cudaSuccess) e = mark(2);
     if (e != cudaSuccess) return e;
     // peaks and the association's candidate tile lists of every event slot

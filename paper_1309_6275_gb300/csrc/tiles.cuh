@@ -4,6 +4,7 @@
 // x all n_d0 bins.  Each translation unit that includes it gets its own copy
 // of these kernels (anonymous namespace).
 #pragma once
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -598,7 +599,12 @@ __device__ __forceinline__ int keep_allowed(unsigned bm, const uint8_t *jmask, i
 // cell is written.
 // hl (optional): the tile scans only the nl hits hl[0 .. nl) of the event
 // (a superset of those that can vote in its columns); otherwise all n.
-template <int KT, typename OutT, bool PACK, int MODE = kModePlain>
+// CL > 1: the CTA's cluster of CL holds the tiles of CL KT neighbouring
+// columns (same rows, all packed), and each CTA writes its share of the rows
+// and bins for all of them: its own tile alone would write 2 KT bytes of a
+// row at a time.  The caller keeps the counters of every tile until the
+// cluster has written (a cluster barrier after this call).
+template <int KT, typename OutT, bool PACK, int MODE = kModePlain, int CL = 1>
 __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restrict__ x,
                                           const float *__restrict__ y, int n,
                                           OutT *__restrict__ acc,
@@ -756,34 +762,66 @@ __device__ __forceinline__ void vote_tile(const DevGeom &G, const float *__restr
             if (threadIdx.x == 0) rn = 0;
         }
     }
-    __syncthreads();
-
-    // write-back: thread = (row, d0 bin); the KT counts of a row go out as
-    // one vector of KT * sizeof(OutT) bytes.  Votes are summed here (tile
-    // counters never saturate: they hold at most 2 n).
     unsigned long long my_votes = 0;
-    for (int t = threadIdx.x; t < TR * ND; t += kThreads) {
-        const int il = t & (TR - 1), j = t / TR;   // il == lane
-        const int i = T.i0 + il;
-        if (i >= G.n_rho) continue;
-        const bool keep = MODE != kModeEvent || halo_bin(M.bm, j, ND);
-        __align__(16) OutT e[KT];
+    if constexpr (CL > 1) {
+        static_assert(PACK && KT > 1 && sizeof(OutT) == 2 && (CL * KT) % 8 == 0,
+                      "a counter word is the output of two columns");
+        // thread = (row, d0 bin, 8 columns): the columns' counter words of 8 / KT
+        // tiles are 16 bytes of the row, and kPer threads hold its 2 CL KT
+        namespace cg = cooperative_groups;
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();
+        constexpr int kPer = CL * KT / 8, kRanks = 8 / KT, kWords = KT / 2;
+        const int q = (int)cluster.block_rank(), kb = T.k0 - q * KT;
+        const uint32_t *src[kRanks];
+        const int part = threadIdx.x % kPer;
 #pragma unroll
-        for (int kl = 0; kl < KT; ++kl) {
-            const uint32_t v = keep ? tile_get<KT, PACK>(cnt, ND, kl, j, il) : 0u;
-            my_votes += v;
-            e[kl] = saturate<OutT>(v);
+        for (int r = 0; r < kRanks; ++r) src[r] = cluster.map_shared_rank(cnt, part * kRanks + r);
+        for (int t = threadIdx.x / kPer; t < TR * ND / CL; t += kThreads / kPer) {
+            const int pr = q * (TR * ND / CL) + t, il = pr & (TR - 1), j = pr / TR;
+            const int i = T.i0 + il;
+            if (i >= G.n_rho) continue;
+            uint32_t e[4];
+#pragma unroll
+            for (int r = 0; r < kRanks; ++r)
+#pragma unroll
+                for (int w = 0; w < kWords; ++w)
+                    e[r * kWords + w] = src[r][(w * ND + j) * TR + il];
+            if (MODE == kModeEvent && !halo_bin(halo_row_blocks(mask, i, G.n_rho), j, ND))
+                e[0] = e[1] = e[2] = e[3] = 0u;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) my_votes += (e[w] & 0xffffu) + (e[w] >> 16);
+            *reinterpret_cast<uint4 *>(acc + ((size_t)i * ND + j) * G.n_phi0 + kb + part * 8) =
+                make_uint4(e[0], e[1], e[2], e[3]);
         }
-        OutT *dst = acc + ((size_t)i * ND + j) * G.n_phi0 + T.k0;
-        if constexpr (KT * sizeof(OutT) == 16) {
-            *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(e);
-        } else if constexpr (KT * sizeof(OutT) == 8) {
-            *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(e);
-        } else if constexpr (KT * sizeof(OutT) == 4) {
-            *reinterpret_cast<uint32_t *>(dst) = *reinterpret_cast<const uint32_t *>(e);
-        } else {
+    } else {
+        __syncthreads();
+        // write-back: thread = (row, d0 bin); the KT counts of a row go out as
+        // one vector of KT * sizeof(OutT) bytes.  Votes are summed here (tile
+        // counters never saturate: they hold at most 2 n).
+        for (int t = threadIdx.x; t < TR * ND; t += kThreads) {
+            const int il = t & (TR - 1), j = t / TR;   // il == lane
+            const int i = T.i0 + il;
+            if (i >= G.n_rho) continue;
+            const bool keep = MODE != kModeEvent || halo_bin(M.bm, j, ND);
+            __align__(16) OutT e[KT];
 #pragma unroll
-            for (int kl = 0; kl < KT; ++kl) dst[kl] = e[kl];
+            for (int kl = 0; kl < KT; ++kl) {
+                const uint32_t v = keep ? tile_get<KT, PACK>(cnt, ND, kl, j, il) : 0u;
+                my_votes += v;
+                e[kl] = saturate<OutT>(v);
+            }
+            OutT *dst = acc + ((size_t)i * ND + j) * G.n_phi0 + T.k0;
+            if constexpr (KT * sizeof(OutT) == 16) {
+                *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(e);
+            } else if constexpr (KT * sizeof(OutT) == 8) {
+                *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(e);
+            } else if constexpr (KT * sizeof(OutT) == 4) {
+                *reinterpret_cast<uint32_t *>(dst) = *reinterpret_cast<const uint32_t *>(e);
+            } else {
+#pragma unroll
+                for (int kl = 0; kl < KT; ++kl) dst[kl] = e[kl];
+            }
         }
     }
 
@@ -820,24 +858,45 @@ k_vote(DevGeom G, const float *__restrict__ x, const float *__restrict__ y, int 
 // set per hit of the batch (indexed like x).
 // bk (optional, ent null for none): per-event hit lists by column group; a
 // tile scans its group's list instead of the whole event.
-template <int KT, typename OutT, bool PACK, int MODE>
+// The events are order[0 .. *d_nev); with CL > 1 clusters of CL CTAs pop CL
+// neighbouring tiles at a time, which must all be packed: the first
+// *d_skip events, whose hit lists may pass the packed limit, are left out.
+template <int KT, typename OutT, bool PACK, int MODE, int CL>
 __global__ void __launch_bounds__(kThreads, PACK ? 3 : 2)
 k_vote_batch(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
              const int *__restrict__ off, const int *__restrict__ order,
-             const int *__restrict__ d_nev,
+             const int *__restrict__ d_nev, const int *__restrict__ d_skip,
              OutT *__restrict__ acc, size_t acc_stride, unsigned long long *__restrict__ stats,
              int *__restrict__ head, const unsigned long long *__restrict__ masks,
              BucketView bk)
 {
-    __shared__ int s_item;
+    namespace cg = cooperative_groups;
+    __shared__ int s_item[2];
     const int ntx = G.n_phi0 / KT, nty = (G.n_rho + 31) / 32, ntiles = ntx * nty;
-    const int total = *d_nev * ntiles;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(head, 1);
-        __syncthreads();
-        const int item = s_item;
+    int skip = 0, q = 0;
+    if constexpr (CL > 1) {
+        skip = *d_skip;
+        q = (int)cg::this_cluster().block_rank();
+    }
+    const int total = (*d_nev - skip) * ntiles;   // ntx is a multiple of CL
+    // the next item is popped before the barrier that ends the current one
+    auto pop = [&](int slot) {
+        if (q == 0 && threadIdx.x == 0) s_item[slot] = atomicAdd(head, CL);
+    };
+    pop(0);
+    for (int slot = 0;; slot ^= 1) {
+        int item;
+        if constexpr (CL > 1) {
+            // (also ends the reads of this CTA's counters by the others)
+            cg::cluster_group cluster = cg::this_cluster();
+            cluster.sync();
+            item = *cluster.map_shared_rank(&s_item[slot], 0) + q;
+        } else {
+            __syncthreads();
+            item = s_item[slot];
+        }
         if (item >= total) break;
-        const int e = order[item / ntiles], t = item % ntiles;
+        const int e = order[skip + item / ntiles], t = item % ntiles;
         const int a = off[e], n = off[e + 1] - a;
         const int *hl = nullptr;
         int nl = 0;
@@ -845,15 +904,17 @@ k_vote_batch(DevGeom G, const float *__restrict__ x, const float *__restrict__ y
         // Packed 16-bit counters take the tiles that scan at most kPackMaxHits
         // hits (a cell then holds at most 2 kPackMaxHits < 2^16 votes, so no
         // count carries into its neighbour), unpacked counters the others:
-        // the two launches of a batch split every event's tiles between them
-        // by the scanned list's length (uniform over the CTA).
+        // the launches of a batch split every event's tiles between them by the
+        // scanned list's length (uniform over the CTA, and with CL > 1 over the
+        // cluster: every list of these events is short enough).
         if (PACK == ((bk.ent ? nl : n) <= kPackMaxHits))
-            vote_tile<KT, OutT, PACK, MODE>(G, x + a, y + a, n, acc + (size_t)e * acc_stride,
-                                            stats ? stats + 2 * e : nullptr, t % ntx, t / ntx,
-                                            MODE == kModeEvent ? masks[e] : ~0ull,
-                                            MODE == kModeHit ? masks + a : nullptr, hl, nl);
-        __syncthreads();
+            vote_tile<KT, OutT, PACK, MODE, CL>(G, x + a, y + a, n, acc + (size_t)e * acc_stride,
+                                                stats ? stats + 2 * e : nullptr, t % ntx, t / ntx,
+                                                MODE == kModeEvent ? masks[e] : ~0ull,
+                                                MODE == kModeHit ? masks + a : nullptr, hl, nl);
+        pop(slot ^ 1);
     }
+    if constexpr (CL > 1) cg::this_cluster().sync();   // the first CTA's items are read
 }
 
 template <int KT>
@@ -905,48 +966,94 @@ cudaError_t launch_vote_t(const DevGeom &G, const float *x, const float *y, int 
 #undef HT_V
 }
 
+// CTAs per cluster of a batch's packed tiles: 4 tiles of 4 (2) columns write
+// 32 (16) bytes of a row instead of 8 (4).
+constexpr int kVoteCluster = 4;
+
+template <int KT, bool PACK, int MODE, int CL>
+cudaError_t launch_vote_batch_kt(const DevGeom &G, const float *x, const float *y, const int *off,
+                                 const int *order, const int *d_nev, const int *d_skip,
+                                 uint16_t *acc, size_t acc_stride, unsigned long long *stats,
+                                 int *head, int sms, const unsigned long long *masks,
+                                 cudaStream_t st, const BucketView &bk)
+{
+    const auto kernel = k_vote_batch<KT, uint16_t, PACK, MODE, CL>;
+    const size_t smem = vote_smem<KT>(G, PACK, MODE);
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = CL;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.gridDim = dim3(CL);
+    int occ = 0;
+    if (CL > 1) {
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&occ, kernel, &cfg);
+        if (e != cudaSuccess) return e;
+        cfg.gridDim = dim3(CL * (occ > 0 ? occ : 1));
+    } else {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kThreads, smem);
+        cfg.gridDim = dim3(sms * (occ > 0 ? occ : 1));
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, G, x, y, off, order, d_nev, d_skip, acc, acc_stride,
+                              stats, head, masks, bk);
+}
+
 // Persistent vote of a batch: `order` lists d_nev[0] event slots; every CTA
 // slot of the GPU (SMs x resident CTAs) pops items until the queue is empty.
 // kt selects the tile width (0 = default).  pack: this launch takes the
 // listed events' tiles that scan at most kPackMaxHits hits (a column group's
 // hit list with buckets, else the event) with 16-bit packed counters;
-// otherwise it takes their other tiles with 32-bit counters.  *head must
-// be zero.
+// otherwise it takes their other tiles with 32-bit counters.  With d_big, the
+// first *d_big events of order[] are those of more than kPackMaxHits hits:
+// where the tiles divide into clusters, these events' tiles and the others'
+// take a launch each.  *head and *head_big must be zero.
+//
+// Clusters, measured on 25 events of 400 hits (256 x 128 x 512 cells, 0.84 GB of
+// counts, 4 columns a tile): 1294 us alone, 1130 us in clusters of 4 (32-byte
+// writes), 1302 us of 8: the wait for the slowest tile and the remote reads cost
+// more than the wider writes give.  Most of the rest is each tile's chain of
+// barriers (zero, phases 1 and 2, write) with 24 warps per SM.
 template <int MODE>
 cudaError_t launch_vote_batch_t(const DevGeom &G, const float *x, const float *y, const int *off,
                                 const int *order, const int *d_nev, uint16_t *acc,
                                 size_t acc_stride, unsigned long long *stats, int *head,
-                                bool pack, int kt, int sms, const unsigned long long *masks,
-                                cudaStream_t st, BucketView bk = BucketView{})
+                                const int *d_big, int *head_big, bool pack, int kt, int sms,
+                                const unsigned long long *masks, cudaStream_t st,
+                                BucketView bk = BucketView{})
 {
-#define HT_VB(KTV, PK)                                                                        \
-    do {                                                                                      \
-        int occ = 0;                                                                          \
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                        \
-            &occ, k_vote_batch<KTV, uint16_t, PK, MODE>, kThreads,                       \
-            vote_smem<KTV>(G, PK, MODE));                                                \
-        k_vote_batch<KTV, uint16_t, PK, MODE><<<sms * (occ > 0 ? occ : 1), kThreads,    \
-                                                     vote_smem<KTV>(G, PK, MODE), st>>>( \
-            G, x, y, off, order, d_nev, acc, acc_stride, stats, head, masks, bk);             \
-        return cudaGetLastError();                                                            \
-    } while (0)
-    // the per-hit mode's larger items would drop a tuned width to two CTAs
-    // per SM: it keeps three
-    const size_t budget = MODE == kModeHit ? kSmemBudget3 : kSmemBudget2;
+#define HT_VB(KTV, PK, CL)                                                                    \
+    launch_vote_batch_kt<KTV, PK, MODE, CL>(G, x, y, off, order, d_nev, d_big, acc,           \
+                                            acc_stride, stats, head, sms, masks, st, bk)
     if (pack) {
+        // the per-hit mode's larger items would drop a tuned width to two CTAs
+        // per SM: it keeps three
+        const size_t budget = MODE == kModeHit ? kSmemBudget3 : kSmemBudget2;
         if (kt == 0) kt = vote_smem<4>(G, true, MODE) <= kSmemBudget3 ? 4
                         : vote_smem<2>(G, true, MODE) <= kSmemBudget3 ? 2 : 1;
-        if (kt == 4 && vote_smem<4>(G, true, MODE) <= budget) HT_VB(4, true);
-        if (kt >= 2 && vote_smem<2>(G, true, MODE) <= budget) HT_VB(2, true);
-        HT_VB(1, true);
+        if (kt == 4 && vote_smem<4>(G, true, MODE) > budget) kt = 2;
+        if (kt >= 2 && vote_smem<2>(G, true, MODE) > budget) kt = 1;
+        if (d_big && kt >= 2 && (G.n_phi0 / kt) % kVoteCluster == 0) {
+            const cudaError_t e = kt == 4 ? HT_VB(4, true, kVoteCluster)
+                                          : HT_VB(2, true, kVoteCluster);
+            if (e != cudaSuccess) return e;
+            d_nev = d_big;   // the packed tiles of the others
+            head = head_big;
+        }
+        if (kt == 4) return HT_VB(4, true, 1);
+        return kt >= 2 ? HT_VB(2, true, 1) : HT_VB(1, true, 1);
     }
     if (kt == 0) kt = vote_smem<8>(G, false, MODE) <= kSmemBudget2 ? 8
                     : vote_smem<4>(G, false, MODE) <= kSmemBudget2 ? 4
                     : vote_smem<2>(G, false, MODE) <= kSmemBudget2 ? 2 : 1;
-    if (kt == 8 && vote_smem<8>(G, false, MODE) <= kSmemBudget2) HT_VB(8, false);
-    if (kt >= 4 && vote_smem<4>(G, false, MODE) <= kSmemBudget2) HT_VB(4, false);
-    if (kt >= 2 && vote_smem<2>(G, false, MODE) <= kSmemBudget2) HT_VB(2, false);
-    HT_VB(1, false);
+    if (kt == 8 && vote_smem<8>(G, false, MODE) <= kSmemBudget2) return HT_VB(8, false, 1);
+    if (kt >= 4 && vote_smem<4>(G, false, MODE) <= kSmemBudget2) return HT_VB(4, false, 1);
+    if (kt >= 2 && vote_smem<2>(G, false, MODE) <= kSmemBudget2) return HT_VB(2, false, 1);
+    return HT_VB(1, false, 1);
 #undef HT_VB
 }
 
@@ -979,13 +1086,15 @@ cudaError_t prepare_vote_kernels_t(int max_smem)
         (const void *)k_vote<4, int32_t, false, MODE>,
         (const void *)k_vote<2, int32_t, false, MODE>,
         (const void *)k_vote<1, int32_t, false, MODE>,
-        (const void *)k_vote_batch<4, uint16_t, true, MODE>,
-        (const void *)k_vote_batch<2, uint16_t, true, MODE>,
-        (const void *)k_vote_batch<1, uint16_t, true, MODE>,
-        (const void *)k_vote_batch<8, uint16_t, false, MODE>,
-        (const void *)k_vote_batch<4, uint16_t, false, MODE>,
-        (const void *)k_vote_batch<2, uint16_t, false, MODE>,
-        (const void *)k_vote_batch<1, uint16_t, false, MODE>};
+        (const void *)k_vote_batch<4, uint16_t, true, MODE, kVoteCluster>,
+        (const void *)k_vote_batch<2, uint16_t, true, MODE, kVoteCluster>,
+        (const void *)k_vote_batch<4, uint16_t, true, MODE, 1>,
+        (const void *)k_vote_batch<2, uint16_t, true, MODE, 1>,
+        (const void *)k_vote_batch<1, uint16_t, true, MODE, 1>,
+        (const void *)k_vote_batch<8, uint16_t, false, MODE, 1>,
+        (const void *)k_vote_batch<4, uint16_t, false, MODE, 1>,
+        (const void *)k_vote_batch<2, uint16_t, false, MODE, 1>,
+        (const void *)k_vote_batch<1, uint16_t, false, MODE, 1>};
     return allow_smem(fns, (int)(sizeof fns / sizeof fns[0]), max_smem);
 }
 
