@@ -373,6 +373,9 @@ __device__ __forceinline__ void assoc32_tile(const DevGeom &G, const float *__re
     __syncthreads();
     const int m_min = s_mrange[0];
     const bool offs = s_mrange[1] - m_min < (1 << 20) && s_mrange[2] < 4096;   // uniform
+    // no candidate of the tile beats this key
+    const unsigned long long most =
+        ((unsigned long long)(unsigned)s_mrange[2] << 32) | (0xffffffffull - (unsigned)m_min);
     if (offs) {
         for (int t = threadIdx.x; t < L; t += kThreads) local[t] = tlist[l0 + t];
     } else {
@@ -476,8 +479,11 @@ __device__ __forceinline__ void assoc32_tile(const DevGeom &G, const float *__re
         int ha;
         float xh, yh;
         pf.next(x, y, S, base, ha, xh, yh);
-        collect<KT, kModeEvent>(G, T, xh, yh, S.n, base + threadIdx.x, ha, lane, qn[parity], W,
-                                &M);
+        // a hit that holds a key no candidate here beats is done with the tile
+        // (its key only grows, so an old one is safe)
+        int h = base + threadIdx.x;
+        if (h < S.n && __ldcg(gbest + ha) >= most) h = S.n;
+        collect<KT, kModeEvent>(G, T, xh, yh, S.n, h, ha, lane, qn[parity], W, &M);
         __syncthreads();
         const int nf = qn[parity][0], ns = qn[parity][1];
         if (threadIdx.x == 0) {
