@@ -611,7 +611,8 @@ size_t assoc_smem(const DevGeom &G)
 template <int KT>
 int assoc32_lcap(const DevGeom &G)
 {
-    return 17 * ((KT + 3) / 2) * ((G.n_d0 + 1) / 2) + 32;
+    // a multiple of four: the 16-byte items lie behind it in shared memory
+    return (17 * ((KT + 3) / 2) * ((G.n_d0 + 1) / 2) + 32 + 3) / 4 * 4;
 }
 
 template <int KT>
