@@ -67,65 +67,7 @@ __device__ __forceinline__ int event_of_hit(const int *off, int n_ev, int h)
 
 #include "mlp_tc.cuh"
 
-// Split z of C[M][N] = sum_h A[h][M] B[h][N] (A BF16 with row stride lda,
-// B float32 with row stride ldb) and, when bias is set, of bias[N] =
-// sum_h B[h][N], on the CUDA cores, for the first layer (M = 6 inputs; the
-// 128-row layers use k_wgrad_tc): the hits are split across gridDim.z and
-// split z stores its partial sums at C + z pstride and bias + z pstride
-// (plain stores: every entry of a split is written by exactly one CTA);
-// k_wgrad_reduce adds the splits in a fixed order, so a training step is
-// bit-reproducible.  CTA: 256 threads, a 64 x 64 output tile (4 x 4 per
-// thread).
-constexpr int kGT = 64, kGH = 32;
 constexpr int kMaxSplits = 128;
-__global__ void __launch_bounds__(256)
-k_wgrad(const __nv_bfloat16 *__restrict__ A, int lda, const float *__restrict__ B, int ldb,
-        int n, int M, int N, float *__restrict__ C, float *__restrict__ bias, size_t pstride)
-{
-    C += (size_t)blockIdx.z * pstride;
-    if (bias) bias += (size_t)blockIdx.z * pstride;
-    __shared__ float sA[kGH][kGT], sB[kGH][kGT];
-    const int m0 = blockIdx.x * kGT, n0 = blockIdx.y * kGT;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc[4][4] = {};
-    float bacc = 0.f;
-    const int per = (n + gridDim.z - 1) / gridDim.z;
-    const int h0 = blockIdx.z * per, h1 = min(n, h0 + per);
-    for (int hb = h0; hb < h1; hb += kGH) {
-        for (int t = threadIdx.x; t < kGH * kGT; t += 256) {
-            const int r = t / kGT, c = t % kGT;
-            const int hh = hb + r;
-            sA[r][c] = (hh < h1 && m0 + c < M) ? __bfloat162float(A[(size_t)hh * lda + m0 + c]) : 0.f;
-            sB[r][c] = (hh < h1 && n0 + c < N) ? B[(size_t)hh * ldb + n0 + c] : 0.f;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int r = 0; r < kGH; ++r) {
-            float a[4], b[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = sA[r][ty * 4 + u];
-                b[u] = sB[r][tx * 4 + u];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
-        }
-        if (bias && blockIdx.x == 0 && threadIdx.x < kGT)
-            for (int r = 0; r < kGH; ++r) bacc += sB[r][threadIdx.x];
-        __syncthreads();
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int m = m0 + ty * 4 + u, nn = n0 + tx * 4 + v;
-            if (m < M && nn < N) C[(size_t)m * N + nn] = acc[u][v];
-        }
-    if (bias && blockIdx.x == 0 && threadIdx.x < kGT && n0 + threadIdx.x < N)
-        bias[n0 + threadIdx.x] = bacc;
-}
 
 // grad[i] += the splits' partial sums of parameter i, added in split order.
 __global__ void k_wgrad_reduce(const float *__restrict__ part, int splits, float *__restrict__ grad)
@@ -133,6 +75,7 @@ __global__ void k_wgrad_reduce(const float *__restrict__ part, int splits, float
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kParams) return;
     float s = 0.f;
+#pragma unroll 16
     for (int z = 0; z < splits; ++z) s += part[(size_t)z * kParams + i];
     grad[i] += s;
 }
@@ -256,7 +199,7 @@ cudaError_t prepare_mlp_kernels()
         e = cudaFuncSetAttribute(k_mlp_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kBwdTcSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kWgTcSmem);
     return e;
 }
@@ -364,14 +307,11 @@ ht_status ht_mlp_backward(const void *params_bf16, const int32_t *labels, int32_
     k_mlp_bwd_tc<<<blocks, kTcM, kBwdTcSmem, st>>>((const __nv_bfloat16 *)params_bf16, prob,
                                                    labels, (const __nv_bfloat16 *)h1,
                                                    (const __nv_bfloat16 *)h2, n, nl, dL, dH2, dH1);
-    // dW3 = h2^T dL, db3 and dW2 = h1^T dH2, db2 on the tensor cores
-    k_wgrad_tc<<<splits, kTcM, kWgTcSmem, st>>>((const __nv_bfloat16 *)h2, kH, dL, kOut, n, kOut,
-                                                part + oW3, part + ob3, kParams);
-    k_wgrad_tc<<<splits, kTcM, kWgTcSmem, st>>>((const __nv_bfloat16 *)h1, kH, dH2, kH, n, kH,
-                                                part + oW2, part + ob2, kParams);
-    // dW1 = f^T dH1, db1
-    k_wgrad<<<dim3(1, kH / kGT, splits), 256, 0, st>>>((const __nv_bfloat16 *)feat, 8, dH1, kH, n,
-                                                       kIn, kH, part + oW1, part + ob1, kParams);
+    // dW3 = h2^T dL, db3; dW2 = h1^T dH2, db2; dW1 = f^T dH1, db1
+    const WgradJob j3{(const __nv_bfloat16 *)h2, dL, part + oW3, part + ob3, kH, kOut};
+    const WgradJob j2{(const __nv_bfloat16 *)h1, dH2, part + oW2, part + ob2, kH, kH};
+    const WgradJob j1{(const __nv_bfloat16 *)feat, dH1, part + oW1, part + ob1, 8, kH};
+    k_wgrad<<<dim3(splits, 3), kWgThreads, kWgTcSmem, st>>>(j3, j2, j1, n, kParams);
     k_wgrad_reduce<<<(kParams + 255) / 256, 256, 0, st>>>(part, splits, grad);
     e = cudaGetLastError();
     return e == cudaSuccess ? HT_OK : set_error(HT_ERR_CUDA, cudaGetErrorString(e));

@@ -127,13 +127,20 @@ k_mlp_fwd_tc(const __nv_bfloat16 *__restrict__ w, const float *__restrict__ x,
     const int tid = threadIdx.x, warp = tid >> 5;
     if (out.d_n) n = *out.d_n;
 
-    for (int t = tid; t < kH * kH; t += kTcM) {                  // B2(n = o, k = i) = W2[i][o]
-        const int i = t / kH, o = t % kH;
-        *reinterpret_cast<__nv_bfloat16 *>(sB2 + core_off(o, i)) = w[oW2 + t];
+    // eight k of a row are 16 bytes of the core layout: eight loads, one store
+    for (int t = tid; t < kH * kH / 8; t += kTcM) {              // B2(n = o, k = i) = W2[i][o]
+        const int i = t / kH * 8, o = t % kH;
+        __align__(16) __nv_bfloat16 b[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) b[u] = w[oW2 + (i + u) * kH + o];
+        *reinterpret_cast<uint4 *>(sB2 + core_off(o, i)) = *reinterpret_cast<uint4 *>(b);
     }
-    for (int t = tid; t < kH * kOut; t += kTcM) {                // B3(n = c, k = i) = W3[i][c]
-        const int i = t / kOut, c = t % kOut;
-        *reinterpret_cast<__nv_bfloat16 *>(sB3 + core_off(c, i)) = w[oW3 + t];
+    for (int t = tid; t < kH * kOut / 8; t += kTcM) {            // B3(n = c, k = i) = W3[i][c]
+        const int i = t / kOut * 8, c = t % kOut;
+        __align__(16) __nv_bfloat16 b[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) b[u] = w[oW3 + (i + u) * kOut + c];
+        *reinterpret_cast<uint4 *>(sB3 + core_off(c, i)) = *reinterpret_cast<uint4 *>(b);
     }
     for (int t = tid; t < kIn * kH; t += kTcM) sW1[t] = w[oW1 + t];
     for (int t = tid; t < kH; t += kTcM) {
@@ -369,13 +376,13 @@ k_mlp_fwd_tc(const __nv_bfloat16 *__restrict__ w, const float *__restrict__ x,
 // tensor cores rounded to BF16; the accumulators and the stored gradients
 // are float32.
 //
-// Weight gradients (k_wgrad_tc): C[m][n] = sum_h A[h][m] B[h][n] for one
-// split of the hits, M = 128, N = 128 or 64, K = 128 hits per step: A^T and
-// B^T are staged K-major (eight hits per 16-byte core-matrix row) and the
-// split's sum accumulates in tensor memory.  B (a float32 gradient) enters
-// rounded to BF16; the bias sum over the same hits is float32 in hit order.
-// Splits are reduced in a fixed order (k_wgrad_reduce), so a training step is
-// reproducible bit for bit.
+// Weight gradients (k_wgrad): C[m][n] = sum_h A[h][m] B[h][n] for one split of
+// the hits.  The 128-row layers: M = 128, N = 128 or 64, K = 128 hits per step:
+// A^T and B^T are staged K-major (eight hits per 16-byte core-matrix row) and
+// the split's sum accumulates in tensor memory.  B (a float32 gradient) enters
+// rounded to BF16; the bias sum over the same hits is float32.  The first layer
+// (six inputs) is summed on the CUDA cores.  Splits are reduced in a fixed order
+// (k_wgrad_reduce), so a training step is reproducible bit for bit.
 
 constexpr uint32_t kSBO64 = 1024;                 // 8-row group stride for K = 64
 constexpr size_t kBwdTcSmem = (size_t)kH * kOut * 2 + (size_t)kH * kH * 2 +
@@ -455,10 +462,19 @@ k_mlp_bwd_tc(const __nv_bfloat16 *__restrict__ w, const float *__restrict__ prob
     __shared__ __align__(8) unsigned long long s_mbar;
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5;
-    for (int t = tid; t < kH * kOut; t += kTcM)         // B3(n = o, k = c) = W3[o][c]
-        *reinterpret_cast<__nv_bfloat16 *>(sB3 + core_off64(t / kOut, t % kOut)) = w[oW3 + t];
-    for (int t = tid; t < kH * kH; t += kTcM)           // B2(n = i, k = o) = W2[i][o]
-        *reinterpret_cast<__nv_bfloat16 *>(sB2 + core_off(t / kH, t % kH)) = w[oW2 + t];
+    // (parameters the caller need not align: eight elements by one load or by eight)
+    const bool wide = (reinterpret_cast<uintptr_t>(w) & 15) == 0;
+    auto eight = [&](const __nv_bfloat16 *q) -> uint4 {
+        if (wide) return __ldg(reinterpret_cast<const uint4 *>(q));
+        __align__(16) __nv_bfloat16 b[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) b[u] = q[u];
+        return *reinterpret_cast<uint4 *>(b);
+    };
+    for (int t = tid * 8; t < kH * kOut; t += kTcM * 8)   // B3(n = o, k = c) = W3[o][c]
+        *reinterpret_cast<uint4 *>(sB3 + core_off64(t / kOut, t % kOut)) = eight(w + oW3 + t);
+    for (int t = tid * 8; t < kH * kH; t += kTcM * 8)     // B2(n = i, k = o) = W2[i][o]
+        *reinterpret_cast<uint4 *>(sB2 + core_off(t / kH, t % kH)) = eight(w + oW2 + t);
     const uint32_t mbar = smem_u32(&s_mbar);
     const uint32_t tmem = tc_setup(mbar, &s_tmem, kTcCols);
     const uint32_t d1 = tmem, d2 = tmem + kH;
@@ -568,47 +584,110 @@ k_mlp_bwd_tc(const __nv_bfloat16 *__restrict__ w, const float *__restrict__ prob
     tc_teardown(failed, mbar, phase, tmem, kTcCols);
 }
 
-// Split blockIdx.x of C[128][N] = sum_h A[h][m] B[h][n] (A BF16, row stride
-// lda; B float32, row stride ldb) and of bias[n] = sum_h B[h][n], over the
-// split's hits; stored at C + split pstride and bias + split pstride.
-__global__ void __launch_bounds__(kTcM)
-k_wgrad_tc(const __nv_bfloat16 *__restrict__ A, int lda, const float *__restrict__ B, int ldb,
-           int n, int N, float *__restrict__ C, float *__restrict__ bias, size_t pstride)
+// One layer's weight gradient: C[M][N] = sum_h A[h][m] B[h][n] and bias[n] =
+// sum_h B[h][n] (A BF16, row stride lda; B float32, row stride N).
+struct WgradJob {
+    const __nv_bfloat16 *A;
+    const float *B;
+    float *C, *bias;
+    int lda, N;
+};
+
+constexpr int kWgThreads = 512;
+
+// blockIdx.x: the split of the hits, its sums at C, bias + split pstride;
+// blockIdx.y: the layer (2 the first one, M = kIn; else M = 128).
+//
+// Bound by the latency of the loads (a split is some hundred hits): with 128
+// threads a CTA, a launch per layer and 64 rows of the 6-row product the three
+// took 210 + 75 us for 80k hits; with all layers in one launch, 512 threads and
+// each thread's loads of a step issued together 88 us (the step: 475 -> 250 us).
+__global__ void __launch_bounds__(kWgThreads, 2)
+k_wgrad(WgradJob j0, WgradJob j1, WgradJob j2, int n, size_t pstride)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    const WgradJob J = blockIdx.y == 0 ? j0 : blockIdx.y == 1 ? j1 : j2;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    constexpr int kParts = kWgThreads / kTcM;           // threads per row
+    const int row = tid % kTcM, part = tid / kTcM;      // row == TMEM lane of the thread
+    float *const C = J.C + (size_t)blockIdx.x * pstride;
+    float *const bias = J.bias + (size_t)blockIdx.x * pstride;
+    const int per = (n + gridDim.x - 1) / gridDim.x;
+    const int h0 = blockIdx.x * per, h1 = min(n, h0 + per);
+    if (blockIdx.y == 2) {
+        // ---- first layer: thread = (column n, a quarter of the split's hits)
+        const bool wide = (reinterpret_cast<uintptr_t>(J.A) & 15) == 0;   // lda = 8
+        const int q = (max(h1 - h0, 0) + kParts - 1) / kParts;
+        const int a = h0 + part * q, b = min(h1, a + q);
+        float acc[kIn + 1] = {};
+#pragma unroll 8
+        for (int h = a; h < b; ++h) {
+            const float g = J.B[(size_t)h * J.N + row];
+            __align__(16) __nv_bfloat16 f[8];
+            if (wide) {
+                *reinterpret_cast<uint4 *>(f) =
+                    __ldg(reinterpret_cast<const uint4 *>(J.A + (size_t)h * 8));
+            } else {
+#pragma unroll
+                for (int m = 0; m < kIn; ++m) f[m] = J.A[(size_t)h * 8 + m];
+            }
+#pragma unroll
+            for (int m = 0; m < kIn; ++m) acc[m] = fmaf(__bfloat162float(f[m]), g, acc[m]);
+            acc[kIn] += g;
+        }
+        float(*s)[kIn + 1][kTcM] = reinterpret_cast<float(*)[kIn + 1][kTcM]>(smem);
+#pragma unroll
+        for (int m = 0; m <= kIn; ++m) s[part][m][row] = acc[m];
+        __syncthreads();
+        for (int t = tid; t < (kIn + 1) * kTcM; t += kWgThreads) {
+            const int m = t / kTcM, c = t % kTcM;
+            float v = s[0][m][c];
+#pragma unroll
+            for (int p = 1; p < kParts; ++p) v += s[p][m][c];
+            if (m < kIn) C[(size_t)m * J.N + c] = v;
+            else bias[c] = v;
+        }
+        return;
+    }
     unsigned char *sA = smem;                           // A^T: M 128 x K 128 hits
     unsigned char *sB = smem + kTcM * kTcM * 2;         // B^T: N x K 128 hits
     __shared__ __align__(8) unsigned long long s_mbar;
     __shared__ uint32_t s_tmem;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    C += (size_t)blockIdx.x * pstride;
-    bias += (size_t)blockIdx.x * pstride;
-    const int per = (n + gridDim.x - 1) / gridDim.x;
-    const int h0 = blockIdx.x * per, h1 = min(n, h0 + per);
+    __shared__ float s_bias[kParts][kTcM];
     const uint32_t mbar = smem_u32(&s_mbar);
     const uint32_t tmem = tc_setup(mbar, &s_tmem, kWgTcCols);
     const uint32_t aA = smem_u32(sA), aB = smem_u32(sB);
+    const int N = J.N;
+    const bool col = row < N;
     uint32_t phase = 0;
     bool failed = false, any = false;
     float bacc = 0.f;
     for (int hb = h0; hb < h1; hb += kTcM) {
-        // ---- stage: thread = row m of A^T (and n of B^T), eight hits per store
-        for (int g = 0; g < kTcM / 8; ++g) {
-            __align__(16) __nv_bfloat16 av[8], bv[8];
+        // ---- stage: thread = row m of A^T (and n of B^T) of 32 hits, eight per
+        // store; every load of the step is issued before the first store
+        constexpr int kG = kTcM / 8 / kParts;
+        __align__(16) __nv_bfloat16 av[kG][8];
+        float bf[kG][8];
+#pragma unroll
+        for (int g = 0; g < kG; ++g)
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int hh = hb + 8 * g + u;
+                const int hh = hb + 8 * (part * kG + g) + u;
                 const bool in = hh < h1;
-                av[u] = in ? A[(size_t)hh * lda + tid] : __float2bfloat16_rn(0.f);
-                float b = 0.f;
-                if (tid < N && in) b = B[(size_t)hh * ldb + tid];
-                bacc += b;
-                bv[u] = __float2bfloat16_rn(b);
+                av[g][u] = in ? J.A[(size_t)hh * J.lda + row] : __float2bfloat16_rn(0.f);
+                bf[g][u] = col && in ? J.B[(size_t)hh * N + row] : 0.f;
             }
-            *reinterpret_cast<uint4 *>(sA + core_off(tid, 8 * g)) = *reinterpret_cast<uint4 *>(av);
-            if (tid < N)
-                *reinterpret_cast<uint4 *>(sB + core_off(tid, 8 * g)) =
-                    *reinterpret_cast<uint4 *>(bv);
+#pragma unroll
+        for (int g = 0; g < kG; ++g) {
+            __align__(16) __nv_bfloat16 bv[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                bacc += bf[g][u];
+                bv[u] = __float2bfloat16_rn(bf[g][u]);
+            }
+            const uint32_t at = core_off(row, 8 * (part * kG + g));
+            *reinterpret_cast<uint4 *>(sA + at) = *reinterpret_cast<uint4 *>(av[g]);
+            if (col) *reinterpret_cast<uint4 *>(sB + at) = *reinterpret_cast<uint4 *>(bv);
         }
         tc_publish();
         if (tid == 0) {
@@ -627,15 +706,24 @@ k_wgrad_tc(const __nv_bfloat16 *__restrict__ A, int lda, const float *__restrict
         tc_fence_after();   // the tiles may be overwritten: the MMAs are done
     }
     if (!failed) {
-        // thread = row m: the split's sums (zero when it had no hits)
-        for (int c0 = 0; c0 < N; c0 += 32) {
+        // thread = (row m, 32 columns): the split's sums (zero when it had no hits)
+        const int c0 = part * 32;
+        if (c0 < N) {   // uniform over the warp
             uint32_t r[32];
-            if (any) tc_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, r);
+            if (any) tc_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0, r);
 #pragma unroll
             for (int q = 0; q < 32; ++q)
-                C[(size_t)tid * N + c0 + q] = any ? __uint_as_float(r[q]) : 0.f;
+                C[(size_t)row * N + c0 + q] = any ? __uint_as_float(r[q]) : 0.f;
         }
-        if (tid < N) bias[tid] = bacc;
+        s_bias[part][row] = bacc;
+        __syncthreads();   // uniform: failed is the barrier's vote
+        if (part == 0 && col) {
+            float v = s_bias[0][row];
+#pragma unroll
+            for (int p = 1; p < kParts; ++p) v += s_bias[p][row];
+            bias[row] = v;
+        }
     }
     tc_teardown(failed, mbar, phase, tmem, kWgTcCols);
 }
+static_assert(kWgThreads / kTcM * 32 == kH, "a thread's 32 columns cover the widest layer");
