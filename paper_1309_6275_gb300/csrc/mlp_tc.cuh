@@ -651,7 +651,9 @@ constexpr int kWgThreads = 512;
 // Bound by the latency of the loads (a split is some hundred hits): with 128
 // threads a CTA, a launch per layer and 64 rows of the 6-row product the three
 // took 210 + 75 us for 80k hits; with all layers in one launch, 512 threads and
-// each thread's loads of a step issued together 88 us (the step: 475 -> 250 us).
+// each thread's loads of a step issued together 76 us.  Two CTAs per SM (64
+// registers, a few spills) and one (no spills, 71 us, but the reduction after
+// it 2 us slower) are equal; the first layer's blocks first: 82 us.
 __global__ void __launch_bounds__(kWgThreads, 2)
 k_wgrad(WgradJob j0, WgradJob j1, WgradJob j2, int n, size_t pstride)
 {
@@ -665,25 +667,38 @@ k_wgrad(WgradJob j0, WgradJob j1, WgradJob j2, int n, size_t pstride)
     const int per = (n + gridDim.x - 1) / gridDim.x;
     const int h0 = blockIdx.x * per, h1 = min(n, h0 + per);
     if (blockIdx.y == 2) {
-        // ---- first layer: thread = (column n, a quarter of the split's hits)
+        // ---- first layer: thread = (column n, a quarter of the hits of a chunk),
+        // the chunk's features staged so that a hit costs one global load
+        constexpr int kChunk = 2048;
+        uint4 *const sf = reinterpret_cast<uint4 *>(smem);
         const bool wide = (reinterpret_cast<uintptr_t>(J.A) & 15) == 0;   // lda = 8
-        const int q = (max(h1 - h0, 0) + kParts - 1) / kParts;
-        const int a = h0 + part * q, b = min(h1, a + q);
         float acc[kIn + 1] = {};
-#pragma unroll 8
-        for (int h = a; h < b; ++h) {
-            const float g = J.B[(size_t)h * J.N + row];
-            __align__(16) __nv_bfloat16 f[8];
-            if (wide) {
-                *reinterpret_cast<uint4 *>(f) =
-                    __ldg(reinterpret_cast<const uint4 *>(J.A + (size_t)h * 8));
-            } else {
+        for (int hc = h0; hc < h1; hc += kChunk) {
+            const int m = min(kChunk, h1 - hc), q = (m + kParts - 1) / kParts;
+            for (int t = tid; t < m; t += kWgThreads) {
+                const __nv_bfloat16 *a = J.A + (size_t)(hc + t) * 8;
+                __align__(16) __nv_bfloat16 f[8];
+                if (wide) {
+                    *reinterpret_cast<uint4 *>(f) = __ldg(reinterpret_cast<const uint4 *>(a));
+                } else {
 #pragma unroll
-                for (int m = 0; m < kIn; ++m) f[m] = J.A[(size_t)h * 8 + m];
+                    for (int u = 0; u < 8; ++u) f[u] = a[u];
+                }
+                sf[t] = *reinterpret_cast<uint4 *>(f);
             }
+            __syncthreads();
+            const int end = min(m, (part + 1) * q);
+            const float *g = J.B + (size_t)hc * J.N + row;
+#pragma unroll 16
+            for (int t = part * q; t < end; ++t) {
+                const float v = g[(size_t)t * J.N];
+                __align__(16) __nv_bfloat16 f[8];
+                *reinterpret_cast<uint4 *>(f) = sf[t];
 #pragma unroll
-            for (int m = 0; m < kIn; ++m) acc[m] = fmaf(__bfloat162float(f[m]), g, acc[m]);
-            acc[kIn] += g;
+                for (int u = 0; u < kIn; ++u) acc[u] = fmaf(__bfloat162float(f[u]), v, acc[u]);
+                acc[kIn] += v;
+            }
+            __syncthreads();
         }
         float(*s)[kIn + 1][kTcM] = reinterpret_cast<float(*)[kIn + 1][kTcM]>(smem);
 #pragma unroll
