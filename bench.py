@@ -632,10 +632,11 @@ def launches_per_batch(ne, learned=False):
 
 def track_launches(learned=False):
     """Kernels one ht_batch_run_tracks replays, whatever its number of events:
-    the hit index (3 + scan 3), the vote, the peaks of all events (2 + scan
-    3), the confirmation (prefix, confirmation, decode) and the z vote (6);
-    with the proposal one more (the network's top-k per hit)."""
-    return 6 + 1 + 5 + 3 + 6 + (1 if learned else 0)
+    the hit index (3 + scan 3), the vote (the large events' hits put in order,
+    their tiles, the others'), the peaks of all events (2 + scan 3), the
+    confirmation (prefix, confirmation, decode) and the z vote (6); with the
+    proposal the network's top-k per hit and one vote."""
+    return 6 + (2 if learned else 3) + 5 + 3 + 6
 
 
 def run_ours(args):
