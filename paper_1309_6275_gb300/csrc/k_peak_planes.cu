@@ -25,9 +25,9 @@
 //    its segment's position plus its rank, in column order.
 //
 // Bound by issue and by the latency of the sweep's loads.  Peak stage, GB300,
-// 25 events of 256 x 128 x 512 cells: 1.75 -> 0.51 ms (the launches were five
+// 25 events of 256 x 128 x 512 cells: 1.75 -> 0.44 ms (the launches were five
 // per event, the stencil 49 us of each event); two of 512 x 256 x 1024: 0.80
-// -> 0.38.
+// -> 0.29.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -36,7 +36,11 @@
 namespace ht {
 namespace {
 
-constexpr int kSegCols = 128;   // a row has at most 64 peaks in a segment: counts fit a byte
+// Short segments give few events enough warps (one event of 2000 hits: its
+// batch 384 us with 128 columns, 321 with 64, 293 with 32); the two columns
+// more that a segment reads cost 25 events less than their fuller last wave
+// gains (peak stage 512, 436, 444 us).  A row's peaks in a segment fit a byte.
+constexpr int kSegCols = 32;
 constexpr int kPpWarps = 4, kPpThreads = 32 * kPpWarps;
 constexpr int kLaneBins = 30;
 constexpr unsigned kAll = 0xffffffffu;
