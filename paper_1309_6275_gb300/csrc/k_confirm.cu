@@ -665,7 +665,8 @@ __device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P
     }
     const long long tol_bits = __double_as_longlong(P.tol);
     const bool single = total <= kCfCap;
-    const int jp0 = max(pk.j_d0 - P.pool, 0), jp1 = min(pk.j_d0 + P.pool + 1, G.n_d0);
+    const int pool = min(P.pool, G.n_d0);   // (any int32 is accepted)
+    const int jp0 = max(pk.j_d0 - pool, 0), jp1 = min(pk.j_d0 + pool + 1, G.n_d0);
     EdgePair E;
     E.init(G, rho, jp0, jp1);
     const float sk = G.sn32[pk.k_phi0], ck = G.cs32[pk.k_phi0];
