@@ -38,8 +38,8 @@
 // Bound by latency and issue (59% of slots; index loads and fixed latencies
 // lead the stalls): 1540 warp instructions per candidate, where scanning and
 // binning the whole pool (435 hits) with a frame per warp took 6800.  Stage on
-// GB300: 25 events of 2k-60k hits (1.25 M candidates) 11.7 -> 2.3 ms, 25 of 10k
-// hits (2.7 M) 16.7 -> 4.6, two of 50k (512 x 256 x 1024) 8.7 -> 1.6.
+// GB300: 25 events of 2k-60k hits (1.25 M candidates) 11.7 -> 2.1 ms, 25 of 10k
+// hits (2.7 M) 16.7 -> 4.2, two of 50k (512 x 256 x 1024) 8.7 -> 1.5.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -97,10 +97,14 @@ __device__ __forceinline__ int column_bins(const DevGeom &G, const ColumnCtx &C,
     return nv;
 }
 
+// circle3 and seed_frame are calls: inlined, their code and registers stand in
+// the loop that nearly every candidate leaves before (stage of 25 events of 10k
+// hits 4.65 ms, called 4.2).
+//
 // Circle through three points: centre = P1 + ((b_y |a|^2 - a_y |b|^2) / d,
 // (a_x |b|^2 - b_x |a|^2) / d) with a = P2 - P1, b = P3 - P1,
 // d = 2 (a_x b_y - a_y b_x); false when d == 0 (collinear).
-__device__ __forceinline__ bool circle3(double x1, double y1, double x2, double y2, double x3,
+static __device__ __noinline__ bool circle3(double x1, double y1, double x2, double y2, double x3,
                                         double y3, double &xc, double &yc, double &R)
 {
     const double ax = __dsub_rn(x2, x1), ay = __dsub_rn(y2, y1);
@@ -153,7 +157,7 @@ struct SeedFrame {
     float x1, y1, nx, ny, kap, B0, B1, B2;
 };
 
-__device__ __forceinline__ bool seed_frame(float x1, float y1, float x2, float y2, float x3,
+static __device__ __noinline__ bool seed_frame(float x1, float y1, float x2, float y2, float x3,
                                            float y3, SeedFrame &F)
 {
     const double ax = __dsub_rn((double)x2, (double)x1), ay = __dsub_rn((double)y2, (double)y1);
@@ -193,7 +197,9 @@ __device__ __forceinline__ bool seed_frame(float x1, float y1, float x2, float y
 }
 
 constexpr int kCfThreads = 128, kCfWarps = kCfThreads / 32;
-constexpr int kCfCap = 128;        // hits near the circle held per pass (more: further passes)
+// Hits near the circle held per pass (more: further passes).  128, 160 and 192,
+// 10k hits, pool 4: tol 0.01 cm 277, 276 and 285 us, 1.5 cm 1043, 947 and 950.
+constexpr int kCfCap = 160;
 constexpr int kCfChunk = 32;       // candidates of a warp's chunk, at most
 
 // A candidate's seeds and, once computed, its float32 seed frame with the
@@ -215,9 +221,9 @@ struct CfWarp {
     unsigned lbmin[16], ubmin[16];
     int ncont[16], cq[16], qs[16], qe[16];
     int2 rr[32];            // non-empty runs scanned: start less the positions before it, layer
-    int pool_p[kCfCap], pool_h[kCfCap];   // index position and event-local hit index
-    float pool_lo[kCfCap], pool_hi[kCfCap];   // bounds on the hit's float64 distance
-    unsigned char pool_l[kCfCap];
+    int pool_p[kCfCap + 1], pool_h[kCfCap + 1];   // index position and event-local hit index
+    float pool_lo[kCfCap + 1], pool_hi[kCfCap + 1];   // bounds on the hit's float64 distance
+    unsigned char pool_l[kCfCap + 1];
     double xc, yc, R;       // the float64 seed circle, once computed
     CfSeed seed[kCfChunk];
 };
@@ -252,6 +258,16 @@ struct Runs {
         if (len > 0)
             g_cfw[wid].rr[__popc(ne & ((1u << lane) - 1u))] = make_int2(start - excl, layer);
         __syncwarp();
+    }
+
+    // The place of index position p, which is in one of the runs (every lane).
+    __device__ __forceinline__ int place(int p, int lane) const
+    {
+        constexpr unsigned kAll = 0xffffffffu;
+        const unsigned ne = __ballot_sync(kAll, len > 0);
+        const int t = len > 0 ? p - g_cfw[wid].rr[__popc(ne & ((1u << lane) - 1u))].x : -1;
+        const unsigned m = __ballot_sync(kAll, len > 0 && t >= excl && t < excl + len);
+        return __shfl_sync(kAll, t, __ffs(m) - 1);
     }
 
     __device__ __forceinline__ bool at(int base, int lane, int &p, int &l) const
@@ -429,6 +445,22 @@ __device__ __forceinline__ void window_run(const int *__restrict__ offs, int cel
     len = o[b] - start;
 }
 
+// The run (window_run) of layer l's hits that can have a root in the bins
+// [j0, j1) of column (rho, phi0_k): the bins' edges, a hundredth of a bin and
+// 1e-4 cm beyond.
+__device__ __forceinline__ void bin_run(const DevGeom &G, const HitIndex &I, int e, int l, int part,
+                                        float rho, float phik, int j0, int j1, int &start, int &len)
+{
+    const float lo = fmaf((float)j0 - G.off_f - 0.01f, G.delta_f, -1e-4f);
+    const float hi = fmaf((float)j1 - G.off_f + 0.01f, G.delta_f, 1e-4f);
+    const float rmin = __uint_as_float(I.rmm[2 * (e * 16 + l)]);
+    const float rmax = __uint_as_float(I.rmm[2 * (e * 16 + l) + 1]);
+    bool full, empty;
+    float w0, w1;
+    layer_window(rho, phik, lo, hi, rmin, rmax, full, empty, w0, w1);
+    window_run(I.offs, (e * 16 + l) * kIdxAz, part, full, empty, w0, w1, start, len);
+}
+
 // Whether the root of a hit in column (rho, phi0) that grows through F = 0 is
 // between da and db (cm): F(d) = rho d^2 + 2 (1 + rho s) d + rho r^2 + 2 s of
 // the circle equation is linear in s and r^2, so its signs at the two ends
@@ -498,18 +530,8 @@ __device__ __forceinline__ void find_seeds(const DevGeom &G, const ConfirmDev &P
     {
         const int l = lane >> 1;
         int start = 0, len = 0;
-        if (l < P.n_layers) {
-            // the bin's edges, a hundredth of a bin and 1e-4 cm beyond
-            const float jo = (float)pk.j_d0 - G.off_f;
-            const float lo = fmaf(jo - 0.01f, G.delta_f, -1e-4f);
-            const float hi = fmaf(jo + 1.01f, G.delta_f, 1e-4f);
-            const float rmin = __uint_as_float(I.rmm[2 * (e * 16 + l)]);
-            const float rmax = __uint_as_float(I.rmm[2 * (e * 16 + l) + 1]);
-            bool full, empty;
-            float w0, w1;
-            layer_window(rho, phik, lo, hi, rmin, rmax, full, empty, w0, w1);
-            window_run(I.offs, (e * 16 + l) * kIdxAz, lane & 1, full, empty, w0, w1, start, len);
-        }
+        if (l < P.n_layers)
+            bin_run(G, I, e, l, lane & 1, rho, phik, pk.j_d0, pk.j_d0 + 1, start, len);
         R.set(start, len, l, wid, lane);
     }
     const float sk = G.sn32[pk.k_phi0], ck = G.cs32[pk.k_phi0];
@@ -593,8 +615,16 @@ __device__ __forceinline__ void make_frame(const HitIndex &I, CfSeed &C)
 // contender has no inlier, a single contender certainly below tol is the
 // inlier, and otherwise the float64 distances of the contenders decide (the
 // definition's seed circle is computed then, once per candidate).  More than
-// kCfCap hits go in passes of kCfCap, every contender by its float64
-// distance.
+// kCfCap hits go in passes of as many whole layers as fit, each scan going on
+// where the pass before it ended; of a layer with more hits than that, every
+// contender goes by its float64 distance.
+//
+// WIDE: the tolerance is of the size of the pool, so the circle's cells can
+// hold more hits than the pool's, and most pool hits are near it.  Each layer
+// then scans whichever cells hold fewer, the pool test comes first, and only
+// the pool's hits are kept.  10k hits, bins of 0.31 cm: pool 4, tol 1.5 and 100
+// cm 1.66 -> 0.95 and 80 -> 0.99 ms; pool 0 1.52 -> 0.47 and 80 -> 0.47.
+template <bool WIDE>
 __device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P,
                                            const HitIndex &I, const ht_peak pk, const CfSeed &C,
                                            float tol_lo, float tol_hi, int wid, int lane,
@@ -605,6 +635,8 @@ __device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P
     const float kInf = __int_as_float(0x7f800000);
     const int e = C.ev;
     const float rho = G.rho32[pk.i_rho], phik = G.phi32[pk.k_phi0];
+    const int pool = min(P.pool, G.n_d0);   // (any int32 is accepted)
+    const int jp0 = max(pk.j_d0 - pool, 0), jp1 = min(pk.j_d0 + pool + 1, G.n_d0);
     Runs R;
     {
         const int l = lane >> 1;
@@ -617,36 +649,61 @@ __device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P
             circle_window(C, phik, tol_hi, rmin, rmax, full, empty, w0, w1);
             window_run(I.offs, (e * 16 + l) * kIdxAz, lane & 1, full, empty, w0, w1, start, len);
         }
+        if (WIDE) {
+            int ps = 0, pl = 0;
+            if (l < P.n_layers) bin_run(G, I, e, l, lane & 1, rho, phik, jp0, jp1, ps, pl);
+            if (pl + __shfl_xor_sync(kAll, pl, 1) < len + __shfl_xor_sync(kAll, len, 1)) {
+                start = ps;
+                len = pl;
+            }
+        }
         R.set(start, len, l, wid, lane);
     }
     in_l = false;
     const SeedFrame F = C.F;
+    EdgePair E;   // the pool's edges (where most candidates end before: not yet)
+    float sk, ck;
+    auto pool_init = [&]() {
+        E.init(G, rho, jp0, jp1);
+        sk = G.sn32[pk.k_phi0];
+        ck = G.cs32[pk.k_phi0];
+    };
+    auto in_pool = [&](float x, float y) -> bool {
+        const int st = E.root(x, y, sk, ck);
+        return st == 2 ? exact_root(G, pk.i_rho, pk.k_phi0, x, y, jp0, jp1) : st == 1;
+    };
+    if (WIDE) pool_init();
     int total = 0;
-    // hits of rank [r0, r0 + kCfCap) near the circle, in layer order; returns
-    // their layers
-    auto scan = [&](int r0) {
+    // hits of rank [r0, r0 + kCfCap) near the circle (WIDE: and in the pool), in
+    // layer order, and the one behind them, the first at place t0 of the sequence;
+    // the first scan (r0 = 0) goes through all hits, sets total and returns their
+    // layers
+    auto scan = [&](int r0, int t0) {
         unsigned lm = 0u;
-        int rank = 0;
-        for (int base = 0; base < R.n; base += 32) {
+        int rank = r0;
+        for (int base = t0; base < R.n && (r0 == 0 || rank <= r0 + kCfCap); base += 32) {
             int p = 0, l = 0;
             float lo = kInf, hi = kInf;
             if (R.at(base, lane, p, l)) {
-                const float wx = I.x[p] - F.x1, wy = I.y[p] - F.y1;
-                const float w2 = fmaf(wx, wx, wy * wy);
-                const float wn = fmaf(wx, F.nx, wy * F.ny);
-                const float num = fmaf(F.kap, w2, -2.0f * wn);
-                const float qx = fmaf(F.kap, wx, -F.nx), qy = fmaf(F.kap, wy, -F.ny);
-                const float d = fabsf(num / (sqrtf(fmaf(qx, qx, qy * qy)) + 1.0f));
-                const float er = fmaf(F.B2, w2, fmaf(F.B1, fabsf(wx) + fabsf(wy), F.B0));
-                const float dl = __fsub_rd(d, er);
-                lo = dl > 0.0f ? dl : 0.0f;   // +0 (the bits order as the values)
-                hi = __fadd_ru(d, er);
+                const float x = I.x[p], y = I.y[p];
+                if (!WIDE || in_pool(x, y)) {
+                    const float wx = x - F.x1, wy = y - F.y1;
+                    const float w2 = fmaf(wx, wx, wy * wy);
+                    const float wn = fmaf(wx, F.nx, wy * F.ny);
+                    const float num = fmaf(F.kap, w2, -2.0f * wn);
+                    const float qx = fmaf(F.kap, wx, -F.nx), qy = fmaf(F.kap, wy, -F.ny);
+                    const float d = fabsf(num / (sqrtf(fmaf(qx, qx, qy * qy)) + 1.0f));
+                    const float er = fmaf(F.B2, w2, fmaf(F.B1, fabsf(wx) + fabsf(wy), F.B0));
+                    const float dl = __fsub_rd(d, er);
+                    lo = dl > 0.0f ? dl : 0.0f;   // +0 (the bits order as the values)
+                    hi = __fadd_ru(d, er);
+                }
             }
             const bool near = lo < tol_hi;
             const unsigned bal = __ballot_sync(kAll, near);
             if (!bal) continue;
             const int r = rank + __popc(bal & ((1u << lane) - 1u)) - r0;
-            if (near && r >= 0 && r < kCfCap) {
+            if (near && r <= kCfCap) {
                 W.pool_p[r] = p;
                 W.pool_l[r] = (unsigned char)l;
                 W.pool_lo[r] = lo;
@@ -655,31 +712,43 @@ __device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P
             lm |= __reduce_or_sync(kAll, near ? 1u << l : 0u);
             rank += __popc(bal);
         }
-        total = rank;
+        if (r0 == 0) total = rank;
         return lm;
     };
-    if (__popc(scan(0)) < P.min_layers) return 0;
+    if (__popc(scan(0, 0)) < P.min_layers) return 0;
     if (lane < 16) {
         W.best_h[lane] = -1;
         W.best_d[lane] = 0.0;
     }
     const long long tol_bits = __double_as_longlong(P.tol);
     const bool single = total <= kCfCap;
-    const int pool = min(P.pool, G.n_d0);   // (any int32 is accepted)
-    const int jp0 = max(pk.j_d0 - pool, 0), jp1 = min(pk.j_d0 + pool + 1, G.n_d0);
-    EdgePair E;
-    E.init(G, rho, jp0, jp1);
-    const float sk = G.sn32[pk.k_phi0], ck = G.cs32[pk.k_phi0];
+    if (!WIDE) pool_init();
     bool exact = false;
-    for (int r0 = 0; r0 < total; r0 += kCfCap) {
-        if (r0 > 0) scan(r0);
+    unsigned split = 0u;   // layers that one pass does not hold
+    for (int r0 = 0, t0 = 0, next = 0; r0 < total; r0 = next) {
+        if (r0 > 0) scan(r0, t0);
         int nq = min(total - r0, kCfCap);
+        __syncwarp();
+        if (r0 + nq < total) {   // the layer that the pass ends in waits for the next one
+            const int first = W.pool_l[0], last = W.pool_l[nq - 1];
+            if (first != last) {
+                int n = 0;
+                for (int q0 = 0; q0 < nq; q0 += 32)
+                    n += __popc(__ballot_sync(kAll, q0 + lane < nq && W.pool_l[q0 + lane] != last));
+                nq = n;
+            } else {
+                split |= 1u << last;
+            }
+            t0 = R.place(W.pool_p[nq], lane);
+        }
+        next = r0 + nq;
         __syncwarp();
         // the pool's hits among them, kept in order
         int kept = 0;
         for (int q0 = 0; q0 < nq; q0 += 32) {
             const int q = q0 + lane;
-            int p = 0, st = 0;
+            int p = 0;
+            bool in = false;
             unsigned char l = 0;
             float lo = 0.0f, hi = 0.0f;
             if (q < nq) {
@@ -687,12 +756,10 @@ __device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P
                 l = W.pool_l[q];
                 lo = W.pool_lo[q];
                 hi = W.pool_hi[q];
-                const float x = I.x[p], y = I.y[p];
-                st = E.root(x, y, sk, ck);
-                if (st == 2) st = exact_root(G, pk.i_rho, pk.k_phi0, x, y, jp0, jp1) ? 1 : 0;
+                in = WIDE || in_pool(I.x[p], I.y[p]);
             }
-            const unsigned bal = __ballot_sync(kAll, st == 1);
-            if (st == 1) {
+            const unsigned bal = __ballot_sync(kAll, in);
+            if (in) {
                 const int r = kept + __popc(bal & ((1u << lane) - 1u));
                 W.pool_p[r] = p;   // r <= q: read before
                 W.pool_l[r] = l;
@@ -751,7 +818,7 @@ __device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P
         bool need = false;
         if (lane < P.n_layers) {
             const int nc = W.ncont[lane];
-            if (single && nc == 1 && W.pool_hi[W.cq[lane]] < tol_lo) {
+            if (!((split >> lane) & 1u) && nc == 1 && W.pool_hi[W.cq[lane]] < tol_lo) {
                 W.best_h[lane] = W.pool_h[W.cq[lane]];   // certainly the inlier
                 W.best_d[lane] = 0.0;                     // (below tol)
             } else {
@@ -816,6 +883,7 @@ __device__ __forceinline__ int confirm_one(const DevGeom &G, const ConfirmDev &P
 // must be zero, k_assoc_final_batch decodes it.  score per slot (0 = not
 // confirmed); inl (may be null): 16 inlier hits per slot, -1 none.  I: the
 // batch's hit index (k_hitindex.cu).
+template <bool WIDE>
 __global__ void __launch_bounds__(kCfThreads, 8)
 k_confirm(DevGeom G, ConfirmDev P, HitIndex I, const int *__restrict__ off,
           const int *__restrict__ d_nev, const ht_peak *__restrict__ peaks, int cap,
@@ -850,7 +918,8 @@ k_confirm(DevGeom G, ConfirmDev P, HitIndex I, const int *__restrict__ off,
             const size_t slot = (size_t)C.ev * cap + m;
             bool in_l = false;
             int sc = 0;
-            if (C.pa >= 0) sc = confirm_one(G, P, I, peaks[slot], C, tol_lo, tol_hi, wid, lane, in_l);
+            if (C.pa >= 0)
+                sc = confirm_one<WIDE>(G, P, I, peaks[slot], C, tol_lo, tol_hi, wid, lane, in_l);
             if (lane == 0) score[slot] = sc;
             if (inl && lane < 16) inl[slot * 16 + lane] = sc > 0 && in_l ? W.best_h[lane] : -1;
             if (sc > 0 && in_l)
@@ -951,9 +1020,15 @@ cudaError_t launch_confirm_batch(const DevGeom &G, const ConfirmDev &P, const in
     if (e == cudaSuccess) e = cudaMemsetAsync(w.gbest, 0, (size_t)max_hits * 8, st);
     if (e != cudaSuccess) return e;
     k_cand_prefix<<<1, 1024, 0, st>>>(counts, d_nev, cap, w.cpre);
+    // Half the pool's width: below it the circle's cells are the fewer.  10k hits,
+    // narrow and wide kernel: pool 0 (0.31 cm) tol 0.1 364 and 397 us, 0.4 485 and
+    // 452; pool 4 (2.8 cm) 0.8 629 and 648, 1.5 1006 and 897; pool 20 (12.8 cm)
+    // 3 1461 and 1509, 6 2260 and 2208.
+    const bool wide = P.tol > 0.5 * (2.0 * (double)P.pool + 1.0) * G.delta;
+    const auto kernel = wide ? k_confirm<true> : k_confirm<false>;
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_confirm, kCfThreads, 0);
-    k_confirm<<<sms * (occ > 0 ? occ : 1), kCfThreads, 0, st>>>(
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kCfThreads, 0);
+    kernel<<<sms * (occ > 0 ? occ : 1), kCfThreads, 0, st>>>(
         G, P, idx, off, d_nev, peaks, cap, w.cpre, score, inl, w.gbest, w.head);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
