@@ -76,7 +76,10 @@
 // k_hitindex.cu: a column scans, per layer, the run of azimuth cells whose
 // hits can reach it, and a warp's hits have about the same curve, so its
 // lanes walk about the same number of bins.  The single-event call has no
-// scratch for an index and scans the event in the caller's order.
+// scratch for an index: each tile goes through the event in the caller's
+// order, and a warp's hits that can vote in it wait in shared memory until they
+// fill the warp's lanes.  One event of 50k hits (512 x 256 x 1024): 20.6 -> 15.4
+// ms; 20k hits (256 x 128 x 512): 1.19 -> 0.93.
 #include <cooperative_groups.h>
 
 #include "tiles.cuh"
@@ -87,7 +90,12 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr int kVrCluster = 8;         // columns whose counts one event's tiles exchange
-constexpr int kVrThreads = 320, kVrWarps = kVrThreads / 32;
+// Threads of a tile: 320, three tiles per SM; cell by cell 512, two.  A single
+// event's tiles of at most two words of rows take 256, four per SM, where three
+// per SM are not one wave: 512 columns, 20k hits, 1 row 210 -> 155 us, 8 rows
+// 376 -> 272, 48 rows 556 -> 469; where shared memory allows only three anyway
+// (512 bins) they would lose: 646 -> 723.
+constexpr int kVrThreads = 320, kClThreads = 512, kVrNarrow = 256;
 constexpr int kRes = 10;              // layers resident in a tile (more: a second round)
 constexpr int kVrRedo = 96;           // redo slots per warp
 constexpr int kVrPad = 4;             // words between rows of words: spreads one bin's words over banks
@@ -96,7 +104,7 @@ constexpr float kEdgeSlope = 0.5f;    // and up to which a lane takes a bin
 constexpr float kWalkEps = 8.0f;      // rows of uncertainty at a crossing
 constexpr float kEdgeEps = 0.25f;     // (an edge lane's at most one row)
 constexpr size_t kVrBitmap = 43 * 1024;
-constexpr int kClThreads = 512;       // cell-by-cell tiles: two CTAs of 16 warps per SM
+constexpr int kGather = 64;           // hits a warp of the single-event call looks at per step, at most
 constexpr int kClMaxHits = 4096;      // hits of a layer in a column's window, at most
 constexpr int kCellMin = 160;         // and at least, to go cell by cell
 constexpr int kClTab = 2048;          // table entries over a layer's s
@@ -132,10 +140,10 @@ struct VrSmem {
     uint8_t *jmask;           // HIT: [ND] d0 blocks of bins j - 1, j, j + 1
 };
 
-__host__ __device__ constexpr size_t vr_smem(int nwb, int nd, bool hit, bool cells)
+__host__ __device__ constexpr size_t vr_smem(int nwb, int nd, bool hit, bool cells, int threads)
 {
     const size_t rows = (size_t)32 * nwb;
-    const size_t warps = cells ? kClThreads / 32 : kVrWarps;
+    const size_t warps = threads / 32;
     size_t b = warps * 32 * (sizeof(VrSlot) + 16) + warps * kVrRedo * 8 +
                (size_t)kRes * nwb * (nd + kVrPad) * 4 + rows * 4;
     b = (b + 15) / 16 * 16;
@@ -143,7 +151,7 @@ __host__ __device__ constexpr size_t vr_smem(int nwb, int nd, bool hit, bool cel
     if (cells) b += (size_t)kClTab * 2;
     return b;
 }
-static_assert((kClThreads / 32) * 32 * (sizeof(VrSlot) + 16) >= (kClMaxHits + 1) * sizeof(float),
+static_assert(kClThreads * (sizeof(VrSlot) + 16) >= (kClMaxHits + 1) * sizeof(float),
               "a layer's hits fit the slots' space");
 
 // Words of rows per band: the largest power of two whose bitmap fits, at
@@ -158,10 +166,10 @@ __host__ __device__ inline int vr_nwb(int n_rho, int nd)
     return nwb;
 }
 
-template <int NWB, bool HIT, bool CELLS>
+template <int NWB, bool HIT, bool CELLS, int kThr>
 __device__ __forceinline__ VrSmem vr_carve(unsigned char *p, int nd)
 {
-    constexpr size_t warps = CELLS ? kClThreads / 32 : kVrWarps;
+    constexpr size_t warps = kThr / 32;
     VrSmem S{};
     // 16-byte items first: the slots, then the rest
     S.slot = reinterpret_cast<VrSlot *>(p);
@@ -325,28 +333,30 @@ __device__ __forceinline__ float row_coord(const DevGeom &G, float s, float c2, 
 // One tile of one event: votes, then the layer counts.
 // PLANES: out is the event's bit planes (see k_peak_planes.cu); otherwise the
 // accumulator of OutT counts.
-template <int NWB, bool HIT, bool PLANES, bool CELLS, typename OutT>
+template <int NWB, bool HIT, bool PLANES, bool CELLS, int kThr, typename OutT>
 __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, int e,
                                         const unsigned long long *__restrict__ hmask,
                                         void *__restrict__ out,
                                         unsigned long long *__restrict__ stats, int k, int band)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int kThr = CELLS ? kClThreads : kVrThreads, kWarps = kThr / 32;
+    constexpr int kWarps = kThr / 32;
     // runs of positions [rs, re) (index: layer << 2 | part << 1 | side), chunks
     // before each, rows first | last << 16 they vote in
     __shared__ int s_rs[64], s_re[64], s_cp[65], s_row[64];
-    __shared__ int s_next, s_more, s_full;
+    __shared__ int s_next, s_more, s_full, s_any;
     __shared__ int s_nredo[kWarps];
     __shared__ unsigned long long s_stats[2];
     __shared__ int s_ws[32], s_we[32];   // CELLS: window runs (layer << 1 | part)
     __shared__ int s_bad, s_val[16];   // CELLS: a cell layer's rows first | last << 16, else -1
+    // single event: the warps' hits that can vote here and wait for a full warp
+    __shared__ int s_wait[PLANES ? 1 : kWarps][32 + kGather];
     constexpr unsigned kAll = 0xffffffffu;
     constexpr int kBand = 32 * NWB;
     constexpr int IPW = 32 / NWB;                  // hits per walk step
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ND = G.n_d0, NDp = ND + kVrPad, NW = (G.n_rho + 31) / 32;
-    const VrSmem S = vr_carve<NWB, HIT, CELLS>(smem, ND);
+    const VrSmem S = vr_carve<NWB, HIT, CELLS, kThr>(smem, ND);
     const int i0 = band * kBand, nrow = min(kBand, G.n_rho - i0);
     const float tc = 0.5f * (float)(G.n_rho - 1) - (float)i0;   // row of rho = 0
 
@@ -416,7 +426,9 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             }
             s_ws[lane] = start;
             s_we[lane] = end;
+            const bool any = __any_sync(kAll, end > start);
             if (lane == 0) {
+                s_any = any;
                 s_cp[0] = 0;
                 s_next = 0;
             }
@@ -426,9 +438,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
         if (threadIdx.x < kWarps) s_nredo[threadIdx.x] = 0;
         if (CELLS && threadIdx.x < 16) s_val[threadIdx.x] = -1;
         __syncthreads();
-        bool none = true;
-        for (int q = 0; q < 32; ++q) none = none && s_we[q] <= s_ws[q];
-        if (l0 > 0 && none) continue;   // uniform
+        if (l0 > 0 && !s_any) continue;   // uniform
         {
             uint4 *z4 = reinterpret_cast<uint4 *>(S.bm);
             const int n4 = kRes * NWB * NDp / 4;   // NDp is a multiple of 2, kRes NWB too
@@ -611,7 +621,13 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             }
             __syncthreads();
         }
-        // ---- chunks of 32 hits of the runs; a cell layer's runs twice, below and
+        // (single event: of a size that gives every warp as many chunks)
+        int step = 32;
+        if (!PLANES) {
+            const int rounds = max((H.n + kGather * kWarps - 1) / (kGather * kWarps), 1);
+            step = max((H.n + rounds * kWarps - 1) / (rounds * kWarps), 1);
+        }
+        // ---- chunks of step hits of the runs; a cell layer's runs twice, below and
         // above its rows
         if (warp == 0) {
             int n[2];
@@ -628,7 +644,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                 s_rs[q] = s_ws[lane];
                 s_re[q] = use ? s_we[lane] : s_ws[lane];
                 s_row[q] = r0 | (max(r1, 0) << 16);
-                n[side] = (s_re[q] - s_rs[q] + 31) >> 5;
+                n[side] = (s_re[q] - s_rs[q] + step - 1) / step;
             }
             int incl = n[0] + n[1];
 #pragma unroll
@@ -641,23 +657,72 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
         }
         __syncthreads();
         const int nchunk = s_cp[64];
-
-        for (;;) {
+        auto pop = [&]() -> int {
             int ch = 0;
             if (lane == 0) ch = atomicAdd(&s_next, 1);
-            ch = __shfl_sync(kAll, ch, 0);
-            if (ch >= nchunk) break;
-            int run = 0;
-            {
+            return __shfl_sync(kAll, ch, 0);
+        };
+        int nwait = 0;   // single event: hits in s_wait
+
+        for (;;) {
+            int run = 0, p = 0;
+            bool live = false;
+            if constexpr (PLANES) {
+                const int ch = pop();
+                if (ch >= nchunk) break;
                 int hi = 63;   // the last run with s_cp[run] <= ch
                 while (run < hi) {
                     const int mid = (run + hi + 1) >> 1;
                     if (s_cp[mid] <= ch) run = mid;
                     else hi = mid - 1;
                 }
+                p = s_rs[run] + (ch - s_cp[run]) * 32 + lane;
+                live = p < s_re[run];
+            } else {
+                // The event's hits in the caller's order: those of this round's layers
+                // that can vote in the tile's rows (the tests below, on the plain s and
+                // c that the filters' margins are for) wait until they fill the warp.
+                const float sk = G.sn32[k], ck = G.cs32[k];
+                while (nwait < 32) {
+                    const int ch = pop();
+                    if (ch >= nchunk) break;
+                    bool keep[kGather / 32];
+#pragma unroll
+                    for (int u = 0; u < kGather / 32; ++u) {
+                        const int q = ch * step + 32 * u + lane;
+                        const bool in = 32 * u + lane < step && q < H.n;
+                        const int l = in ? H.l[q] & 15 : 0;
+                        const float xf = in ? H.x[q] : 0.0f, yf = in ? H.y[q] : 0.0f;
+                        if (l >= l1) s_more = 1;
+                        const float c = fmaf(xf, ck, yf * sk), s = fmaf(xf, sk, -(yf * ck));
+                        const float R1 = fabsf(xf) + fabsf(yf);
+                        keep[u] = in && l >= l0 && l < l1 &&
+                                  !(c < hit_cos_window(G, fmaf(xf, xf, yf * yf))) &&
+                                  !(c < -(kSafe * 3.0f * kEps) * R1);
+                        if (nrow < G.n_rho && keep[u] && c > 1.0f) {   // more than one band
+                            float gmin, gmax;
+                            rho_range(G, s, c, 4e-7f * R1, gmin, gmax);
+                            keep[u] = floorf(fmaf(gmin, G.inv_drho_f, tc - 0.5f)) <= (float)(nrow - 1) &&
+                                      ceilf(fmaf(gmax, G.inv_drho_f, tc + 0.5f)) >= 0.0f;
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kGather / 32; ++u) {
+                        const unsigned m = __ballot_sync(kAll, keep[u]);
+                        if (keep[u])
+                            s_wait[warp][nwait + __popc(m & ((1u << lane) - 1u))] =
+                                ch * step + 32 * u + lane;
+                        nwait += __popc(m);
+                    }
+                }
+                if (nwait == 0) break;
+                __syncwarp();
+                const int take = min(nwait, 32);
+                nwait -= take;
+                live = lane < take;
+                if (live) p = s_wait[warp][nwait + lane];
+                __syncwarp();   // the places are free again
             }
-            const int p = s_rs[run] + (ch - s_cp[run]) * 32 + lane;
-            bool live = p < s_re[run];
             // ---- one hit per lane: its kind and its constants
             enum { kWalk, kEdge8, kEdge16, kEdge32, kEdge64, kRow, kKinds, kNone = kKinds };
             int kind = kNone;
@@ -667,23 +732,14 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             float4 ma = make_float4(0.f, 0.f, 0.f, 0.f), mb = ma;
             unsigned long long hm = 0ull;
             if (live) {
-                int l = run >> 2;
-                if (!H.offs) {
-                    l = H.l[p] & 15;
-                    if (l < l0 || l >= l1) {
-                        live = false;
-                        if (l >= l1) s_more = 1;
-                    }
-                }
+                const int l = PLANES ? run >> 2 : H.l[p] & 15;
                 const float sk = G.sn32[k], ck = G.cs32[k], sl = G.snlo[k], cl = G.cslo[k];
                 const float xf = H.x[p], yf = H.y[p];
                 const float c = dot2(xf, ck, cl, yf, sk, sl);
                 const float s = dot2(xf, sk, sl, -yf, ck, cl);
                 const float R1 = fabsf(xf) + fabsf(yf);
-                const float r2 = fmaf(xf, xf, yf * yf);
                 const float Ec = (kSafe * 3.0f * kEps) * R1;
                 const float eR = 4e-7f * R1;   // what the shared filters take for s and c
-                if (!H.offs && c < hit_cos_window(G, r2)) live = false;
                 if (c < -Ec) live = false;
                 float hwlo = G.d0lo_f, hwhi = G.d0hi_f;
                 int jhi = ND;   // the highest bin of interest, plus one
@@ -938,11 +994,17 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
 
             // ---- row: lane = row of the window; a lane's bit and the step of its word
             // are the same for all its rows
+            // (a band of one word: as many hits per step as their rows fit the lanes;
+            // 8 rows, 20k hits: 564 -> 376 us)
+            const int lgr = NWB > 1 ? 5 : 32 - __clz(nrow - 1);   // nrow = 1: 0
 #pragma unroll 1
-            for (int q = first[kRow]; q < first[kKinds]; ++q) {
+            for (int q0 = first[kRow]; q0 < first[kKinds]; q0 += 32 >> lgr) {
+                const int q = NWB > 1 ? q0 : q0 + (lane >> lgr);
+                if (NWB == 1 && q >= first[kKinds]) continue;
                 const float4 a = slot[q].a, b = slot[q].b;
                 const int rend = __float_as_int(b.y) >> 16;
-                int row = (__float_as_int(b.y) & 0xffff) + lane;
+                const int sub = NWB > 1 ? lane : lane & ((1 << lgr) - 1);
+                int row = (__float_as_int(b.y) & 0xffff) + sub;
                 const uint32_t bit = 1u << (row & 31);
                 uint32_t *wp = S.bm + (__float_as_int(b.z) & 0xffff) + (row >> 5) * NDp;
                 unsigned long long hs = 0ull;
@@ -973,6 +1035,10 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                         push(__float_as_int(b.w), rw, __float_as_int(b.z) >> 16);
                     }
                 };
+                if (NWB == 1) {
+                    one(row, wp);
+                    continue;
+                }
 #pragma unroll 1
                 for (int left = rend - (row - lane); left >= 0; left -= 64) {   // uniform
                     one(row, wp);
@@ -998,7 +1064,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                     slot[q].b = make_float4(it.E1, it.E2, it.Qa, it.Qb);
                     const bool sure = c > (kSafe * 3.0f * kEps) * R1;   // sign of c proven
                     const bool nb = needs_b(G, rt, s, c, 4e-7f * R1);
-                    imeta[q] = make_int4((int)rest, (H.offs ? run >> 2 : H.l[p] & 15) |
+                    imeta[q] = make_int4((int)rest, (PLANES ? run >> 2 : H.l[p] & 15) |
                                                         (sure ? 32 : 0) | (nb ? 64 : 0), p, 0);
                     if (HIT) shm[q] = hm;
                 }
@@ -1180,7 +1246,7 @@ k_vote_rows_batch(DevGeom G, HitSource H, const int *__restrict__ off,
         const int item = s_item;
         if (item >= total) break;
         const int e = order[first + item / nt], t = item % nt;
-        vr_tile<NWB, HIT, true, CELLS, uint16_t>(G, H, e, HIT ? masks + off[e] : nullptr,
+        vr_tile<NWB, HIT, true, CELLS, CELLS ? kClThreads : kVrThreads, uint16_t>(G, H, e, HIT ? masks + off[e] : nullptr,
                                                  out + (size_t)e * out_stride,
                                                  stats ? stats + 2 * e : nullptr, t % G.n_phi0,
                                                  t / G.n_phi0);
@@ -1189,12 +1255,12 @@ k_vote_rows_batch(DevGeom G, HitSource H, const int *__restrict__ off,
 
 // One event (hits in the caller's order), one CTA per tile, clusters of
 // neighbouring columns (n_phi0 is a multiple of 8).
-template <int NWB, typename OutT>
-__global__ void __cluster_dims__(kVrCluster, 1, 1) __launch_bounds__(kVrThreads, 3)
+template <int NWB, int kThr, typename OutT>
+__global__ void __cluster_dims__(kVrCluster, 1, 1) __launch_bounds__(kThr, kThr == kVrNarrow ? 4 : 3)
 k_vote_rows(DevGeom G, HitSource H, OutT *__restrict__ acc,
             unsigned long long *__restrict__ stats)
 {
-    vr_tile<NWB, false, false, false, OutT>(G, H, 0, nullptr, acc, stats, blockIdx.x, blockIdx.y);
+    vr_tile<NWB, false, false, false, kThr, OutT>(G, H, 0, nullptr, acc, stats, blockIdx.x, blockIdx.y);
 }
 
 }  // namespace
@@ -1211,20 +1277,25 @@ cudaError_t launch_vote_layers(const DevGeom &G, const float *x, const float *y,
     const HitSource H{x, y, nullptr, layer, nullptr, nullptr, n, nullptr};
     const int nwb = vr_nwb(G.n_rho, G.n_d0);
     const dim3 grid(G.n_phi0, (G.n_rho + 32 * nwb - 1) / (32 * nwb));
-    const size_t sm = vr_smem(nwb, G.n_d0, false, false);
-#define HT_VR(N)                                                                              \
+    const long long tiles = (long long)grid.x * grid.y, sms = device_sms();
+    const bool narrow = nwb <= 2 && tiles > 3 * sms &&
+                        vr_smem(nwb, G.n_d0, false, false, kVrNarrow) <= 50 * 1024;
+    const size_t sm = vr_smem(nwb, G.n_d0, false, false, narrow ? kVrNarrow : kVrThreads);
+#define HT_VR(N, THR)                                                                         \
     do {                                                                                      \
         if (G.count_bits == 16)                                                               \
-            k_vote_rows<N, uint16_t><<<grid, kVrThreads, sm, st>>>(                           \
+            k_vote_rows<N, THR, uint16_t><<<grid, THR, sm, st>>>(                             \
                 G, H, reinterpret_cast<uint16_t *>(acc), stats);                              \
         else                                                                                  \
-            k_vote_rows<N, int32_t><<<grid, kVrThreads, sm, st>>>(                            \
+            k_vote_rows<N, THR, int32_t><<<grid, THR, sm, st>>>(                              \
                 G, H, reinterpret_cast<int32_t *>(acc), stats);                               \
     } while (0)
-    if (nwb == 8) HT_VR(8);
-    else if (nwb == 4) HT_VR(4);
-    else if (nwb == 2) HT_VR(2);
-    else HT_VR(1);
+    if (nwb == 8) HT_VR(8, kVrThreads);
+    else if (nwb == 4) HT_VR(4, kVrThreads);
+    else if (nwb == 2 && narrow) HT_VR(2, kVrNarrow);
+    else if (nwb == 2) HT_VR(2, kVrThreads);
+    else if (narrow) HT_VR(1, kVrNarrow);
+    else HT_VR(1, kVrThreads);
 #undef HT_VR
     return cudaGetLastError();
 }
@@ -1237,8 +1308,8 @@ void run_vote_batch(const DevGeom &G, const HitSource &H, const int *off, const 
                     unsigned long long *stats, int *head, int sms,
                     const unsigned long long *hit_masks, cudaStream_t st)
 {
-    const size_t sm = vr_smem(NWB, G.n_d0, HIT, CELLS);
-    const int threads = CELLS ? kClThreads : kVrThreads;
+    constexpr int threads = CELLS ? kClThreads : kVrThreads;
+    const size_t sm = vr_smem(NWB, G.n_d0, HIT, CELLS, threads);
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_vote_rows_batch<NWB, HIT, CELLS>, threads,
                                                   sm);
@@ -1293,11 +1364,19 @@ cudaError_t launch_vote_batch_layers(const DevGeom &G, const HitIndex &I, const 
 cudaError_t prepare_layer_vote_kernels(int max_smem)
 {
 #define HT_VRP(N)                                                                             \
-    (const void *)k_vote_rows<N, uint16_t>, (const void *)k_vote_rows<N, int32_t>,            \
+    (const void *)k_vote_rows<N, kVrThreads, uint16_t>,                                       \
+        (const void *)k_vote_rows<N, kVrThreads, int32_t>,                                    \
         (const void *)k_vote_rows_batch<N, false, false>,                                     \
         (const void *)k_vote_rows_batch<N, true, false>,                                      \
         (const void *)k_vote_rows_batch<N, false, true>
-    const void *fns[] = {HT_VRP(8), HT_VRP(4), HT_VRP(2), HT_VRP(1)};
+    const void *fns[] = {HT_VRP(8),
+                         HT_VRP(4),
+                         HT_VRP(2),
+                         HT_VRP(1),
+                         (const void *)k_vote_rows<2, kVrNarrow, uint16_t>,
+                         (const void *)k_vote_rows<2, kVrNarrow, int32_t>,
+                         (const void *)k_vote_rows<1, kVrNarrow, uint16_t>,
+                         (const void *)k_vote_rows<1, kVrNarrow, int32_t>};
 #undef HT_VRP
     return allow_smem(fns, (int)(sizeof fns / sizeof fns[0]), max_smem);
 }
