@@ -97,6 +97,8 @@ constexpr int kVrCluster = 8;         // columns whose counts one event's tiles 
 // (512 bins) they would lose: 646 -> 723.
 constexpr int kVrThreads = 320, kClThreads = 512, kVrNarrow = 256;
 constexpr int kRes = 10;              // layers resident in a tile (more: a second round)
+constexpr int kKept = 16 - kRes;      // its first free place: the first round's counts, four bits
+static_assert(kKept + 4 <= kRes, "the second round's layers leave room for the counts");
 constexpr int kVrRedo = 96;           // redo slots per warp
 constexpr int kVrPad = 4;             // words between rows of words: spreads one bin's words over banks
 constexpr float kWalkSlope = 1.0f / 64.0f;   // bins per row up to which a curve is walked
@@ -387,6 +389,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
     int my_cast = 0;   // votes (cell rows subtract what lies below the axis)
     int my_fb = 0;
 
+#pragma unroll 1
     for (int l0 = 0; l0 < 16; l0 += kRes) {
         const int l1 = min(l0 + kRes, 16);
         // ---- the runs of positions that hold the column's hits
@@ -441,7 +444,7 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
         if (l0 > 0 && !s_any) continue;   // uniform
         {
             uint4 *z4 = reinterpret_cast<uint4 *>(S.bm);
-            const int n4 = kRes * NWB * NDp / 4;   // NDp is a multiple of 2, kRes NWB too
+            const int n4 = (!PLANES && l0 > 0 ? kKept : kRes) * NWB * NDp / 4;   // NDp is a multiple of 2, kRes NWB too
             for (int t = threadIdx.x; t < n4; t += kThr) z4[t] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();
@@ -1135,13 +1138,29 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
             const int w = t / ND, j = t - w * ND, wg = band * NWB + w;
             if (wg >= NW) continue;
             uint32_t n0 = 0, n1 = 0, n2 = 0, n3 = 0, n4 = 0;
+            if (!PLANES && l0 > 0) {   // on from the first round's counts
+                n0 = S.bm[(kKept * NWB + w) * NDp + j];
+                n1 = S.bm[((kKept + 1) * NWB + w) * NDp + j];
+                n2 = S.bm[((kKept + 2) * NWB + w) * NDp + j];
+                n3 = S.bm[((kKept + 3) * NWB + w) * NDp + j];
 #pragma unroll
-            for (int l = 0; l < kRes; ++l) {
-                uint32_t x = S.bm[(l * NWB + w) * NDp + j], y;
-                y = n0 & x; n0 ^= x; x = y;
-                y = n1 & x; n1 ^= x; x = y;
-                y = n2 & x; n2 ^= x; x = y;
-                n3 ^= x;
+                for (int l = 0; l < kKept; ++l) {
+                    uint32_t x = S.bm[(l * NWB + w) * NDp + j], y;
+                    y = n0 & x; n0 ^= x; x = y;
+                    y = n1 & x; n1 ^= x; x = y;
+                    y = n2 & x; n2 ^= x; x = y;
+                    y = n3 & x; n3 ^= x; n4 |= y;
+                }
+                S.bm[(4 * NWB + w) * NDp + j] = n4;
+            } else {
+#pragma unroll
+                for (int l = 0; l < kRes; ++l) {
+                    uint32_t x = S.bm[(l * NWB + w) * NDp + j], y;
+                    y = n0 & x; n0 ^= x; x = y;
+                    y = n1 & x; n1 ^= x; x = y;
+                    y = n2 & x; n2 ^= x; x = y;
+                    n3 ^= x;
+                }
             }
             if (PLANES) {
                 uint32_t *o = reinterpret_cast<uint32_t *>(out) + ((size_t)k * kPlanes * NW + wg) * ND + j;
@@ -1159,13 +1178,18 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                 o[3 * ps] = n3;
                 if (s_full) o[4 * ps] = n4;   // read only where 16 layers hold hits
             } else {   // this thread was the only reader of (l, w, j)
-                S.bm[w * NDp + j] = n0;
-                S.bm[(NWB + w) * NDp + j] = n1;
-                S.bm[(2 * NWB + w) * NDp + j] = n2;
-                S.bm[(3 * NWB + w) * NDp + j] = n3;
+                uint32_t *o = S.bm + w * NDp + j;
+                if (l0 == 0 && s_more) o += kKept * NWB * NDp;   // kept for the second round
+                o[0] = n0;
+                o[NWB * NDp] = n1;
+                o[2 * NWB * NDp] = n2;
+                o[3 * NWB * NDp] = n3;
             }
         }
         if constexpr (!PLANES) {
+            // hits on layers of the second round (uniform over the cluster: every tile
+            // looks at all hits): their votes first, then one write of the counts
+            if (l0 == 0 && s_more) continue;
             // The accumulator is phi0-fastest: the cluster's eight columns exchange
             // their bit planes through distributed shared memory, and each tile
             // writes an eighth of the (word, bin)s, eight counts of a row at a time
@@ -1194,13 +1218,17 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                                       (((pl[v][2] >> r) & 1u) << 2) | (((pl[v][3] >> r) & 1u) << 3));
                     constexpr int NV = kVrCluster * (int)sizeof(OutT) / 16;
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        uint4 x = reinterpret_cast<const uint4 *>(o)[v];
-                        if (l0 > 0) {   // counts are at most 16: no carry between halves
-                            const uint4 y = reinterpret_cast<const uint4 *>(d)[v];
-                            x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
-                        }
-                        reinterpret_cast<uint4 *>(d)[v] = x;
+                    for (int v = 0; v < NV; ++v)
+                        reinterpret_cast<uint4 *>(d)[v] = reinterpret_cast<const uint4 *>(o)[v];
+                }
+                if (l0 > 0) {   // cells of all 16 layers (the other bits are 0)
+#pragma unroll 1
+                    for (int v = 0; v < kVrCluster; ++v) {
+                        uint32_t m = cluster.map_shared_rank(S.bm, v)[(4 * NWB + w) * NDp + j];
+                        m = (m >> (8 * (t & 3))) & 0xffu;
+                        for (; m; m &= m - 1u)
+                            reinterpret_cast<OutT *>(out)[((size_t)(r0 + __ffs(m) - 1) * ND + j) * G.n_phi0 +
+                                                          k0 + v] = (OutT)16;
                     }
                 }
             }

@@ -91,3 +91,21 @@ def test_few_rows_cost_no_more_than_the_plain_vote():
     """8 rows, 20k hits: about 0.4 of the plain vote (a lane per row and hits
     that cannot vote among the others' lanes made it over 1.3)."""
     assert layer_over_plain(geometry(8, 64, 512), 20000, range(10)) < 1.3
+
+
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("layers", [range(11), range(10, 16), [15], [9, 10], range(16)],
+                         ids=["11", "last6", "one", "both_sides", "16"])
+def test_layers_of_the_second_round(layers, bits):
+    """Layers past the ten that a tile holds at once: a second round of votes on
+    the first one's counts, up to 16 in a cell."""
+    o = check(geometry(70, 36, 16, bits), *hits(12000, layers, len(layers)))
+    if len(layers) == 16:
+        assert o.max() == 16
+
+
+def test_sixteen_layers_write_the_counts_once():
+    """300 hits, where writing the accumulator is most of the time: about 1.4
+    of the plain vote (over 1.8 when the second round read it back and wrote
+    it again)."""
+    assert layer_over_plain(geometry(256, 128, 512), 300, range(16)) < 1.8
