@@ -109,3 +109,16 @@ def test_sixteen_layers_write_the_counts_once():
     of the plain vote (over 1.8 when the second round read it back and wrote
     it again)."""
     assert layer_over_plain(geometry(256, 128, 512), 300, range(16)) < 1.8
+
+
+@pytest.mark.parametrize("nphi", [8, 16, 40])
+@pytest.mark.parametrize("nr", [64, 65, 256, 300])
+def test_few_columns(nr, nphi):
+    """Fewer tiles than SMs at the widest bands: narrower ones."""
+    check(geometry(nr, 40, nphi), *hits(700, range(10), nr))
+
+
+def test_few_columns_use_the_sms():
+    """8 columns of 256 rows, 20k hits: about a quarter of the plain vote (one
+    tile per column on 8 SMs took about 0.7 of it)."""
+    assert layer_over_plain(geometry(256, 128, 8), 20000, range(10)) < 0.45
