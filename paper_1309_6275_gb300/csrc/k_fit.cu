@@ -25,7 +25,8 @@
 // thread, its hits in turn, its hit selection kept as a bit mask, the sine
 // and cosine computed once per parameter vector; by eight lanes where the
 // candidates would not fill the GPU one to a thread (64 threads per SM: two
-// warps keep its float64 pipe busy).  Larger candidates take a warp each.
+// warps keep its float64 pipe busy), by sixteen where not even sixteen each do.
+// Larger candidates take a warp each.
 // GB300, 21,855 candidates of 7 to 10 hits, road, cut and eight steps: 3.67 ->
 // 0.265 ms.
 #include <cuda_runtime.h>
@@ -96,7 +97,7 @@ struct FitArgs {
     int n_phi0, min_hits, iters, iters2;
 };
 
-constexpr int kFitSmall = 32;       // hits of a candidate fitted by one thread or eight lanes
+constexpr int kFitSmall = 32;       // hits of a candidate fitted by one thread or some lanes
 constexpr int kFitThreads = 64;     // small blocks spread few candidates over the SMs
 
 // One candidate's hits as W consecutive lanes of a warp see them: lane sub
@@ -188,7 +189,7 @@ struct Fitter {
     // this one still steps).
     __device__ __forceinline__ bool steps(int iters, bool active)
     {
-        for (int it = 0; it < iters; ++it) {
+        for (int it = 0; it < iters && __any_sync(0xffffffffu, active); ++it) {
             double A[6], g[3], rr, L[6];
             normal_eq(A, g, rr);
             if (active && !chol3(A, L)) active = false;
@@ -347,9 +348,13 @@ k_fit_tracks(FitArgs F, const float *__restrict__ x, const float *__restrict__ y
              const int *__restrict__ n, int dense, ht_track *__restrict__ out)
 {
     const int small = n[0], big = n[1];
-    // a thread each where the candidates fill `dense` threads, else eight lanes
+    // a thread each where the candidates fill `dense` threads, else eight lanes,
+    // or sixteen where those fill no more: with so few a candidate's own latency
+    // counts (50 of 10, 20 and 32 hits 109, 120 and 132 -> 104, 114 and 115 us; a
+    // warp each 107, 107 and 108, but 3 and 6 hits 113 and 107 against 109 and 104)
     if (small >= dense) fit_list<1>(F, x, y, peaks, start, list, todo, 1, small, out);
-    else fit_list<8>(F, x, y, peaks, start, list, todo, 1, small, out);
+    else if (small > dense / 16) fit_list<8>(F, x, y, peaks, start, list, todo, 1, small, out);
+    else fit_list<16>(F, x, y, peaks, start, list, todo, 1, small, out);
     fit_list<32>(F, x, y, peaks, start, list, todo + ns - 1, -1, big, out);
 }
 
