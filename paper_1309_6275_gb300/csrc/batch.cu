@@ -34,7 +34,7 @@ namespace ht {
 cudaError_t launch_vote_batch(const DevGeom &G, const float *x, const float *y, const int *off,
                               const int *order, const int *d_nev, uint16_t *acc,
                               size_t acc_stride, unsigned long long *stats, int *head,
-                              const int *d_big, int *head_big, bool pack, int kt, int sms,
+                              const int *d_dense, int *head_dense, bool pack, int kt, int sms,
                               cudaStream_t st, const HitBuckets *hb);
 int assoc32_kt(const DevGeom &G);
 int assoc32_ntiles(const DevGeom &G, int kt);
@@ -58,7 +58,7 @@ cudaError_t prepare_batch_kernels(int max_smem);
 cudaError_t launch_vote_batch_masked(const DevGeom &G, const float *x, const float *y,
                                      const int *off, const int *order, const int *d_nev,
                                      uint16_t *acc, size_t acc_stride, unsigned long long *stats,
-                                     int *head, const int *d_big, int *head_big, bool pack,
+                                     int *head, const int *d_dense, int *head_dense, bool pack,
                                      int kt, int sms,
                                      const unsigned long long *masks, cudaStream_t st,
                                      const HitBuckets *hb);
@@ -69,8 +69,8 @@ cudaError_t launch_region_mask(const void *params_bf16, const float *x, const fl
 cudaError_t launch_vote_batch_hitmask(const DevGeom &G, const float *x, const float *y,
                                       const int *off, const int *order, const int *d_nev,
                                       uint16_t *acc, size_t acc_stride,
-                                      unsigned long long *stats, int *head, const int *d_big,
-                                      int *head_big, bool pack, int kt,
+                                      unsigned long long *stats, int *head, const int *d_dense,
+                                      int *head_dense, bool pack, int kt,
                                       int sms, const unsigned long long *hit_masks,
                                       cudaStream_t st, const HitBuckets *hb);
 cudaError_t launch_hit_masks(const void *params_bf16, const float *x, const float *y,
@@ -119,7 +119,8 @@ struct ht_batch {
     size_t slot_words;  // 32-bit words of an event's slot in acc
     uint16_t *acc;      // plain path: counts, cells apart; track path: bit planes
                         // and peak bits, slot_words apart
-    int *meta;          // [0] n_big [1] events of at least kCellHits hits [2] n_all [3] pad,
+    int *meta;          // [0] n_big [1] events of at least kCellHits hits [2] n_all
+                        // [3] events above cluster_hits hits,
                         // off[max_events + 1],
                         // order_big[max_events], order_all[max_events] (largest first),
                         // thr[max_events] (peak threshold of each event slot)
@@ -288,21 +289,22 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
     // vote: the tiles whose hit lists pass the packed-counter limit (only
     // events above it can have such tiles), then every other tile of every
     // event with packed counters
-    auto vote = [&](const int *order, const int *d_nev, int *head, const int *d_big,
-                    int *head_big, bool pack, int kt) {
+    auto vote = [&](const int *order, const int *d_nev, int *head, const int *d_dense,
+                    int *head_dense, bool pack, int kt) {
         if (R.hit_masks)
             return ht::launch_vote_batch_hitmask(G, x, y, off, order, d_nev, b->acc, b->cells,
-                                                 st64, head, d_big, head_big, pack, kt, b->sms,
+                                                 st64, head, d_dense, head_dense, pack, kt, b->sms,
                                                  R.hit_masks, st, &b->bk);
         return masks ? ht::launch_vote_batch_masked(G, x, y, off, order, d_nev, b->acc, b->cells,
-                                                    st64, head, d_big, head_big, pack, kt, b->sms,
-                                                    masks, st, &b->bk)
+                                                    st64, head, d_dense, head_dense, pack, kt,
+                                                    b->sms, masks, st, &b->bk)
                      : ht::launch_vote_batch(G, x, y, off, order, d_nev, b->acc, b->cells, st64,
-                                             head, d_big, head_big, pack, kt, b->sms, st, &b->bk);
+                                             head, d_dense, head_dense, pack, kt, b->sms, st,
+                                             &b->bk);
     };
     e = vote(order_big_of(meta, me), meta + 0, b->heads + 0, nullptr, nullptr, false, b->kt_big);
     if (e == cudaSuccess)
-        e = vote(order_all_of(meta, me), meta + 2, b->heads + 1, meta + 0, b->heads + 3, true,
+        e = vote(order_all_of(meta, me), meta + 2, b->heads + 1, meta + 3, b->heads + 3, true,
                  b->kt_pack);
     if (e == cudaSuccess) e = mark(2);
     if (e != cudaSuccess) return e;
@@ -332,7 +334,7 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
 }
 
 // Upload offsets and the largest-first event orders for this batch.
-ht_status stage_meta(ht_batch *b, const int32_t *h_off, int n_ev, cudaStream_t st)
+ht_status stage_meta(ht_batch *b, const int32_t *h_off, int n_ev, const Restrict &R, cudaStream_t st)
 {
     if (b->meta_pending) {
         cudaError_t e = cudaEventSynchronize(b->meta_done);
@@ -347,16 +349,19 @@ ht_status stage_meta(ht_batch *b, const int32_t *h_off, int n_ev, cudaStream_t s
     std::stable_sort(idx.begin(), idx.end(), [&](int a, int c) {
         return h_off[a + 1] - h_off[a] > h_off[c + 1] - h_off[c];
     });
-    int nb = 0, ncell = 0;
+    int nb = 0, ncell = 0, ndense = 0;
+    const int cluster = ht::cluster_hits(b->g->G, R.hit_masks != nullptr, R.masks != nullptr);
     for (int i = 0; i < n_ev; ++i) {
         const int ev = idx[i];
         if (h_off[ev + 1] - h_off[ev] >= ht::kCellHits) ++ncell;   // a prefix: largest first
+        if (h_off[ev + 1] - h_off[ev] > cluster) ++ndense;
         if (h_off[ev + 1] - h_off[ev] > ht::kPackMaxHits) order_big_of(hm, me)[nb++] = ev;
         order_all_of(hm, me)[i] = ev;
     }
     hm[0] = nb;
     hm[1] = ncell;
     hm[2] = n_ev;
+    hm[3] = ndense;
     // peak threshold of each event slot (track path): the first band holding
     // the event's hit count, else the geometry's threshold
     for (int ev = 0; ev < n_ev; ++ev) {
@@ -503,7 +508,7 @@ ht_status run_impl(ht_batch *b, const float *x, const float *y, const float *z,
     ht_status s = check_offsets(b, h_off, n_events);
     if (s != HT_OK) return s;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s = stage_meta(b, h_off, n_events, st);
+    s = stage_meta(b, h_off, n_events, R, st);
     if (s != HT_OK) return s;
     if (!b->use_graph) {
         cudaError_t e = enqueue(b, x, y, z, n_events, peaks, counts, assign, zres, stats, R, st,

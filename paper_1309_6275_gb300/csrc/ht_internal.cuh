@@ -345,6 +345,25 @@ constexpr int kGroupCols = 8;
 // Packed 16-bit tile counters are exact for tiles scanning up to this many
 // hits (two votes per hit at most in a cell: 2 * 32767 < 2^16).
 constexpr int kPackMaxHits = 32767;
+// Events of up to this many hits vote their plain tiles in clusters (tiles.cuh).
+// A cluster saves on the write-back, which grows with the bins, twice where
+// they halve the tile's columns (from 128), and waits for its slowest tile,
+// which grows with the hits; region sets per hit leave each fewer votes.  Vote
+// stage in clusters and single, 256 x 128 x 512 cells: 25 events of 400 hits
+// 1.34 and 1.46 ms, 1500 2.77 and 2.77, 3000 4.70 and 4.57, 4 of 30k 6.75 and
+// 6.24; 512 x 256 x 1024: two of 5000 4.02 and 4.25, of 20k 14.46 and 14.15.
+// With top-8 sets 25 of 400 1.60 and 2.04, 7000 7.14 and 7.20, 16 of 12k 7.33
+// and 7.16; two of 5000 2.95 and 3.15, of 20k 9.95 and 9.52.  Under an event's
+// region mask tiles end early or not and clusters wait: 25 of 400 1.22 and 1.10;
+// only narrow tiles gain, two of 1000 0.89 and 1.06, of 5000 2.19 and 2.23, of
+// 20k 7.04 and 6.85.
+inline int cluster_hits(const DevGeom &G, bool hit_sets, bool event_masks)
+{
+    const int nd = G.n_d0;   // 2 to 512
+    const int n = hit_sets ? 64 * nd : event_masks ? (nd > 128 ? 24 * nd : 0)
+                                                   : nd * (nd > 128 ? nd : 128) * 3 / 32;
+    return n < kPackMaxHits ? n : kPackMaxHits;   // (a cluster's tiles are all packed)
+}
 struct HitBuckets {
     int *cnt, *start, *cursor, *ent;
     int *hg;   // per hit: first group | group count << 16

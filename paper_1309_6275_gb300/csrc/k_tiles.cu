@@ -736,11 +736,11 @@ cudaError_t launch_associate(const DevGeom &G, const float *x, const float *y, i
 cudaError_t launch_vote_batch(const DevGeom &G, const float *x, const float *y, const int *off,
                               const int *order, const int *d_nev, uint16_t *acc,
                               size_t acc_stride, unsigned long long *stats, int *head,
-                              const int *d_big, int *head_big, bool pack, int kt, int sms,
+                              const int *d_dense, int *head_dense, bool pack, int kt, int sms,
                               cudaStream_t st, const HitBuckets *hb)
 {
     return launch_vote_batch_t<kModePlain>(G, x, y, off, order, d_nev, acc, acc_stride, stats,
-                                           head, d_big, head_big, pack, kt, sms, nullptr, st,
+                                           head, d_dense, head_dense, pack, kt, sms, nullptr, st,
                                            bucket_view(hb));
 }
 

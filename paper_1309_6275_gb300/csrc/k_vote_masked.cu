@@ -28,13 +28,13 @@ cudaError_t launch_vote_masked(const DevGeom &G, const float *x, const float *y,
 cudaError_t launch_vote_batch_masked(const DevGeom &G, const float *x, const float *y,
                                      const int *off, const int *order, const int *d_nev,
                                      uint16_t *acc, size_t acc_stride, unsigned long long *stats,
-                                     int *head, const int *d_big, int *head_big, bool pack,
+                                     int *head, const int *d_dense, int *head_dense, bool pack,
                                      int kt, int sms,
                                      const unsigned long long *masks, cudaStream_t st,
                                      const HitBuckets *hb)
 {
     return launch_vote_batch_t<kModeEvent>(G, x, y, off, order, d_nev, acc, acc_stride, stats,
-                                           head, d_big, head_big, pack, kt, sms, masks, st,
+                                           head, d_dense, head_dense, pack, kt, sms, masks, st,
                                            bucket_view(hb));
 }
 
@@ -48,13 +48,13 @@ cudaError_t launch_vote_hitmask(const DevGeom &G, const float *x, const float *y
 cudaError_t launch_vote_batch_hitmask(const DevGeom &G, const float *x, const float *y,
                                       const int *off, const int *order, const int *d_nev,
                                       uint16_t *acc, size_t acc_stride,
-                                      unsigned long long *stats, int *head, const int *d_big,
-                                      int *head_big, bool pack, int kt,
+                                      unsigned long long *stats, int *head, const int *d_dense,
+                                      int *head_dense, bool pack, int kt,
                                       int sms, const unsigned long long *hit_masks,
                                       cudaStream_t st, const HitBuckets *hb)
 {
     return launch_vote_batch_t<kModeHit>(G, x, y, off, order, d_nev, acc, acc_stride, stats,
-                                         head, d_big, head_big, pack, kt, sms, hit_masks, st,
+                                         head, d_dense, head_dense, pack, kt, sms, hit_masks, st,
                                          bucket_view(hb));
 }
 

@@ -859,8 +859,8 @@ k_vote(DevGeom G, const float *__restrict__ x, const float *__restrict__ y, int 
 // bk (optional, ent null for none): per-event hit lists by column group; a
 // tile scans its group's list instead of the whole event.
 // The events are order[0 .. *d_nev); with CL > 1 clusters of CL CTAs pop CL
-// neighbouring tiles at a time, which must all be packed: the first
-// *d_skip events, whose hit lists may pass the packed limit, are left out.
+// neighbouring tiles at a time, which must all be packed; the first *d_skip
+// events are left out.
 template <int KT, typename OutT, bool PACK, int MODE, int CL>
 __global__ void __launch_bounds__(kThreads, PACK ? 3 : 2)
 k_vote_batch(DevGeom G, const float *__restrict__ x, const float *__restrict__ y,
@@ -879,12 +879,14 @@ k_vote_batch(DevGeom G, const float *__restrict__ x, const float *__restrict__ y
         q = (int)cg::this_cluster().block_rank();
     }
     const int total = (*d_nev - skip) * ntiles;   // ntx is a multiple of CL
-    // the next item is popped before the barrier that ends the current one
+    // CL > 1: the next item is popped before the barrier that ends the current one
+    // (single tiles pop when they begin: kept across the tile, the second item
+    // costs registers; 188 bytes of spills and 16% of the vote under event masks)
     auto pop = [&](int slot) {
         if (q == 0 && threadIdx.x == 0) s_item[slot] = atomicAdd(head, CL);
     };
-    pop(0);
-    for (int slot = 0;; slot ^= 1) {
+    if constexpr (CL > 1) pop(0);
+    for (int slot = 0;;) {
         int item;
         if constexpr (CL > 1) {
             // (also ends the reads of this CTA's counters by the others)
@@ -892,8 +894,9 @@ k_vote_batch(DevGeom G, const float *__restrict__ x, const float *__restrict__ y
             cluster.sync();
             item = *cluster.map_shared_rank(&s_item[slot], 0) + q;
         } else {
+            pop(0);
             __syncthreads();
-            item = s_item[slot];
+            item = s_item[0];
         }
         if (item >= total) break;
         const int e = order[skip + item / ntiles], t = item % ntiles;
@@ -906,13 +909,14 @@ k_vote_batch(DevGeom G, const float *__restrict__ x, const float *__restrict__ y
         // count carries into its neighbour), unpacked counters the others:
         // the launches of a batch split every event's tiles between them by the
         // scanned list's length (uniform over the CTA, and with CL > 1 over the
-        // cluster: every list of these events is short enough).
+        // cluster: every list of its events is short enough).
         if (PACK == ((bk.ent ? nl : n) <= kPackMaxHits))
             vote_tile<KT, OutT, PACK, MODE, CL>(G, x + a, y + a, n, acc + (size_t)e * acc_stride,
                                                 stats ? stats + 2 * e : nullptr, t % ntx, t / ntx,
                                                 MODE == kModeEvent ? masks[e] : ~0ull,
                                                 MODE == kModeHit ? masks + a : nullptr, hl, nl);
-        pop(slot ^ 1);
+        if constexpr (CL > 1) pop(slot ^= 1);
+        else __syncthreads();
     }
     if constexpr (CL > 1) cg::this_cluster().sync();   // the first CTA's items are read
 }
@@ -1008,26 +1012,27 @@ cudaError_t launch_vote_batch_kt(const DevGeom &G, const float *x, const float *
 // kt selects the tile width (0 = default).  pack: this launch takes the
 // listed events' tiles that scan at most kPackMaxHits hits (a column group's
 // hit list with buckets, else the event) with 16-bit packed counters;
-// otherwise it takes their other tiles with 32-bit counters.  With d_big, the
-// first *d_big events of order[] are those of more than kPackMaxHits hits:
-// where the tiles divide into clusters, these events' tiles and the others'
-// take a launch each.  *head and *head_big must be zero.
+// otherwise it takes their other tiles with 32-bit counters.  With d_dense, the
+// first *d_dense events of order[] are those of more than cluster_hits hits:
+// where the tiles divide into clusters, these events' tiles (single) and the
+// others' (clusters) take a launch each.  *head and *head_dense must be zero.
 //
 // Clusters, measured on 25 events of 400 hits (256 x 128 x 512 cells, 0.84 GB of
 // counts, 4 columns a tile): 1294 us alone, 1130 us in clusters of 4 (32-byte
 // writes), 1302 us of 8: the wait for the slowest tile and the remote reads cost
 // more than the wider writes give.  Most of the rest is each tile's chain of
-// barriers (zero, phases 1 and 2, write) with 24 warps per SM.
+// barriers (zero, phases 1 and 2, write) with 24 warps per SM.  With more hits
+// the wait grows and the writes count less (cluster_hits).
 template <int MODE>
 cudaError_t launch_vote_batch_t(const DevGeom &G, const float *x, const float *y, const int *off,
                                 const int *order, const int *d_nev, uint16_t *acc,
                                 size_t acc_stride, unsigned long long *stats, int *head,
-                                const int *d_big, int *head_big, bool pack, int kt, int sms,
+                                const int *d_dense, int *head_dense, bool pack, int kt, int sms,
                                 const unsigned long long *masks, cudaStream_t st,
                                 BucketView bk = BucketView{})
 {
 #define HT_VB(KTV, PK, CL)                                                                    \
-    launch_vote_batch_kt<KTV, PK, MODE, CL>(G, x, y, off, order, d_nev, d_big, acc,           \
+    launch_vote_batch_kt<KTV, PK, MODE, CL>(G, x, y, off, order, d_nev, d_dense, acc,           \
                                             acc_stride, stats, head, sms, masks, st, bk)
     if (pack) {
         // the per-hit mode's larger items would drop a tuned width to two CTAs
@@ -1037,12 +1042,14 @@ cudaError_t launch_vote_batch_t(const DevGeom &G, const float *x, const float *y
                         : vote_smem<2>(G, true, MODE) <= kSmemBudget3 ? 2 : 1;
         if (kt == 4 && vote_smem<4>(G, true, MODE) > budget) kt = 2;
         if (kt >= 2 && vote_smem<2>(G, true, MODE) > budget) kt = 1;
-        if (d_big && kt >= 2 && (G.n_phi0 / kt) % kVoteCluster == 0) {
-            const cudaError_t e = kt == 4 ? HT_VB(4, true, kVoteCluster)
-                                          : HT_VB(2, true, kVoteCluster);
+        // (under event masks four-column tiles lose at any size)
+        constexpr int kWide = MODE == kModeEvent ? 2 : 4;
+        if (d_dense && (kt == 2 || kt == kWide) && (G.n_phi0 / kt) % kVoteCluster == 0) {
+            const cudaError_t e = kt == kWide ? HT_VB(kWide, true, kVoteCluster)
+                                              : HT_VB(2, true, kVoteCluster);
             if (e != cudaSuccess) return e;
-            d_nev = d_big;   // the packed tiles of the others
-            head = head_big;
+            d_nev = d_dense;   // the packed tiles of the others
+            head = head_dense;
         }
         if (kt == 4) return HT_VB(4, true, 1);
         return kt >= 2 ? HT_VB(2, true, 1) : HT_VB(1, true, 1);
@@ -1076,6 +1083,8 @@ template <int MODE>
 cudaError_t prepare_vote_kernels_t(int max_smem)
 {
     const void *fns[] = {
+        (const void *)k_vote_batch<MODE == kModeEvent ? 2 : 4, uint16_t, true, MODE, kVoteCluster>,
+        (const void *)k_vote_batch<2, uint16_t, true, MODE, kVoteCluster>,
         (const void *)k_vote<4, uint16_t, true, MODE>,
         (const void *)k_vote<2, uint16_t, true, MODE>,
         (const void *)k_vote<1, uint16_t, true, MODE>,
@@ -1086,8 +1095,6 @@ cudaError_t prepare_vote_kernels_t(int max_smem)
         (const void *)k_vote<4, int32_t, false, MODE>,
         (const void *)k_vote<2, int32_t, false, MODE>,
         (const void *)k_vote<1, int32_t, false, MODE>,
-        (const void *)k_vote_batch<4, uint16_t, true, MODE, kVoteCluster>,
-        (const void *)k_vote_batch<2, uint16_t, true, MODE, kVoteCluster>,
         (const void *)k_vote_batch<4, uint16_t, true, MODE, 1>,
         (const void *)k_vote_batch<2, uint16_t, true, MODE, 1>,
         (const void *)k_vote_batch<1, uint16_t, true, MODE, 1>,
