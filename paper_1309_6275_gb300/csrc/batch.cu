@@ -116,9 +116,10 @@ struct ht_batch {
     int max_events, max_hits, cap, sms;
     int kt_pack, kt_big, kt_assoc;
     size_t cells;
-    size_t slot_words;  // 32-bit words of an event's slot in acc
-    uint16_t *acc;      // plain path: counts, cells apart; track path: bit planes
-                        // and peak bits, slot_words apart
+    uint16_t *acc;      // plain path: counts, cells apart
+    size_t slot_words;  // track path: 32-bit words of an event's bit planes and peak bits
+    uint32_t *planes;   // where they lie: in acc where they fit, else planes_ws
+    void *planes_ws;
     int *meta;          // [0] n_big [1] events of at least kCellHits hits [2] n_all
                         // [3] events above cluster_hits hits,
                         // off[max_events + 1],
@@ -147,7 +148,8 @@ struct ht_batch {
     char *cf_ws;            // track path: confirmation scratch
     char *idx_ws;           // track path: the hit index (k_hitindex.cu)
     ht::HitIndex idx;
-    char *pp_ws;            // track path: peak finding's scratch
+    char *pp_ws;            // track path: peak finding's scratch, for pp_events at a time
+    int pp_events;
     struct HostPath {       // buffers of ht_batch_run_tracks_host (allocated on first use)
         float *x, *y, *z;
         uint8_t *layer;
@@ -195,6 +197,7 @@ void free_batch(ht_batch *b)
     cudaFree(b->cf_ws);
     cudaFree(b->idx_ws);
     cudaFree(b->pp_ws);
+    cudaFree(b->planes_ws);
     {
         ht_batch::HostPath &h = b->hp;
         void *bufs[] = {h.x, h.y, h.z, h.layer, h.hmasks, h.peaks, h.zres, h.counts, h.score,
@@ -260,15 +263,14 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
         // events at their staged thresholds, confirmation and final
         // assignment, z vote
         e = ht::launch_hit_index(x, y, R.layer, off, meta + 2, me, b->max_hits, b->idx, b->sms, st);
-        uint32_t *planes = reinterpret_cast<uint32_t *>(b->acc);
         if (e == cudaSuccess)
             e = ht::launch_vote_batch_layers(G, b->idx, off, order_all_of(meta, me), meta + 2,
-                                             meta + 1, planes, b->slot_words, st64, b->heads + 1,
-                                             b->sms, R.hit_masks, st);
+                                             meta + 1, b->planes, b->slot_words, st64,
+                                             b->heads + 1, b->sms, R.hit_masks, st);
         if (e == cudaSuccess) e = mark(2);
         if (e == cudaSuccess)
-            e = ht::launch_plane_peaks(G, planes, b->slot_words, b->idx.rmm, thr_of(meta, me),
-                                       n_ev, me, peaks, b->cap, counts, b->pp_ws, st);
+            e = ht::launch_plane_peaks(G, b->planes, b->slot_words, b->idx.rmm, thr_of(meta, me),
+                                       n_ev, b->pp_events, peaks, b->cap, counts, b->pp_ws, st);
         if (e == cudaSuccess) e = mark(3);
         const ht::ConfirmDev P{b->conf.pool, b->conf.min_layers, b->conf.n_layers, b->conf.tol};
         if (e == cudaSuccess)
@@ -430,8 +432,6 @@ ht_status ht_batch_create(const ht_geometry *g, int32_t max_events, int32_t max_
     b->kt_big = 0;
     b->kt_assoc = ht::assoc32_kt(G);
     b->cells = (size_t)G.n_rho * G.n_d0 * G.n_phi0;
-    b->slot_words = std::max((b->cells + 1) / 2,
-                             ht::layer_planes_words(G) + ht::plane_flag_words(G));
     b->meta_ints = 4 + (size_t)max_events + 1 + 3 * (size_t)max_events;
     b->pk_stride = ht::peaks_workspace_bytes(G) + ht::peaks_flag_bytes(G);
     b->ntiles = ht::assoc32_ntiles(G, 1);   // the most tiles any tile width gives
@@ -441,11 +441,10 @@ ht_status ht_batch_create(const ht_geometry *g, int32_t max_events, int32_t max_
     auto M = [&](void **p, size_t bytes) {
         if (e == cudaSuccess) e = cudaMalloc(p, bytes);
     };
-    M((void **)&b->acc, b->slot_words * 4 * max_events);
+    M((void **)&b->acc, b->cells * 2 * max_events);
     M((void **)&b->meta, b->meta_ints * 4);
     M((void **)&b->heads, 256);
     M((void **)&b->gbest, (size_t)max_hits * 8);
-    M((void **)&b->pk_ws, b->pk_stride * max_events);
     M((void **)&b->tcnt, tl);
     M((void **)&b->toff, tl);
     M((void **)&b->tcur, tl);
@@ -455,6 +454,12 @@ ht_status ht_batch_create(const ht_geometry *g, int32_t max_events, int32_t max_
     M((void **)&b->mass, (size_t)max_events * 64 * sizeof(float));
     M((void **)&b->bk_ws, ht::hit_bucket_bytes(G, max_events, max_hits));
     if (e == cudaSuccess) b->bk = ht::carve_hit_buckets(G, max_events, max_hits, b->bk_ws);
+    // the peak bits only save a second comparison: without room for them it is made
+    if (e == cudaSuccess && cudaMalloc((void **)&b->pk_ws, b->pk_stride * max_events) != cudaSuccess) {
+        cudaGetLastError();
+        b->pk_stride = ht::peaks_workspace_bytes(G);
+        M((void **)&b->pk_ws, b->pk_stride * max_events);
+    }
     if (e == cudaSuccess) e = cudaMallocHost((void **)&b->h_meta, b->meta_ints * 4);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->meta_done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
@@ -639,20 +644,35 @@ ht_status ht_batch_set_confirm(ht_batch *b, const ht_confirm_desc *c)
         b->meta_pending = false;
     }
     if (!b->cf_ws) {
+        const ht::DevGeom &G = b->g->G;
+        const size_t need = ht::layer_planes_words(G) + ht::plane_flag_words(G);
+        const bool fits = need <= b->cells / 2;   // (n_rho below 12: a word holds 32 rows)
+        b->slot_words = fits ? b->cells / 2 : need;
         cudaError_t e = cudaMalloc((void **)&b->cf_ws,
                                    ht::confirm_workspace_bytes(b->max_events, b->max_hits));
         if (e == cudaSuccess)
             e = cudaMalloc((void **)&b->idx_ws, ht::hit_index_bytes(b->max_events, b->max_hits));
-        if (e == cudaSuccess)
-            e = cudaMalloc((void **)&b->pp_ws, ht::plane_peaks_bytes(b->g->G, b->max_events));
-        if (e == cudaSuccess) b->idx = ht::carve_hit_index(b->max_events, b->max_hits, b->idx_ws);
+        if (e == cudaSuccess && !fits)
+            e = cudaMalloc(&b->planes_ws, b->slot_words * 4 * b->max_events);
+        // peak finding's scratch for all events at a time, or for as many as there is room
+        for (b->pp_events = b->max_events; e == cudaSuccess; b->pp_events /= 2) {
+            e = cudaMalloc((void **)&b->pp_ws, ht::plane_peaks_bytes(G, b->pp_events));
+            if (e == cudaSuccess) break;
+            cudaGetLastError();
+            if (b->pp_events > 1) e = cudaSuccess;
+        }
         if (e != cudaSuccess) {
+            cudaGetLastError();
             cudaFree(b->cf_ws);
             cudaFree(b->idx_ws);
+            cudaFree(b->planes_ws);
             cudaFree(b->pp_ws);
             b->cf_ws = b->idx_ws = b->pp_ws = nullptr;
+            b->planes_ws = nullptr;
             return ht::set_error(HT_ERR_CUDA, "ht_batch_set_confirm: allocation failed");
         }
+        b->idx = ht::carve_hit_index(b->max_events, b->max_hits, b->idx_ws);
+        b->planes = reinterpret_cast<uint32_t *>(fits ? (void *)b->acc : b->planes_ws);
     }
     b->conf = *c;
     b->conf_set = true;
