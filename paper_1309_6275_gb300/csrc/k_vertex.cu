@@ -54,7 +54,10 @@ struct VtxArgs {
 };
 
 constexpr int kVtxThreads = 256;
-constexpr int kVtxGroup = 32;     // events per peak launch that the workspace is sized for
+// Events per peak launch that the workspace is sized for, and the most that it
+// takes for them (a large accumulator's events fill the GPU by themselves).
+constexpr int kVtxGroup = 32;
+constexpr size_t kVtxBytes = 32u << 20;
 
 __global__ void __launch_bounds__(kVtxThreads)
 k_vertex_vote(VtxArgs A, const ht_peak *__restrict__ peaks, const int *__restrict__ counts,
@@ -144,6 +147,11 @@ __global__ void k_vertex_first(const ht_peak *__restrict__ peaks, const int *__r
 }
 
 size_t vtx_scratch(const DevGeom &P) { return peaks_workspace_bytes(P) + peaks_flag_bytes(P); }
+
+int vtx_group(const DevGeom &P)
+{
+    return (int)std::max((size_t)1, std::min((size_t)kVtxGroup, kVtxBytes / vtx_scratch(P)));
+}
 
 ht_status vfail(ht_status s, const char *msg) { return set_error(s, msg); }
 
@@ -237,7 +245,7 @@ size_t ht_vertex_accumulator_bytes(const ht_vertex *v)
 
 size_t ht_vertex_workspace_size(const ht_vertex *v)
 {
-    return v ? ht::kVtxGroup * ht::vtx_scratch(v->P) : 0;
+    return v ? ht::vtx_group(v->P) * ht::vtx_scratch(v->P) : 0;
 }
 
 ht_status ht_vertex_vote(const ht_vertex *v, const ht_peak *cands, const int32_t *d_count,

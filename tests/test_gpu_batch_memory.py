@@ -116,3 +116,17 @@ def test_a_batch_that_has_no_room_for_the_peak_bits():
         for k in ("peaks", "assign", "zres"):
             assert np.array_equal(a[k], b[k])
     G.close()
+
+
+@pytest.mark.parametrize("n_r,n_theta", [(32, 64), (500, 4096), (1024, 65536)])
+def test_a_vertex_workspace_stays_below_the_accumulators(n_r, n_theta):
+    """The peaks' scratch of several events at a time, at most 32 MB or one
+    event's (40 bytes per 256 cells), whatever the accumulator's size."""
+    import ctypes
+    from paper_1309_6275_gb300 import ht
+    G = ht.Geometry(geometry(16, 32, 64, 0.0114, 3))
+    V = ht.Vertex(G, dict(n_r=n_r, n_theta=n_theta, r_max=30.0, r_keep=1.0, threshold=3), 1, 16)
+    one = n_r * -(-n_theta // 256) * 40
+    assert V.ws.numel() <= max(32 * MB, 1.05 * one + 4096)
+    V.close()
+    G.close()
