@@ -206,9 +206,46 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-# Minimal float32 issue slots of one vote: b, rho*c, D (3 FMA/MUL), rsqrt,
-# sqrt(D), q, C, 1/q, d0, bin coordinate, floor, range test, shared atomic.
-OPS_PER_VOTE = 13
+# Minimal float32 issue slots of one run of votes (the rho rows of a column in
+# which a hit's root stays in one d0 bin): w = d + s, w^2 + c^2, its reciprocal,
+# the row coordinate, its floor, the run's two masks, their product, the word's
+# address, shared atomic.
+OPS_PER_RUN = 10
+
+
+def count_runs(g, x, y, columns=None):
+    """(votes, runs) of the hits in the given columns (all when None), by the
+    definition's float64 roots."""
+    nr, nd, nphi = g["n_rho"], g["n_d0"], g["n_phi0"]
+    k = np.arange(nphi) if columns is None else np.asarray(columns)
+    phi = (2 * k + 1 - nphi) * (np.pi / nphi)
+    rho = ((2 * np.arange(nr) + 1 - nr) * (g["rho_max"] / nr))[:, None]
+    delta, off = 2.0 * g["d0_half"] / nd, nd * 0.5 + 0.5
+    votes = runs = 0
+    for xh, yh in zip(np.asarray(x, np.float64), np.asarray(y, np.float64)):
+        s, c = xh * np.sin(phi) - yh * np.cos(phi), xh * np.cos(phi) + yh * np.sin(phi)
+        s, c = s[c > 0], c[c > 0]
+        b, D = 1.0 + rho * s, 1.0 - (rho * c) ** 2
+        with np.errstate(divide="ignore", invalid="ignore"):
+            q = -(b + np.where(b >= 0, 1.0, -1.0) * np.sqrt(D))
+            for root in (q / rho, (rho * (xh * xh + yh * yh) + 2.0 * s) / q):
+                u = np.where(D >= 0, root / delta + off, -1.0)
+                j = np.where((u >= 0) & (u < nd), np.floor(u), -1.0)
+                votes += int((j >= 0).sum())
+                runs += int(((j[1:] >= 0) & (j[1:] != j[:-1])).sum() + (j[0] >= 0).sum())
+    return votes, runs
+
+
+def runs_per_vote(g, events, hits=600, columns=64, seed=0):
+    """Runs per vote, from a random sample of the events' hits and columns."""
+    rng = np.random.default_rng(seed)
+    at = np.sort(rng.integers(0, sum(e.n_hits for e in events), hits))
+    first = np.cumsum([0] + [e.n_hits for e in events])
+    e = np.searchsorted(first, at, side="right") - 1
+    x, y = (np.array([getattr(events[a], q)[h - first[a]] for a, h in zip(e, at)]) for q in "xy")
+    k = rng.choice(g["n_phi0"], min(columns, g["n_phi0"]), replace=False)
+    votes, runs = count_runs(g, x, y, k)
+    return runs / max(votes, 1)
 
 
 def alu_peak_ops(dev_props, peaks):
@@ -459,7 +496,7 @@ def secondary_leg(args, ht, name, flush):
                        f"layers, pool {tk['pool']}, {tk['min_layers']} inlier layers within "
                        f"{tk['tol'] * 1e4:.0f} um",
            "stage_ms_per_event": {s: round(v / n, 4) for s, v in zip(STAGES, prof["stage_ms"])},
-           "vote_alu_frac": OPS_PER_VOTE * prof["votes"] / vote_s / peak_ops,
+           "vote_alu_frac": OPS_PER_RUN * runs_per_vote(g, evs) * prof["votes"] / vote_s / peak_ops,
            "candidates_per_event": prof["candidates_per_event"],
            "confirmed_per_event": prof["confirmed_per_event"],
            "quality": prof["quality"],
@@ -625,8 +662,8 @@ def kernel_sha():
 
 
 def launches_per_batch(ne, learned=False):
-    """Kernels of a batch whose events' peaks are found one event after
-    another, two passes and a 3-kernel scan each (5 per event)."""
+    """Kernels of a batch that finds its events' peaks one event after another,
+    two passes and a 3-kernel scan each; no path does now (track_launches)."""
     return 5 + 1 + 5 * ne + 15 + 7 + (1 if learned else 0)
 
 
@@ -730,7 +767,8 @@ def run_ours(args):
     roof = {"kernel": {1: "k_vote_rows_batch", 3: "k_confirm"}.get(dom, STAGES[dom]),
             "stage_ms_per_event": {s: round(1e3 * v / n_ev, 4) for s, v in zip(STAGES, stage_s)}}
     if dom == 1:
-        achieved = OPS_PER_VOTE * votes / stage_s[1]
+        rpv = runs_per_vote(g, events)
+        achieved = OPS_PER_RUN * rpv * votes / stage_s[1]
         prof = PROFILED_TRAFFIC.get("k_vote_rows_batch")
         from paper_1309_6275_gb300 import probe
         atom = probe.shared_atomic_rate(1 << 14)
@@ -740,8 +778,10 @@ def run_ours(args):
                                  if prof and prof["sha"] == kernel_sha() else None),
                      "peak_source": f"derived: {props.multi_processor_count} SMs x 128 FP32 "
                                     f"lanes x {peaks.get('sm_max_mhz', 2070.0):.0f} MHz "
-                                    f"(issue-limited), {OPS_PER_VOTE} algorithmic ops per vote",
-                     "shared_atomic_frac": (votes / stage_s[1]) / atom,
+                                    f"(issue-limited), {OPS_PER_RUN} algorithmic ops per run of votes "
+                                    f"(rows of a column in one bin; {rpv:.3f} runs per vote, "
+                                    "sampled)",
+                     "shared_atomic_frac": (rpv * votes / stage_s[1]) / atom,
                      "shared_atomic_peak_gops": atom / 1e9})
     else:
         roof.update({"bound": "alu", "achieved": None, "peak": peak_ops / 1e9, "unit": "Gop/s",
