@@ -92,26 +92,29 @@ def test_a_batch_that_has_no_room_for_the_peak_bits():
     cat = lambda k, t: to_dev(np.concatenate([getattr(e, k) for e in evs]).astype(t))
     hits = [cat(k, np.float32) for k in "xyz"] + [cat("layer", np.uint8)]
     G = ht.Geometry(g)
-    results = []
-    rest = None
-    for short in (False, True):
-        before = free()
-        if short:
-            rest = torch.empty(before - took + 130 * MB, dtype=torch.uint8, device="cuda")
+
+    def run():
         B = ht.Batch(G, max_events=4, max_hits=int(off[-1]), cap=1 << 12)
         B.set_confirm(CP)
-        if not short:
-            took = before - free()
+        took = before - free()
         out = []
         B.run(*hits[:3], off)
         out += [batch_event(B, off, e) for e in range(4)]
         B.run_tracks(*hits, off)
         out += [batch_event(B, off, e) for e in range(4)]
-        results.append(out)
         B.close()
+        return took, out
+
+    before = free()
+    took, full = run()
+    before = free()
+    rest = torch.empty(before - took + 130 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        short = run()[1]
+    finally:
         del rest
-        rest = None
-    for a, b in zip(*results):
+        torch.cuda.empty_cache()
+    for a, b in zip(full, short):
         assert a["count"] == b["count"] > 0 and a["votes"] == b["votes"]
         for k in ("peaks", "assign", "zres"):
             assert np.array_equal(a[k], b[k])
@@ -122,7 +125,6 @@ def test_a_batch_that_has_no_room_for_the_peak_bits():
 def test_a_vertex_workspace_stays_below_the_accumulators(n_r, n_theta):
     """The peaks' scratch of several events at a time, at most 32 MB or one
     event's (40 bytes per 256 cells), whatever the accumulator's size."""
-    import ctypes
     from paper_1309_6275_gb300 import ht
     G = ht.Geometry(geometry(16, 32, 64, 0.0114, 3))
     V = ht.Vertex(G, dict(n_r=n_r, n_theta=n_theta, r_max=30.0, r_keep=1.0, threshold=3), 1, 16)
