@@ -465,7 +465,7 @@ cudaError_t launch_hit_sort(const HitIndex &I, const int *order, const int *d_n,
                             cudaStream_t st);
 // Events of at least this many hits vote their dense layers cell by cell
 // (k_vote_rows.cu).
-constexpr int kCellHits = 24000;
+constexpr int kCellHits = 28000;
 
 // Candidate confirmation (k_confirm.cu): parameters as ht_confirm_desc.
 struct ConfirmDev {

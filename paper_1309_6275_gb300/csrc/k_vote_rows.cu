@@ -42,10 +42,12 @@
 // Why here: the tile kernel this replaces evaluated every (hit, row) of a
 // column (52.7 thread instructions per vote; 29.5 lanes) and built each (hit,
 // column) item three times, once per 64-row tile.  Of a 17k-hit event's 24.5k
-// votes per hit, 4.0k runs of rows remain.  Issue-bound now (76% of slots).
+// votes per hit, 5.0k runs of rows remain.  Issue-bound now (70% of the slots;
+// 19.8k warp instructions per 10k-hit event's hit, 27.8 lanes).
 // Vote stage with hit index, GB300, 25 events of 2k-60k hits (256 x 128 x 512
-// cells): 18.3 -> 8.5 ms; 25 of 10k: 11.2 -> 5.2; with top-8 region sets 14.6
-// -> 6.1; two of 50k (512 x 256 x 1024): 32.2 -> 17.7.
+// cells): 18.3 -> 8.6 ms; 25 of 10k: 11.2 -> 5.3; with top-8 region sets 14.6
+// -> 6.0; two of 50k (512 x 256 x 1024): 32.2 -> 17.8; the last two lines' dense
+// events cell by cell (below): 7.5 and 14.1.
 //
 // Constants, each measured on those batches: kEdgeSlope 0.5 (0.45 to 0.6
 // equal, 1.0 5% slower: a steep curve has fewer rows than bins); kWalkSlope
@@ -66,11 +68,13 @@
 // The number of votes telescopes: per row, the hits between the axis' ends.
 // A layer's rows where S is not monotone (tight curls) keep the hit-by-hit
 // vote, as do sparse layers (kCellMin: 160, 300 and 500 time alike), layers
-// whose radii spread, and smaller events: kCellHits = 24000 measured, for 25
-// events of 2k-60k hits on 256 x 128 x 512 cells, 7.49 ms (20000: 7.67, 16000:
-// 7.88, 12000: 8.25, none: 8.67), and for two of 50k hits on 512 x 256 x 1024 14.2 ms
-// instead of 18.1.  It is bound
-// by instructions (3.25 G for 6 events of 30k hits, the issue slots 75% busy).
+// whose radii spread, and smaller events.  kCellHits lies where the two cost the
+// same: 8 events on 256 x 128 x 512 cells, cell by cell and hit by hit, of 20k
+// hits 4.18 and 3.33 ms, 24k 4.30 and 3.91, 28k 4.41 and 4.55, 32k 4.53 and
+// 5.20, 60k 5.40 and 9.58; two on 512 x 256 x 1024, of 20k 9.50 and 7.52, 30k
+// 11.05 and 10.91, 50k 14.1 and 17.8.  (25 of 2k-60k hits: 12000 8.23 ms, 16000
+// 7.83, 20000 7.52, 24000 7.43, 28000 7.50, 32000 7.41, none 8.61.)  It is bound
+// by instructions (1.53 G for 3 events of 30k hits, the issue slots 69% busy).
 //
 // In the batch the hits come from the (layer, azimuth) index of
 // k_hitindex.cu: a column scans, per layer, the run of azimuth cells whose
