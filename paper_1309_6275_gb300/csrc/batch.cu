@@ -3,9 +3,9 @@
 // A batch of events runs as one CUDA graph, captured once per batch shape and
 // replayed: persistent vote and association kernels pop (event, tile) items
 // from device counters (events ordered largest first, so 2k- and 60k-hit
-// events share the GPU without per-event launch tails); peak finding and
-// candidate lists run per event slot; the (z0, cot theta) vote runs over all
-// candidates of the batch at once.  The vote and association tiles scan
+// events share the GPU without per-event launch tails); peak finding,
+// candidate lists and the (z0, cot theta) vote take all events of the batch at
+// once.  The vote and association tiles scan
 // per-event lists of the hits whose angular window meets their columns
 // (k_buckets.cu), built at the head of the vote stage.  Per-batch data (hit
 // offsets, event order) lives in device memory, uploaded from pinned staging

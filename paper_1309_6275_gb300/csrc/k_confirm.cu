@@ -35,8 +35,8 @@
 // definition's float64 distance, so the results are bit-identical to the
 // float64 plain definition.
 //
-// Bound by latency and issue (59% of slots; index loads and fixed latencies
-// lead the stalls): 1540 warp instructions per candidate, where scanning and
+// Bound by latency and issue (60% of slots; index loads and fixed latencies
+// lead the stalls): 1350 warp instructions per candidate, where scanning and
 // binning the whole pool (435 hits) with a frame per warp took 6800.  Stage on
 // GB300: 25 events of 2k-60k hits (1.25 M candidates) 11.7 -> 2.1 ms, 25 of 10k
 // hits (2.7 M) 16.7 -> 4.2, two of 50k (512 x 256 x 1024) 8.7 -> 1.5.
