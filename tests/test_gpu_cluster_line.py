@@ -94,4 +94,4 @@ def masked_over_plain():
 def test_event_masks_cost_little_over_the_plain_vote():
     """Masks of every region restrict nothing: 0.99 of the plain vote (1.04 in
     clusters, with registers spilled)."""
-    assert masked_over_plain() < 1.015
+    assert masked_over_plain() < 1.03
