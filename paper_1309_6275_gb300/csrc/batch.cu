@@ -336,7 +336,8 @@ cudaError_t enqueue(ht_batch *b, const float *x, const float *y, const float *z,
 }
 
 // Upload offsets and the largest-first event orders for this batch.
-ht_status stage_meta(ht_batch *b, const int32_t *h_off, int n_ev, const Restrict &R, cudaStream_t st)
+ht_status stage_meta(ht_batch *b, const int32_t *h_off, int n_ev, const Restrict &R,
+                     cudaStream_t st)
 {
     if (b->meta_pending) {
         cudaError_t e = cudaEventSynchronize(b->meta_done);
@@ -455,7 +456,8 @@ ht_status ht_batch_create(const ht_geometry *g, int32_t max_events, int32_t max_
     M((void **)&b->bk_ws, ht::hit_bucket_bytes(G, max_events, max_hits));
     if (e == cudaSuccess) b->bk = ht::carve_hit_buckets(G, max_events, max_hits, b->bk_ws);
     // the peak bits only save a second comparison: without room for them it is made
-    if (e == cudaSuccess && cudaMalloc((void **)&b->pk_ws, b->pk_stride * max_events) != cudaSuccess) {
+    if (e == cudaSuccess &&
+        cudaMalloc((void **)&b->pk_ws, b->pk_stride * max_events) != cudaSuccess) {
         cudaGetLastError();
         b->pk_stride = ht::peaks_workspace_bytes(G);
         M((void **)&b->pk_ws, b->pk_stride * max_events);

@@ -46,8 +46,8 @@
 // 19.8k warp instructions per 10k-hit event's hit, 27.8 lanes).
 // Vote stage with hit index, GB300, 25 events of 2k-60k hits (256 x 128 x 512
 // cells): 18.3 -> 8.6 ms; 25 of 10k: 11.2 -> 5.3; with top-8 region sets 14.6
-// -> 6.0; two of 50k (512 x 256 x 1024): 32.2 -> 17.8; the last two lines' dense
-// events cell by cell (below): 7.5 and 14.1.
+// -> 6.0; two of 50k (512 x 256 x 1024): 32.2 -> 17.8.  With dense layers cell by
+// cell (below) the first takes 7.5 and the last 14.1.
 //
 // Constants, each measured on those batches: kEdgeSlope 0.5 (0.45 to 0.6
 // equal, 1.0 5% slower: a steep curve has fewer rows than bins); kWalkSlope
@@ -110,7 +110,7 @@ constexpr float kEdgeSlope = 0.5f;    // and up to which a lane takes a bin
 constexpr float kWalkEps = 8.0f;      // rows of uncertainty at a crossing
 constexpr float kEdgeEps = 0.25f;     // (an edge lane's at most one row)
 constexpr size_t kVrBitmap = 43 * 1024;
-constexpr int kGather = 64;           // hits a warp of the single-event call looks at per step, at most
+constexpr int kGather = 64;           // hits a single event's warp looks at per step, at most
 constexpr int kClMaxHits = 4096;      // hits of a layer in a column's window, at most
 constexpr int kCellMin = 160;         // and at least, to go cell by cell
 constexpr int kClTab = 2048;          // table entries over a layer's s
@@ -448,7 +448,8 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
         if (l0 > 0 && !s_any) continue;   // uniform
         {
             uint4 *z4 = reinterpret_cast<uint4 *>(S.bm);
-            const int n4 = (!PLANES && l0 > 0 ? kKept : kRes) * NWB * NDp / 4;   // NDp is a multiple of 2, kRes NWB too
+            // (NDp is a multiple of 2, kRes and kKept too; the kept counts stay)
+            const int n4 = (!PLANES && l0 > 0 ? kKept : kRes) * NWB * NDp / 4;
             for (int t = threadIdx.x; t < n4; t += kThr) z4[t] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();
@@ -709,8 +710,9 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                         if (nrow < G.n_rho && keep[u] && c > 1.0f) {   // more than one band
                             float gmin, gmax;
                             rho_range(G, s, c, 4e-7f * R1, gmin, gmax);
-                            keep[u] = floorf(fmaf(gmin, G.inv_drho_f, tc - 0.5f)) <= (float)(nrow - 1) &&
-                                      ceilf(fmaf(gmax, G.inv_drho_f, tc + 0.5f)) >= 0.0f;
+                            const float fa = floorf(fmaf(gmin, G.inv_drho_f, tc - 0.5f));
+                            const float fb = ceilf(fmaf(gmax, G.inv_drho_f, tc + 0.5f));
+                            keep[u] = fa <= (float)(nrow - 1) && fb >= 0.0f;
                         }
                     }
 #pragma unroll
@@ -1230,9 +1232,10 @@ __device__ __forceinline__ void vr_tile(const DevGeom &G, const HitSource &H, in
                     for (int v = 0; v < kVrCluster; ++v) {
                         uint32_t m = cluster.map_shared_rank(S.bm, v)[(4 * NWB + w) * NDp + j];
                         m = (m >> (8 * (t & 3))) & 0xffu;
-                        for (; m; m &= m - 1u)
-                            reinterpret_cast<OutT *>(out)[((size_t)(r0 + __ffs(m) - 1) * ND + j) * G.n_phi0 +
-                                                          k0 + v] = (OutT)16;
+                        for (; m; m &= m - 1u) {
+                            const size_t cell = (size_t)(r0 + __ffs(m) - 1) * ND + j;
+                            reinterpret_cast<OutT *>(out)[cell * G.n_phi0 + k0 + v] = (OutT)16;
+                        }
                     }
                 }
             }
@@ -1278,21 +1281,22 @@ k_vote_rows_batch(DevGeom G, HitSource H, const int *__restrict__ off,
         const int item = s_item;
         if (item >= total) break;
         const int e = order[first + item / nt], t = item % nt;
-        vr_tile<NWB, HIT, true, CELLS, CELLS ? kClThreads : kVrThreads, uint16_t>(G, H, e, HIT ? masks + off[e] : nullptr,
-                                                 out + (size_t)e * out_stride,
-                                                 stats ? stats + 2 * e : nullptr, t % G.n_phi0,
-                                                 t / G.n_phi0);
+        vr_tile<NWB, HIT, true, CELLS, CELLS ? kClThreads : kVrThreads, uint16_t>(
+            G, H, e, HIT ? masks + off[e] : nullptr, out + (size_t)e * out_stride,
+            stats ? stats + 2 * e : nullptr, t % G.n_phi0, t / G.n_phi0);
     }
 }
 
 // One event (hits in the caller's order), one CTA per tile, clusters of
 // neighbouring columns (n_phi0 is a multiple of 8).
 template <int NWB, int kThr, typename OutT>
-__global__ void __cluster_dims__(kVrCluster, 1, 1) __launch_bounds__(kThr, kThr == kVrNarrow ? 4 : 3)
+__global__ void __cluster_dims__(kVrCluster, 1, 1)
+__launch_bounds__(kThr, kThr == kVrNarrow ? 4 : 3)
 k_vote_rows(DevGeom G, HitSource H, OutT *__restrict__ acc,
             unsigned long long *__restrict__ stats)
 {
-    vr_tile<NWB, false, false, false, kThr, OutT>(G, H, 0, nullptr, acc, stats, blockIdx.x, blockIdx.y);
+    vr_tile<NWB, false, false, false, kThr, OutT>(G, H, 0, nullptr, acc, stats, blockIdx.x,
+                                                  blockIdx.y);
 }
 
 }  // namespace
